@@ -2,6 +2,7 @@
 // systems for each implicit weight, and the order of kernel launches for the
 // multistep (Eq. multistep1) and diagonally implicit (Eq. dirks) schemes of
 // Section 4 of Gastine, pizza, GJI 2019.
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -73,6 +74,23 @@ std::vector<double2> fft_twiddles(int L) {
     for (int j = 0; j < L; ++j) {
         long double a = 2.0L * pi * (long double)j / (long double)L;
         t[j] = make_double2((double)cosl(a), (double)(-sinl(a)));
+    }
+    return t;
+}
+
+std::vector<int4> fft_twiddles_fx(int L) {
+    std::vector<int4> t(L);
+    const long double pi = 3.141592653589793238462643383279502884L;
+    auto split = [](long double c, int& hi, int& lo) {
+        const long long v = llroundl(c * 4611686018427387904.0L);
+        lo = (int)(unsigned)(unsigned long long)v;
+        hi = (int)((v - lo) >> 32);
+        if (lo == INT_MIN) ++lo;  // the kernels negate both words
+    };
+    for (int j = 0; j < L; ++j) {
+        const long double a = 2.0L * pi * (long double)j / (long double)L;
+        split(cosl(a), t[j].x, t[j].y);
+        split(-sinl(a), t[j].z, t[j].w);
     }
     return t;
 }
@@ -1504,30 +1522,6 @@ int pizza_init(pizza_ctx** out, int n_r, int n_phi, double E, double Ra, double 
         P.s_f = fs;
         P.h2_f = fh;
         P.inv_s_f = fi;
-        // double-float copies: hi the nearest float, lo the float nearest the rest
-        std::vector<float2> sd(n_r), hd(n_r), idd(n_r);
-        auto split = [](double v) {
-            const float h = (float)v;
-            return make_float2(h, (float)(v - (double)h));
-        };
-        for (int k = 0; k < n_r; ++k) {
-            sd[k] = split(s[k]);
-            hd[k] = split(h2[k]);
-            idd[k] = split(is[k]);
-        }
-        float2* ds2 = dalloc<float2>(ctx, n_r, al);
-        float2* dh2 = dalloc<float2>(ctx, n_r, al);
-        float2* di2 = dalloc<float2>(ctx, n_r, al);
-        if (!ds2 || !dh2 || !di2) {
-            ctx->err = "device allocation failed";
-            return bail(PIZZA_ENOMEM);
-        }
-        up(ds2, sd.data(), n_r * 8);
-        up(dh2, hd.data(), n_r * 8);
-        up(di2, idd.data(), n_r * 8);
-        P.s_dd = ds2;
-        P.h2_dd = dh2;
-        P.inv_s_dd = di2;
     }
 
     if (!make_fft_plan(2 * ctx->K, P.plan_r) || !make_fft_plan(n_phi, P.plan_p)) {
@@ -1546,6 +1540,19 @@ int pizza_init(pizza_ctx** out, int n_r, int n_phi, double E, double Ra, double 
     P.plan_r.tw = dtwr;
     P.plan_p.tw = dtwp;
     {
+        const auto fr = fft_twiddles_fx(2 * ctx->K), fp = fft_twiddles_fx(n_phi);
+        int4* dfr = dalloc<int4>(ctx, fr.size(), al);
+        int4* dfp = dalloc<int4>(ctx, fp.size(), al);
+        if (!dfr || !dfp) {
+            ctx->err = "device allocation failed";
+            return bail(PIZZA_ENOMEM);
+        }
+        up(dfr, fr.data(), fr.size() * sizeof(int4));
+        up(dfp, fp.data(), fp.size() * sizeof(int4));
+        P.fx_r = dfr;
+        P.fx_p = dfp;
+    }
+    {
         // the same twiddles rounded to FP32 for the mixed-precision explicit stage
         std::vector<float2> fr(twr.size()), fp(twp.size());
         for (size_t i = 0; i < twr.size(); ++i) fr[i] = make_float2((float)twr[i].x, (float)twr[i].y);
@@ -1561,25 +1568,7 @@ int pizza_init(pizza_ctx** out, int n_r, int n_phi, double E, double Ra, double 
         P.plan_r.twf = ftr;
         P.plan_p.twf = ftp;
     }
-    {
-        // the azimuthal twiddles as double-float pairs for the double-float products
-        std::vector<float4> dd(n_phi);
-        const long double pi = 3.141592653589793238462643383279502884L;
-        for (int j = 0; j < n_phi; ++j) {
-            const long double a = 2.0L * pi * (long double)j / (long double)n_phi;
-            const long double c = cosl(a), sn = -sinl(a);
-            const float ch = (float)c, sh = (float)sn;
-            dd[j] = make_float4(ch, (float)(c - (long double)ch), sh, (float)(sn - (long double)sh));
-        }
-        float4* dtw = dalloc<float4>(ctx, dd.size(), al);
-        if (!dtw) {
-            ctx->err = "device allocation failed";
-            return bail(PIZZA_ENOMEM);
-        }
-        up(dtw, dd.data(), dd.size() * sizeof(float4));
-        P.plan_p.twdd = dtw;
-        P.phi_dd = 1;
-    }
+    P.phi_dd = 1;
     P.solve_roles = -1;
     P.radial_lean = -1;
     P.psi_dd = -1;
@@ -1591,26 +1580,6 @@ int pizza_init(pizza_ctx** out, int n_r, int n_phi, double E, double Ra, double 
     P.plan_h.tw = P.plan_r.tw;
     P.plan_h.twf = P.plan_r.twf;
     P.plan_h.tws = 2;
-    {
-        // the radial twiddles as double-float pairs (double-float lean transforms)
-        const int L = 2 * ctx->K;
-        std::vector<float4> dd(L);
-        const long double pi = 3.141592653589793238462643383279502884L;
-        for (int j = 0; j < L; ++j) {
-            const long double a = 2.0L * pi * (long double)j / (long double)L;
-            const long double c = cosl(a), sn = -sinl(a);
-            const float ch = (float)c, sh = (float)sn;
-            dd[j] = make_float4(ch, (float)(c - (long double)ch), sh, (float)(sn - (long double)sh));
-        }
-        float4* dtw = dalloc<float4>(ctx, dd.size(), al);
-        if (!dtw) {
-            ctx->err = "device allocation failed";
-            return bail(PIZZA_ENOMEM);
-        }
-        up(dtw, dd.data(), dd.size() * sizeof(float4));
-        P.plan_r.twdd = dtw;
-        P.plan_h.twdd = dtw;
-    }
     P.radial_dd = -1;
 
     // m-independent banded operators and tau rows

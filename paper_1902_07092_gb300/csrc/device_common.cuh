@@ -64,31 +64,15 @@ struct Cx<float2> {
     __device__ static float2 from(double2 a) { return make_float2((float)a.x, (float)a.y); }
     __device__ static const float2* tw(const FftPlan& p) { return p.twf; }
 };
-template <>
-struct Cx<ddc> {
-    using R = ddf;
-    __device__ static ddc make(double a, double b) { return ddc{dd_from(a), dd_from(b)}; }
-    __device__ static ddc from(double2 a) { return dd_from(a); }
-    __device__ static const ddc* tw(const FftPlan& p) { return reinterpret_cast<const ddc*>(p.twdd); }
-};
 // a real constant in the real type of a complex type
 template <class RT>
 __device__ __forceinline__ RT rconst(double c) {
     return (RT)c;
 }
-template <>
-__device__ __forceinline__ ddf rconst<ddf>(double c) {
-    return dd_from(c);
-}
 // twiddle load through the read-only cache
 template <class T>
 __device__ __forceinline__ T ldg_tw(const T* p) {
     return __ldg(p);
-}
-template <>
-__device__ __forceinline__ ddc ldg_tw<ddc>(const ddc* p) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-    return ddc{ddf{v.x, v.y}, ddf{v.z, v.w}};
 }
 // radial tables in the precision of the complex type
 template <class T>
@@ -257,15 +241,15 @@ __device__ __forceinline__ void stockham_pass(const T* __restrict__ src, T* __re
 // Batched FFT of nb transforms stored contiguously in buf0 (each length pl.L);
 // buf1 is scratch of the same size.  Ends with __syncthreads(); returns the buffer
 // holding the result.
-template <int SIGN, class T, bool R8 = false>
+template <int SIGN, class T>
 __device__ __forceinline__ T* fft_batched(T* buf0, T* buf1, const FftPlan& pl, int nb) {
     T* a = buf0;
     T* b = buf1;
     int Ns = 1;
     const int tid = threadIdx.x, nth = blockDim.x;
     const T* tw = Cx<T>::tw(pl);
-    // FP32 (and R8 callers): the radix-8 factorisation, fewer passes
-    constexpr bool f32 = R8 || sizeof(typename Cx<T>::R) == sizeof(float);
+    // FP32: the radix-8 factorisation, fewer passes
+    constexpr bool f32 = sizeof(typename Cx<T>::R) == sizeof(float);
     const int npass = f32 ? pl.npass8 : pl.npass;
     __syncthreads();
     for (int p = 0; p < npass; ++p) {

@@ -11,7 +11,10 @@
 //   e       [M][nc] integrated explicit right-hand sides
 // The change from mode-major to radius-major order (the paper's MPI transpose)
 // is folded into the stores of spec_to_grid and the loads of grid_to_spec.
+#include <algorithm>
+
 #include "device_common.cuh"
+#include "fixfft.cuh"
 
 namespace pz {
 
@@ -23,17 +26,25 @@ constexpr int MAXPER = 12;       // azimuthal points per thread held in register
 __device__ __forceinline__ int g_index(int k, int f, int m, int M) { return (k * 4 + f) * M + m; }
 
 // number of radial transforms batched together in shared memory (the
-// autotuner's choice, else up to n_r = 513 four in FP64 -- all four synthesised
-// fields of a mode in one pass -- and two in FP32, measured fastest at n_r = 257)
+// autotuner's choice, else four in FP64 up to n_r = 257 -- all four synthesised
+// fields of a mode in one pass -- and two in FP32 and at n_r = 513: measured
+// fastest at n_r = 257 and, 99 against 107 us for a1 at 513 x 1536, at 513)
 __host__ __device__ inline int radial_batch(const StepParams& P) {
     if (P.nb_r > 0) return P.nb_r;
     if (2 * P.K > 1024) return 1;
-    return P.fp32 ? 2 : 4;
+    return (P.fp32 || P.K > 256) ? 2 : 4;
 }
 // threads of the per-radius azimuthal kernels
 inline int phi_threads(const StepParams& P) {
     if (P.phi_threads > 0) return P.phi_threads;
     return P.n_phi > 256 * MAXPER ? 512 : 256;
+}
+
+// of the fixed-point one: a divisor of the n_phi/2 radix-4 butterflies of a pass over
+// both pairs (96 2^j of them), at most 384 (two CTAs share an SM's registers)
+inline int phi_threads_fx(const StepParams& P) {
+    if (P.phi_threads > 0 || P.n_phi > 256 * MAXPER) return phi_threads(P);
+    return P.n_phi >= 768 ? 384 : 192;
 }
 
 // ---------------------------------------------------------------------------
@@ -264,8 +275,6 @@ __device__ __forceinline__ double re_abs(float2 z) { return fabs((double)z.x); }
 __device__ __forceinline__ double im_abs(float2 z) { return fabs((double)z.y); }
 __device__ __forceinline__ double re_abs(double2 z) { return fabs(z.x); }
 __device__ __forceinline__ double im_abs(double2 z) { return fabs(z.y); }
-__device__ __forceinline__ double re_abs(ddc z) { return fabs(dd_to(z.x)); }
-__device__ __forceinline__ double im_abs(ddc z) { return fabs(dd_to(z.y)); }
 
 template <class T>
 __device__ void cfl_rates(const StepParams& P, const T* R, int Pn, double l1, int k, double* red) {
@@ -374,202 +383,6 @@ __global__ void __launch_bounds__(512, 1) k_phi_products(StepParams P, const T* 
     S = fft_batched<-1>(X, Y, P.plan_p, 1);
     // g1 Im(g2) = l2 (v theta + i l1 u_phi theta)
     store_split_spectrum(S, G2 + g_index(k, 2, 0, M), M, Pn, n_m, iP * P2<T>::v(-e2), iP * P2<T>::v(-e1 - e2));
-}
-
-// ---------------------------------------------------------------------------
-// K2 of the FP64 stage in double-float arithmetic (ddfloat.cuh): the FP64
-// spectra are split into float pairs on load, the transforms and products run
-// on the FP32 pipe with ~48-bit significands, and the product spectra are
-// rounded back to FP64 on store.  The same steps as k_phi_products; the packed
-// pairs are balanced within float range (|exponent difference| <= 40).
-// The m = 0 modes of the products are taken in FP64 from the input spectra
-// instead: with band-limited fields (2 n_m < n_phi, no aliasing) the mean of
-// a b is a_0 b_0 + 2 sum_{m >= 1} Re(a_m conj(b_m)).  These means (the zonal
-// forcing [v omega]_0 above all) cancel to ~1e-4 of their terms, which would
-// magnify the double-float rounding beyond FP64 accuracy.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void load_packed_spectrum_dd(ddc* Z, const double2* __restrict__ src, int M, int Pn,
-                                                        int n_m, float sb) {
-    // each spectral value converted once, written to m and to its mirror Pn - m
-    for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
-        if (m == 0) {
-            Z[0] = ddc{dd_from_bits(src[0].x), dd_scale2(dd_from_bits(src[M].x), sb)};
-            continue;
-        }
-        const ddc a = dd_from_bits(src[m]);
-        ddc b = dd_from_bits(src[M + m]);
-        b.x = dd_scale2(b.x, sb);
-        b.y = dd_scale2(b.y, sb);
-        Z[m] = ddc{a.x - b.y, a.y + b.x};        // a + i b
-        Z[Pn - m] = ddc{a.x + b.y, b.x - a.y};   // conj(a) + i conj(b)
-    }
-    for (int j = n_m + 1 + threadIdx.x; j < Pn - n_m; j += blockDim.x) Z[j] = ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}};
-}
-
-__device__ __forceinline__ void store_split_spectrum_dd(const ddc* Y, double2* __restrict__ dst, int M, int Pn,
-                                                        int n_m, ddf ia, ddf ib) {
-    for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
-        ddc a, b;
-        if (m == 0) {
-            a = ddc{Y[0].x * ia, ddf{0.f, 0.f}};
-            b = ddc{Y[0].y * ib, ddf{0.f, 0.f}};
-        } else {
-            const ddc y1 = Y[m], y2 = Y[Pn - m];
-            // a = (y1 + conj(y2))/2,  b = (y1 - conj(y2))/(2i)
-            a.x = dd_scale2(y1.x + y2.x, 0.5f) * ia;
-            a.y = dd_scale2(y1.y - y2.y, 0.5f) * ia;
-            b.x = dd_scale2(y1.y + y2.y, 0.5f) * ib;
-            b.y = -(dd_scale2(y1.x - y2.x, 0.5f) * ib);
-        }
-        dst[m] = dd_compose(a);
-        dst[M + m] = dd_compose(b);
-    }
-}
-
-// |x| as the high word of its bits (monotone in |x|: its biased exponent and
-// leading fraction bits), on the integer pipe
-__device__ __forceinline__ unsigned hi_word_abs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-// the power of two a / b rounded down to exponents, from the high words of a and b,
-// clamped to [-lim, lim]; 0 where either is zero or subnormal
-__device__ __forceinline__ int pow2_exponent_words(unsigned wa, unsigned wb, int lim) {
-    const int ea = (int)(wa >> 20), eb = (int)(wb >> 20);
-    if (ea == 0 || eb == 0) return 0;
-    return max(-lim, min(lim, ea - eb));
-}
-
-__global__ void __launch_bounds__(512, 1) k_phi_products_dd(StepParams P, const double2* __restrict__ G1,
-                                                            double2* __restrict__ G2, int pair) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    ddc* sm = reinterpret_cast<ddc*>(smraw);
-    const int k = P.k_lo + blockIdx.x;
-    const int Pn = P.n_phi, M = P.M, n_m = P.n_m;
-    ddc* X = sm;
-    ddc* Y = sm + Pn;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    ddc reg[MAXPER];
-    __shared__ double red[4 * 32];
-    const ddf iP = dd_from(P.inv_nphi);  // 1/n_phi
-    // One pass over the four fields (v, u_phi, omega, theta):
-    // * the FP64 means of the four products, pairs (v, omega), (u_phi, omega),
-    //   (v, theta), (u_phi, theta): a_0 b_0 + 2 sum_{m >= 1} Re(a_m conj(b_m)), with
-    //   the real parts only at m = 0 (the transforms read no more of mode 0);
-    // * the largest biased exponent of |Re|, |Im| of each field, from the high
-    //   words on the integer pipe: the powers of two that balance the packed pairs.
-    __shared__ double msum[4][16];
-    __shared__ unsigned wmx[4][16];
-    {
-        double acc[4] = {0.0, 0.0, 0.0, 0.0}, a0[4] = {0.0, 0.0, 0.0, 0.0};
-        unsigned hx[4] = {0u, 0u, 0u, 0u};
-        const double2* f = G1 + g_index(k, 0, 0, M);  // f[q * M + m]: v, u_phi, omega, theta
-        for (int m = tid; m <= n_m; m += nth) {
-            const double2 v = f[m], up = f[M + m], om = f[2 * M + m], th = f[3 * M + m];
-            hx[0] = max(hx[0], max(hi_word_abs(v.x), hi_word_abs(v.y)));
-            hx[1] = max(hx[1], max(hi_word_abs(up.x), hi_word_abs(up.y)));
-            hx[2] = max(hx[2], max(hi_word_abs(om.x), hi_word_abs(om.y)));
-            hx[3] = max(hx[3], max(hi_word_abs(th.x), hi_word_abs(th.y)));
-            if (m == 0) {
-                a0[0] = v.x * om.x;
-                a0[1] = up.x * om.x;
-                a0[2] = v.x * th.x;
-                a0[3] = up.x * th.x;
-            } else {
-                acc[0] = fma(v.x, om.x, fma(v.y, om.y, acc[0]));
-                acc[1] = fma(up.x, om.x, fma(up.y, om.y, acc[1]));
-                acc[2] = fma(v.x, th.x, fma(v.y, th.y, acc[2]));
-                acc[3] = fma(up.x, th.x, fma(up.y, th.y, acc[3]));
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            acc[q] = fma(2.0, acc[q], a0[q]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-            hx[q] = __reduce_max_sync(0xffffffffu, hx[q]);
-        }
-        if ((tid & 31) == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                msum[q][tid >> 5] = acc[q];
-                wmx[q][tid >> 5] = hx[q];
-            }
-    }
-    __syncthreads();
-    int e1, e2;
-    {
-        unsigned w[4] = {0u, 0u, 0u, 0u};
-        for (int i = 0; i < (nth >> 5); ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) w[q] = max(w[q], wmx[q][i]);
-        e1 = pow2_exponent_words(w[0], w[1], 40);
-        e2 = pow2_exponent_words(w[2], w[3], 40);
-    }
-
-    if (pair) {
-        // both packed pairs in one batched transform each way (X, Y hold 2 Pn):
-        // half the barrier-separated passes, the same arithmetic per transform
-        Y = X + 2 * Pn;
-        load_packed_spectrum_dd(X, G1 + g_index(k, 0, 0, M), M, Pn, n_m, pow2f(e1));
-        load_packed_spectrum_dd(X + Pn, G1 + g_index(k, 2, 0, M), M, Pn, n_m, pow2f(e2));
-        ddc* R = fft_batched<+1, ddc, true>(X, Y, P.plan_p, 2);
-        if (P.cfl_max) cfl_rates(P, R, Pn, (double)pow2f(e1), k, red);
-        ddc* O = (R == X) ? Y : X;
-        for (int j = tid; j < Pn; j += nth) {
-            const ddc g1 = R[j], g2 = R[Pn + j];
-            O[j] = cscale(g1, g2.x);
-            O[Pn + j] = cscale(g1, g2.y);
-        }
-        ddc* S = fft_batched<-1, ddc, true>(O, R, P.plan_p, 2);
-        store_split_spectrum_dd(S, G2 + g_index(k, 0, 0, M), M, Pn, n_m, iP, dd_scale2(iP, pow2f(-e1)));
-        store_split_spectrum_dd(S + Pn, G2 + g_index(k, 2, 0, M), M, Pn, n_m, dd_scale2(iP, pow2f(-e2)),
-                                dd_scale2(dd_scale2(iP, pow2f(-e1)), pow2f(-e2)));
-        __syncthreads();  // the stores above are done (thread 0 wrote the m = 0 entries replaced here)
-        if (tid < 4) {
-            double t = 0.0;
-            for (int w = 0; w < (nth >> 5); ++w) t += msum[tid][w];
-            G2[g_index(k, tid, 0, M)] = make_double2(t, 0.0);
-        }
-        return;
-    }
-    load_packed_spectrum_dd(X, G1 + g_index(k, 0, 0, M), M, Pn, n_m, pow2f(e1));
-    ddc* R = fft_batched<+1, ddc, true>(X, Y, P.plan_p, 1);
-    if (P.cfl_max) cfl_rates(P, R, Pn, (double)pow2f(e1), k, red);
-#pragma unroll
-    for (int i = 0; i < MAXPER; ++i) {
-        const int j = tid + i * nth;
-        if (j < Pn) reg[i] = R[j];
-    }
-    __syncthreads();
-    load_packed_spectrum_dd(X, G1 + g_index(k, 2, 0, M), M, Pn, n_m, pow2f(e2));
-    R = fft_batched<+1, ddc, true>(X, Y, P.plan_p, 1);
-#pragma unroll
-    for (int i = 0; i < MAXPER; ++i) {
-        const int j = tid + i * nth;
-        if (j < Pn) {
-            const ddc g2 = R[j], g1 = reg[i];
-            R[j] = cscale(g1, g2.x);
-            reg[i] = cscale(g1, g2.y);
-        }
-    }
-    ddc* other = (R == X) ? Y : X;
-    ddc* S = fft_batched<-1, ddc, true>(R, other, P.plan_p, 1);
-    // g1 Re(g2) = v omega + i l1 u_phi omega
-    store_split_spectrum_dd(S, G2 + g_index(k, 0, 0, M), M, Pn, n_m, iP, dd_scale2(iP, pow2f(-e1)));
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < MAXPER; ++i) {
-        const int j = tid + i * nth;
-        if (j < Pn) X[j] = reg[i];
-    }
-    S = fft_batched<-1, ddc, true>(X, Y, P.plan_p, 1);
-    // g1 Im(g2) = l2 (v theta + i l1 u_phi theta)
-    store_split_spectrum_dd(S, G2 + g_index(k, 2, 0, M), M, Pn, n_m, dd_scale2(iP, pow2f(-e2)),
-                            dd_scale2(dd_scale2(iP, pow2f(-e1)), pow2f(-e2)));
-    __syncthreads();  // the stores above are done (thread 0 wrote the m = 0 entries replaced here)
-    if (tid < 4) {
-        double t = 0.0;
-        for (int w = 0; w < (nth >> 5); ++w) t += msum[tid][w];
-        G2[g_index(k, tid, 0, M)] = make_double2(t, 0.0);  // G2 fields follow the pair order
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -735,6 +548,700 @@ __global__ void __launch_bounds__(NTHREADS_R) k_grid_to_spec(StepParams P, const
 }
 
 // ---------------------------------------------------------------------------
+// Radial DCT-I in fixed point (fixfft.cuh), the FP64 stage's transform: the even
+// extension of K + 1 FP64 values as 64-bit integers, one complex transform of
+// length 2K for each vector, the outputs back in FP64.
+//
+// A vector's components are normalised separately by the exponents of their
+// largest magnitudes; FxScale keeps the exponents and the transforms' schedules of
+// up to FX_VEC vectors of a kernel.  The work around the transforms is split by
+// component (task t: entry t/2, part t & 1): an FP64 instruction of a warp takes
+// 64 cycles, so twice the warps with half the instructions each is twice as fast
+// until all four sub-partitions issue FP64 without a pause.
+// ---------------------------------------------------------------------------
+constexpr int FX_VEC = 6;
+constexpr int FX_L1 = 43;  // 1-norms are summed in units of 2^FX_L1 (up to 2^13 points)
+struct FxScale {
+    unsigned e[FX_VEC][2];  // biased exponent of the largest |re|, |im|
+    unsigned l1[FX_VEC];    // 1-norm of the extension in units of 2^FX_L1
+    unsigned back[FX_VEC];  // fx_schedule
+    int S[FX_VEC];
+};
+// threads of the fixed-point radial kernels: every (entry, part) at once, at
+// least eight warps (the derivative scans' roles)
+constexpr int NTHREADS_FX = 544;
+inline int fx_threads(const StepParams& P) { return std::max(256, std::min(NTHREADS_FX, (2 * P.n_r + 31) / 32 * 32)); }
+
+// Whole CTA, before the first use; the caller's next barrier publishes it.
+__device__ __forceinline__ void fx_scale_clear(FxScale& sc) {
+    for (int i = threadIdx.x; i < (int)(sizeof(FxScale) / 4); i += blockDim.x) reinterpret_cast<unsigned*>(&sc)[i] = 0u;
+}
+// exponent ex of part of vector v joins the block's; whole warps
+__device__ __forceinline__ void fx_scale_max(FxScale& sc, int v, int part, unsigned ex) {
+    const unsigned x = __reduce_max_sync(0xffffffffu, part ? 0u : ex), y = __reduce_max_sync(0xffffffffu, part ? ex : 0u);
+    if ((threadIdx.x & 31) == 0) {
+        if (x) atomicMax(&sc.e[v][0], x);
+        if (y) atomicMax(&sc.e[v][1], y);
+    }
+}
+// at least |q| 2^-FX_L1, from the leading word
+__device__ __forceinline__ unsigned fx_l1_part(fx64 q) {
+    int h, l;
+    fx_words(q, h, l);
+    return (unsigned)abs(h) / (1u << (FX_L1 - 32)) + 1u;
+}
+__device__ __forceinline__ int fx_l1_bits(unsigned l1) { return FX_L1 + 32 - __clz((int)l1); }
+
+// DCT-I of vectors v0 .. v0 + nb - 1 of the kernel, val(i, t) the FP64 part t & 1 of
+// entry t / 2 of vector v0 + i for t < 2 n (entries from n to K are zero), whose
+// exponents have been gathered before a barrier.  twice: the entries at both ends
+// count twice (a synthesis).  a, b: 2K nb points each.  Vector i's transform Z_n
+// (n <= K) is at the returned pointer + 2K i; dct_part gives it in FP64.  Ends with
+// a barrier.
+template <class V>
+__device__ __forceinline__ fxc* dct1_fx(const StepParams& P, FxScale& sc, int v0, int nb, int n, bool twice, fxc* a,
+                                        fxc* b, V val) {
+    const int K = P.K, L = 2 * K;
+    for (int i = 0; i < nb; ++i) {
+        fx64* z = reinterpret_cast<fx64*>(a + (size_t)i * L);
+        unsigned l1 = 0u;
+        for (int t = threadIdx.x; t < 2 * (K + 1); t += blockDim.x) {
+            const int j = t >> 1, part = t & 1;
+            const int e = (int)sc.e[v0 + i][part];
+            fx64 q = 0;
+            if (j < n && e != 0x7ff) {  // (a block with an infinity or NaN: outputs are NaN)
+                q = fx_from(val(i, t), e);
+                if (twice && (j == 0 || j == K)) q = 2 * q;  // its exponent entered e plus one
+            }
+            z[t] = q;
+            const unsigned w = fx_l1_part(q);
+            if (j > 0 && j < K) {
+                z[2 * (L - j) + part] = q;
+                l1 += 2u * w;
+            } else {
+                l1 += w;
+            }
+        }
+        l1 = __reduce_add_sync(0xffffffffu, l1);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&sc.l1[v0 + i], l1);
+    }
+    __syncthreads();
+    const int lg = 32 - __clz(K);  // L = 2^lg
+    if ((int)threadIdx.x < nb) {
+        const int v = v0 + threadIdx.x;
+        int S;
+        sc.back[v] = fx_schedule(lg, false, fx_l1_bits(sc.l1[v]), S);
+        sc.S[v] = S;
+    }
+    return fx_fft(a, b, reinterpret_cast<const fxw*>(P.fx_r), 1, lg, false, nb, sc.back + v0);
+}
+// 2^p times part of an output of vector v
+__device__ __forceinline__ double dct_part(const FxScale& sc, int v, const fxc* z, int part, int p) {
+    const int ex = (int)sc.e[v][part];
+    return fx_to(part ? z->y : z->x, sc.S[v] - 1022 - FX_BITS + p + ex, ex == 0x7ff);
+}
+
+// Chebyshev derivative of FP64 plain coefficients c[0 .. n-1] into d (another
+// array), the sums of cheb_derivative_scan, by four warps: role 0..3 takes one
+// index parity of one component, -1 none.  The exponents of d (as a synthesis's
+// input: the first entry twice) join vector v.  The caller's next barrier publishes d.
+__device__ __forceinline__ void cheb_derivative_part(const double2* c, double2* d, int n, double scale, int role,
+                                                     FxScale& sc, int v) {
+    if (role < 0) return;
+    const int lane = threadIdx.x & 31;
+    const int q = role & 1, part = role >> 1;
+    const double* cs = reinterpret_cast<const double*>(c) + part;
+    double* ds = reinterpret_cast<double*>(d) + part;
+    const int len = (n - q + 1) / 2;
+    const int per = (len + 31) / 32;
+    const int i0 = lane * per, i1 = min(i0 + per, len);
+    double acc = 0.0;
+    for (int i = i1 - 1; i >= i0; --i) {
+        const int k = 2 * i + q;
+        if (k > 0) {
+            acc = fma((double)(2 * k), cs[2 * k], acc);
+            ds[2 * (k - 1)] = acc;
+        }
+    }
+    double sfx = acc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double x = __shfl_down_sync(0xffffffffu, sfx, o);
+        if (lane + o < 32) sfx += x;
+    }
+    const double off = sfx - acc;
+    unsigned ex = 0u;
+    for (int i = i0; i < i1; ++i) {
+        const int k = 2 * i + q;
+        if (k > 0) {
+            const double x = (ds[2 * (k - 1)] + off) * ((k == 1) ? 0.5 * scale : scale);
+            ds[2 * (k - 1)] = x;
+            ex = max(ex, fx_exponent(x) + (k == 1 && fx_exponent(x) ? 1u : 0u));
+        }
+    }
+    if (q == 0 && lane == 0) ds[2 * (n - 1)] = 0.0;
+    ex = __reduce_max_sync(0xffffffffu, min(ex, 0x7ffu));
+    if (lane == 0) atomicMax(&sc.e[v][part], ex);
+}
+
+// K1 of the FP64 stage in the batched layout: the equations of k_spec_to_grid with
+// the DCT-I in fixed point.  Bound by the latency of its phases (45 % of the issue
+// slots, 30 % of the FP64 pipe busy at 257 x 768, where the FP64 transforms kept
+// that pipe 60 % busy): 50 -> 25.6 us there, 23 -> 14.9 us at 129 x 384, 67 -> 36 us
+// at 513 x 384 (against the double-float lean layout it replaces at that size).
+__global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P, VecSet y, double2* __restrict__ G1) {
+    __shared__ FxScale sc;
+    const int m = P.m_lo + blockIdx.x;
+    const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
+    const int NB = radial_batch(P);
+    fxc* bufA = fx_shared;
+    fxc* bufB = bufA + NB * L;
+    double2* cc0 = reinterpret_cast<double2*>(bufB + NB * L);  // Psi (or u_bar) plain coefficients, length nc
+    double2* cc1 = cc0 + N;                                    // first derivative
+    double2* cc2 = cc1 + N;                                    // second derivative
+    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
+    const double Cw = P.cnorm, Cw0 = 0.5 * P.cnorm;
+    // vectors: 0 Psi, 1 Psi', 2 Psi'', 3 theta (m >= 1); 0 u_bar, 1 u_bar', 3 theta (m = 0)
+    const int th_v = 3;
+    const double* ps = reinterpret_cast<const double*>(y.psi + (size_t)m * nc);
+    const double* th = reinterpret_cast<const double*>(y.th + (size_t)m * nc);
+    fx_scale_clear(sc);
+    __syncthreads();
+    for (int b = 0; b < 2; ++b) {
+        unsigned ex = 0u;
+        for (int t = tid; t < 2 * nc; t += nth) {
+            const double w = (t < 2) ? Cw0 : Cw;
+            double x;
+            if (b) {
+                x = th[t] * w;  // (formed again when it is converted)
+            } else {
+                x = (m > 0) ? ps[t] * w : (t & 1) ? 0.0 : y.u[t >> 1] * w;
+                reinterpret_cast<double*>(cc0)[t] = x;
+            }
+            const unsigned e = fx_exponent(x);
+            ex = max(ex, (t < 2 && e) ? min(e + 1u, 0x7ffu) : e);  // the first entry counts twice
+        }
+        fx_scale_max(sc, b ? th_v : 0, tid & 1, ex);
+    }
+    __syncthreads();
+    cheb_derivative_part(cc0, cc1, nc, P.inv_a, warp < 4 ? warp : -1, sc, 1);
+    __syncthreads();
+    if (m > 0) {
+        cheb_derivative_part(cc1, cc2, nc, P.inv_a, warp < 4 ? warp : -1, sc, 2);
+        __syncthreads();
+    }
+    auto value = [&](int v, int t) -> double {
+        if (v == th_v) return th[t] * ((t < 2) ? Cw0 : Cw);
+        return reinterpret_cast<const double*>(v == 0 ? cc0 : v == 1 ? cc1 : cc2)[t];
+    };
+    const double dm = (double)m;
+    double* PF = P.pump ? reinterpret_cast<double*>(P.pump_F + (size_t)m * N) : nullptr;
+    for (int f0 = 0; f0 < 4; f0 += NB) {
+        const fxc* R = dct1_fx(P, sc, f0, NB, nc, true, bufA, bufB, [&](int i, int t) { return value(f0 + i, t); });
+        for (int t = tid; t < 2 * N; t += nth) {
+            const int k = t >> 1, part = t & 1;
+            const double s = P.s[k], h2 = P.h2[k], is = P.inv_s[k];
+            double* out = reinterpret_cast<double*>(G1 + g_index(k, 0, m, M));
+            // out: fields v, u_phi, omega, theta, 2M doubles apart.  u_phi and omega are summed
+            // over the vectors of a batch in a register, over batches in out.
+            double up = 0.0, om = 0.0, pf = 0.0;
+            if (f0 > 0) {
+                up = out[2 * M + part];
+                om = out[4 * M + part];
+                if (PF) pf = PF[t];
+            }
+            for (int i = 0; i < NB; ++i) {
+                const int v = f0 + i;
+                const double g = dct_part(sc, v, R + (size_t)i * L + k, part, -1);  // value of the series at x_k
+                if (v == th_v) {
+                    out[6 * M + part] = g;
+                } else if (m == 0) {
+                    if (v == 0) {
+                        out[part] = 0.0;
+                        up = g;
+                        om = __dmul_rn(g, is);
+                    } else if (v == 1) {
+                        om += g;
+                        if (PF) pf = part ? 0.0 : P.pump_ups[k] * up * (1.0 + (0.5 * P.E) * om);
+                    }
+                } else if (v == 0) {
+                    const double c = fma(__dmul_rn(dm * dm, h2), __dmul_rn(is, is), 6.0);
+                    out[part ^ 1] = part ? -dm * g : dm * g;
+                    up = __dmul_rn(__dmul_rn(3.0, s), g);
+                    om = __dmul_rn(c, g);
+                    if (PF) {
+                        const double go = dct_part(sc, v, R + (size_t)i * L + k, part ^ 1, -1), U = P.pump_ups[k];
+                        const double ci = __dmul_rn(__dmul_rn(U, dm), P.pump_ci[k]);
+                        pf = fma(part ? -ci : ci, go, __dmul_rn(__dmul_rn(-U, fma(dm, dm, P.pump_cr[k])), g));
+                    }
+                } else if (v == 1) {
+                    const double c = fma(-5.0, s, __dmul_rn(h2, is));
+                    up = fma(-h2, g, up);
+                    om = fma(-c, g, om);
+                    if (PF) pf = fma(__dmul_rn(P.pump_ups[k], __dmul_rn(0.5, s)), g, pf);
+                } else {
+                    om = fma(-h2, g, om);
+                    if (PF) pf = fma(-P.pump_ups[k], om, pf);
+                }
+            }
+            out[2 * M + part] = up;
+            out[4 * M + part] = om;
+            if (PF) PF[t] = pf;
+        }
+        __syncthreads();
+    }
+}
+
+// row k of a real band applied to one component of complex values: x points at
+// that component (stride 2)
+template <int H>
+__device__ __forceinline__ double band_part(const double* __restrict__ band, const double* x, int k, int nc) {
+    const double* row = band + (size_t)k * (2 * H + 1);
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d <= 2 * H; ++d) {
+        const int n = k - H + d;
+        if (n >= 0 && n < nc) acc = fma(__ldg(&row[d]), x[2 * n], acc);
+    }
+    return acc;
+}
+
+// K3 of the FP64 stage in the batched layout: the equations of k_grid_to_spec with
+// the DCT-I in fixed point, the buoyancy added to N_omega_hat before the one C^I
+// apply (Eq. psi_int applies C^I to their sum), and the banded applies spread
+// over (row, component, operator) so that every warp issues FP64.  257 x 768:
+// 75 -> 43 us (FP64 pipe 66 -> 38 % busy), 129 x 384: 43 -> 24.5, 513 x 384: 114 -> 49 us
+// (from the double-float lean layout).
+// Vectors 0, 1: F1, F2 (to coefficients); 2, 3: their derivatives (to the grid);
+// 4, 5: N_omega (N_u), N_theta (to coefficients).
+__global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P, const double2* __restrict__ G2,
+                                                                    VecSet y, VecSet e) {
+    __shared__ FxScale sc;
+    const int m = P.m_lo + blockIdx.x;
+    const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
+    const int NB = min(2, radial_batch(P));
+    fxc* bufA = fx_shared;
+    fxc* bufB = bufA + NB * L;
+    double2* cc0 = reinterpret_cast<double2*>(bufB + NB * L);
+    double2* cc1 = cc0 + N;
+    double2* cc2 = cc1 + N;
+    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
+    const double dm = (double)m;
+    const int lgK = 31 - __clz(K);
+    const double* g2 = reinterpret_cast<const double*>(G2);
+    auto flat = [](double2* c) { return reinterpret_cast<double*>(c); };
+    fx_scale_clear(sc);
+    __syncthreads();
+    // pass A: plain Chebyshev coefficients of F1 = h^2 [v omega]_m, F2 = h^2 [v theta]_m
+    for (int b = 0; b < 2; ++b) {
+        double* dst = flat(b ? cc1 : cc0);
+        unsigned ex = 0u;
+        for (int t = tid; t < 2 * N; t += nth) {
+            const double v = g2[2 * (size_t)g_index(t >> 1, 2 * b, m, M) + (t & 1)] * P.h2[t >> 1];
+            dst[t] = v;
+            ex = max(ex, fx_exponent(v));
+        }
+        fx_scale_max(sc, b, tid & 1, ex);
+    }
+    __syncthreads();
+    for (int b0 = 0; b0 < 2; b0 += NB) {
+        const fxc* R = dct1_fx(P, sc, b0, NB, N, false, bufA, bufB,
+                               [&](int i, int t) { return flat((b0 + i) ? cc1 : cc0)[t]; });
+        for (int i = 0; i < NB; ++i) {
+            double* dst = flat((b0 + i) ? cc1 : cc0);
+            for (int t = tid; t < 2 * N; t += nth) {
+                const int n = t >> 1;
+                dst[t] = dct_part(sc, b0 + i, R + (size_t)i * L + n, t & 1, (n == 0 || n == K) ? -lgK - 1 : -lgK);
+            }
+        }
+        __syncthreads();
+    }
+    // d/ds of both: F1' -> cc2, F2' -> the free transform buffer beside it (two
+    // vectors in it) or, one vector at a time, cc0 once F1 is done with
+    double2* d1 = cc0;
+    if (NB == 2) {
+        d1 = reinterpret_cast<double2*>(bufB);
+        if (warp < 4)
+            cheb_derivative_part(cc0, cc2, N, P.inv_a, warp, sc, 2);
+        else
+            cheb_derivative_part(cc1, d1, N, P.inv_a, warp < 8 ? warp - 4 : -1, sc, 3);
+    } else {
+        cheb_derivative_part(cc0, cc2, N, P.inv_a, warp < 4 ? warp : -1, sc, 2);
+        __syncthreads();
+        cheb_derivative_part(cc1, d1, N, P.inv_a, warp < 4 ? warp : -1, sc, 3);
+    }
+    __syncthreads();
+    // pass B: derivative values on the grid, then N_omega (or N_u) -> cc1 and N_theta
+    // -> cc2; with Ekman pumping N_omega - F_eps and N_u + Ups_eps u_bar (1 + (E/2) omega_0)
+    const double* PF = P.pump ? reinterpret_cast<const double*>(P.pump_F + (size_t)m * N) : nullptr;
+    for (int b0 = 0; b0 < 2; b0 += NB) {
+        // (the last coefficient of a derivative is zero)
+        const fxc* R = dct1_fx(P, sc, 2 + b0, NB, K, true, bufA, bufB,
+                               [&](int i, int t) { return flat((b0 + i) ? d1 : cc2)[t]; });
+        for (int i = 0; i < NB; ++i) {
+            const int fld = b0 + i;  // 0: omega, 1: theta
+            double* dst = flat(fld ? cc2 : cc1);
+            unsigned ex = 0u;
+            for (int t = tid; t < 2 * N; t += nth) {
+                const int k = t >> 1, part = t & 1;
+                const double dF = dct_part(sc, 2 + fld, R + (size_t)i * L + k, part, -1);
+                const double is = P.inv_s[k];
+                const double* g = g2 + 2 * (size_t)g_index(k, 0, m, M);  // fields 2M doubles apart
+                double val;
+                if (fld == 0 && m == 0) {
+                    val = g[part] * (P.h2[k] * is);
+                    if (PF) val += PF[t];
+                } else {  // dF + i m [u_phi omega] (or [u_phi theta]), over s
+                    const double u = g[(fld ? 6 : 2) * M + (part ^ 1)];
+                    const double w = fma(part ? dm : -dm, u, dF);
+                    if (fld == 0) {
+                        val = w * is;
+                        if (PF) val -= PF[t];
+                    } else {
+                        val = fma(w, is, -g[4 * M + part]);
+                    }
+                }
+                dst[t] = val;
+                ex = max(ex, fx_exponent(val));
+            }
+            fx_scale_max(sc, 4 + fld, tid & 1, ex);
+        }
+        __syncthreads();
+    }
+    // pass C: Eq. icheb of N_omega (cc1) and N_theta (cc2), truncated to n < nc:
+    // N_omega_hat, with the buoyancy, -> cc0, N_theta_hat -> cc1
+    const double hc = 0.5 * P.cnorm, bfac = P.Ra / P.Pr * dm / P.s_o;
+    const bool buoy = m > 0 && !P.buoy_imp;
+    const double* th = reinterpret_cast<const double*>(y.th + (size_t)m * nc);
+    for (int b0 = 0; b0 < 2; b0 += NB) {
+        const fxc* R = dct1_fx(P, sc, 4 + b0, NB, N, false, bufA, bufB,
+                               [&](int i, int t) { return flat((b0 + i) ? cc2 : cc1)[t]; });
+        for (int i = 0; i < NB; ++i)
+            for (int t = tid; t < 2 * nc; t += nth) {
+                const int part = t & 1;
+                double v = dct_part(sc, 4 + b0 + i, R + (size_t)i * L + (t >> 1), part, 0) * hc;
+                if (b0 + i) {
+                    flat(cc1)[t] = v;
+                } else {
+                    if (buoy) v = fma(part ? bfac : -bfac, th[t ^ 1], v);
+                    flat(cc0)[t] = v;
+                }
+            }
+        __syncthreads();
+    }
+    // integrated right-hand sides; the linear couplings read the FP64 state
+    //   e_psi = C^I N_omega_hat,  e_theta = -D^I N_theta_hat - (alpha/ln eta) i m G^I Psi_hat,
+    //   e_u = -D^I N_u_hat
+    double* eps = reinterpret_cast<double*>(e.psi + (size_t)m * nc);
+    double* eth = reinterpret_cast<double*>(e.th + (size_t)m * nc);
+    const double* ps = reinterpret_cast<const double*>(y.psi + (size_t)m * nc);
+    for (int t = tid; t < 4 * nc; t += nth) {
+        const int r = (t < 2 * nc) ? t : t - 2 * nc;
+        const int k = r >> 1, part = r & 1;
+        if (t < 2 * nc) {
+            double v = 0.0;
+            if (m > 0) {
+                if (k >= 4) v = band_part<8>(P.ops.band[OP_C], flat(cc0) + part, k, nc);
+            } else if (part == 0) {
+                e.u[k] = (k >= 2) ? -band_part<4>(P.ops.band[OP_D], flat(cc0), k, nc) : 0.0;
+            }
+            eps[r] = v;
+        } else {
+            double v = 0.0;
+            if (k >= 2) {
+                v = -band_part<4>(P.ops.band[OP_D], flat(cc1) + part, k, nc);
+                if (m > 0) {
+                    const double gp = band_part<4>(P.ops.band[OP_G], ps + (part ^ 1), k, nc);
+                    v = fma(part ? -P.tc * dm : P.tc * dm, gp, v);
+                }
+            }
+            eth[r] = v;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// K2 of the FP64 stage in fixed point: the steps of k_phi_products on 64-bit
+// integers.  Each field is normalised by the exponent of its largest
+// coefficient on load; the physical values of each field are shifted up by the
+// free leading bits of their largest before the products, whose 60-bit results
+// are transformed back.  FP64 is used for conversions only.  The mean of a product
+// (m = 0) needs no separate sum: the transforms are accurate to about 2^-53 of
+// their largest value (the double-float products needed an FP64 one; the zonal
+// explicit term at 2049 x 6144 is now 1.1e-11 from an FP64 evaluation, 4.9e-11
+// then).  Bound by instruction issue (43-54 % of the slots; 16 warps an SM at
+// n_phi = 6144, where two buffers fill its shared memory).  Against the
+// double-float kernel: 257 x 768 37 -> 24.4 us, 33 x 96 22 -> 12.2, 1025 x 3072
+// 443 -> 313, 2049 x 6144 1706 -> 1265 us.
+// ---------------------------------------------------------------------------
+struct PhiScale {
+    unsigned e[4];      // biased exponents of v, u_phi, omega, theta
+    unsigned top[4];    // OR of the leading words of the fields' physical values
+    unsigned l1[4];     // 1-norms of the packed spectra, then of the packed products
+    unsigned back[4];
+    int S[4];
+    double cfl[2 * 16];
+};
+
+// 2/3 of a: 1/n_phi = (2/3) 2^-(lg + 1) for n_phi = 3 2^lg
+__device__ __forceinline__ fx64 fx_two_thirds(fx64 a) {
+    constexpr long long c = 3074457345618258603ll;  // in units of 2^-62
+    constexpr int lo = (int)(unsigned)(unsigned long long)c;
+    return fx_mulc(a, (int)((c - lo) >> 32), lo);
+}
+// a b 2^-62, |a|, |b| < 2^61
+__device__ __forceinline__ fx64 fx_mul62(fx64 a, fx64 b) {
+    int ah, al, bh, bl;
+    fx_split(a, ah, al);
+    fx_split(b, bh, bl);
+    return (fx64)((unsigned long long)fx_mulw(ah, bh) << 2) + ((fx_mad(al, bh, fx_mulw(ah, bl)) + ((fx64)1 << 29)) >> 30);
+}
+__device__ __forceinline__ unsigned fx_top(fx64 a) { return (unsigned)((a < 0 ? ~a : a) >> 32); }
+
+// the pair of fields (f, f + 1) packed as a + i b into Z, components exchanged
+// (fx_fft then runs the backward transform); 1-norm into l1
+__device__ __forceinline__ void phi_pack(const double2* __restrict__ src, int M, int Pn, int n_m, unsigned ea, unsigned eb,
+                                         fxc* Z, unsigned* l1) {
+    unsigned w = 0u;
+    for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
+        const double2 a = src[m], b = src[M + m];
+        fxc p, q;
+        p.x = (ea == 0x7ff) ? 0 : fx_from(a.x, ea) >> 1;  // below 2^59: the packed values below 2^60
+        p.y = (ea == 0x7ff) ? 0 : fx_from(a.y, ea) >> 1;
+        q.x = (eb == 0x7ff) ? 0 : fx_from(b.x, eb) >> 1;
+        q.y = (eb == 0x7ff) ? 0 : fx_from(b.y, eb) >> 1;
+        if (m == 0) {
+            Z[0] = fxc{q.x, p.x};
+            w += fx_l1_part(p.x) + fx_l1_part(q.x);
+        } else {
+            const fxc z1 = fxc{p.y + q.x, p.x - q.y};  // (im, re) of a + i b
+            const fxc z2 = fxc{q.x - p.y, p.x + q.y};  // of conj(a) + i conj(b)
+            Z[m] = z1;
+            Z[Pn - m] = z2;
+            w += fx_l1_part(z1.x) + fx_l1_part(z1.y) + fx_l1_part(z2.x) + fx_l1_part(z2.y);
+        }
+    }
+    for (int j = n_m + 1 + threadIdx.x; j < Pn - n_m; j += blockDim.x) Z[j] = fxc{0, 0};
+    w = __reduce_add_sync(0xffffffffu, w);
+    if ((threadIdx.x & 31) == 0) atomicAdd(l1, w);
+}
+// the spectra of a + i b from its transform Y (scaled by 2^-S), over n_phi
+__device__ __forceinline__ void phi_split(const fxc* Y, double2* __restrict__ dst, int M, int Pn, int n_m, bool three,
+                                          int exa, int exb, bool bada, bool badb) {
+    for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
+        const fxc y1 = Y[m], y2 = Y[m ? Pn - m : 0];
+        // a = (y1 + conj(y2))/2,  b = (y1 - conj(y2))/(2i)
+        fx64 v[4] = {(y1.x >> 1) + (y2.x >> 1), (y1.y >> 1) - (y2.y >> 1), (y1.y >> 1) + (y2.y >> 1),
+                     (y2.x >> 1) - (y1.x >> 1)};
+        double d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            d[i] = fx_to(three ? fx_two_thirds(v[i]) : v[i], i < 2 ? exa : exb, i < 2 ? bada : badb);
+        dst[m] = make_double2(d[0], d[1]);
+        dst[M + m] = make_double2(d[2], d[3]);
+    }
+}
+
+// Courant rates (cfl_rates) from the packed physical pair (u_phi, v) in R
+__device__ void cfl_rates_fx(const StepParams& P, const fxc* R, int k, int sv, int su, bool bad, double* red) {
+    fx64 a = 0, b = 0;
+    for (int j = threadIdx.x; j < P.n_phi; j += blockDim.x) {
+        const fxc g = R[j];
+        a = max(a, g.y < 0 ? -g.y : g.y);
+        b = max(b, g.x < 0 ? -g.x : g.x);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+        red[2 * w] = fx_to(a, sv, bad);
+        red[2 * w + 1] = fx_to(b, su, bad);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double ra = red[0], rb = red[1];
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
+            ra = fmax(ra, red[2 * i]);
+            rb = fmax(rb, red[2 * i + 1]);
+        }
+        const double s = P.s[k];
+        const double fs = P.coll ? 1.0 / s : P.h2[k] / s;
+        const double rs = fs * ra / P.cfl_ds[k], rp = rb / (s * P.cfl_dphi);
+        atomicMax(reinterpret_cast<unsigned long long*>(P.cfl_max), (unsigned long long)__double_as_longlong(rs));
+        atomicMax(reinterpret_cast<unsigned long long*>(P.cfl_max + 1), (unsigned long long)__double_as_longlong(rp));
+    }
+    __syncthreads();
+}
+
+// PAIR: both packed pairs in one batched transform each way (buffers of 2 n_phi
+// points each); else one after the other, the first pair's physical values
+// and the second products waiting in registers.
+template <bool PAIR>
+__global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParams P, const double2* __restrict__ G1,
+                                                            double2* __restrict__ G2) {
+    __shared__ PhiScale sc;
+    const int k = P.k_lo + blockIdx.x;
+    const int Pn = P.n_phi, M = P.M, n_m = P.n_m;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const bool three = Pn % 3 == 0;
+    const int lg = 31 - __clz(three ? Pn / 3 : Pn);
+    const fxw* tw = reinterpret_cast<const fxw*>(P.fx_p);
+    fxc* X = fx_shared;
+    fxc* Y = X + (PAIR ? 2 : 1) * Pn;
+    const double2* src = G1 + g_index(k, 0, 0, M);
+    double2* dst = G2 + g_index(k, 0, 0, M);
+    if (tid < (int)(offsetof(PhiScale, cfl) / 4)) reinterpret_cast<unsigned*>(&sc)[tid] = 0u;
+    __syncthreads();
+    {
+        unsigned ex[4] = {0u, 0u, 0u, 0u};
+        for (int m = tid; m <= n_m; m += nth)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const double2 v = src[q * M + m];
+                ex[q] = max(ex[q], max(fx_exponent(v.x), fx_exponent(v.y)));
+            }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            ex[q] = __reduce_max_sync(0xffffffffu, ex[q]);
+            if ((tid & 31) == 0) atomicMax(&sc.e[q], ex[q]);
+        }
+    }
+    __syncthreads();
+    const unsigned ev = sc.e[0], eu = sc.e[1], ew = sc.e[2], et = sc.e[3];
+    // schedules of transforms i0 .. i0 + n - 1 from their 1-norms
+    auto schedule = [&](int i0, int n) {
+        __syncthreads();
+        if (tid < n) {
+            int S;
+            sc.back[i0 + tid] = fx_schedule(lg, three, fx_l1_bits(sc.l1[i0 + tid]), S);
+            sc.S[i0 + tid] = S;
+        }
+    };
+    // leading bits in use of the fields of pair i, from the physical values
+    auto tops = [&](int i, unsigned x, unsigned yv) {
+        x = __reduce_or_sync(0xffffffffu, x);
+        yv = __reduce_or_sync(0xffffffffu, yv);
+        if ((tid & 31) == 0) {
+            atomicOr(&sc.top[2 * i], yv);  // first field of the pair: the exchanged y
+            atomicOr(&sc.top[2 * i + 1], x);
+        }
+    };
+    fxc reg[PAIR ? 1 : MAXPER];
+    const fxc *R1 = nullptr, *R2 = nullptr;
+    if (PAIR) {
+        phi_pack(src, M, Pn, n_m, ev, eu, X, &sc.l1[0]);
+        phi_pack(src + 2 * M, M, Pn, n_m, ew, et, X + Pn, &sc.l1[1]);
+        schedule(0, 2);
+        R1 = fx_fft(X, Y, tw, 1, lg, three, 2, sc.back);
+        R2 = R1 + Pn;
+        for (int i = 0; i < 2; ++i) {
+            unsigned x = 0u, yv = 0u;
+            for (int j = tid; j < Pn; j += nth) {
+                x |= fx_top(R1[i * Pn + j].x);
+                yv |= fx_top(R1[i * Pn + j].y);
+            }
+            tops(i, x, yv);
+        }
+    } else {
+        for (int i = 0; i < 2; ++i) {
+            phi_pack(src + 2 * i * M, M, Pn, n_m, i ? ew : ev, i ? et : eu, X, &sc.l1[i]);
+            schedule(i, 1);
+            R2 = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + i);
+            unsigned x = 0u, yv = 0u;
+            for (int j = tid; j < Pn; j += nth) {
+                x |= fx_top(R2[j].x);
+                yv |= fx_top(R2[j].y);
+            }
+            tops(i, x, yv);
+            if (i == 0) {
+                if (P.cfl_max)
+                    cfl_rates_fx(P, R2, k, sc.S[0] + (int)ev - 1022 - FX_BITS + 1, sc.S[0] + (int)eu - 1022 - FX_BITS + 1,
+                                 ev == 0x7ff || eu == 0x7ff, sc.cfl);
+#pragma unroll
+                for (int n = 0; n < (PAIR ? 1 : MAXPER); ++n) {
+                    const int j = tid + n * nth;
+                    if (j < Pn) reg[n] = R2[j];
+                }
+                __syncthreads();
+            }
+        }
+    }
+    __syncthreads();
+    if (PAIR && P.cfl_max)
+        cfl_rates_fx(P, R1, k, sc.S[0] + (int)ev - 1022 - FX_BITS + 1, sc.S[0] + (int)eu - 1022 - FX_BITS + 1,
+                     ev == 0x7ff || eu == 0x7ff, sc.cfl);
+    // free leading bits: |value| < 2^(32 + bits of top), shifted up to below 2^61
+    int sh[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sh[q] = __clz((int)sc.top[q]) - 3;  // (-2 at least)
+    // exponents of the shifted physical fields: value = integer 2^x
+    const int xv = sc.S[0] + (int)ev - 1022 - FX_BITS + 1 - sh[0], xu = sc.S[0] + (int)eu - 1022 - FX_BITS + 1 - sh[1];
+    const int xw = sc.S[1] + (int)ew - 1022 - FX_BITS + 1 - sh[2], xt = sc.S[1] + (int)et - 1022 - FX_BITS + 1 - sh[3];
+    unsigned l0 = 0u, l1 = 0u;
+    auto up = [](fx64 a, int s) { return s >= 0 ? (fx64)((unsigned long long)a << s) : a >> -s; };
+    // (v omega, u_phi omega) and (v theta, u_phi theta), each 2^-62 of the integers' product
+    auto prods = [&](fxc g1, fxc g2, fxc& p, fxc& r) {
+        const fx64 v = up(g1.y, sh[0]), u = up(g1.x, sh[1]), w = up(g2.y, sh[2]), t = up(g2.x, sh[3]);
+        p = fxc{fx_mul62(v, w), fx_mul62(u, w)};
+        r = fxc{fx_mul62(v, t), fx_mul62(u, t)};
+        l0 += fx_l1_part(p.x) + fx_l1_part(p.y);
+        l1 += fx_l1_part(r.x) + fx_l1_part(r.y);
+    };
+    auto norms = [&]() {
+        l0 = __reduce_add_sync(0xffffffffu, l0);
+        l1 = __reduce_add_sync(0xffffffffu, l1);
+        if ((tid & 31) == 0) {
+            atomicAdd(&sc.l1[2], l0);
+            atomicAdd(&sc.l1[3], l1);
+        }
+    };
+    const int ln = three ? -(lg + 1) : -lg;  // 1/n_phi
+    const bool bv = ev == 0x7ff, bu = eu == 0x7ff, bw = ew == 0x7ff, bt = et == 0x7ff;
+    if (PAIR) {
+        fxc* O = (R1 == X) ? Y : X;
+        for (int j = tid; j < Pn; j += nth) {
+            fxc p, r;
+            prods(R1[j], R2[j], p, r);
+            O[j] = p;
+            O[Pn + j] = r;
+        }
+        norms();
+        schedule(2, 2);
+        const fxc* Z = fx_fft(O, const_cast<fxc*>(R1), tw, 1, lg, three, 2, sc.back + 2);
+        phi_split(Z, dst, M, Pn, n_m, three, xv + xw + 62 + sc.S[2] + ln, xu + xw + 62 + sc.S[2] + ln, bv || bw, bu || bw);
+        phi_split(Z + Pn, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln,
+                  bv || bt, bu || bt);
+    } else {
+        fxc* O = (R2 == X) ? Y : X;
+#pragma unroll
+        for (int n = 0; n < (PAIR ? 1 : MAXPER); ++n) {
+            const int j = tid + n * nth;
+            if (j < Pn) {
+                fxc p;
+                prods(reg[n], R2[j], p, reg[n]);
+                O[j] = p;
+            }
+        }
+        norms();
+        schedule(2, 2);
+        const fxc* Z = fx_fft(O, const_cast<fxc*>(R2), tw, 1, lg, three, 1, sc.back + 2);
+        phi_split(Z, dst, M, Pn, n_m, three, xv + xw + 62 + sc.S[2] + ln, xu + xw + 62 + sc.S[2] + ln, bv || bw, bu || bw);
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < (PAIR ? 1 : MAXPER); ++n) {
+            const int j = tid + n * nth;
+            if (j < Pn) X[j] = reg[n];
+        }
+        Z = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + 3);
+        phi_split(Z, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln, bv || bt,
+                  bu || bt);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Diagnostics from G1 (radial-grid Fourier coefficients written by K1):
 // per mode, sums over the Gauss-Lobatto points with quadrature weights q_k
 // (int f s ds ~ sum_k q_k f_k) of |u_s|^2 + |u_phi|^2 and |omega|^2;
@@ -878,13 +1385,16 @@ size_t smem_spec_to_grid(const StepParams& P) {
 size_t smem_phi_products(const StepParams& P) {
     return (P.fp32 ? sizeof(float2) : sizeof(double2)) * 2 * P.n_phi;
 }
-size_t smem_grid_to_spec(const StepParams& P) { return smem_spec_to_grid(P); }
+// a3: two vectors at a time at most in the fixed-point kernel
+size_t smem_grid_to_spec(const StepParams& P) {
+    if (P.fp32) return smem_spec_to_grid(P);
+    return sizeof(double2) * (2 * (size_t)std::min(2, radial_batch(P)) * 2 * P.K + 3 * P.n_r);
+}
 
 // The explicit stage runs on double2 (FP64) or float2 (option "precision" =
 // mixed) grid arrays; G1, G2 hold either type.
 // ---------------------------------------------------------------------------
-// Large radial grids in FP64 (K = n_r - 1 >= LEAN_K, the half-length DCT-I;
-// measured faster than the batched layout from n_r = 513, slower at 257):
+// Large radial grids (K = n_r - 1 >= LEAN_K, the half-length DCT-I):
 // a1 and a3 with three shared arrays of K + 1 entries, X, C, Y (98 KB at
 // n_r = 2049), instead of the batched layout's 2 x 2K + 3 n_r entries (229 KB),
 // so that two CTAs share an SM and hide each other's barrier and shared-memory
@@ -893,7 +1403,7 @@ size_t smem_grid_to_spec(const StepParams& P) { return smem_spec_to_grid(P); }
 // C with X as scratch; the DCT-I works in place on the pair (X, Y).  The same
 // equations, in the same precision, as k_spec_to_grid / k_grid_to_spec.
 // ---------------------------------------------------------------------------
-constexpr int LEAN_K = 512;
+constexpr int LEAN_K = 1024;
 
 __device__ __forceinline__ double2 warp_sum(double2 v) {
 #pragma unroll
@@ -916,10 +1426,10 @@ __host__ __device__ inline bool lean_radial(const StepParams& P) {
     return P.radial_lean > 0 || P.K >= LEAN_K;
 }
 
-// double-float radial transforms in the lean kernels (option "radial_dd"):
+// fixed-point radial transforms in the lean kernels (option "radial_dd"):
 // 1 always, 0 never, -1 (default) as the lean layout's own default
-__host__ __device__ inline bool radial_dd(const StepParams& P) {
-    if (!P.plan_r.twdd || !P.s_dd || P.radial_dd == 0) return false;
+__host__ __device__ inline bool radial_fx(const StepParams& P) {
+    if (!P.fx_r || P.radial_dd == 0) return false;
     return P.radial_dd > 0 || P.K >= LEAN_K;
 }
 
@@ -1030,140 +1540,6 @@ __device__ T* dct1_pair(T* X, T* Y, const StepParams& P) {
     }
     __syncthreads();
     return O;
-}
-
-// ---------------------------------------------------------------------------
-// Double-float radial transforms (option "radial_dd", lean layout).  The same
-// DCT-I and derivative scan as dct1_pair and cheb_derivative_scan with complex
-// double-floats (ddfloat.cuh: about 48 significant bits) on the FP32 pipe, which
-// issues 64 times the FP64 rate on GB300; grid and coefficient values cross to
-// and from FP64 at the kernels' loads and stores only.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ ddf dd_shfl_xor(ddf v, int o) {
-    return ddf{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-}
-__device__ __forceinline__ ddf dd_shfl_up(ddf v, int o) {
-    return ddf{__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
-}
-__device__ __forceinline__ ddf dd_shfl_down(ddf v, int o) {
-    return ddf{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-}
-__device__ __forceinline__ ddc dd_warp_sum(ddc v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x = v.x + dd_shfl_xor(v.x, o);
-        v.y = v.y + dd_shfl_xor(v.y, o);
-    }
-    return v;
-}
-// an integer |k| < 2^24 as a double-float (exact)
-__device__ __forceinline__ ddf dd_int(int k) { return ddf{(float)k, 0.f}; }
-__device__ __forceinline__ ddc dd_scale2c(ddc a, float s) { return ddc{dd_scale2(a.x, s), dd_scale2(a.y, s)}; }
-
-// dct1_pair in double-float: X, Y hold K + 1 (resp. the FFT's K) complex
-// double-floats; the same steps, the C_1 sum and the prefix sums in double-float.
-__device__ ddc* dct1_pair_dd(ddc* X, ddc* Y, const StepParams& P) {
-    const int K = P.plan_h.L, H = K / 2;
-    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nth >> 5;
-    const ddc* tw = reinterpret_cast<const ddc*>(P.plan_r.twdd);  // (cos(pi j/K), -sin(pi j/K))
-    __shared__ ddc wsum[NTHREADS_R / 32];
-    __shared__ ddc c1;
-    __syncthreads();
-    ddc acc = ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}};
-    for (int j = tid; j < H; j += nth) {
-        if (j == 0) {
-            const ddc a = X[0], b = X[K];
-            X[0] = dd_scale2c(cadd(a, b), 0.5f);
-            acc = csub(a, b);
-        } else {
-            const ddc a = X[j], b = X[K - j];
-            const ddc t = ldg_tw(tw + j);
-            const ddf sn = -t.y, cs2 = dd_scale2(t.x, 2.f);
-            const ddc hs = dd_scale2c(cadd(a, b), 0.5f), dif = csub(a, b);
-            X[j] = ddc{hs.x - sn * dif.x, hs.y - sn * dif.y};
-            X[K - j] = ddc{hs.x + sn * dif.x, hs.y + sn * dif.y};
-            acc = ddc{acc.x + cs2 * dif.x, acc.y + cs2 * dif.y};
-        }
-    }
-    acc = dd_warp_sum(acc);
-    if (lane == 0) wsum[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        ddc t = wsum[0];
-        for (int w = 1; w < nw; ++w) t = cadd(t, wsum[w]);
-        c1 = t;
-    }
-    ddc* F = fft_batched<+1, ddc, true>(X, Y, P.plan_h, 1);  // begins with a barrier
-    ddc* O = (F == X) ? Y : X;
-    for (int k = tid; k <= H; k += nth) O[2 * k] = cadd(F[k], F[k == 0 ? 0 : K - k]);
-    const int chunk = (H + nth - 1) / nth;
-    const int lo = min(tid * chunk, H), hi = min(lo + chunk, H);
-    ddc tot = ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}};
-    for (int k = max(lo, 1); k < hi; ++k) {
-        const ddc df = csub(F[k], F[K - k]);
-        tot = ddc{tot.x + df.y, tot.y - df.x};
-    }
-    ddc inc = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const ddf ux = dd_shfl_up(inc.x, o), uy = dd_shfl_up(inc.y, o);
-        if (lane >= o) inc = ddc{inc.x + ux, inc.y + uy};
-    }
-    __syncthreads();
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    ddc run = c1;
-    for (int w = 0; w < warp; ++w) run = cadd(run, wsum[w]);
-    run = cadd(run, csub(inc, tot));
-    for (int k = lo; k < hi; ++k) {
-        if (k > 0) {
-            const ddc df = csub(F[k], F[K - k]);
-            run = ddc{run.x + df.y, run.y - df.x};
-        }
-        O[2 * k + 1] = run;
-    }
-    __syncthreads();
-    return O;
-}
-
-// cheb_derivative_scan in double-float (scale: the x -> s factor, rounded to
-// double-float once)
-__device__ void cheb_derivative_scan_dd(const ddc* c, ddc* d, ddc* tmp, int n, double scale) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const ddc zero = ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}};
-    if (warp < 2) {
-        const int q = warp;
-        const int len = (n - q + 1) / 2;
-        const int per = (len + 31) / 32;
-        const int i0 = lane * per, i1 = min(i0 + per, len);
-        ddc acc = zero;
-        for (int i = i1 - 1; i >= i0; --i) {
-            const int k = 2 * i + q;
-            if (k > 0) {
-                const ddf f = dd_int(2 * k);
-                acc = ddc{acc.x + f * c[k].x, acc.y + f * c[k].y};
-            }
-            tmp[k] = acc;
-        }
-        ddc sfx = acc;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const ddf x = dd_shfl_down(sfx.x, o), y = dd_shfl_down(sfx.y, o);
-            if (lane + o < 32) sfx = ddc{sfx.x + x, sfx.y + y};
-        }
-        const ddc off = csub(sfx, acc);
-        for (int i = i0; i < i1; ++i) {
-            const int k = 2 * i + q;
-            tmp[k] = cadd(tmp[k], off);
-        }
-    }
-    __syncthreads();
-    const ddf fs = dd_from(scale), f0 = dd_from(0.5 * scale);
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const ddf f = (j == 0) ? f0 : fs;
-        d[j] = (j + 1 < n) ? cscale(tmp[j + 1], f) : zero;
-    }
-    __syncthreads();
 }
 
 // The FP64 coefficients as the lean kernels' element type: unchanged in FP64,
@@ -1369,215 +1745,396 @@ __global__ void __launch_bounds__(NTHREADS_R, lean_ctas<T>()) k_grid_to_spec_lea
     }
 }
 
-// k_spec_to_grid_lean with double-float transforms: the coefficients become
-// double-floats when loaded (the Chebyshev weights applied in double-float), the
-// field arithmetic at each radius runs in double-float with double-float tables
-// of s, h^2 and 1/s, and each grid value becomes FP64 once, when it is final.
-// Between the passes over psi, dpsi/ds and d2psi/ds2 the partial sums of the
-// u_phi and omega columns wait in the grid array in double-float form (each CTA
-// owns its column m); the pumping flux and the m = 0 column stay FP64.
-__global__ void __launch_bounds__(NTHREADS_R, 2) k_spec_to_grid_lean_dd(StepParams P, VecSet y,
-                                                                         double2* __restrict__ G1) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int m = P.m_lo + blockIdx.x;
-    const int K = P.K, N = P.n_r, nc = P.nc, M = P.M;
-    ddc* X = reinterpret_cast<ddc*>(smraw);
-    ddc* C = X + N;
-    ddc* Y = C + N;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const double dm = (double)m;
-    const ddf Cw = dd_from(P.cnorm), Cw0 = dd_scale2(Cw, 0.5f);
-    const float fm = (float)m;  // exact: m < 2^24
-    const ddf fm2 = dd_from(dm * dm);
-    const ddf* s_dd = reinterpret_cast<const ddf*>(P.s_dd);
-    const ddf* h2_dd = reinterpret_cast<const ddf*>(P.h2_dd);
-    const ddf* is_dd = reinterpret_cast<const ddf*>(P.inv_s_dd);
-    const ddc zero = ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}};
-    for (int n = tid; n < N; n += nth) {
-        ddc a = zero;
-        if (n < nc) {
-            const ddf w = (n == 0) ? Cw0 : Cw;
-            a = (m > 0) ? cscale(dd_from_bits(y.psi[(size_t)m * nc + n]), w)
-                        : ddc{dd_from_bits(y.u[n]) * w, ddf{0.f, 0.f}};
+// ---------------------------------------------------------------------------
+// The lean layout in fixed point (option "radial_dd", the FP64 stage's default from
+// n_r = 1025): two buffers of K fixed-point entries and one array of n_r FP64 values
+// (98 KB at n_r = 2049: two CTAs of 512 threads share an SM), the vectors of a mode
+// one after another through a half-length DCT-I.  Against double-float transforms
+// in the same layout: 1025 x 3072 343 -> 310 (a1) and 581 -> 433 us (a3), 2049 x 6144
+// 1124 -> 1090 and 1607 -> 1594 us, with roundings about 2^5 smaller; from n_r = 1025,
+// since at 513 the batched layout is faster (a1 52 -> 36, a3 90 -> 49 us at 513 x 384).
+// ---------------------------------------------------------------------------
+constexpr int NTHREADS_LX = 512;
+
+struct DctHalf {
+    long long c1h[NTHREADS_LX / 32][2], c1l[NTHREADS_LX / 32][2];  // partial sums of C_1
+    long long c1[2];                                              // C_1 2^-(S + 1)
+    long long run[NTHREADS_LX / 32][2];                           // odd outputs' increments of a warp
+    double tot[NTHREADS_LX / 32];                                 // derivative sums of a warp
+};
+
+// DCT-I of K + 1 values by one complex transform of length K, as dct1_pair: y_j = (x_j + x_{K-j})/2
+// - sin(pi j/K)(x_j - x_{K-j}), F = FFT(y), C_{2k} = F_k + F_{K-k}, and the odd outputs
+// from C_1 = sum_j (x_j - x_{K-j}) cos(pi j/K) by prefix sums of -i (F_k - F_{K-k})
+// (the transform here is the forward one, F_{K-k} in the place of F_k, which
+// changes the sign).  The integer prefix sums are exact; what accumulates is the
+// rounding of F, about 2^-55 of its largest value a term.
+// The schedule takes the 1-norms of x and y together: the outputs are bounded by
+// x's, and y's can be far below it (sin(pi j/K) is small near the ends).
+// val(t): FP64 part t & 1 of entry t / 2, t < 2 n, exponents gathered before a
+// barrier; twice: the end entries count twice.  X, Y: K points each.  On return F holds
+// the transform and O[k] the odd outputs C_{2k+1}; half_part reads an output.
+// Ends with a barrier.
+template <class V>
+__device__ __forceinline__ void dct1_half_fx(const StepParams& P, FxScale& sc, DctHalf& dh, int v, int n, bool twice,
+                                             fxc* X, fxc* Y, fxc*& F, fxc*& O, V val) {
+    const int K = P.K, H = K >> 1;
+    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nth >> 5;
+    const fxw* tw = reinterpret_cast<const fxw*>(P.fx_r);  // (cos(pi j/K), -sin(pi j/K))
+    {
+        const int part = tid & 1;
+        const int e = (int)sc.e[v][part];
+        fx64* x = reinterpret_cast<fx64*>(X) + part;
+        unsigned l1 = 0u;
+        fx64 ch = 0, cl = 0;
+        auto get = [&](int j) -> fx64 {
+            if (j >= n || e == 0x7ff) return 0;
+            const fx64 q = fx_from(val(2 * j + part), e) >> 2;  // pairs grow by less than four
+            return (twice && (j == 0 || j == K)) ? 2 * q : q;
+        };
+        for (int j = tid >> 1; j <= H; j += nth >> 1) {
+            const fx64 a = get(j);
+            l1 += fx_l1_part(a);
+            if (j == H) {
+                x[2 * H] = a;
+                continue;
+            }
+            const fx64 b = get(K - j);
+            l1 += fx_l1_part(b);
+            const fx64 hs = (a + b) >> 1, dif = a - b;
+            fx64 c;
+            if (j == 0) {
+                x[0] = hs;
+                c = dif;
+            } else {
+                const fxw w = fx_ldw(tw + j);
+                const fx64 sd = fx_mulc(dif, w.y1, w.y0);  // -sin(pi j/K) dif
+                x[2 * j] = hs + sd;
+                x[2 * (K - j)] = hs - sd;
+                l1 += fx_l1_part(hs + sd) + fx_l1_part(hs - sd);
+                c = 2 * fx_mulc(dif, w.x1, w.x0);
+            }
+            ch += c >> 32;
+            cl += (fx64)(unsigned)c;
         }
-        C[n] = a;
+        l1 = __reduce_add_sync(0xffffffffu, l1);
+        if (lane == 0) atomicAdd(&sc.l1[v], l1);
+#pragma unroll
+        for (int o = 2; o < 32; o <<= 1) {
+            ch += __shfl_xor_sync(0xffffffffu, ch, o);
+            cl += __shfl_xor_sync(0xffffffffu, cl, o);
+        }
+        if (lane < 2) {
+            dh.c1h[warp][lane] = ch;
+            dh.c1l[warp][lane] = cl;
+        }
     }
     __syncthreads();
-    double2* PF = P.pump ? P.pump_F + (size_t)m * N : nullptr;
-    __shared__ double red[4 * 32], mx[4];
-    float lam = 1.f;
-    if (m == 0) {  // u_bar and lam u_bar' packed into one transform (lam a power of two)
-        cheb_derivative_scan_dd(C, Y, X, N, P.inv_a);
-        double a0 = 0.0, a1 = 0.0;  // max |u_bar|, max |u_bar'| (leading parts)
-        for (int i = tid; i < N; i += nth) {
-            a0 = fmax(a0, fabs((double)C[i].x.hi) + fabs((double)C[i].y.hi));
-            a1 = fmax(a1, fabs((double)Y[i].x.hi) + fabs((double)Y[i].y.hi));
+    const int lg = 31 - __clz(K);  // transform length 2^lg
+    if (tid < 2) {
+        int S;
+        const unsigned bk = fx_schedule(lg, false, fx_l1_bits(sc.l1[v]), S);
+        if (tid == 0) {
+            sc.back[v] = bk;
+            sc.S[v] = S;
         }
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int o = 16; o > 0; o >>= 1) {
-            a0 = fmax(a0, __shfl_xor_sync(0xffffffffu, a0, o));
-            a1 = fmax(a1, __shfl_xor_sync(0xffffffffu, a1, o));
+        fx64 h = 0, l = 0;
+        for (int w = 0; w < nw; ++w) {
+            h += dh.c1h[w][tid];
+            l += dh.c1l[w][tid];
         }
-        if (lane == 0) {
-            red[warp] = a0;
-            red[32 + warp] = a1;
-        }
-        __syncthreads();
-        if (tid < 2) {
-            double r = 0.0;
-            for (int w = 0; w < (nth >> 5); ++w) r = fmax(r, red[tid * 32 + w]);
-            mx[tid] = r;
-        }
-        __syncthreads();
-        lam = (float)pow2_ratio(mx[0], mx[1]);
+        h += l >> 32;
+        l &= 0xffffffffll;
+        dh.c1[tid] = (fx64)((unsigned long long)h << (31 - S)) + (l >> (S + 1));  // rounded down (S < 31)
     }
-    const int nf = (m > 0) ? 4 : 2;
-    for (int i = 0; i < nf; ++i) {
-        const int fid = (m > 0) ? i : (i == 0 ? 4 : 3);
-        if (m > 0 && (fid == 1 || fid == 2)) cheb_derivative_scan_dd(C, C, X, N, P.inv_a);  // C <- dC/ds
-        for (int j = tid; j <= K; j += nth) {
-            ddc v;
-            if (fid <= 2)
-                v = C[j];
-            else if (fid == 3)
-                v = (j < nc) ? cscale(dd_from_bits(y.th[(size_t)m * nc + j]), (j == 0) ? Cw0 : Cw) : zero;
-            else
-                v = ddc{C[j].x, dd_scale2(Y[j].x, lam)};
-            X[j] = (j == 0 || j == K) ? dd_scale2c(v, 2.f) : v;
+    F = fx_fft(X, Y, tw, 2, lg, false, 1, sc.back + v);
+    O = (F == X) ? Y : X;
+    // odd outputs: each thread a run of k, its increments, a scan over the CTA
+    const int chunk = (H + nth - 1) / nth;
+    const int lo = min(tid * chunk, H), hi = min(lo + chunk, H);
+    auto inc = [&](int k) {
+        const fxc p = F[k], q = F[K - k];
+        return fxc{(q.y >> 1) - (p.y >> 1), (p.x >> 1) - (q.x >> 1)};
+    };
+    fxc tot = fxc{0, 0};
+    for (int k = max(lo, 1); k < hi; ++k) tot = fx_add(tot, inc(k));
+    fxc sum = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const fx64 ux = __shfl_up_sync(0xffffffffu, sum.x, o), uy = __shfl_up_sync(0xffffffffu, sum.y, o);
+        if (lane >= o) sum = fx_add(sum, fxc{ux, uy});
+    }
+    if (lane == 31) {
+        dh.run[warp][0] = sum.x;
+        dh.run[warp][1] = sum.y;
+    }
+    __syncthreads();
+    // C_1 and the runs of the warps below: lane l those of warp l
+    fxc run = fxc{0, 0};
+    if (lane < warp) run = fxc{dh.run[lane][0], dh.run[lane][1]};
+#pragma unroll
+    for (int o = 1; o < NTHREADS_LX / 32; o <<= 1)
+        run = fx_add(run, fxc{__shfl_xor_sync(0xffffffffu, run.x, o), __shfl_xor_sync(0xffffffffu, run.y, o)});
+    run.x = __shfl_sync(0xffffffffu, run.x, 0) + dh.c1[0];
+    run.y = __shfl_sync(0xffffffffu, run.y, 0) + dh.c1[1];
+    run = fx_add(run, fx_sub(sum, tot));
+    for (int k = lo; k < hi; ++k) {
+        if (k > 0) run = fx_add(run, inc(k));
+        O[k] = run;
+    }
+    __syncthreads();
+}
+// 2^p times part of output C_k of vector v
+__device__ __forceinline__ double half_part(const FxScale& sc, int v, const fxc* F, const fxc* O, int K, int k, int part,
+                                            int p) {
+    const int kk = k >> 1;
+    fx64 c;
+    if (k & 1) {
+        c = part ? O[kk].y : O[kk].x;
+    } else {
+        const fxc* f0 = F + kk;
+        const fxc* f1 = F + (kk ? K - kk : 0);
+        c = part ? (f0->y >> 1) + (f1->y >> 1) : (f0->x >> 1) + (f1->x >> 1);
+    }
+    const int ex = (int)sc.e[v][part];
+    return fx_to(c, sc.S[v] + 1 - 1022 - (FX_BITS - 2) + p + ex, ex == 0x7ff);
+}
+
+// Chebyshev derivative of FP64 plain coefficients (the sums of cheb_derivative_scan)
+// by the whole CTA: warp w takes one index parity of one component (w & 3) in
+// the w >> 2-th of nw / 4 segments.  The exponents of d join vector v.  Ends
+// with a barrier.
+__device__ __forceinline__ void cheb_derivative_cta(const double2* c, double2* d, int n, int nd, double scale, DctHalf& dh,
+                                                    FxScale& sc, int v) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nseg = blockDim.x >> 7;
+    const int q = warp & 1, part = (warp >> 1) & 1, seg = warp >> 2;
+    const double* cs = reinterpret_cast<const double*>(c) + part;
+    double* ds = reinterpret_cast<double*>(d) + part;
+    const int len = (n - q + 1) / 2;
+    const int per = (len + 32 * nseg - 1) / (32 * nseg);
+    const int i0 = min((seg * 32 + lane) * per, len), i1 = min(i0 + per, len);
+    double acc = 0.0;
+    for (int i = i1 - 1; i >= i0; --i) {
+        const int k = 2 * i + q;
+        if (k > 0) {
+            acc = fma((double)(2 * k), cs[2 * k], acc);
+            ds[2 * (k - 1)] = acc;
         }
-        const ddc* Z = dct1_pair_dd(X, Y, P);
-        for (int k = tid; k < N; k += nth) {
-            const ddc gd = dd_scale2c(Z[k], 0.5f);  // value of the series at x_k
-            double2* out = G1 + g_index(k, 0, m, M);
-            ddc* outd = reinterpret_cast<ddc*>(out);  // the partial sums, double-float
-            if (fid == 0) {
-                const ddf h2 = h2_dd[k], is = is_dd[k];
-                out[0] = dd_compose(cmul_if(gd, fm));
-                outd[M] = cscale(gd, dd_mulf(s_dd[k], 3.f));
-                outd[2 * M] = cscale(gd, h2 * (is * is) * fm2 + ddf{6.f, 0.f});
-                if (PF) {
-                    const double2 g = dd_compose(gd);
-                    const double U = P.pump_ups[k];
-                    PF[k] = cadd(cscale(g, -U * (P.pump_cr[k] + dm * dm)), cmul_i(g, -U * dm * P.pump_ci[k]));
-                }
-            } else if (fid == 1) {
-                const ddf s_ = s_dd[k], h2 = h2_dd[k];
-                out[M] = dd_compose(csub(outd[M], cscale(gd, h2)));
-                outd[2 * M] = csub(outd[2 * M], cscale(gd, h2 * is_dd[k] - dd_mulf(s_, 5.f)));
-                if (PF) PF[k] = cadd(PF[k], cscale(dd_compose(gd), P.pump_ups[k] * 0.5 * P.s[k]));
-            } else if (fid == 2) {
-                const double2 o2 = dd_compose(csub(outd[2 * M], cscale(gd, h2_dd[k])));
-                out[2 * M] = o2;
-                if (PF) PF[k] = csub(PF[k], cscale(o2, P.pump_ups[k]));
-            } else if (fid == 3) {
-                out[3 * M] = dd_compose(gd);
+    }
+    double sfx = acc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double x = __shfl_down_sync(0xffffffffu, sfx, o);
+        if (lane + o < 32) sfx += x;
+    }
+    if (lane == 0) dh.tot[warp] = sfx;
+    __syncthreads();
+    double off = sfx - acc;
+    for (int s = seg + 1; s < nseg; ++s) off += dh.tot[4 * s + (warp & 3)];
+    unsigned ex = 0u;
+    for (int i = i0; i < i1; ++i) {
+        const int k = 2 * i + q;
+        if (k > 0) {
+            const double x = (ds[2 * (k - 1)] + off) * ((k == 1) ? 0.5 * scale : scale);
+            ds[2 * (k - 1)] = x;
+            const unsigned e = fx_exponent(x);
+            ex = max(ex, (k == 1 && e) ? e + 1u : e);
+        }
+    }
+    if (n <= nd && q == 0 && seg == 0 && lane == 0) ds[2 * (n - 1)] = 0.0;  // (unless d ends before it)
+    ex = __reduce_max_sync(0xffffffffu, min(ex, 0x7ffu));
+    if (lane == 0) atomicMax(&sc.e[v][part], ex);
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepParams P, VecSet y,
+                                                                         double2* __restrict__ G1) {
+    __shared__ FxScale sc;
+    __shared__ DctHalf dh;
+    const int m = P.m_lo + blockIdx.x;
+    const int K = P.K, N = P.n_r, nc = P.nc, M = P.M;
+    fxc* X = fx_shared;
+    fxc* Y = X + K;
+    double2* C = reinterpret_cast<double2*>(Y + K);  // plain coefficients of Psi and then of its derivatives (u_bar)
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const double Cw = P.cnorm, Cw0 = 0.5 * P.cnorm, dm = (double)m;
+    const double* ps = reinterpret_cast<const double*>(y.psi + (size_t)m * nc);
+    const double* th = reinterpret_cast<const double*>(y.th + (size_t)m * nc);
+    double* PF = P.pump ? reinterpret_cast<double*>(P.pump_F + (size_t)m * N) : nullptr;
+    fx_scale_clear(sc);
+    __syncthreads();
+    for (int b = 0; b < 2; ++b) {
+        unsigned ex = 0u;
+        for (int t = tid; t < 2 * nc; t += nth) {
+            const double w = (t < 2) ? Cw0 : Cw;
+            double x;
+            if (b) {
+                x = th[t] * w;
             } else {
-                const double2 g = dd_compose(gd);
-                const double is = P.inv_s[k];
-                out[0] = make_double2(0.0, 0.0);
-                out[M] = make_double2(g.x, 0.0);
-                out[2 * M] = make_double2(g.y / (double)lam + g.x * is, 0.0);
-                if (PF) {
-                    const double w0 = g.y / (double)lam + g.x * is;
-                    PF[k] = make_double2(P.pump_ups[k] * g.x * (1.0 + 0.5 * P.E * w0), 0.0);
+                x = (m > 0) ? ps[t] * w : (t & 1) ? 0.0 : y.u[t >> 1] * w;
+                reinterpret_cast<double*>(C)[t] = x;
+            }
+            const unsigned e = fx_exponent(x);
+            ex = max(ex, (t < 2 && e) ? min(e + 1u, 0x7ffu) : e);
+        }
+        fx_scale_max(sc, b ? 3 : 0, tid & 1, ex);
+    }
+    __syncthreads();
+    // vectors 0 Psi, 1 Psi', 2 Psi'' (u_bar, u_bar' for m = 0), 3 theta
+    for (int v = 0; v < 4; ++v) {
+        if (m == 0 && v == 2) continue;
+        double2* D = C;
+        if (v == 1 || v == 2) {
+            D = reinterpret_cast<double2*>(Y);
+            cheb_derivative_cta(C, D, nc, nc, P.inv_a, dh, sc, v);
+            for (int t = tid; t < 2 * nc; t += nth) reinterpret_cast<double*>(C)[t] = reinterpret_cast<double*>(D)[t];
+        }
+        fxc *F, *O;
+        if (v == 3)
+            dct1_half_fx(P, sc, dh, v, nc, true, X, Y, F, O, [&](int t) { return th[t] * ((t < 2) ? Cw0 : Cw); });
+        else
+            dct1_half_fx(P, sc, dh, v, nc, true, X, Y, F, O, [&](int t) { return reinterpret_cast<const double*>(D)[t]; });
+        for (int t = tid; t < 2 * N; t += nth) {
+            const int k = t >> 1, part = t & 1;
+            const double g = half_part(sc, v, F, O, K, k, part, -1);  // value of the series at x_k
+            double* out = reinterpret_cast<double*>(G1 + g_index(k, 0, m, M));  // fields 2M doubles apart
+            if (v == 3) {
+                out[6 * M + part] = g;
+                continue;
+            }
+            const double s = P.s[k], h2 = P.h2[k], is = P.inv_s[k];
+            if (m == 0) {
+                if (v == 0) {
+                    out[part] = 0.0;
+                    out[2 * M + part] = g;
+                    out[4 * M + part] = g * is;
+                } else {
+                    const double om = out[4 * M + part] + g;
+                    out[4 * M + part] = om;
+                    if (PF) PF[t] = part ? 0.0 : P.pump_ups[k] * out[2 * M] * (1.0 + (0.5 * P.E) * om);
                 }
+            } else if (v == 0) {
+                out[part ^ 1] = part ? -dm * g : dm * g;
+                out[2 * M + part] = (3.0 * s) * g;
+                out[4 * M + part] = fma(dm * dm * h2, is * is, 6.0) * g;
+                if (PF) {
+                    const double go = half_part(sc, v, F, O, K, k, part ^ 1, -1), U = P.pump_ups[k];
+                    const double ci = U * dm * P.pump_ci[k];
+                    PF[t] = fma(part ? -ci : ci, go, -U * fma(dm, dm, P.pump_cr[k]) * g);
+                }
+            } else if (v == 1) {
+                out[2 * M + part] = fma(-h2, g, out[2 * M + part]);
+                out[4 * M + part] = fma(-fma(-5.0, s, h2 * is), g, out[4 * M + part]);
+                if (PF) PF[t] = fma(P.pump_ups[k] * (0.5 * s), g, PF[t]);
+            } else {
+                const double om = fma(-h2, g, out[4 * M + part]);
+                out[4 * M + part] = om;
+                if (PF) PF[t] = fma(-P.pump_ups[k], om, PF[t]);
             }
         }
         __syncthreads();
     }
 }
 
-// k_grid_to_spec_lean with double-float transforms: grid values become
-// double-floats when loaded, the flux divergence is formed in double-float at
-// each radius from the double-float derivative (double-float tables of h^2 and
-// 1/s), and the analysed coefficients, with the explicit buoyancy added in
-// double-float, are FP64 again (in C, over the double-float data) before the
-// FP64 banded applies.  The pumping flux is read in FP64.
-__global__ void __launch_bounds__(NTHREADS_R, 2) k_grid_to_spec_lean_dd(StepParams P, const double2* __restrict__ G2,
+__global__ void __launch_bounds__(NTHREADS_LX, 2) k_grid_to_spec_lean_fx(StepParams P, const double2* __restrict__ G2,
                                                                          VecSet y, VecSet e) {
-    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ FxScale sc;
+    __shared__ DctHalf dh;
     const int m = P.m_lo + blockIdx.x;
     const int K = P.K, N = P.n_r, nc = P.nc, M = P.M;
-    ddc* X = reinterpret_cast<ddc*>(smraw);
-    ddc* C = X + N;
-    ddc* Y = C + N;
-    double2* Cd = reinterpret_cast<double2*>(C);  // the analysed coefficients, FP64
+    fxc* X = fx_shared;
+    fxc* Y = X + K;
+    double* C = reinterpret_cast<double*>(Y + K);  // n_r complex values
+    double* D = reinterpret_cast<double*>(Y);      // derivative coefficients 0 .. K-1 (the last one is zero)
     const int tid = threadIdx.x, nth = blockDim.x;
-    const double dm = (double)m;
-    const ddf hc = dd_from(0.5 * P.cnorm);
-    const float iK = 1.f / (float)K, hK = 0.5f / (float)K;  // K a power of two: exact
-    const float fm = (float)m;                               // exact: m < 2^24
-    const double2* PF = P.pump ? P.pump_F + (size_t)m * N : nullptr;
-    const ddf bfac = dd_from(P.Ra / P.Pr * (double)m / P.s_o);
-    const ddf* h2_dd = reinterpret_cast<const ddf*>(P.h2_dd);
-    const ddf* is_dd = reinterpret_cast<const ddf*>(P.inv_s_dd);
+    const double dm = (double)m, hc = 0.5 * P.cnorm;
+    const int lgK = 31 - __clz(K);
+    const double* PF = P.pump ? reinterpret_cast<const double*>(P.pump_F + (size_t)m * N) : nullptr;
+    const double bfac = P.Ra / P.Pr * dm / P.s_o;
+    const double* g2 = reinterpret_cast<const double*>(G2);
+    const double* th = reinterpret_cast<const double*>(y.th + (size_t)m * nc);
+    const double* ps = reinterpret_cast<const double*>(y.psi + (size_t)m * nc);
+    double* eps = reinterpret_cast<double*>(e.psi + (size_t)m * nc);
+    double* eth = reinterpret_cast<double*>(e.th + (size_t)m * nc);
+    fx_scale_clear(sc);
+    __syncthreads();
+    fxc *F, *O;
+    auto coef = [&](int t) { return C[t]; };
+    // field 0: N_omega (m >= 1) or N_u (m = 0); field 1: N_theta; vectors 3 fld ..: the flux, its
+    // derivative, N
     for (int fld = 0; fld < 2; ++fld) {
-        ddc* W = X;
+        const int v = 3 * fld;
+        unsigned ex = 0u;
         if (fld == 1 || m > 0) {
-            const int f = (fld == 0) ? 0 : 2;
-            for (int j = tid; j <= K; j += nth) X[j] = cscale(dd_from_bits(G2[g_index(j, f, m, M)]), h2_dd[j]);
-            const ddc* Z = dct1_pair_dd(X, Y, P);
-            for (int n = tid; n <= K; n += nth) C[n] = dd_scale2c(Z[n], (n == 0 || n == K) ? hK : iK);
+            for (int t = tid; t < 2 * N; t += nth) {
+                const double x = g2[2 * (size_t)g_index(t >> 1, 2 * fld, m, M) + (t & 1)] * P.h2[t >> 1];
+                C[t] = x;
+                ex = max(ex, fx_exponent(x));
+            }
+            fx_scale_max(sc, v, tid & 1, ex);
             __syncthreads();
-            cheb_derivative_scan_dd(C, C, X, N, P.inv_a);
-            for (int j = tid; j <= K; j += nth) X[j] = (j == 0 || j == K) ? dd_scale2c(C[j], 2.f) : C[j];
-            const ddc* D = dct1_pair_dd(X, Y, P);
-            W = (D == X) ? Y : X;
-            for (int k = tid; k <= K; k += nth) {
-                const ddc dF = dd_scale2c(D[k], 0.5f);
-                const ddf is = is_dd[k];
-                ddc val;
-                if (fld == 0) {
-                    val = cscale(cadd(dF, cmul_if(dd_from_bits(G2[g_index(k, 1, m, M)]), fm)), is);
-                    if (PF) val = csub(val, dd_from_bits(PF[k]));
-                } else {
-                    val = csub(cscale(cadd(dF, cmul_if(dd_from_bits(G2[g_index(k, 3, m, M)]), fm)), is),
-                               dd_from_bits(G2[g_index(k, 2, m, M)]));
-                }
-                W[k] = val;
+            dct1_half_fx(P, sc, dh, v, N, false, X, Y, F, O, coef);
+            for (int t = tid; t < 2 * N; t += nth) {
+                const int n = t >> 1;
+                C[t] = half_part(sc, v, F, O, K, n, t & 1, (n == 0 || n == K) ? -lgK - 1 : -lgK);
             }
-        } else {  // N_u = (h^2/s) [v omega]_0 (+ pumping)
-            for (int k = tid; k <= K; k += nth) {
-                ddc val = cscale(dd_from_bits(G2[g_index(k, 0, m, M)]), h2_dd[k] * is_dd[k]);
-                if (PF) val = cadd(val, dd_from_bits(PF[k]));
-                W[k] = val;
-            }
+            __syncthreads();
+            cheb_derivative_cta(reinterpret_cast<double2*>(C), reinterpret_cast<double2*>(D), N, K, P.inv_a, dh, sc, v + 1);
+            dct1_half_fx(P, sc, dh, v + 1, K, true, X, Y, F, O, [&](int t) { return D[t]; });
         }
-        const ddc* Z = dct1_pair_dd(W, (W == X) ? Y : X, P);
-        const bool buoy = (fld == 0 && m > 0 && !P.buoy_imp);
-        // Z lives in X or Y, never in C: the FP64 coefficients overwrite C
-        for (int n = tid; n < nc; n += nth) {
-            const ddc v = cscale(Z[n], hc);
-            if (buoy) {
-                const ddc t = dd_from_bits(y.th[(size_t)m * nc + n]);
-                Cd[n] = dd_compose(ddc{v.x - t.y * bfac, v.y + t.x * bfac});  // + i bfac theta
+        ex = 0u;
+        for (int t = tid; t < 2 * N; t += nth) {
+            const int k = t >> 1, part = t & 1;
+            const double is = P.inv_s[k];
+            const double* g = g2 + 2 * (size_t)g_index(k, 0, m, M);  // fields 2M doubles apart
+            double val;
+            if (fld == 0 && m == 0) {
+                val = g[part] * (P.h2[k] * is);
+                if (PF) val += PF[t];
             } else {
-                Cd[n] = dd_compose(v);
+                const double dF = half_part(sc, v + 1, F, O, K, k, part, -1);
+                const double w = fma(part ? dm : -dm, g[(fld ? 6 : 2) * M + (part ^ 1)], dF);
+                if (fld == 0) {
+                    val = w * is;
+                    if (PF) val -= PF[t];
+                } else {
+                    val = fma(w, is, -g[4 * M + part]);
+                }
             }
+            C[t] = val;
+            ex = max(ex, fx_exponent(val));
+        }
+        fx_scale_max(sc, v + 2, tid & 1, ex);
+        __syncthreads();
+        // Eq. icheb of the grid values, truncated to n < nc, N_omega_hat with the buoyancy
+        dct1_half_fx(P, sc, dh, v + 2, N, false, X, Y, F, O, coef);
+        const bool buoy = (fld == 0 && m > 0 && !P.buoy_imp);
+        for (int t = tid; t < 2 * nc; t += nth) {
+            const int part = t & 1;
+            double x = half_part(sc, v + 2, F, O, K, t >> 1, part, 0) * hc;
+            if (buoy) x = fma(part ? bfac : -bfac, th[t ^ 1], x);
+            C[t] = x;
         }
         __syncthreads();
-        for (int k = tid; k < nc; k += nth) {
+        for (int t = tid; t < 2 * nc; t += nth) {
+            const int k = t >> 1, part = t & 1;
+            double x = 0.0;
             if (fld == 0) {
                 if (m > 0) {
-                    double2 ep = make_double2(0.0, 0.0);
-                    if (k >= 4) ep = band_row<8>(P.ops.band[OP_C], Cd, k, nc);
-                    e.psi[(size_t)m * nc + k] = ep;
-                } else {
-                    e.psi[k] = make_double2(0.0, 0.0);
-                    e.u[k] = (k >= 2) ? -band_row<4>(P.ops.band[OP_D], Cd, k, nc).x : 0.0;
+                    if (k >= 4) x = band_part<8>(P.ops.band[OP_C], C + part, k, nc);
+                } else if (part == 0) {
+                    e.u[k] = (k >= 2) ? -band_part<4>(P.ops.band[OP_D], C, k, nc) : 0.0;
                 }
+                eps[t] = x;
             } else {
-                double2 et = make_double2(0.0, 0.0);
                 if (k >= 2) {
-                    const double2 dn = band_row<4>(P.ops.band[OP_D], Cd, k, nc);
+                    x = -band_part<4>(P.ops.band[OP_D], C + part, k, nc);
                     if (m > 0) {
-                        const double2 gp = band_row<4>(P.ops.band[OP_G], y.psi + (size_t)m * nc, k, nc);
-                        et = csub(cmul_i(gp, -P.tc * dm), dn);
-                    } else {
-                        et = cscale(dn, -1.0);
+                        const double gp = band_part<4>(P.ops.band[OP_G], ps + (part ^ 1), k, nc);
+                        x = fma(part ? -P.tc * dm : P.tc * dm, gp, x);
                     }
                 }
-                e.th[(size_t)m * nc + k] = et;
+                eth[t] = x;
             }
         }
         __syncthreads();
@@ -1642,28 +2199,35 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, cuda
     }
     if (lean_radial(P)) {
         const size_t sm = smem_radial_lean(P);
-        auto kern = radial_dd(P) ? k_spec_to_grid_lean_dd : k_spec_to_grid_lean<double2>;
+        const bool fx = radial_fx(P);
+        auto kern = fx ? k_spec_to_grid_lean_fx : k_spec_to_grid_lean<double2>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        kern<<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, G1);
+        kern<<<slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st>>>(P, y, G1);
         return cudaGetLastError();
     }
-    return P.fp32 ? spec_to_grid_t<float2>(P, y, G1, st) : spec_to_grid_t<double2>(P, y, G1, st);
+    if (P.fp32) return spec_to_grid_t<float2>(P, y, G1, st);
+    const size_t sm = smem_spec_to_grid(P);
+    cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (err != cudaSuccess) return err;
+    k_spec_to_grid_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, y, G1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_phi_products(const StepParams& P, const double2* G1, double2* G2, cudaStream_t st) {
     if (P.fp32) return phi_products_t<float2>(P, G1, G2, st);
-    if (P.phi_dd && P.plan_p.twdd) {
-        const int nth = phi_threads(P);
+    if (P.phi_dd && P.fx_p) {
+        const int nth = phi_threads_fx(P);
         if (P.n_phi > nth * MAXPER || nth > 512) return cudaErrorInvalidValue;
         // the batched pair of transforms needs twice the buffers (n_phi <= 3072)
         cudaError_t err;
         const int pair = phi_pair(P, err);
         if (err != cudaSuccess) return err;
         const size_t sm = (pair ? 2 : 1) * smem_phi_products(P);
-        err = cudaFuncSetAttribute(k_phi_products_dd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        auto kern = pair ? k_phi_products_fx<true> : k_phi_products_fx<false>;
+        err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        k_phi_products_dd<<<slab_radii(P), nth, sm, st>>>(P, G1, G2, pair);
+        kern<<<slab_radii(P), nth, sm, st>>>(P, G1, G2);
         return cudaGetLastError();
     }
     return phi_products_t<double2>(P, G1, G2, st);
@@ -1680,13 +2244,19 @@ cudaError_t launch_grid_to_spec(const StepParams& P, const double2* G2, VecSet y
     }
     if (lean_radial(P)) {
         const size_t sm = smem_radial_lean(P);
-        auto kern = radial_dd(P) ? k_grid_to_spec_lean_dd : k_grid_to_spec_lean<double2>;
+        const bool fx = radial_fx(P);
+        auto kern = fx ? k_grid_to_spec_lean_fx : k_grid_to_spec_lean<double2>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        kern<<<slab_modes(P), NTHREADS_R, sm, st>>>(P, G2, y, e);
+        kern<<<slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st>>>(P, G2, y, e);
         return cudaGetLastError();
     }
-    return P.fp32 ? grid_to_spec_t<float2>(P, G2, y, e, st) : grid_to_spec_t<double2>(P, G2, y, e, st);
+    if (P.fp32) return grid_to_spec_t<float2>(P, G2, y, e, st);
+    const size_t sm = smem_grid_to_spec(P);
+    cudaError_t err = cudaFuncSetAttribute(k_grid_to_spec_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (err != cudaSuccess) return err;
+    k_grid_to_spec_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, G2, y, e);
+    return cudaGetLastError();
 }
 
 }  // namespace pz

@@ -17,12 +17,11 @@ struct FftPlan {
     int L;
     int npass;
     int tws;  // stride of the twiddle table: tw[tws * j] = exp(-2 pi i j / L)
-    int radix[MAX_PASSES];   // FP64 and double-float transforms: radix 3, then 4s and 2s
+    int radix[MAX_PASSES];   // FP64 transforms: radix 3, then 4s and 2s
     int npass8;
     int radix8[MAX_PASSES];  // FP32 transforms: radix 3, then 8s, 4s and 2s (fewer passes)
     const double2* tw;  // tw[j] = exp(-2 pi i j / L), j < L
     const float2* twf;  // the same, rounded to FP32 (mixed-precision explicit stage)
-    const float4* twdd; // the same as double-float pairs (hi, lo) of (re, im), or null
 };
 
 // One set of per-field vectors: Psi and theta complex [M][nc], u real [nc]; the
@@ -115,10 +114,11 @@ struct StepParams {
     const double* h2;     // [n_r]
     const double* inv_s;  // [n_r]
     const float *s_f, *h2_f, *inv_s_f;  // the same in FP32 (mixed-precision explicit stage)
-    const float2 *s_dd, *h2_dd, *inv_s_dd;  // the same as double-floats (hi, lo): lean radial kernels
     FftPlan plan_r;       // length 2K (radial DCT-I as an FFT of the even extension)
     FftPlan plan_h;       // length K, plan_r's twiddles at stride 2 (radial DCT-I, dct1_batched)
     FftPlan plan_p;       // length n_phi (azimuthal)
+    // twiddles exp(-2 pi i j/L) in fixed point (fixfft.cuh's fxw): L = 2K and n_phi
+    const int4 *fx_r, *fx_p;
     DevOps ops;
     // explicit stage in FP32 (option "precision" = mixed): 1 when selected
     int fp32;
@@ -142,8 +142,8 @@ struct StepParams {
     // implicit buoyancy (option "buoy_implicit", Section 4): 1 when the buoyancy
     // term is part of the implicit operator of the streamfunction equation
     int buoy_imp;
-    // azimuthal products of the FP64 explicit stage in double-float arithmetic on
-    // the FP32 pipe (option "azimuthal_dd"): 1 when selected (plan_p.twdd set)
+    // azimuthal products of the FP64 explicit stage in fixed point (option
+    // "azimuthal_dd"): 1 when selected (fx_p set)
     int phi_dd;
     double2* pump_F;
     // m-slab decomposition (pizza_set_slab): the per-mode kernels (a1, a3, solve)
@@ -157,10 +157,10 @@ struct StepParams {
     // mode (option "solve_roles"): 1 always, 0 never, -1 (default) from N_c > 600
     int solve_roles;
     // FP64 radial kernels in the three-array layout (option "radial_lean"):
-    // 1 from n_r = 129 (the half-length DCT-I), 0 never, -1 (default) from n_r = 513
+    // 1 from n_r = 129 (the half-length DCT-I), 0 never, -1 (default) from n_r = 1025
     int radial_lean;
-    // double-float DCT-I and derivative scans in the lean radial kernels (option
-    // "radial_dd"): 1 always, 0 never, -1 (default) from n_r = 513
+    // fixed-point DCT-I in the lean radial kernels (option "radial_dd"): 1 always,
+    // 0 never (FP64), -1 (default) from n_r = 1025
     int radial_dd;
     // streamfunction block chains of the solve in double-float arithmetic
     // (option "psi_chain_dd", explicit buoyancy): 1 always, 0 never, -1
@@ -222,6 +222,8 @@ void set_global_error(const char* msg);
 // Stockham radix plan (3 * 2^j or 2^j) and twiddle table exp(-2 pi i j/L), j < L.
 bool make_fft_plan(int L, FftPlan& pl);
 std::vector<double2> fft_twiddles(int L);
+// the same in units of 2^-62, components split as hi 2^32 + lo (fixfft.cuh's fxw)
+std::vector<int4> fft_twiddles_fx(int L);
 
 size_t smem_spec_to_grid(const StepParams& P);
 size_t smem_adj_grid_to_spec(const StepParams& P);
