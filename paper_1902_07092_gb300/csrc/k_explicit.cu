@@ -609,7 +609,7 @@ __device__ __forceinline__ fxc* dct1_fx(const StepParams& P, FxScale& sc, int v0
             const int j = t >> 1, part = t & 1;
             const int e = (int)sc.e[v0 + i][part];
             fx64 q = 0;
-            if (j < n && e != 0x7ff) {  // (a block with an infinity or NaN: outputs are NaN)
+            if (j < n && e && e != 0x7ff) {  // (zero, or with an infinity or NaN in the block: outputs are NaN)
                 q = fx_from(val(i, t), e);
                 if (twice && (j == 0 || j == K)) q = 2 * q;  // its exponent entered e plus one
             }
@@ -965,13 +965,10 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P
 // integers.  Each field is normalised by the exponent of its largest
 // coefficient on load; the physical values of each field are shifted up by the
 // free leading bits of their largest before the products, whose 60-bit results
-// are transformed back.  FP64 is used for conversions only.  The mean of a product
-// (m = 0) needs no separate sum: the transforms are accurate to about 2^-53 of
-// their largest value (the double-float products needed an FP64 one; the zonal
-// explicit term at 2049 x 6144 is now 1.1e-11 from an FP64 evaluation, 4.9e-11
-// then).  Bound by instruction issue (43-54 % of the slots; 16 warps an SM at
-// n_phi = 6144, where two buffers fill its shared memory).  Against the
-// double-float kernel: 257 x 768 37 -> 24.4 us, 33 x 96 22 -> 12.2, 1025 x 3072
+// are transformed back.  FP64 is used for conversions only.  The means of the
+// products (m = 0), which cancel, are summed over the modes in FP64.  Bound by
+// instruction issue (43-54 % of the slots; 16 warps an SM at n_phi = 6144, where
+// two buffers fill its shared memory).  Against the double-float kernel: 257 x 768 37 -> 24.4 us, 33 x 96 22 -> 12.2, 1025 x 3072
 // 443 -> 313, 2049 x 6144 1706 -> 1265 us.
 // ---------------------------------------------------------------------------
 struct PhiScale {
@@ -980,6 +977,8 @@ struct PhiScale {
     unsigned l1[4];     // 1-norms of the packed spectra, then of the packed products
     unsigned back[4];
     int S[4];
+    double mean[16][4];  // per warp: sums of the four products over the modes
+    double mean0[4];     // the products' means
     double cfl[2 * 16];
 };
 
@@ -998,32 +997,25 @@ __device__ __forceinline__ fx64 fx_mul62(fx64 a, fx64 b) {
 }
 __device__ __forceinline__ unsigned fx_top(fx64 a) { return (unsigned)((a < 0 ? ~a : a) >> 32); }
 
-// the pair of fields (f, f + 1) packed as a + i b into Z, components exchanged
-// (fx_fft then runs the backward transform); 1-norm into l1
-__device__ __forceinline__ void phi_pack(const double2* __restrict__ src, int M, int Pn, int n_m, unsigned ea, unsigned eb,
-                                         fxc* Z, unsigned* l1) {
-    unsigned w = 0u;
-    for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
-        const double2 a = src[m], b = src[M + m];
-        fxc p, q;
-        p.x = (ea == 0x7ff) ? 0 : fx_from(a.x, ea) >> 1;  // below 2^59: the packed values below 2^60
-        p.y = (ea == 0x7ff) ? 0 : fx_from(a.y, ea) >> 1;
-        q.x = (eb == 0x7ff) ? 0 : fx_from(b.x, eb) >> 1;
-        q.y = (eb == 0x7ff) ? 0 : fx_from(b.y, eb) >> 1;
-        if (m == 0) {
-            Z[0] = fxc{q.x, p.x};
-            w += fx_l1_part(p.x) + fx_l1_part(q.x);
-        } else {
-            const fxc z1 = fxc{p.y + q.x, p.x - q.y};  // (im, re) of a + i b
-            const fxc z2 = fxc{q.x - p.y, p.x + q.y};  // of conj(a) + i conj(b)
-            Z[m] = z1;
-            Z[Pn - m] = z2;
-            w += fx_l1_part(z1.x) + fx_l1_part(z1.y) + fx_l1_part(z2.x) + fx_l1_part(z2.y);
-        }
+// a field's coefficient in fixed point, components below 2^FX_BITS
+__device__ __forceinline__ fxc phi_coef(double2 v, unsigned e) {
+    return (e == 0x7ff) ? fxc{0, 0} : fxc{fx_from(v.x, (int)e), fx_from(v.y, (int)e)};
+}
+// mode m of the fields a and b packed as a + i b into Z, halved (the packed values
+// stay below 2^FX_BITS) and with the components exchanged (fx_fft then runs the
+// backward transform); returns the 1-norm written
+__device__ __forceinline__ unsigned phi_pack(fxc a, fxc b, int m, int Pn, fxc* Z) {
+    a = fx_shr(a, 1);
+    b = fx_shr(b, 1);
+    if (m == 0) {
+        Z[0] = fxc{b.x, a.x};
+        return fx_l1_part(a.x) + fx_l1_part(b.x);
     }
-    for (int j = n_m + 1 + threadIdx.x; j < Pn - n_m; j += blockDim.x) Z[j] = fxc{0, 0};
-    w = __reduce_add_sync(0xffffffffu, w);
-    if ((threadIdx.x & 31) == 0) atomicAdd(l1, w);
+    const fxc z1 = fxc{a.y + b.x, a.x - b.y};  // (im, re) of a + i b
+    const fxc z2 = fxc{b.x - a.y, a.x + b.y};  // of conj(a) + i conj(b)
+    Z[m] = z1;
+    Z[Pn - m] = z2;
+    return fx_l1_part(z1.x) + fx_l1_part(z1.y) + fx_l1_part(z2.x) + fx_l1_part(z2.y);
 }
 // the spectra of a + i b from its transform Y (scaled by 2^-S), over n_phi
 __device__ __forceinline__ void phi_split(const fxc* Y, double2* __restrict__ dst, int M, int Pn, int n_m, bool three,
@@ -1093,23 +1085,57 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
     fxc* Y = X + (PAIR ? 2 : 1) * Pn;
     const double2* src = G1 + g_index(k, 0, 0, M);
     double2* dst = G2 + g_index(k, 0, 0, M);
-    if (tid < (int)(offsetof(PhiScale, cfl) / 4)) reinterpret_cast<unsigned*>(&sc)[tid] = 0u;
+    if (tid < (int)(offsetof(PhiScale, mean) / 4)) reinterpret_cast<unsigned*>(&sc)[tid] = 0u;
     __syncthreads();
     {
+        // exponents of the fields and, in FP64 (its pipe is idle here), the means of the
+        // products, a_0 b_0 + 2 sum_{m >= 1} Re(a_m conj(b_m)), exact for these band-limited fields:
+        // they cancel (the zonal forcing [v omega]_0 down to 1e-7 of its terms), where even a
+        // few units of rounding of the transforms' m = 0 entries show
         unsigned ex[4] = {0u, 0u, 0u, 0u};
-        for (int m = tid; m <= n_m; m += nth)
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int m = tid; m <= n_m; m += nth) {
+            double2 f[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const double2 v = src[q * M + m];
-                ex[q] = max(ex[q], max(fx_exponent(v.x), fx_exponent(v.y)));
+                f[q] = src[q * M + m];
+                ex[q] = max(ex[q], max(fx_exponent(f[q].x), fx_exponent(f[q].y)));
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {  // (v, omega), (u_phi, omega), (v, theta), (u_phi, theta)
+                const double2 a = f[q & 1], b = f[2 + (q >> 1)];
+                acc[q] = m ? fma(a.x, b.x, fma(a.y, b.y, acc[q])) : 0.5 * (a.x * b.x);
+            }
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             ex[q] = __reduce_max_sync(0xffffffffu, ex[q]);
             if ((tid & 31) == 0) atomicMax(&sc.e[q], ex[q]);
         }
+        // four sums over the warp: halves exchanged twice, then lanes of equal l >> 3 added up
+        const int lane = tid & 31;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int o = 16 >> s, half = 2 >> s;
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < half; ++i) {
+                const double send = up ? acc[i] : acc[i + half];
+                acc[i] = (up ? acc[i + half] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+        if ((lane & 7) == 0) sc.mean[tid >> 5][lane >> 3] = acc[0];
     }
     __syncthreads();
+    if (tid >= nth - 32) {  // one warp: lane 4 w + q adds warps w and w + 8 of product q
+        const int q = tid & 3, w = (tid & 31) >> 2, nw = nth >> 5;
+        double v = (w < nw ? sc.mean[w][q] : 0.0) + (w + 8 < nw ? sc.mean[w + 8][q] : 0.0);
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (w == 0) sc.mean0[q] = 2.0 * v;
+    }
     const unsigned ev = sc.e[0], eu = sc.e[1], ew = sc.e[2], et = sc.e[3];
     // schedules of transforms i0 .. i0 + n - 1 from their 1-norms
     auto schedule = [&](int i0, int n) {
@@ -1131,9 +1157,24 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
     };
     fxc reg[PAIR ? 1 : MAXPER];
     const fxc *R1 = nullptr, *R2 = nullptr;
+    for (int j = n_m + 1 + tid; j < Pn - n_m; j += nth) {
+        X[j] = fxc{0, 0};
+        if (PAIR) X[Pn + j] = fxc{0, 0};
+    }
+    {
+        unsigned w0 = 0u, w1 = 0u;
+        for (int m = tid; m <= n_m; m += nth) {
+            w0 += phi_pack(phi_coef(src[m], ev), phi_coef(src[M + m], eu), m, Pn, X);
+            if (PAIR) w1 += phi_pack(phi_coef(src[2 * M + m], ew), phi_coef(src[3 * M + m], et), m, Pn, X + Pn);
+        }
+        w0 = __reduce_add_sync(0xffffffffu, w0);
+        if ((tid & 31) == 0) atomicAdd(&sc.l1[0], w0);
+        if (PAIR) {
+            w1 = __reduce_add_sync(0xffffffffu, w1);
+            if ((tid & 31) == 0) atomicAdd(&sc.l1[1], w1);
+        }
+    }
     if (PAIR) {
-        phi_pack(src, M, Pn, n_m, ev, eu, X, &sc.l1[0]);
-        phi_pack(src + 2 * M, M, Pn, n_m, ew, et, X + Pn, &sc.l1[1]);
         schedule(0, 2);
         R1 = fx_fft(X, Y, tw, 1, lg, three, 2, sc.back);
         R2 = R1 + Pn;
@@ -1147,7 +1188,14 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         }
     } else {
         for (int i = 0; i < 2; ++i) {
-            phi_pack(src + 2 * i * M, M, Pn, n_m, i ? ew : ev, i ? et : eu, X, &sc.l1[i]);
+            if (i) {
+                unsigned w1 = 0u;
+                for (int m = tid; m <= n_m; m += nth)
+                    w1 += phi_pack(phi_coef(src[2 * M + m], ew), phi_coef(src[3 * M + m], et), m, Pn, X);
+                for (int j = n_m + 1 + tid; j < Pn - n_m; j += nth) X[j] = fxc{0, 0};
+                w1 = __reduce_add_sync(0xffffffffu, w1);
+                if ((tid & 31) == 0) atomicAdd(&sc.l1[1], w1);
+            }
             schedule(i, 1);
             R2 = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + i);
             unsigned x = 0u, yv = 0u;
@@ -1198,8 +1246,13 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
             atomicAdd(&sc.l1[3], l1);
         }
     };
-    const int ln = three ? -(lg + 1) : -lg;  // 1/n_phi
     const bool bv = ev == 0x7ff, bu = eu == 0x7ff, bw = ew == 0x7ff, bt = et == 0x7ff;
+    const int ln = three ? -(lg + 1) : -lg;  // 1/n_phi
+    // after the stores of phi_split: the means in the place of the transforms' m = 0 entries
+    auto means = [&]() {
+        __syncthreads();
+        if (tid < 4) dst[tid * M] = make_double2(sc.mean0[tid], 0.0);
+    };
     if (PAIR) {
         fxc* O = (R1 == X) ? Y : X;
         for (int j = tid; j < Pn; j += nth) {
@@ -1214,6 +1267,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         phi_split(Z, dst, M, Pn, n_m, three, xv + xw + 62 + sc.S[2] + ln, xu + xw + 62 + sc.S[2] + ln, bv || bw, bu || bw);
         phi_split(Z + Pn, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln,
                   bv || bt, bu || bt);
+        means();
     } else {
         fxc* O = (R2 == X) ? Y : X;
 #pragma unroll
@@ -1238,6 +1292,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         Z = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + 3);
         phi_split(Z, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln, bv || bt,
                   bu || bt);
+        means();
     }
 }
 
@@ -2200,8 +2255,9 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, cuda
     if (lean_radial(P)) {
         const size_t sm = smem_radial_lean(P);
         const bool fx = radial_fx(P);
-        auto kern = fx ? k_spec_to_grid_lean_fx : k_spec_to_grid_lean<double2>;
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t err = fx ? cudaFuncSetAttribute(k_spec_to_grid_lean_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
+                             : cudaFuncSetAttribute(k_spec_to_grid_lean<double2>,
+                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
         kern<<<slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st>>>(P, y, G1);
         return cudaGetLastError();
