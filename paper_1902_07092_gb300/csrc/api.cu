@@ -778,7 +778,7 @@ int explicit_eval(pizza_ctx* ctx, VecSet y, VecSet e) {
         double2* g1 = static_cast<double2*>(ctx->slab.g1);
         double2* g2 = static_cast<double2*>(ctx->slab.g2);
         const int eb = ctx->P.fp32 ? 8 : 16;
-        CK(timed_launch(ctx, 0, [&] { return launch_spec_to_grid(ctx->P, y, g1, ctx->stream); }));
+        CK(timed_launch(ctx, 0, [&] { return launch_spec_to_grid(ctx->P, y, g1, ctx->G2, ctx->stream); }));
         if (int rc = ctx->slab.fn(ctx->slab.user, 1, g1, eb, ctx->stream))
             return fail(ctx, PIZZA_ECUDA, "slab exchange after the synthesis failed (%d)", rc);
         CK(timed_launch(ctx, 1, [&] { return launch_phi_products(ctx->P, g1, g2, ctx->stream); }));
@@ -787,7 +787,7 @@ int explicit_eval(pizza_ctx* ctx, VecSet y, VecSet e) {
         CK(timed_launch(ctx, 2, [&] { return launch_grid_to_spec(ctx->P, g2, y, e, ctx->stream); }));
         return PIZZA_OK;
     }
-    CK(timed_launch(ctx, 0, [&] { return launch_spec_to_grid(ctx->P, y, ctx->G1, ctx->stream); }));
+    CK(timed_launch(ctx, 0, [&] { return launch_spec_to_grid(ctx->P, y, ctx->G1, ctx->G2, ctx->stream); }));
     CK(timed_launch(ctx, 1, [&] { return launch_phi_products(ctx->P, ctx->G1, ctx->G2, ctx->stream); }));
     CK(timed_launch(ctx, 2, [&] { return launch_grid_to_spec(ctx->P, ctx->G2, y, e, ctx->stream); }));
     return PIZZA_OK;
@@ -2038,7 +2038,7 @@ int pizza_diagnostics(pizza_ctx* ctx, pizza_diag* out) {
     if (ctx->coll)
         CK(launch_coll_spec_to_grid(P64, y, ctx->G1, ctx->stream));
     else
-        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->stream));
+        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->G2, ctx->stream));
     CK(launch_diagnostics(P64, ctx->G1, ctx->diag_q, ctx->diag_modes, ctx->diag_radii, ctx->stream));
     std::vector<double> ms(2 * (size_t)M), rm(2 * (size_t)n_r);
     std::vector<double2> th0(nc);
@@ -2098,7 +2098,7 @@ int pizza_get_grid(pizza_ctx* ctx, double* us, double* uphi, double* omega, doub
     if (ctx->coll)
         CK(launch_coll_spec_to_grid(P64, y, ctx->G1, ctx->stream));
     else
-        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->stream));
+        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->G2, ctx->stream));
     double* g = ctx->grid_out;
     CK(launch_phi_fields(P64, ctx->G1, g, g + n, g + 2 * n, g + 3 * n, ctx->stream));
     double* outs[4] = {us, uphi, omega, theta};
@@ -2179,7 +2179,7 @@ int pizza_adjoint_step(pizza_ctx* ctx, const double* g_theta, const double* g_ps
     if (i < a.seg_g1n)
         g1 = a.seg_G1[i];  // recorded by the recomputation
     else
-        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->stream));
+        CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->G2, ctx->stream));
     CK(launch_adj_explicit(P64, a.w, y, a.lam, g1, a.Gb2, a.Gb1, a.ra, ctx->stream));
     CK(launch_ra_accumulate(a.ra, ctx->M, a.dRa_dev, ctx->stream));
     a.rcur = 1 - a.rcur;
@@ -2221,7 +2221,7 @@ int pizza_explicit_adjoint(pizza_ctx* ctx, const double* e_psi_bar, const double
     VecSet y = ctx->vec[ctx->ys[0]];
     StepParams P64 = ctx->P;
     P64.fp32 = 0;
-    CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->stream));
+    CK(launch_spec_to_grid(P64, y, ctx->G1, ctx->G2, ctx->stream));
     CK(launch_adj_explicit(P64, a.w, y, a.g, ctx->G1, a.Gb2, a.Gb1, a.ra, ctx->stream));
     const size_t vsz = (size_t)ctx->M * ctx->nc;
     if (theta_bar) CK(cudaMemcpyAsync(theta_bar, a.g.th, vsz * 16, cudaMemcpyDefault, ctx->stream));

@@ -54,6 +54,10 @@ inline int phi_threads_fx(const StepParams& P) {
 //   m = 0:  v = 0, u_phi = u_bar, omega = u_bar' + u_bar/s
 // (Section 3.2: u_s = (h^2/s) dPsi/dphi, u_phi = u_bar - h^2 dPsi/ds + 3 s Psi,
 //  omega = (1/s) d(s u_bar)/ds - L_I Psi.)
+// u_phi and omega are built up over the passes of Psi, Psi' and Psi''.  Their partial
+// sums wait in W[m][2][n_r] (contiguous for a mode; the grid array's columns are
+// strided by 4 M entries, and rereading and rewriting those took 175 of the 305
+// thousand cycles of a mode at 2049 x 6144): the grid array is only written, once.
 // With Ekman pumping it also writes P.pump_F[m][k]: for m >= 1 the approximate
 // pumping of Eq. approx_pump,
 //   F_eps = Ups_eps [ -omega + (s/2) Psi' - (3 s^2/(2 h_eps^2) + m^2 + i m 5 s_o/(2 h_eps)) Psi ]
@@ -62,7 +66,7 @@ inline int phi_threads_fx(const StepParams& P) {
 // uphicoll.
 // ---------------------------------------------------------------------------
 template <class T>
-__global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSet y, T* __restrict__ G1) {
+__global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSet y, T* __restrict__ G1, T* __restrict__ W) {
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
@@ -133,6 +137,8 @@ __global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSe
     }
     const RT dm = (RT)m;
     T* PF = P.pump ? reinterpret_cast<T*>(P.pump_F) + (size_t)m * N : nullptr;
+    T* wu = W + (size_t)m * 2 * N;
+    T* wo = wu + N;
     for (int f0 = 0; f0 < nf; f0 += NB) {
         const int nb = min(NB, nf - f0);
         for (int b = 0; b < nb; ++b) {
@@ -165,19 +171,20 @@ __global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSe
                 // out[0] = v, out[M] = u_phi, out[2M] = omega, out[3M] = theta
                 if (fid == 0) {
                     out[0] = cmul_i(g, dm);
-                    out[M] = cscale(g, (RT)3 * s);
-                    out[2 * M] = cscale(g, (RT)6 + dm * dm * h2 * is * is);
+                    wu[k] = cscale(g, (RT)3 * s);
+                    wo[k] = cscale(g, (RT)6 + dm * dm * h2 * is * is);
                     if (PF) {
                         const RT U = (RT)P.pump_ups[k];
                         PF[k] = cadd(cscale(g, -U * ((RT)P.pump_cr[k] + dm * dm)), cmul_i(g, -U * dm * (RT)P.pump_ci[k]));
                     }
                 } else if (fid == 1) {
-                    out[M] = csub(out[M], cscale(g, h2));
-                    out[2 * M] = csub(out[2 * M], cscale(g, h2 * is - (RT)5 * s));
+                    out[M] = csub(wu[k], cscale(g, h2));
+                    wo[k] = csub(wo[k], cscale(g, h2 * is - (RT)5 * s));
                     if (PF) PF[k] = cadd(PF[k], cscale(g, (RT)P.pump_ups[k] * (RT)0.5 * s));
                 } else if (fid == 2) {
-                    out[2 * M] = csub(out[2 * M], cscale(g, h2));
-                    if (PF) PF[k] = csub(PF[k], cscale(out[2 * M], (RT)P.pump_ups[k]));
+                    const T om = csub(wo[k], cscale(g, h2));
+                    out[2 * M] = om;
+                    if (PF) PF[k] = csub(PF[k], cscale(om, (RT)P.pump_ups[k]));
                 } else if (fid == 3) {
                     out[3 * M] = g;
                 } else {
@@ -689,7 +696,8 @@ __device__ __forceinline__ void cheb_derivative_part(const double2* c, double2* 
 // slots, 30 % of the FP64 pipe busy at 257 x 768, where the FP64 transforms kept
 // that pipe 60 % busy): 50 -> 25.6 us there, 23 -> 14.9 us at 129 x 384, 67 -> 36 us
 // at 513 x 384 (against the double-float lean layout it replaces at that size).
-__global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P, VecSet y, double2* __restrict__ G1) {
+__global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P, VecSet y, double2* __restrict__ G1,
+                                                                   double2* __restrict__ W) {
     __shared__ FxScale sc;
     const int m = P.m_lo + blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
@@ -736,6 +744,7 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P
     };
     const double dm = (double)m;
     double* PF = P.pump ? reinterpret_cast<double*>(P.pump_F + (size_t)m * N) : nullptr;
+    double* wu = reinterpret_cast<double*>(W + (size_t)m * 2 * N);  // partial sums of u_phi, then of omega
     for (int f0 = 0; f0 < 4; f0 += NB) {
         const fxc* R = dct1_fx(P, sc, f0, NB, nc, true, bufA, bufB, [&](int i, int t) { return value(f0 + i, t); });
         for (int t = tid; t < 2 * N; t += nth) {
@@ -743,11 +752,11 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P
             const double s = P.s[k], h2 = P.h2[k], is = P.inv_s[k];
             double* out = reinterpret_cast<double*>(G1 + g_index(k, 0, m, M));
             // out: fields v, u_phi, omega, theta, 2M doubles apart.  u_phi and omega are summed
-            // over the vectors of a batch in a register, over batches in out.
+            // over the vectors of a batch in a register, over batches in W.
             double up = 0.0, om = 0.0, pf = 0.0;
             if (f0 > 0) {
-                up = out[2 * M + part];
-                om = out[4 * M + part];
+                up = wu[t];
+                om = wu[2 * N + t];
                 if (PF) pf = PF[t];
             }
             for (int i = 0; i < NB; ++i) {
@@ -784,8 +793,14 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P
                     if (PF) pf = fma(-P.pump_ups[k], om, pf);
                 }
             }
-            out[2 * M + part] = up;
-            out[4 * M + part] = om;
+            // u_phi is complete after vector 1, omega after vector 2 (1 for m = 0, whose
+            // vector 2 is zero)
+            if (f0 <= 1 && f0 + NB > 1) out[2 * M + part] = up;
+            if (f0 <= 2 && f0 + NB > 2) out[4 * M + part] = om;
+            if (f0 + NB < 3) {
+                wu[t] = up;
+                wu[2 * N + t] = om;
+            }
             if (PF) PF[t] = pf;
         }
         __syncthreads();
@@ -2003,7 +2018,8 @@ __device__ __forceinline__ void cheb_derivative_cta(const double2* c, double2* d
 }
 
 __global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepParams P, VecSet y,
-                                                                         double2* __restrict__ G1) {
+                                                                         double2* __restrict__ G1,
+                                                                         double2* __restrict__ W) {
     __shared__ FxScale sc;
     __shared__ DctHalf dh;
     const int m = P.m_lo + blockIdx.x;
@@ -2016,6 +2032,8 @@ __global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepPar
     const double* ps = reinterpret_cast<const double*>(y.psi + (size_t)m * nc);
     const double* th = reinterpret_cast<const double*>(y.th + (size_t)m * nc);
     double* PF = P.pump ? reinterpret_cast<double*>(P.pump_F + (size_t)m * N) : nullptr;
+    double* wu = reinterpret_cast<double*>(W + (size_t)m * 2 * N);  // partial sums of u_phi
+    double* wo = wu + 2 * N;                                         // and of omega
     fx_scale_clear(sc);
     __syncthreads();
     for (int b = 0; b < 2; ++b) {
@@ -2062,27 +2080,28 @@ __global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepPar
                 if (v == 0) {
                     out[part] = 0.0;
                     out[2 * M + part] = g;
-                    out[4 * M + part] = g * is;
+                    wu[t] = g;
+                    wo[t] = g * is;
                 } else {
-                    const double om = out[4 * M + part] + g;
+                    const double om = wo[t] + g;
                     out[4 * M + part] = om;
-                    if (PF) PF[t] = part ? 0.0 : P.pump_ups[k] * out[2 * M] * (1.0 + (0.5 * P.E) * om);
+                    if (PF) PF[t] = part ? 0.0 : P.pump_ups[k] * wu[t] * (1.0 + (0.5 * P.E) * om);
                 }
             } else if (v == 0) {
                 out[part ^ 1] = part ? -dm * g : dm * g;
-                out[2 * M + part] = (3.0 * s) * g;
-                out[4 * M + part] = fma(dm * dm * h2, is * is, 6.0) * g;
+                wu[t] = (3.0 * s) * g;
+                wo[t] = fma(dm * dm * h2, is * is, 6.0) * g;
                 if (PF) {
                     const double go = half_part(sc, v, F, O, K, k, part ^ 1, -1), U = P.pump_ups[k];
                     const double ci = U * dm * P.pump_ci[k];
                     PF[t] = fma(part ? -ci : ci, go, -U * fma(dm, dm, P.pump_cr[k]) * g);
                 }
             } else if (v == 1) {
-                out[2 * M + part] = fma(-h2, g, out[2 * M + part]);
-                out[4 * M + part] = fma(-fma(-5.0, s, h2 * is), g, out[4 * M + part]);
+                out[2 * M + part] = fma(-h2, g, wu[t]);
+                wo[t] = fma(-fma(-5.0, s, h2 * is), g, wo[t]);
                 if (PF) PF[t] = fma(P.pump_ups[k] * (0.5 * s), g, PF[t]);
             } else {
-                const double om = fma(-h2, g, out[4 * M + part]);
+                const double om = fma(-h2, g, wo[t]);
                 out[4 * M + part] = om;
                 if (PF) PF[t] = fma(-P.pump_ups[k], om, PF[t]);
             }
@@ -2203,11 +2222,11 @@ static size_t smem_radial_lean32(const StepParams& P, bool analysis) {
 }
 
 template <class T>
-static cudaError_t spec_to_grid_t(const StepParams& P, VecSet y, void* G1, cudaStream_t st) {
+static cudaError_t spec_to_grid_t(const StepParams& P, VecSet y, void* G1, void* W, cudaStream_t st) {
     const size_t sm = smem_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_spec_to_grid<T><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, static_cast<T*>(G1));
+    k_spec_to_grid<T><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, static_cast<T*>(G1), static_cast<T*>(W));
     return cudaGetLastError();
 }
 
@@ -2243,7 +2262,7 @@ static cudaError_t grid_to_spec_t(const StepParams& P, const void* G2, VecSet y,
     return cudaGetLastError();
 }
 
-cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, cudaStream_t st) {
+cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, double2* W, cudaStream_t st) {
     if (lean_radial(P) && P.fp32) {
         const size_t sm = smem_radial_lean32(P, false);
         cudaError_t err =
@@ -2259,14 +2278,17 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, cuda
                              : cudaFuncSetAttribute(k_spec_to_grid_lean<double2>,
                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        kern<<<slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st>>>(P, y, G1);
+        if (fx)
+            k_spec_to_grid_lean_fx<<<slab_modes(P), NTHREADS_LX, sm, st>>>(P, y, G1, W);
+        else
+            k_spec_to_grid_lean<double2><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, G1);
         return cudaGetLastError();
     }
-    if (P.fp32) return spec_to_grid_t<float2>(P, y, G1, st);
+    if (P.fp32) return spec_to_grid_t<float2>(P, y, G1, W, st);
     const size_t sm = smem_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_spec_to_grid_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, y, G1);
+    k_spec_to_grid_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, y, G1, W);
     return cudaGetLastError();
 }
 

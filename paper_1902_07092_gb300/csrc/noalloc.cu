@@ -200,7 +200,7 @@ extern "C" int pizza_explicit_terms_noalloc(int n_r, int n_phi, double Ra, doubl
     VecSet y{const_cast<double2*>(reinterpret_cast<const double2*>(psi_hat)),
              const_cast<double2*>(reinterpret_cast<const double2*>(theta_hat)), const_cast<double*>(uphi0_hat)};
     VecSet e{reinterpret_cast<double2*>(e_psi), reinterpret_cast<double2*>(e_theta), e_uphi};
-    cudaError_t err = launch_spec_to_grid(P, y, G1, st);
+    cudaError_t err = launch_spec_to_grid(P, y, G1, G2, st);
     if (err == cudaSuccess) err = launch_phi_products(P, G1, G2, st);
     if (err == cudaSuccess) err = launch_grid_to_spec(P, G2, y, e, st);
     if (err != cudaSuccess) return na_fail(PIZZA_ECUDA, cudaGetErrorString(err));

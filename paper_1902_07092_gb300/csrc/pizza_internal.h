@@ -185,7 +185,8 @@ struct RhsSpec {
 };
 
 // kernel launchers (k_explicit.cu, k_implicit.cu)
-cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, cudaStream_t st);
+// W: working space of 2 M n_r entries (any grid array that holds nothing needed)
+cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, double2* W, cudaStream_t st);
 cudaError_t launch_phi_products(const StepParams& P, const double2* G1, double2* G2, cudaStream_t st);
 cudaError_t launch_grid_to_spec(const StepParams& P, const double2* G2, VecSet y, VecSet e, cudaStream_t st);
 cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFactors& F, VecSet y_out,
