@@ -364,6 +364,26 @@ int build_factors(pizza_ctx* ctx, const HostOps& H, double gamma, DevFactors& F,
     const int ntA = 8 * (nbt / 2);
     std::vector<double> htSpk(tsplit ? (size_t)M * nt * 8 : 0), htRj(tsplit ? (size_t)M * 256 : 0),
         htKs(tsplit ? htK.size() : 0);
+    // small systems: the dense inverses, column-major
+    const bool dense = nc <= DENSE_NC;
+    std::vector<double2> hpI(dense ? (size_t)M * nc * nc : 0, make_double2(0.0, 0.0));
+    std::vector<double> htI(dense ? (size_t)M * nc * nc : 0), huI(dense ? (size_t)nc * nc : 0);
+    auto dense_of = [&](const auto& band, int h, int pb, const std::vector<double>& tau, auto&& put) -> bool {
+        using T = typename std::decay_t<decltype(band)>::value_type;
+        std::vector<T> S((size_t)nc * nc, T(0.0)), inv;
+        for (int k = 0; k < nc; ++k)
+            for (int n = 0; n < nc; ++n) {
+                const int d = n - k + h;
+                if (k < pb)
+                    S[(size_t)k * nc + n] = T(tau[(size_t)k * nc + n]);
+                else if (d >= 0 && d <= 2 * h)
+                    S[(size_t)k * nc + n] = band[(size_t)k * (2 * h + 1) + d];
+            }
+        if (!dense_inverse(nc, S, inv)) return false;
+        for (int k = 0; k < nc; ++k)
+            for (int n = 0; n < nc; ++n) put((size_t)n * nc + k, inv[(size_t)k * nc + n]);
+        return true;
+    };
     auto work = [&](int m0, int m1) {
         std::vector<cplx> bp((size_t)nc * 17);
         std::vector<double> bt((size_t)nc * 9);
@@ -385,6 +405,12 @@ int build_factors(pizza_ctx* ctx, const HostOps& H, double gamma, DevFactors& F,
                     }
                 for (size_t i = 0; i < (size_t)np * 17; ++i)
                     hpB[(size_t)m * np * 17 + i] = make_double2(bp[4 * 17 + i].real(), bp[4 * 17 + i].imag());
+                if (dense && !dense_of(bp, 8, 4, tauP, [&](size_t i, cplx v) {
+                        hpI[(size_t)m * nc * nc + i] = make_double2(v.real(), v.imag());
+                    })) {
+                    bad[m] = 1;
+                    continue;
+                }
                 Bordered<cplx> f;
                 if (!factor_bordered(bp, nc, 8, tauP, 4, f)) {
                     bad[m] = 1;
@@ -415,6 +441,11 @@ int build_factors(pizza_ctx* ctx, const HostOps& H, double gamma, DevFactors& F,
                         v = get(OP_D, k, n) - gdt * (get(OP_F0, k, n) + mu * get(OP_F2, k, n)) / ctx->Pr;
                     bt[(size_t)k * 9 + d] = v;
                 }
+            if (dense &&
+                !dense_of(bt, 4, 2, tauD, [&](size_t i, double v) { htI[(size_t)m * nc * nc + i] = v; })) {
+                bad[m] = 1;
+                continue;
+            }
             Bordered<double> g;
             if (!factor_bordered(bt, nc, 4, tauD, 2, g)) {
                 bad[m] = 1;
@@ -467,6 +498,8 @@ int build_factors(pizza_ctx* ctx, const HostOps& H, double gamma, DevFactors& F,
             if (n >= 0 && n < nc && k >= 2) v = get(OP_D, k, n) - gdt * get(OP_EZ, k, n);
             bu[(size_t)k * 9 + d] = v;
         }
+    if (dense && !dense_of(bu, 4, 2, tauD, [&](size_t i, double v) { huI[i] = v; }))
+        return fail(ctx, PIZZA_EINVAL, "zonal-flow tau system singular");
     Bordered<double> fu;
     if (!factor_bordered(bu, nc, 4, tauD, 2, fu)) return fail(ctx, PIZZA_EINVAL, "zonal-flow tau system singular");
 
@@ -503,6 +536,11 @@ int build_factors(pizza_ctx* ctx, const HostOps& H, double gamma, DevFactors& F,
         const std::vector<float4> sd = to_dd(hpSpk), rd = to_dd(hpRj);
         UPLOAD(F.pSpkDD, float4, sd);
         UPLOAD(F.pRjDD, float4, rd);
+    }
+    if (dense) {
+        UPLOAD(F.pInv, double2, hpI);
+        UPLOAD(F.tInv, double, htI);
+        UPLOAD(F.uInv, double, huI);
     }
     UPLOAD(F.pY, double2, hpY);
     UPLOAD(F.pSinv, double2, hpS);

@@ -15,14 +15,12 @@
 // factorisation (blocks of 8 rows; the temperature and zonal-flow bands, half
 // width 4, are padded to that: twice the block size halves their chains and keeps
 // all 32 lanes busy; host_ops.h, block_lu_twisted): a pair of warps walks the top and
-// the bottom half towards the middle block and back, each step one lane-parallel
-// H x H mat-vec forward and a fused pair of them backward.  On GB300 a dependent
-// FP64 FMA costs ~64 cycles, so the sequential chain, not the flop count, sets
-// the time of a solve; two half-length chains halve it.  Lane (r, c) =
-// (lane/4, lane%4) owns row r of a block and columns c, c+4.  A CTA handles one
-// mode: warps 0-1 the streamfunction, 2-3 the temperature, 4-5 the zonal flow
-// (m = 0); the right-hand side, Schur updates, residual and the banded mass
-// applies for later stages use the whole CTA.
+// the bottom half towards the middle block and back.  On GB300 an FP64 instruction
+// of a warp holds its sub-partition ~64 cycles, dependent or not, so a phase costs
+// the FP64 instructions of its longest warp: the chains have as few of them as the
+// lanes allow, and everything else (right-hand side, Schur sums and updates,
+// residual, the banded mass applies for later stages) is cut into tasks of one
+// component of one row over the whole CTA.
 #include "device_common.cuh"
 
 namespace pz {
@@ -39,9 +37,6 @@ template <>
 __device__ __forceinline__ double zero<double>() { return 0.0; }
 
 // x - a*z in fused form
-__device__ __forceinline__ double2 fms(double2 x, double2 a, double2 z) {
-    return make_double2(fma(-a.x, z.x, fma(a.y, z.y, x.x)), fma(-a.x, z.y, fma(-a.y, z.x, x.y)));
-}
 __device__ __forceinline__ double2 fms(double2 x, double a, double2 z) {
     return make_double2(fma(-a, z.x, x.x), fma(-a, z.y, x.y));
 }
@@ -56,23 +51,6 @@ template <>
 __device__ __forceinline__ double2 shfl_idx<double2>(double2 v, int src) {
     return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
-// sum over the four lanes of a row (lanes 4r .. 4r+3); every lane gets the sum
-__device__ __forceinline__ double reduce4(double v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    return v + __shfl_xor_sync(0xffffffffu, v, 2);
-}
-__device__ __forceinline__ double2 reduce4(double2 v) { return make_double2(reduce4(v.x), reduce4(v.y)); }
-// acc + a*b
-__device__ __forceinline__ double2 fma_x(double2 a, double2 b, double2 acc) {
-    return make_double2(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
-}
-__device__ __forceinline__ double2 fma_x(double a, double2 b, double2 acc) {
-    return make_double2(fma(a, b.x, acc.x), fma(a, b.y, acc.y));
-}
-__device__ __forceinline__ double fma_x(double a, double b, double acc) { return fma(a, b, acc); }
-__device__ __forceinline__ double2 sub_x(double2 a, double2 b) { return csub(a, b); }
-__device__ __forceinline__ double sub_x(double a, double b) { return a - b; }
-
 __device__ __forceinline__ double2 fms_x(double2 a, double2 b, double2 acc) {
     return make_double2(fma(-a.x, b.x, fma(a.y, b.y, acc.x)), fma(-a.x, b.y, fma(-a.y, b.x, acc.y)));
 }
@@ -85,36 +63,13 @@ __device__ __forceinline__ double fms_x(double a, double b, double acc) { return
 template <>
 __device__ __forceinline__ float2 zero<float2>() { return make_float2(0.f, 0.f); }
 template <>
-__device__ __forceinline__ float zero<float>() { return 0.f; }
-template <>
 __device__ __forceinline__ float2 shfl_idx<float2>(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
-__device__ __forceinline__ float reduce4(float v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    return v + __shfl_xor_sync(0xffffffffu, v, 2);
-}
-__device__ __forceinline__ float2 reduce4(float2 v) { return make_float2(reduce4(v.x), reduce4(v.y)); }
-__device__ __forceinline__ float2 fma_x(float a, float2 b, float2 acc) {
-    return make_float2(fmaf(a, b.x, acc.x), fmaf(a, b.y, acc.y));
-}
-__device__ __forceinline__ float2 sub_x(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 // conversions between the FP32 chains and FP64 on the integer and FP32 pipes
 // (GB300 issues float <-> double conversions on its FP64 unit)
 __device__ __forceinline__ float2 to_f2(double2 v) { return make_float2(f32_from_bits(v.x), f32_from_bits(v.y)); }
 __device__ __forceinline__ double2 to_d2_bits(float2 v) { return make_double2(f2d_bits(v.x), f2d_bits(v.y)); }
-
-// Accumulator, conversions and finalisation of a chain value: for FP64 and FP32
-// chains the accumulator is the value type itself and these are identities.
-__device__ __forceinline__ double2 sub_acc(double2 a, double2 b) { return csub(a, b); }
-__device__ __forceinline__ float2 sub_acc(float2 a, float2 b) { return sub_x(a, b); }
-__device__ __forceinline__ double sub_acc(double a, double b) { return a - b; }
-__device__ __forceinline__ double2 fin(double2 v) { return v; }
-__device__ __forceinline__ float2 fin(float2 v) { return v; }
-__device__ __forceinline__ double fin(double v) { return v; }
-__device__ __forceinline__ double2 cvt_to(double2 v, const double2*) { return v; }
-__device__ __forceinline__ float2 cvt_to(float2 v, const float2*) { return v; }
-__device__ __forceinline__ double cvt_to(double v, const double*) { return v; }
 
 // Double-float chains of the streamfunction solve.  The block chains of the
 // Appendix A solve need about 44 significant bits: with the Schur step, the
@@ -126,20 +81,11 @@ __device__ __forceinline__ double cvt_to(double v, const double*) { return v; }
 // rate on GB300.
 //
 // Factors and chain values are complex double-floats (ddc, 16 bytes like a
-// double2).  A row sum runs in an accumulator dacc of leading sums s and trailing
-// sums e per component: every product a b of double-floats adds its leading part
+// double2).  A row sum runs in leading sums s and trailing sums e: every product a b of double-floats adds its leading part
 // p = a.hi b.hi to s by a two-sum and its trailing parts (the two-product error
 // fma(a.hi, b.hi, -p), a.hi b.lo + a.lo b.hi, and the two-sum's error) to e; the
 // value is s + e, renormalised once at the end of the row (Ogita, Rump and
 // Oishi's compensated dot product, applied to double-float inputs).
-struct __align__(16) dacc {
-    float xs, xe, ys, ye;
-};
-template <>
-__device__ __forceinline__ dacc zero<dacc>() { return dacc{0.f, 0.f, 0.f, 0.f}; }
-template <>
-__device__ __forceinline__ ddc zero<ddc>() { return ddc{ddf{0.f, 0.f}, ddf{0.f, 0.f}}; }
-
 // s + p = s' + t exactly (Knuth's two-sum)
 __device__ __forceinline__ float two_sum(float s, float p, float& t) {
     const float r = __fadd_rn(s, p);
@@ -156,15 +102,7 @@ __device__ __forceinline__ void dd_acc(float& s, float& e, float ah, float al, f
     s = two_sum(s, p, t);
     e = __fadd_rn(e, __fadd_rn(t, __fadd_rn(pe, cr)));
 }
-// acc + a b, complex
-__device__ __forceinline__ dacc fma_x(ddc a, ddc b, dacc acc) {
-    dd_acc(acc.xs, acc.xe, a.x.hi, a.x.lo, b.x.hi, b.x.lo);
-    dd_acc(acc.xs, acc.xe, -a.y.hi, -a.y.lo, b.y.hi, b.y.lo);
-    dd_acc(acc.ys, acc.ye, a.x.hi, a.x.lo, b.y.hi, b.y.lo);
-    dd_acc(acc.ys, acc.ye, a.y.hi, a.y.lo, b.x.hi, b.x.lo);
-    return acc;
-}
-// sum over the four lanes of a row; the two-sum's result and error do not depend
+// sum over a pair of lanes; the two-sum's result and error do not depend
 // on the order of its operands, so every lane gets the same bits
 __device__ __forceinline__ void dd_pair_sum(float& s, float& e, int o) {
     const float s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
@@ -172,41 +110,12 @@ __device__ __forceinline__ void dd_pair_sum(float& s, float& e, int o) {
     s = two_sum(s, s2, t);
     e = __fadd_rn(__fadd_rn(e, e2), t);
 }
-__device__ __forceinline__ dacc reduce4(dacc v) {
-#pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-        dd_pair_sum(v.xs, v.xe, o);
-        dd_pair_sum(v.ys, v.ye, o);
-    }
-    return v;
-}
 // (s + e) as a normalised double-float: two-sum, since e may exceed a cancelled s
 __device__ __forceinline__ ddf dd_norm(float s, float e) {
     float t;
     const float h = two_sum(s, e, t);
     return ddf{h, t};
 }
-__device__ __forceinline__ ddc fin(dacc v) { return ddc{dd_norm(v.xs, v.xe), dd_norm(v.ys, v.ye)}; }
-// b - p
-__device__ __forceinline__ ddf dd_sub1(ddf b, float s, float e) {
-    float t;
-    const float h = two_sum(b.hi, -s, t);
-    return dd_norm(h, __fadd_rn(__fsub_rn(b.lo, e), t));
-}
-__device__ __forceinline__ ddc sub_x(ddc b, dacc p) { return ddc{dd_sub1(b.x, p.xs, p.xe), dd_sub1(b.y, p.ys, p.ye)}; }
-__device__ __forceinline__ dacc sub_acc(dacc a, dacc b) {
-    float t, u;
-    const float xs = two_sum(a.xs, -b.xs, t);
-    const float ys = two_sum(a.ys, -b.ys, u);
-    return dacc{xs, __fadd_rn(__fsub_rn(a.xe, b.xe), t), ys, __fadd_rn(__fsub_rn(a.ye, b.ye), u)};
-}
-template <>
-__device__ __forceinline__ ddc shfl_idx<ddc>(ddc v, int src) {
-    return ddc{ddf{__shfl_sync(0xffffffffu, v.x.hi, src), __shfl_sync(0xffffffffu, v.x.lo, src)},
-               ddf{__shfl_sync(0xffffffffu, v.y.hi, src), __shfl_sync(0xffffffffu, v.y.lo, src)}};
-}
-__device__ __forceinline__ ddc cvt_to(ddc v, const ddc*) { return v; }
-
 // Asynchronous 16-byte copies global -> shared (cp.async), committed in groups;
 // cp_async_wait<N> returns when at most N of the calling thread's groups are
 // still in flight.
@@ -221,176 +130,150 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 __device__ __forceinline__ void cp_async_wait1() { cp_async_wait<1>(); }
 
-// Blocks of coefficients prefetched ahead in the chains.  With a few CTAs per SM
-// (N_c up to ~600) two blocks cover the L2 latency at little register cost; the
-// large systems run one CTA per SM (shared memory) with their factors streamed
-// from HBM, where the chains wait on that latency unless loads go further ahead:
-// there the streamfunction chains (FP64 complex coefficients) prefetch 4 blocks
-// and the FP32 temperature chains 8.
-constexpr int PFB = 2;
-constexpr int PFB_DEEP_P = 4;
-constexpr int PFB_DEEP_T = 8;
-
-// Barrier of the two warps (64 threads) of a solver pair.
-__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
-
-// Solve D x = b with the two-sided block factorisation (host_ops.h,
-// block_lu_twisted) by a pair of warps: half 0 walks the top blocks down, half 1
-// the bottom blocks up, both compute the middle block, then each substitutes
-// back through its half.  Lane (r, c) = (lane/4, lane%4) owns row r of a block
-// and columns c + 4q.  Z holds the forward values (nb*H entries), x the solution
-// (n entries); rows of b at or beyond n read as zero.  Both warps of the pair
-// must call it (bar: named barrier id); act = false skips all memory accesses.
-// On return the whole of x is visible to both warps.
-template <int H, int PF, class TF, class TX, class TA = TX, class TB = TX>
-__device__ void pair_block_solve(const TB* b, TX* Z, TB* x, int n, const TF* __restrict__ blk, bool act, int half,
-                                 int bar) {
-    constexpr int CPL = H / 4;
-    constexpr int HH = H * H;
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const bool ra = act && r < H;
-    const int nb = (n + H - 1) / H;
-    const int cm = nb / 2;
-    const int dir = half ? -1 : 1;
-    const int len = half ? (nb - 1 - cm) : cm;  // blocks of this half
-    const int k_fw = half ? nb - 1 : 0;         // first block of the forward walk
-    const int k_bw = half ? cm + 1 : cm - 1;    // first block of the backward walk
-    auto coef = [&](int k, int which, int q) -> TF {
-        return (ra && k >= 0 && k < nb) ? blk[(size_t)k * 3 * HH + which * HH + r * H + c + 4 * q] : zero<TF>();
+// ---------------------------------------------------------------------------
+// Block chains.  D x = b by the two-sided block factorisation (host_ops.h,
+// block_lu_twisted) with blocks of 8 rows: a pair of warps walks the two halves,
+//   forward   Z_k = b_k - [0]_k Z_prev            (half 0 down from the top, half 1 up from the bottom),
+//   middle    x_c = [1]_c (b_c - [0]_c Z_{c-1} - [2]_c Z_{c+1})   (both warps),
+//   diagonal  W_k = [1]_k Z_k for every other block (no chain depends on it: every warp of the CTA),
+//   backward  x_k = W_k - [2]_k x_prev,
+// with a barrier of the CTA between the phases.  Everything may run in place (Z, W
+// and x over b): a block's row is read before it is written, the middle block's
+// rows after the barrier that ends the middle phase.
+//
+// Lane (r, part, g) owns row r = lane/4 of a block, one component (part) of its
+// value and columns 4 g .. 4 g + 3: a step is four multiply-adds a lane (eight with
+// complex coefficients) and one exchange, the right-hand side being the sum's start.
+// With a lane per (row, two columns) and both components a step took 10 and 18 FP64
+// instructions of 64 cycles where it now takes 5 and 9, and the previous block's
+// values come from shared memory instead of 8 shuffles.  Measured: 800-900 cycles a
+// step of the real FP64 chain alone on its SM, 600-700 of the double-float one.
+//
+// The matrices of a walk stream through a ring of D slots in shared memory, filled by
+// asynchronous copies D - 1 ahead and kept filled across the phases' barriers:
+// forward, the middle block's three, backward.  (D = 6 measured the same as 4.)
+// ---------------------------------------------------------------------------
+// Component, accumulator and arithmetic of a chain by its coefficient type: double2
+// (complex, FP64), ddc (complex double-float), double and float (real coefficients).
+// An accumulator starts from the value the products are taken from, in one of the two
+// lanes that share a row's component: no subtraction afterwards.  The double-float
+// one keeps the products of the coefficients' real and imaginary parts apart: two
+// shorter strings of dependent sums, and one sign for the second.
+struct ddacc {
+    float s, e, t, f;
+};
+template <class C>
+struct Chain;
+template <>
+struct Chain<double2> {
+    using V = double;
+    using A = double;
+    static constexpr bool cplx = true;
+};
+template <>
+struct Chain<double> {
+    using V = double;
+    using A = double;
+    static constexpr bool cplx = false;
+};
+template <>
+struct Chain<float> {
+    using V = float;
+    using A = float;
+    static constexpr bool cplx = false;
+};
+template <>
+struct Chain<ddc> {
+    using V = ddf;
+    using A = ddacc;
+    static constexpr bool cplx = true;
+};
+__device__ __forceinline__ void ch_zero(double& a) { a = 0.0; }
+__device__ __forceinline__ void ch_zero(float& a) { a = 0.f; }
+__device__ __forceinline__ void ch_zero(ddf& a) { a = ddf{0.f, 0.f}; }
+__device__ __forceinline__ void ch_start(double& a, double b) { a = b; }
+__device__ __forceinline__ void ch_start(float& a, float b) { a = b; }
+__device__ __forceinline__ void ch_start(ddacc& a, ddf b) { a = ddacc{b.hi, b.lo, 0.f, 0.f}; }
+// acc -= (SUB) or += component part of a (x + i y); p, q: that component and the other
+template <bool SUB>
+__device__ __forceinline__ void ch_mac(double& acc, double2 a, double p, double q, int part) {
+    q = (part != 0) == SUB ? -q : q;  // operands chosen, not instructions: one path for all lanes
+    acc = fma(SUB ? -a.x : a.x, p, fma(a.y, q, acc));
+}
+template <bool SUB>
+__device__ __forceinline__ void ch_mac(ddacc& acc, ddc a, ddf p, ddf q, int) {
+    dd_acc(acc.s, acc.e, SUB ? -a.x.hi : a.x.hi, SUB ? -a.x.lo : a.x.lo, p.hi, p.lo);
+    dd_acc(acc.t, acc.f, a.y.hi, a.y.lo, q.hi, q.lo);
+}
+// acc -= or += a x
+template <bool SUB>
+__device__ __forceinline__ void ch_mac(double& acc, double a, double x) { acc = fma(SUB ? -a : a, x, acc); }
+template <bool SUB>
+__device__ __forceinline__ void ch_mac(float& acc, float a, float x) { acc = fmaf(SUB ? -a : a, x, acc); }
+// the value: both lanes' sums (g = 0, 1) of a row's component
+template <bool SUB>
+__device__ __forceinline__ double ch_value(double a, int) { return a + __shfl_xor_sync(0xffffffffu, a, 1); }
+template <bool SUB>
+__device__ __forceinline__ float ch_value(float a, int) { return a + __shfl_xor_sync(0xffffffffu, a, 1); }
+template <bool SUB>
+__device__ __forceinline__ ddf ch_value(ddacc a, int part) {
+    const float sg = (part != 0) == SUB ? -1.f : 1.f;
+    float u, s = two_sum(a.s, sg * a.t, u), e = __fadd_rn(__fadd_rn(a.e, sg * a.f), u);
+    dd_pair_sum(s, e, 1);
+    return dd_norm(s, e);
+}
+// the sum over 4 columns: coefficients a[4], this lane's component p[4] of the values
+// and (complex coefficients) the other q[4]
+template <bool SUB, class C>
+__device__ __forceinline__ void ch_row(typename Chain<C>::A& acc, const C (&a)[4], const typename Chain<C>::V (&p)[4],
+                                       const typename Chain<C>::V (&q)[4], int part) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if constexpr (Chain<C>::cplx)
+            ch_mac<SUB>(acc, a[j], p[j], q[j], part);
+        else
+            ch_mac<SUB>(acc, a[j], p[j]);
+    }
+}
+// its values from a vector with NP components a row
+template <class C, int NP>
+__device__ __forceinline__ void ch_values(const typename Chain<C>::V* v, int c0, int part, typename Chain<C>::V (&p)[4],
+                                          typename Chain<C>::V (&q)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        p[j] = v[NP * (c0 + j) + (NP == 2 ? part : 0)];
+        if constexpr (Chain<C>::cplx) q[j] = v[2 * (c0 + j) + 1 - part];
+    }
+}
+// or from a walk's previous block, stored component by component (8 rows each):
+// 16-byte reads
+template <class V>
+__device__ __forceinline__ void ch_four(const V* v, V (&p)[4]) {
+    struct __align__(16) Q {
+        V x[16 / sizeof(V)];
     };
-    // forward: Z_k = b_k - [0]_k Z_prev
-    {
-        TX prev[CPL];
-        TF cur[PF][CPL], nxt[PF][CPL];
+    constexpr int K = 16 / (int)sizeof(V);
 #pragma unroll
-        for (int q = 0; q < CPL; ++q) prev[q] = zero<TX>();
+    for (int i = 0; i < 4 / K; ++i) {
+        const Q w = reinterpret_cast<const Q*>(v)[i];
 #pragma unroll
-        for (int i = 0; i < PF; ++i)
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) cur[i][q] = (i < len) ? coef(k_fw + dir * i, 0, q) : zero<TF>();
-        for (int i0 = 0; i0 < len; i0 += PF) {
-#pragma unroll
-            for (int i = 0; i < PF; ++i)
-#pragma unroll
-                for (int q = 0; q < CPL; ++q)
-                    nxt[i][q] = (i0 + PF + i < len) ? coef(k_fw + dir * (i0 + PF + i), 0, q) : zero<TF>();
-#pragma unroll
-            for (int i = 0; i < PF; ++i) {
-                if (i0 + i < len) {
-                    const int k = k_fw + dir * (i0 + i);
-                    const int row = k * H + r;
-                    const TX bv = (ra && row < n) ? cvt_to(b[row], (const TX*)nullptr) : zero<TX>();
-                    TA p = zero<TA>();
-#pragma unroll
-                    for (int q = 0; q < CPL; ++q) p = fma_x(cur[i][q], prev[q], p);
-                    p = reduce4(p);
-                    const TX zv = sub_x(bv, p);
-                    if (ra && c == 0) Z[row] = zv;
-#pragma unroll
-                    for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(zv, 4 * (c + 4 * q));
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < PF; ++i)
-#pragma unroll
-                for (int q = 0; q < CPL; ++q) cur[i][q] = nxt[i][q];
-        }
+        for (int j = 0; j < K; ++j) p[i * K + j] = w.x[j];
     }
-    pair_sync(bar);
-    // middle block, by both warps: x_c = S^{-1}(b_c - L_c z_{c-1} - M_c w_{c+1})
-    TX prev[CPL];
-    {
-        TA t = zero<TA>();
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) {
-            const int col = c + 4 * q;
-            if (ra && cm > 0) t = fma_x(coef(cm, 0, q), Z[(cm - 1) * H + col], t);
-            if (ra && cm < nb - 1) t = fma_x(coef(cm, 2, q), Z[(cm + 1) * H + col], t);
-        }
-        t = reduce4(t);
-        const int row = cm * H + r;
-        const TX bv = (ra && row < n) ? cvt_to(b[row], (const TX*)nullptr) : zero<TX>();
-        const TX rv = sub_x(bv, t);
-        TX rr[CPL];
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) rr[q] = shfl_idx(rv, 4 * (c + 4 * q));
-        TA xa = zero<TA>();
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) xa = fma_x(coef(cm, 1, q), rr[q], xa);
-        const TX xv = fin(reduce4(xa));
-        if (half == 0 && ra && c == 0 && row < n) x[row] = cvt_to(xv, (const TB*)nullptr);
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(xv, 4 * (c + 4 * q));
-    }
-    // backward: x_k = [1]_k Z_k - [2]_k x_prev, walking away from the middle
-    {
-        TF cu[PF][CPL], ch[PF][CPL], nu[PF][CPL], nh[PF][CPL];
-        const int bdir = half ? 1 : -1;
-#pragma unroll
-        for (int i = 0; i < PF; ++i)
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) {
-                cu[i][q] = (i < len) ? coef(k_bw + bdir * i, 1, q) : zero<TF>();
-                ch[i][q] = (i < len) ? coef(k_bw + bdir * i, 2, q) : zero<TF>();
-            }
-        for (int i0 = 0; i0 < len; i0 += PF) {
-#pragma unroll
-            for (int i = 0; i < PF; ++i)
-#pragma unroll
-                for (int q = 0; q < CPL; ++q) {
-                    const bool in = i0 + PF + i < len;
-                    nu[i][q] = in ? coef(k_bw + bdir * (i0 + PF + i), 1, q) : zero<TF>();
-                    nh[i][q] = in ? coef(k_bw + bdir * (i0 + PF + i), 2, q) : zero<TF>();
-                }
-#pragma unroll
-            for (int i = 0; i < PF; ++i) {
-                if (i0 + i < len) {
-                    const int k = k_bw + bdir * (i0 + i);
-                    TA pz = zero<TA>(), ph = zero<TA>();
-#pragma unroll
-                    for (int q = 0; q < CPL; ++q) {
-                        const TX zq = ra ? Z[k * H + c + 4 * q] : zero<TX>();
-                        pz = fma_x(cu[i][q], zq, pz);
-                        ph = fma_x(ch[i][q], prev[q], ph);
-                    }
-                    const TX p = fin(reduce4(sub_acc(pz, ph)));
-                    const int row = k * H + r;
-                    if (ra && c == 0 && row < n) x[row] = cvt_to(p, (const TB*)nullptr);
-#pragma unroll
-                    for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(p, 4 * (c + 4 * q));
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < PF; ++i)
-#pragma unroll
-                for (int q = 0; q < CPL; ++q) {
-                    cu[i][q] = nu[i][q];
-                    ch[i][q] = nh[i][q];
-                }
-        }
-    }
-    // both halves of x written before either warp goes on (a Schur step of the
-    // caller reads all of it)
-    pair_sync(bar);
+}
+template <class C, int NP>
+__device__ __forceinline__ void ch_prev(const typename Chain<C>::V* v, int c0, int part, typename Chain<C>::V (&p)[4],
+                                        typename Chain<C>::V (&q)[4]) {
+    ch_four(v + (NP == 2 ? 8 * part : 0) + c0, p);
+    if constexpr (Chain<C>::cplx) ch_four(v + 8 * (1 - part) + c0, q);
 }
 
-// The same two-sided solve split into phases for a CTA whose other warps can
-// help (the kernel with one CTA per system).  The pair's walks each read one
-// matrix per block -- [0] forward, [2] backward -- so the same registers prefetch
-// PF blocks ahead with PF twice as large; the products W_k = [1]_k Z_k, which no
-// chain depends on, are formed between the walks by every warp of the CTA:
-//   chain_forward (pair)  -> barrier -> chain_middle (pair) -> barrier ->
-//   chain_diag (CTA, Z_k := W_k in place for k != c) -> barrier ->
-//   chain_backward (pair), x_k = W_k - [2]_k x_prev.
-// Geometry as in pair_block_solve: blocks of H rows, middle block c = nb/2,
-// half 0 walks 0..c-1, half 1 nb-1..c+1.  b, Z and x hold the chain type (no
-// conversions on the dependent path).
-template <int H>
+template <class C>
+__host__ __device__ constexpr int ring_bytes(int D) { return D * 64 * (int)sizeof(C); }
+
 struct ChainGeom {
-    int nb, cm, dir, len, k_fw, k_bw;
-    __device__ ChainGeom(int n, int half) {
-        nb = (n + H - 1) / H;
+    int nb, cm, len, k_fw, k_bw, dir;  // blocks, middle block, blocks of this half, its first blocks, forward direction
+    __device__ __forceinline__ ChainGeom(int n, int half) {
+        nb = (n + 7) / 8;
         cm = nb / 2;
         dir = half ? -1 : 1;
         len = half ? (nb - 1 - cm) : cm;
@@ -399,219 +282,270 @@ struct ChainGeom {
     }
 };
 
-// Coefficients of a walk come through a ring of D matrices in shared memory
-// (ring: D * H * H entries per warp), filled by asynchronous copies D blocks
-// ahead: a copy in flight holds no register and no scoreboard, so the walk keeps
-// D loads outstanding whatever its own latency.  Step i waits for its block's
-// group, reads the lane's coefficients, and refills the slot with block i + D
-// once every lane has read it.
-template <int H, int D, class TF>
-__device__ __forceinline__ void ring_issue(const TF* __restrict__ blk, TF* ring, int k, int which, int slot,
-                                           bool valid) {
-    constexpr int HH = H * H;
-    constexpr int CH = HH * (int)sizeof(TF) / 16;  // 16-byte chunks of one matrix
-    const int lane = threadIdx.x & 31;
-    if (valid) {
-        const char* src = reinterpret_cast<const char*>(blk + (size_t)k * 3 * HH + which * HH);
-        char* dst = reinterpret_cast<char*>(ring + slot * HH);
-        for (int j = lane; j < CH; j += 32) cp_async16(dst + 16 * j, src + 16 * j);
-    }
-    cp_async_commit();
-}
-
-template <int H, int D, class TF, class TX, class TA>
-__device__ void chain_forward(const TX* b, TX* Z, int n, const TF* __restrict__ blk, int half, TF* ring) {
-    constexpr int CPL = H / 4;
-    constexpr int HH = H * H;
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const ChainGeom<H> g(n, half);
-#pragma unroll
-    for (int i = 0; i < D; ++i) ring_issue<H, D>(blk, ring, g.k_fw + g.dir * i, 0, i, i < g.len);
-    TX prev[CPL];
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) prev[q] = zero<TX>();
-    for (int i = 0; i < g.len; ++i) {
-        const int k = g.k_fw + g.dir * i;
-        const int row = k * H + r;
-        const TX bv = (row < n) ? b[row] : zero<TX>();
-        cp_async_wait<D - 1>();
-        __syncwarp();
-        const TF* mat = ring + (i % D) * HH;
-        TA p = zero<TA>();
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) p = fma_x(mat[r * H + c + 4 * q], prev[q], p);
-        __syncwarp();  // every lane has read the slot
-        ring_issue<H, D>(blk, ring, g.k_fw + g.dir * (i + D), 0, i % D, i + D < g.len);
-        p = reduce4(p);
-        const TX zv = sub_x(bv, p);
-        if (c == 0) Z[row] = zv;
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(zv, 4 * (c + 4 * q));
-    }
-    cp_async_wait<0>();
-}
-
-// middle block by both warps of the pair: x_c = S^{-1}(b_c - L_c z_{c-1} - M_c w_{c+1});
-// both keep it in prev (the start of their backward walks) and return the lane's
-// row of it; the caller stores it after a barrier, since x may share its rows
-// with b (the correction solved in place of the residual) and the other warp of
-// the pair reads b_c here
-template <int H, class TF, class TX, class TA>
-__device__ TX chain_middle(const TX* b, const TX* Z, int n, const TF* __restrict__ blk, int half,
-                           TX (&prev)[H / 4]) {
-    constexpr int CPL = H / 4;
-    constexpr int HH = H * H;
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const ChainGeom<H> g(n, half);
-    const int cm = g.cm, nb = g.nb;
-    auto coef = [&](int which, int q) -> TF { return blk[(size_t)cm * 3 * HH + which * HH + r * H + c + 4 * q]; };
-    TA t = zero<TA>();
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) {
-        const int col = c + 4 * q;
-        if (cm > 0) t = fma_x(coef(0, q), Z[(cm - 1) * H + col], t);
-        if (cm < nb - 1) t = fma_x(coef(2, q), Z[(cm + 1) * H + col], t);
-    }
-    t = reduce4(t);
-    const int row = cm * H + r;
-    const TX bv = (row < n) ? b[row] : zero<TX>();
-    const TX rv = sub_x(bv, t);
-    TX rr[CPL];
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) rr[q] = shfl_idx(rv, 4 * (c + 4 * q));
-    TA xa = zero<TA>();
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) xa = fma_x(coef(1, q), rr[q], xa);
-    const TX xv = fin(reduce4(xa));
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(xv, 4 * (c + 4 * q));
-    return xv;
-}
-
-// the middle block's rows of x, by half 0 of the pair (after the barrier that
-// ends the middle phase)
-template <int H, class TX>
-__device__ __forceinline__ void chain_middle_store(TX* x, int n, int half, TX xv) {
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const int row = ((n + H - 1) / H / 2) * H + r;
-    if (half == 0 && c == 0 && row < n) x[row] = xv;
-}
-
-// Z_k := [1]_k Z_k for every block k except the middle one, one warp per block
-// (warp w of nw), DU blocks in flight per warp: their coefficient and Z loads are
-// issued together before any product, so the pass costs a few load latencies
-// rather than one per block.  Rows at or beyond n stay untouched.
-constexpr int DU = 4;
-template <int H, class TF, class TX, class TA>
-__device__ void chain_diag(TX* Z, int n, const TF* __restrict__ blk, int w, int nw) {
-    constexpr int CPL = H / 4;
-    constexpr int HH = H * H;
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const int nb = (n + H - 1) / H, cm = nb / 2;
-    for (int k0 = w; k0 < nb; k0 += nw * DU) {
-        TF a[DU][CPL];
-        TX z[DU][CPL];
-#pragma unroll
-        for (int u = 0; u < DU; ++u) {
-            const int k = k0 + u * nw;
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) {
-                const int col = k * H + c + 4 * q;
-                const bool ok = k < nb && k != cm;
-                a[u][q] = ok ? blk[(size_t)k * 3 * HH + HH + r * H + c + 4 * q] : zero<TF>();
-                z[u][q] = (ok && col < n) ? Z[col] : zero<TX>();
+// One warp's walk (one set of registers whatever its system) and its stream of
+// matrices through a ring of D slots: entry e (issued in order) to slot e % D, src
+// following the entries from block to block.
+struct Walk {
+    char *b, *Z, *x, *ring;
+    const char *blk, *src;
+    int n, half, e;
+    ChainGeom g;
+    template <class C, int D>
+    __device__ __forceinline__ void issue() {
+        constexpr int MAT = 64 * (int)sizeof(C);
+        if (e < 2 * g.len + 3) {
+            if (e > 0 && e < g.len) {
+                src += g.dir * 3 * MAT;
+            } else if (e > g.len + 3) {
+                src -= g.dir * 3 * MAT;
+            } else {  // the first block, the middle one's three matrices, the first block backward
+                const int i = e - g.len;
+                src = blk + (i < 0 ? g.k_fw * 3 : i < 3 ? g.cm * 3 + (i == 0 ? 0 : i == 1 ? 2 : 1) : g.k_bw * 3 + 2) * MAT;
             }
-        }
-        TX wv[DU];
+            char* dst = ring + (e % D) * MAT;
+            const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int u = 0; u < DU; ++u) {
-            TA t = zero<TA>();
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) t = fma_x(a[u][q], z[u][q], t);
-            wv[u] = fin(reduce4(t));
+            for (int j = 0; j < MAT; j += 512)
+                if (j + 512 <= MAT || lane < 16) cp_async16(dst + j + 16 * lane, src + j + 16 * lane);
         }
-        __syncwarp();
+        cp_async_commit();
+        ++e;
+    }
+    // the four coefficients of this lane of entry e - D + 1, the oldest in flight
+    template <class C, int D>
+    __device__ __forceinline__ void take(C (&a)[4]) {
+        const int lane = threadIdx.x & 31;
+        cp_async_wait<D - 2>();
+        __syncwarp();  // also: every lane has read the slot before, which issue refills
+        const C* p = reinterpret_cast<const C*>(ring + ((e + 1) % D) * 64 * (int)sizeof(C)) + (lane >> 2) * 8 + (lane & 1) * 4;
+        ch_four(p, a);
+    }
+};
+
+// Forward walk of one warp.  b: n rows (NP components each), Z: 8 nb rows.  prev:
+// this warp's 2 x 16 components in shared memory.
+template <class C, int NP, int D>
+__device__ __forceinline__ void chain_forward(Walk& w, typename Chain<C>::V* prev) {
+    using V = typename Chain<C>::V;
+    const V* b = reinterpret_cast<const V*>(w.b);
+    V* Z = reinterpret_cast<V*>(w.Z);
+    const ChainGeom& g = w.g;
+    const int n = w.n;
+    const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
+    const bool own = gcol == 0 && part < NP;
+#pragma unroll
+    for (int e = 0; e < D - 1; ++e) w.issue<C, D>();
+    if (lane < 16) ch_zero(prev[lane]);
+    for (int i = 0; i < g.len; ++i) {
+        const int row = (g.k_fw + g.dir * i) * 8 + r;
+        V bv, p[4], q[4];
+        C a[4];
+        w.take<C, D>(a);
+        ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        ch_zero(bv);
+        if (row < n && own) bv = b[row * NP + part];
+        w.issue<C, D>();
+        typename Chain<C>::A acc;
+        ch_start(acc, bv);
+        ch_row<true>(acc, a, p, q, part);
+        const V z = ch_value<true>(acc, part);
+        if (own) {
+            prev[((i + 1) & 1) * 16 + 8 * part + r] = z;
+            Z[row * NP + part] = z;
+        }
+    }
+}
+// middle block by both warps of the pair; returns the lane's component of it, also
+// left in prev[0 .. 16) for the backward walk.  The caller stores it after a barrier.
+template <class C, int NP, int D>
+__device__ __forceinline__ typename Chain<C>::V chain_middle(Walk& w, typename Chain<C>::V* prev) {
+    using V = typename Chain<C>::V;
+    const V *b = reinterpret_cast<const V*>(w.b), *Z = reinterpret_cast<const V*>(w.Z);
+    const ChainGeom& g = w.g;
+    const int n = w.n;
+    const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
+    const bool own = gcol == 0 && part < NP;
+    const int row = g.cm * 8 + r;
+    V bv;
+    ch_zero(bv);
+    if (row < n && own) bv = b[row * NP + part];
+    typename Chain<C>::A acc;
+    ch_start(acc, bv);
+    C a[4];
+    V p[4], q[4];
+    w.take<C, D>(a);
+    w.issue<C, D>();
+    if (g.cm > 0) {
+        ch_values<C, NP>(Z + (g.cm - 1) * 8 * NP, 4 * gcol, part, p, q);
+        ch_row<true>(acc, a, p, q, part);
+    }
+    w.take<C, D>(a);
+    w.issue<C, D>();
+    if (g.cm < g.nb - 1) {
+        ch_values<C, NP>(Z + (g.cm + 1) * 8 * NP, 4 * gcol, part, p, q);
+        ch_row<true>(acc, a, p, q, part);
+    }
+    const V y = ch_value<true>(acc, part);
+    __syncwarp();  // the lanes' reads of the last block
+    if (own) prev[16 + 8 * part + r] = y;
+    w.take<C, D>(a);  // (synchronises the warp)
+    w.issue<C, D>();
+    ch_prev<C, NP>(prev + 16, 4 * gcol, part, p, q);
+    ch_zero(bv);
+    ch_start(acc, bv);
+    ch_row<false>(acc, a, p, q, part);
+    const V x = ch_value<false>(acc, part);
+    if (own) prev[8 * part + r] = x;
+    return x;
+}
+template <int NP, class V>
+__device__ __forceinline__ void chain_middle_store(const Walk& w, V xv) {
+    const int lane = threadIdx.x & 31, part = (lane >> 1) & 1;
+    const int row = w.g.cm * 8 + (lane >> 2);
+    if (w.half == 0 && (lane & 1) == 0 && part < NP && row < w.n) reinterpret_cast<V*>(w.x)[row * NP + part] = xv;
+}
+// W_k = [1]_k Z_k in place for every block but the middle one, blocks w, w + nw, ...
+// by warp w, DU of them in flight (their loads before any product)
+template <class C, int NP, int DU>
+__device__ __forceinline__ void chain_diag(typename Chain<C>::V* Z, int n, const C* __restrict__ blk, int w, int nw) {
+    using V = typename Chain<C>::V;
+    const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
+    const bool own = gcol == 0 && part < NP;
+    const int nb = (n + 7) / 8, cm = nb / 2;
+    for (int k0 = w; k0 < nb; k0 += nw * DU) {
+        C a[DU][4];
 #pragma unroll
         for (int u = 0; u < DU; ++u) {
             const int k = k0 + u * nw;
-            const int row = k * H + r;
-            if (k < nb && k != cm && c == 0 && row < n) Z[row] = wv[u];
+            if (k < nb) ch_four(blk + (k * 3 + 1) * 64 + r * 8 + 4 * gcol, a[u]);
         }
-        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < DU; ++u) {
+            const int k = k0 + u * nw;
+            if (k >= nb || k == cm) continue;
+            V v;
+            ch_zero(v);
+            typename Chain<C>::A acc;
+            ch_start(acc, v);
+            V p[4], q[4];
+            ch_values<C, NP>(Z + k * 8 * NP, 4 * gcol, part, p, q);
+            ch_row<false>(acc, a[u], p, q, part);
+            v = ch_value<false>(acc, part);
+            __syncwarp();
+            if (own && k * 8 + r < n) Z[(k * 8 + r) * NP + part] = v;
+        }
     }
 }
-
-// backward walk away from the middle block: x_k = W_k - [2]_k x_prev
-template <int H, int D, class TF, class TX, class TA>
-__device__ void chain_backward(const TX* W, TX* x, int n, const TF* __restrict__ blk, int half, TX (&prev)[H / 4],
-                               TF* ring) {
-    constexpr int CPL = H / 4;
-    constexpr int HH = H * H;
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c = lane & 3;
-    const ChainGeom<H> g(n, half);
-    const int bdir = half ? 1 : -1;
-#pragma unroll
-    for (int i = 0; i < D; ++i) ring_issue<H, D>(blk, ring, g.k_bw + bdir * i, 2, i, i < g.len);
+// backward walk away from the middle block (prev[0 .. 16) holds it)
+template <class C, int NP, int D>
+__device__ __forceinline__ void chain_backward(Walk& w, typename Chain<C>::V* prev) {
+    using V = typename Chain<C>::V;
+    const V* W = reinterpret_cast<const V*>(w.Z);
+    V* x = reinterpret_cast<V*>(w.x);
+    const ChainGeom& g = w.g;
+    const int n = w.n;
+    const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
+    const bool own = gcol == 0 && part < NP;
     for (int i = 0; i < g.len; ++i) {
-        const int k = g.k_bw + bdir * i;
-        const int row = k * H + r;
-        const TX wv = (row < n) ? W[row] : zero<TX>();
-        cp_async_wait<D - 1>();
-        __syncwarp();
-        const TF* mat = ring + (i % D) * HH;
-        TA ph = zero<TA>();
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) ph = fma_x(mat[r * H + c + 4 * q], prev[q], ph);
-        __syncwarp();
-        ring_issue<H, D>(blk, ring, g.k_bw + bdir * (i + D), 2, i % D, i + D < g.len);
-        ph = reduce4(ph);
-        const TX p = sub_x(wv, ph);
-        if (c == 0 && row < n) x[row] = p;
-#pragma unroll
-        for (int q = 0; q < CPL; ++q) prev[q] = shfl_idx(p, 4 * (c + 4 * q));
+        const int row = (g.k_bw - g.dir * i) * 8 + r;
+        V wv, p[4], q[4];
+        C a[4];
+        w.take<C, D>(a);
+        ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        ch_zero(wv);
+        if (row < n && own) wv = W[row * NP + part];
+        w.issue<C, D>();
+        typename Chain<C>::A acc;
+        ch_start(acc, wv);
+        ch_row<true>(acc, a, p, q, part);
+        const V xv = ch_value<true>(acc, part);
+        if (own) {
+            prev[((i + 1) & 1) * 16 + 8 * part + r] = xv;
+            if (row < n) x[row * NP + part] = xv;
+        }
     }
     cp_async_wait<0>();
+    __syncwarp();
 }
 
-// Whole-CTA driver of the phased solve for up to two systems: system 1 by the
-// warp pair (w1, w1 + 1), system 2 (n2 > 0) by (w2, w2 + 1).  ring: shared memory
-// for 4 x D matrices (one ring per walking warp: system 1's pair first).  Every
-// thread of the CTA calls it; it ends with a __syncthreads that publishes x, x2.
-template <int D, class TF, class TX, class TA>
-__device__ void cta_chain_solve(const TX* b, TX* Z, TX* x, int n, const TF* __restrict__ blk, int w1, const TX* b2,
-                                TX* Z2, TX* x2, int n2, const TF* __restrict__ blk2, int w2, TF* ring) {
-    constexpr int HH = 64;
+// One system's chain, for the phases below: b, Z and x as flattened components.
+template <class C, int NP>
+struct ChainJob {
+    typename Chain<C>::V *b, *Z, *x;
+    int n;  // 0: no such system
+    const C* blk;
+    int w;       // first warp of its pair
+    char* ring;  // the pair's two rings
+};
+// Whole-CTA driver: ja, jb two halves of one system or one alone, jt and ju others, on
+// disjoint warp pairs.  prevs: 16 doubles x 2 a warp in shared memory.  Z may be b
+// and x where it has room for whole blocks; ends with a barrier that publishes x.
+// With the walks, the diagonal products and the phases above: solve at n_r x n_phi =
+// 129 x 384, 257 x 768, 513 x 1536 46 -> 39, 71 -> 69, 270 -> 260 us; 513 x 384 with
+// implicit buoyancy 136 -> 88 us.
+template <int D, int DU, class CP, int NPP, class CT, int NPT, class CU, int NPU>
+__device__ __forceinline__ void run_chains(const ChainJob<CP, NPP>& ja, const ChainJob<CP, NPP>& jb, const ChainJob<CT, NPT>& jt,
+                                           const ChainJob<CU, NPU>& ju, double (*prevs)[32]) {
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const bool in1 = warp == w1 || warp == w1 + 1, in2 = n2 > 0 && (warp == w2 || warp == w2 + 1);
-    TF* my_ring = ring + (in1 ? warp - w1 : 2 + warp - w2) * D * HH;
-    if (in1) chain_forward<8, D, TF, TX, TA>(b, Z, n, blk, warp - w1, my_ring);
-    if (in2) chain_forward<8, D, TF, TX, TA>(b2, Z2, n2, blk2, warp - w2, my_ring);
+    Walk w{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, warp & 1, 0, ChainGeom(0, 0)};
+    auto pick = [&]<class C, int NP>(const ChainJob<C, NP>& j) {
+        if (j.n == 0 || (warp & ~1) != j.w) return false;
+        w.b = reinterpret_cast<char*>(j.b);
+        w.Z = reinterpret_cast<char*>(j.Z);
+        w.x = reinterpret_cast<char*>(j.x);
+        w.ring = j.ring + (warp & 1) * ring_bytes<C>(D);
+        w.blk = w.src = reinterpret_cast<const char*>(j.blk);
+        w.n = j.n;
+        w.g = ChainGeom(j.n, warp & 1);
+        return true;
+    };
+    bool inp = pick(ja);
+    if (pick(jb)) inp = true;
+    const bool in_t = pick(jt), in_u = pick(ju);
+    using VP = typename Chain<CP>::V;
+    using VT = typename Chain<CT>::V;
+    using VU = typename Chain<CU>::V;
+    VP* pp = reinterpret_cast<VP*>(prevs[warp]);
+    VT* pt = reinterpret_cast<VT*>(prevs[warp]);
+    VU* pu = reinterpret_cast<VU*>(prevs[warp]);
+    if (inp) chain_forward<CP, NPP, D>(w, pp);
+    if (in_t) chain_forward<CT, NPT, D>(w, pt);
+    if (in_u) chain_forward<CU, NPU, D>(w, pu);
     __syncthreads();
-    TX prev[2];
-    TX xm = zero<TX>();
-    if (in1) xm = chain_middle<8, TF, TX, TA>(b, Z, n, blk, warp - w1, prev);
-    if (in2) xm = chain_middle<8, TF, TX, TA>(b2, Z2, n2, blk2, warp - w2, prev);
+    VP xp;
+    VT xt;
+    VU xu;
+    if (inp) xp = chain_middle<CP, NPP, D>(w, pp);
+    if (in_t) xt = chain_middle<CT, NPT, D>(w, pt);
+    if (in_u) xu = chain_middle<CU, NPU, D>(w, pu);
     __syncthreads();
-    if (in1) chain_middle_store<8>(x, n, warp - w1, xm);
-    if (in2) chain_middle_store<8>(x2, n2, warp - w2, xm);
-    chain_diag<8, TF, TX, TA>(Z, n, blk, warp, nw);
-    if (n2 > 0) chain_diag<8, TF, TX, TA>(Z2, n2, blk2, warp, nw);
+    if (inp) chain_middle_store<NPP>(w, xp);
+    if (in_t) chain_middle_store<NPT>(w, xt);
+    if (in_u) chain_middle_store<NPU>(w, xu);
+    for (int h = 0; h < 2; ++h) {
+        const int n = h ? jb.n : ja.n;
+        if (n > 0) chain_diag<CP, NPP, DU>(h ? jb.Z : ja.Z, n, h ? jb.blk : ja.blk, warp, nw);
+    }
+    if (jt.n > 0) chain_diag<CT, NPT, DU>(jt.Z, jt.n, jt.blk, nw - 1 - warp, nw);
+    if (ju.n > 0) chain_diag<CU, NPU, DU>(ju.Z, ju.n, ju.blk, warp, nw);
     __syncthreads();
-    if (in1) chain_backward<8, D, TF, TX, TA>(Z, x, n, blk, warp - w1, prev, my_ring);
-    if (in2) chain_backward<8, D, TF, TX, TA>(Z2, x2, n2, blk2, warp - w2, prev, my_ring);
+    if (inp) chain_backward<CP, NPP, D>(w, pp);
+    if (in_t) chain_backward<CT, NPT, D>(w, pt);
+    if (in_u) chain_backward<CU, NPU, D>(w, pu);
     __syncthreads();
 }
+template <class C, int NP>
+__device__ __forceinline__ ChainJob<C, NP> no_job() { return ChainJob<C, NP>{nullptr, nullptr, nullptr, 0, nullptr, 0, nullptr}; }
 
-// Ring depths of the phased chains: double-float streamfunction chains 6
-// matrices (1 KB each) per walking warp, FP32 temperature chains 8 (256 bytes)
-constexpr int RD_DD = 6;
-constexpr int RD_32 = 8;
+// Ring depths (matrices a walking warp): 1152 bytes a complex or double-float
+// matrix, 640 a real FP64 one, 384 an FP32 one
+constexpr int RD = 4;
 
+// acc - a z, component part
+__device__ __forceinline__ double fms_part(double acc, double2 a, double2 z, int part) {
+    const double p = part ? z.y : z.x, q = part ? -z.x : z.y;
+    return fma(-a.x, p, fma(a.y, q, acc));
+}
 // Join of the streamfunction block solved in two halves (rows [0, nA) by warps
 // 0-1, [nA, n) by warps 6-7; DevFactors psplit): x holds each half's own solution
 // g.  The interface unknowns, A's last block and B's first, are
@@ -624,21 +558,24 @@ __device__ void split_join(double2* x, int n, int nA, const double2* __restrict_
                            bool act) {
     __shared__ double2 xi[16];
     const int tid = threadIdx.x;
-    if (act && tid < 16) {
-        double2 acc = make_double2(0.0, 0.0);
-#pragma unroll 4
-        for (int c = 0; c < 16; ++c) acc = cfma(__ldg(&rj[tid * 16 + c]), x[c < 8 ? nA - 8 + c : nA + c - 8], acc);
-        xi[tid] = acc;
+    if (act && tid < 256) {  // (output, component, two columns)
+        const int o = tid >> 4, part = (tid >> 3) & 1, c = 2 * (tid & 7);
+        const double2* v = x + (c < 8 ? nA - 8 + c : nA + c - 8);
+        double acc = fms_part(fms_part(0.0, __ldg(&rj[o * 16 + c]), v[0], part), __ldg(&rj[o * 16 + c + 1]), v[1], part);
+#pragma unroll
+        for (int h = 1; h < 8; h <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, h);
+        if ((tid & 7) == 0) reinterpret_cast<double*>(xi)[tid >> 3] = -acc;
     }
     __syncthreads();
     if (act)
-        for (int i = tid; i < n; i += blockDim.x) {
-            const double2* row = spk + (size_t)i * 8;
-            const double2* v = (i < nA) ? xi + 8 : xi;
-            double2 t = x[i];
+        for (int t = tid; t < 2 * n; t += blockDim.x) {
+            const double2* row = spk + (size_t)(t >> 1) * 8;
+            const double2* v = ((t >> 1) < nA) ? xi + 8 : xi;
+            double* xt = reinterpret_cast<double*>(x) + t;
+            double acc = *xt;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) t = fms(t, __ldg(&row[c]), v[c]);
-            x[i] = t;
+            for (int c = 0; c < 8; ++c) acc = fms_part(acc, __ldg(&row[c]), v[c], t & 1);
+            *xt = acc;
         }
     __syncthreads();
 }
@@ -646,42 +583,36 @@ __device__ void split_join(double2* x, int n, int nA, const double2* __restrict_
 // The same join in double-float arithmetic on the FP32 pipe (double-float
 // chains): x, the spikes and the interface inverse as complex double-floats.  The
 // 16 interface values are summed by 64 threads (four partial sums each, joined
-// by shuffles); the rows go two per thread and pass, loads first.
+// by shuffles).
 __device__ void split_join_dd(ddc* x, int n, int nA, const ddc* __restrict__ spk, const ddc* __restrict__ rj,
                               bool act) {
-    __shared__ ddc xi[16];
+    __shared__ __align__(16) ddf xi[2][16];  // by component
     const int tid = threadIdx.x;
-    if (act && tid < 64) {
-        const int o = tid >> 2, part = tid & 3;  // output o, columns part*4 .. part*4+3
-        dacc acc = zero<dacc>();
+    if (act && tid < 256) {  // (output, component, two columns)
+        const int o = tid >> 4, part = (tid >> 3) & 1, c = 2 * (tid & 7);
+        const ddf* v = reinterpret_cast<const ddf*>(x + (c < 8 ? nA - 8 + c : nA + c - 8));
+        ddacc acc{0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = part * 4 + j;
-            acc = fma_x(rj[o * 16 + c], x[c < 8 ? nA - 8 + c : nA + c - 8], acc);
-        }
-        acc = reduce4(acc);
-        if (part == 0) xi[o] = fin(acc);
+        for (int j = 0; j < 2; ++j) ch_mac<false>(acc, rj[o * 16 + c + j], v[2 * j + part], v[2 * j + 1 - part], part);
+        float u, s = two_sum(acc.s, part ? acc.t : -acc.t, u), e = __fadd_rn(__fadd_rn(acc.e, part ? acc.f : -acc.f), u);
+#pragma unroll
+        for (int h = 1; h < 8; h <<= 1) dd_pair_sum(s, e, h);
+        if ((tid & 7) == 0) xi[part][o] = dd_norm(s, e);
     }
     __syncthreads();
     if (act)
-        for (int i0 = tid; i0 < n; i0 += 2 * blockDim.x) {
-            const int i1 = i0 + blockDim.x;
-            ddc s0[8], s1[8];
+        for (int t = tid; t < 2 * n; t += blockDim.x) {
+            const int part = t & 1, c0 = ((t >> 1) < nA) ? 8 : 0;
+            ddc sp[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                s0[c] = spk[(size_t)i0 * 8 + c];
-                s1[c] = (i1 < n) ? spk[(size_t)i1 * 8 + c] : zero<ddc>();
-            }
-            const ddc* v0 = (i0 < nA) ? xi + 8 : xi;
-            const ddc* v1 = (i1 < nA) ? xi + 8 : xi;
-            dacc a0 = zero<dacc>(), a1 = zero<dacc>();
+            for (int c = 0; c < 8; ++c) sp[c] = spk[(size_t)(t >> 1) * 8 + c];
+            ddf* xt = reinterpret_cast<ddf*>(x) + t;
+            ddacc acc;
+            ch_start(acc, *xt);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                a0 = fma_x(s0[c], v0[c], a0);
-                a1 = fma_x(s1[c], v1[c], a1);
-            }
-            x[i0] = sub_x(x[i0], a0);
-            if (i1 < n) x[i1] = sub_x(x[i1], a1);
+            for (int c = 0; c < 8; ++c) ch_mac<true>(acc, sp[c], xi[part][c0 + c], xi[1 - part][c0 + c], part);
+            float u, s = two_sum(acc.s, part ? -acc.t : acc.t, u);
+            *xt = dd_norm(s, __fadd_rn(__fadd_rn(acc.e, part ? -acc.f : acc.f), u));
         }
     __syncthreads();
 }
@@ -725,51 +656,6 @@ __device__ __forceinline__ double2 warp_sum(double2 v) {
         v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
     }
     return v;
-}
-
-// Schur step of Appendix A by one warp: sol[PB..] = D^{-1} h on entry;
-// sol[0..PB) = S^{-1}(g - B sol[PB..]) on exit.  B: PB x (nc-PB) real tau rows.
-template <int PB, class TF>
-__device__ void warp_schur(double2* sol, const double2* g, int nc, const double* __restrict__ B,
-                           const TF* __restrict__ Sinv) {
-    const int lane = threadIdx.x & 31;
-    const int n = nc - PB;
-    double2 t[PB];
-#pragma unroll
-    for (int r = 0; r < PB; ++r) t[r] = make_double2(0.0, 0.0);
-    for (int j = lane; j < n; j += 32) {
-        const double2 xv = sol[PB + j];
-#pragma unroll
-        for (int r = 0; r < PB; ++r) {
-            const double b = __ldg(&B[(size_t)r * n + j]);
-            t[r].x = fma(b, xv.x, t[r].x);
-            t[r].y = fma(b, xv.y, t[r].y);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < PB; ++r) t[r] = csub(g ? g[r] : make_double2(0.0, 0.0), warp_sum(t[r]));
-    if (lane < PB) {
-        double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int c = 0; c < PB; ++c) acc = cadd(acc, mul(Sinv[lane * PB + c], t[c]));
-        sol[lane] = acc;
-    }
-    __syncwarp();
-}
-
-// y2 -= Y y1 over the rows of one system, threads [t0, t0 + nt)
-template <int PB, class TF>
-__device__ void schur_update(double2* sol, int nc, const TF* __restrict__ Y, int t0, int nt) {
-    const int n = nc - PB;
-    double2 y1[PB];
-#pragma unroll
-    for (int c = 0; c < PB; ++c) y1[c] = sol[c];
-    for (int j = threadIdx.x - t0; j < n; j += nt) {
-        double2 acc = sol[PB + j];
-#pragma unroll
-        for (int c = 0; c < PB; ++c) acc = fms(acc, Y[(size_t)j * PB + c], y1[c]);
-        sol[PB + j] = acc;
-    }
 }
 
 // Row-block dot products by the whole CTA: t_r = sum_{j < nj} R[r nj + j] x[j]
@@ -820,27 +706,6 @@ __device__ TX block_rows_dot(const TX* x, int nj, const TR* __restrict__ R) {
     if (warp == 0 && lane < PB)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = add_x(v, part[w][lane]);
     return v;
-}
-
-// Schur step of Appendix A by the whole CTA: sol[PB..] = D^{-1} h on entry;
-// sol[0..PB) = S^{-1}(g - B sol[PB..]) on exit (g = 0 when null), visible to
-// every thread.  B: PB x (nc-PB) real tau rows; S^{-1} complex or real.
-template <int PB, class TS>
-__device__ void block_schur(double2* sol, const double2* g, int nc, const double* __restrict__ B,
-                            const TS* __restrict__ Sinv) {
-    const double2 t = block_rows_dot<PB>(sol + PB, nc - PB, B);
-    if ((threadIdx.x >> 5) == 0) {
-        const int lane = threadIdx.x & 31;
-        const double2 gv = (lane < PB) ? csub(g ? g[lane] : make_double2(0.0, 0.0), t) : make_double2(0.0, 0.0);
-        double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int c = 0; c < PB; ++c) {
-            const double2 gc = shfl_idx(gv, c);
-            if (lane < PB) acc = cadd(acc, mul(Sinv[lane * PB + c], gc));
-        }
-        if (lane < PB) sol[lane] = acc;
-    }
-    __syncthreads();
 }
 
 // FP32 Schur step of the temperature system by the whole CTA: sol[2..] = D^{-1} r
@@ -1001,9 +866,17 @@ __device__ void epilogue_row(const StepParams& P, const RhsSpec& R, double gdt, 
     double2 mp = make_double2(0.0, 0.0), mt = make_double2(0.0, 0.0);
     double muu = 0.0;
     if (m > 0 && k >= 4) {
-        const double2 a0 = band_row_c<8>(P.ops.band[OP_A0], xp, k, nc);
-        const double2 a2 = band_row_c<8>(P.ops.band[OP_A2], xp, k, nc);
-        mp = make_double2(fma(mu, a2.x, a0.x), fma(mu, a2.y, a0.y));
+        const double* r0 = P.ops.band[OP_A0] + (size_t)k * 17;
+        const double* r2 = P.ops.band[OP_A2] + (size_t)k * 17;
+#pragma unroll
+        for (int d = 0; d < 17; ++d) {
+            const int n = k - 8 + d;
+            if (n >= 0 && n < nc) {
+                const double c = fma(mu, __ldg(&r2[d]), __ldg(&r0[d]));
+                mp.x = fma(c, xp[n].x, mp.x);
+                mp.y = fma(c, xp[n].y, mp.y);
+            }
+        }
     }
     if (k >= 2) {
         mt = band_row_c<4>(P.ops.band[OP_D], xt, k, nc);
@@ -1046,71 +919,258 @@ __device__ void epilogue_row(const StepParams& P, const RhsSpec& R, double gdt, 
     }
 }
 
-// shared-memory layout of one CTA, per mode mi < MB:
-//   streamfunction: pf rhs (then the refinement residual), pw forward-chain
-//                   values, px solution, pd correction
-//   temperature:    tf rhs, tw forward-chain values, tx solution
-// and for the zonal flow (the CTA holding m = 0): uf rhs, ux solution (real); its
-// chain scratch is the temperature warp's, reused after the temperature solve.
+// ---------------------------------------------------------------------------
+// The same steps spread over the CTA by component (k_solve).  An FP64 instruction
+// of a warp takes 64 cycles of its sub-partition whatever it does, so a phase costs
+// its longest warp's FP64 instructions: one warp adding 4 complex sums over its
+// lanes one by one spent 40 of them (2600 cycles), the rows of a system one thread
+// each left most warps idle.  Here a task is (row, component), and the sums of
+// a row block over the CTA are added by exchanging halves of the values.
+// ---------------------------------------------------------------------------
+// v[0 .. 2^LOG): each lane's partial sums; returns the sum over the warp of value
+// (lane >> (5 - LOG)), the same in the lanes that share it.
+template <int LOG>
+__device__ __forceinline__ double warp_sums(double (&v)[1 << LOG]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 0; s < LOG; ++s) {
+        const int o = 16 >> s, half = 1 << (LOG - 1 - s);
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const double send = up ? v[i] : v[i + half];
+            const double keep = up ? v[i + half] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = 16 >> LOG; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+// Partial sums of the PB rows R (PB x nj, real) against a complex vector x, one
+// value per (row, component): part[warp][2 row + component].
+template <int PB>
+__device__ __forceinline__ void rows_dot_part(const double2* x, int nj, const double* __restrict__ R,
+                                              double (*part)[8]) {
+    constexpr int LOG = PB == 4 ? 3 : 2;
+    const int tid = threadIdx.x, lane = tid & 31;
+    double t[1 << LOG];
+#pragma unroll
+    for (int i = 0; i < 2 * PB; ++i) t[i] = 0.0;
+    for (int j = tid; j < nj; j += blockDim.x) {
+        const double2 xv = x[j];
+#pragma unroll
+        for (int r = 0; r < PB; ++r) {
+            const double b = __ldg(&R[(size_t)r * nj + j]);
+            t[2 * r] = fma(b, xv.x, t[2 * r]);
+            t[2 * r + 1] = fma(b, xv.y, t[2 * r + 1]);
+        }
+    }
+    const double v = warp_sums<LOG>(t);
+    if ((lane & ((32 >> LOG) - 1)) == 0) part[tid >> 5][lane >> (5 - LOG)] = v;
+}
+// the sums over the CTA's eight warps: lane l of the calling warp gets value l & 7
+__device__ __forceinline__ double rows_dot_sum(const double (*part)[8], int nval) {
+    const int lane = threadIdx.x & 31, i = lane & 7, w = lane >> 3;
+    double v = (i < nval) ? part[w][i] + part[w + 4][i] : 0.0;
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+// sol[0 .. PB) = S^{-1} (g - t) by one warp, t the sums of rows_dot_sum (value 2 r +
+// component in lane 2 r + component), g = 0 when null.  Lane (row, component, c)
+// takes one term.
+__device__ __forceinline__ double2 as_complex(double2 a) { return a; }
+__device__ __forceinline__ double2 as_complex(double a) { return make_double2(a, 0.0); }
+template <int PB, class TS>
+__device__ __forceinline__ void schur_apply(double2* sol, const double2* g, double t, const TS* __restrict__ Sinv) {
+    const int lane = threadIdx.x & 31;
+    double gv = 0.0;
+    if (lane < 2 * PB) gv = (g ? reinterpret_cast<const double*>(g)[lane] : 0.0) - t;
+    const int c = lane % PB, p = (lane / PB) & 1, r = lane / (2 * PB);
+    const double gx = __shfl_sync(0xffffffffu, gv, 2 * c), gy = __shfl_sync(0xffffffffu, gv, 2 * c + 1);
+    const bool on = r < PB;
+    const double2 a = on ? as_complex(Sinv[r * PB + c]) : make_double2(0.0, 0.0);
+    double v = fma(a.x, p ? gy : gx, a.y * (p ? gx : -gy));
+#pragma unroll
+    for (int o = 1; o < PB; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (on && c == 0) reinterpret_cast<double*>(sol)[2 * r + p] = v;
+}
+// component part of y2 -= Y y1, every (row, component) of the CTA
+__device__ __forceinline__ double fms_part(double acc, double a, double2 z, int part) {
+    return fma(-a, part ? z.y : z.x, acc);
+}
+template <int PB, class TF>
+__device__ __forceinline__ void schur_update_parts(double2* sol, int nc, const TF* __restrict__ Y) {
+    const int part = threadIdx.x & 1;
+    double2 y1[PB];
+#pragma unroll
+    for (int c = 0; c < PB; ++c) y1[c] = sol[c];
+    for (int t = threadIdx.x; t < 2 * (nc - PB); t += blockDim.x) {
+        double* x = reinterpret_cast<double*>(sol + PB) + t;
+        double acc = *x;
+#pragma unroll
+        for (int c = 0; c < PB; ++c) acc = fms_part(acc, Y[(size_t)(t >> 1) * PB + c], y1[c], part);
+        *x = acc;
+    }
+}
+// component part of f_k - (L x)_k, a complex band row of half width 8
+__device__ __forceinline__ double residual_part(double acc, const double2* __restrict__ row, const double2* x, int k, int nc,
+                                                int part) {
+#pragma unroll
+    for (int d = 0; d < 17; ++d) {
+        const int n = k - 8 + d;
+        if (n >= 0 && n < nc) acc = fms_part(acc, __ldg(&row[d]), x[n], part);
+    }
+    return acc;
+}
+// row k, one component, of a real band applied to complex values (x: that component, stride 2)
+template <int H>
+__device__ __forceinline__ double band_part(const double* __restrict__ band, const double* x, int k, int nc) {
+    const double* row = band + (size_t)k * (2 * H + 1);
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d <= 2 * H; ++d) {
+        const int n = k - H + d;
+        if (n >= 0 && n < nc) acc = fma(__ldg(&row[d]), x[2 * n], acc);
+    }
+    return acc;
+}
+// Epilogue of a solve (epilogue_row) for one component of row k: the streamfunction's
+// mass term A^I_m Psi and its implicit term (mass - f)/(gamma dt), f the component
+// of the assembled right-hand side (fps) or, null, its terms summed again.
+__device__ __forceinline__ void epilogue_psi_part(const StepParams& P, const RhsSpec& R, double gdt, int m, int k, int part,
+                                                  const double2* xp, VecSet mass_out, VecSet imp_out, bool want_mass,
+                                                  bool want_imp, const double2* fps) {
+    const int nc = P.nc;
+    const size_t idx = 2 * ((size_t)m * nc + k) + part;
+    const double mu = (double)m * m;
+    double mp = 0.0, im = 0.0;
+    if (m > 0 && k >= 4) {
+        const double* r0 = P.ops.band[OP_A0] + (size_t)k * 17;
+        const double* r2 = P.ops.band[OP_A2] + (size_t)k * 17;
+        const double* x = reinterpret_cast<const double*>(xp) + part;
+        // the row's coefficients, half of them by each component's lane
+        const unsigned both = 3u << (threadIdx.x & 30);
+        double c[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int d = min(2 * i + part, 16);
+            c[i] = fma(mu, __ldg(&r2[d]), __ldg(&r0[d]));
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const double o = __shfl_xor_sync(both, c[i], 1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int n = k - 8 + 2 * i + h;
+                if (2 * i + h < 17 && n >= 0 && n < nc) mp = fma(h == part ? c[i] : o, x[2 * n], mp);
+            }
+        }
+        if (want_imp) {  // before any store: an output may be one of the terms of f
+            double f = 0.0;
+            if (fps)
+                f = reinterpret_cast<const double*>(fps)[2 * k + part];
+            else
+                for (int t = 0; t < R.nterms; ++t) f = fma(R.t[t].c, reinterpret_cast<const double*>(R.t[t].v.psi)[idx], f);
+            im = (mp - f) * (1.0 / gdt);
+        }
+    }
+    if (want_imp) reinterpret_cast<double*>(imp_out.psi)[idx] = im;
+    if (want_mass) reinterpret_cast<double*>(mass_out.psi)[idx] = mp;
+}
+// the same for the temperature (fts always kept) and, for m = 0 and component 0,
+// the zonal flow (fus kept, or null)
+__device__ __forceinline__ void epilogue_theta_part(const StepParams& P, const RhsSpec& R, double gdt, int m, int k,
+                                                    int part, const double2* xt, const double* xu, VecSet mass_out,
+                                                    VecSet imp_out, bool want_mass, bool want_imp, const double2* fts,
+                                                    const double* fus) {
+    const int nc = P.nc;
+    const size_t idx = 2 * ((size_t)m * nc + k) + part;
+    const double ig = 1.0 / gdt;
+    const double mt = (k >= 2) ? band_part<4>(P.ops.band[OP_D], reinterpret_cast<const double*>(xt) + part, k, nc) : 0.0;
+    if (want_imp)
+        reinterpret_cast<double*>(imp_out.th)[idx] =
+            (k >= 2) ? (mt - reinterpret_cast<const double*>(fts)[2 * k + part]) * ig : 0.0;
+    if (want_mass) reinterpret_cast<double*>(mass_out.th)[idx] = mt;
+    if (m == 0 && part == 0) {
+        double mu = 0.0;
+        if (k >= 2) {
+            const double* rd = P.ops.band[OP_D] + (size_t)k * 9;
+            for (int d = 0; d < 9; ++d) {
+                const int n = k - 4 + d;
+                if (n >= 0 && n < nc) mu = fma(__ldg(&rd[d]), xu[n], mu);
+            }
+        }
+        if (want_imp) {
+            double f = 0.0;
+            if (fus)
+                f = fus[k];
+            else
+                for (int t = 0; t < R.nterms; ++t) f = fma(R.t[t].c, R.t[t].v.u[k], f);
+            imp_out.u[k] = (k >= 2) ? (mu - f) * ig : 0.0;
+        }
+        if (want_mass) mass_out.u[k] = mu;
+    }
+}
+
+// shared-memory layout of one CTA (chains run in place in the solution's array):
+//   streamfunction: pf rhs (then the refinement residual), px solution, pd correction
+//   temperature:    tf rhs, tx solution
+// and for the zonal flow (the CTA holding m = 0): uf rhs, ux solution (real).
 struct SolveSmem {
-    double2 *pf[2], *pw[2], *px[2], *pd[2], *tf[2], *tw[2], *tx[2];
+    double2 *pf, *px, *pd, *tf, *tx;
     double *uf, *ux;
-    float2 *tr, *tq, *td;  // refined FP32 temperature solves: residual, chain scratch, correction (MB = 1)
-    float* ring32;         // coefficient rings of the FP32 temperature walks (one CTA per system)
+    float2 *tr, *td;  // refined FP32 temperature solves: residual, correction
+    char *ring_p, *ring_t, *ring_u;  // the walks' rings of matrices (the zonal flow's over the streamfunction's)
+    double (*prevs)[32];             // the walking warps' previous blocks
     // the streamfunction and zonal-flow right-hand sides as assembled (pf and uf
     // become residuals), for the epilogue; past the end of solve_smem_doubles,
-    // present when the launch adds keep_f_doubles (MB = 1)
+    // present when the launch adds keep_f_doubles
     double2* fp;
     double* fu;
 };
 
 __host__ __device__ inline int round8(int n) { return (n + 7) / 8 * 8; }
 
-// DEEP (the FP32-refined temperature solve): the FP64 temperature chain scratch
-// tw is not used, so it is left out (at N_c = 1365 this lets the epilogue keep
-// the assembled right-hand sides in shared memory)
-__host__ __device__ inline size_t solve_smem_doubles(int nc, int MB, bool deep = false) {
-    const int b = round8(nc);
-    return (size_t)MB * 2 * (deep ? 6 : 7) * b + 2 * (size_t)b + 3 * (size_t)b;  // last: 3 b float2
+// rows of an array that a chain solves in place: whole blocks past an offset of up to 4
+__host__ __device__ inline int chain_rows(int nc) { return round8(nc) + 8; }
+
+__host__ __device__ inline size_t solve_smem_doubles(int nc) {
+    return (size_t)14 * chain_rows(nc) + (4 * ring_bytes<double2>(RD) + 2 * ring_bytes<double>(RD)) / 8;
 }
 
 __host__ __device__ inline size_t keep_f_doubles(int nc) { return 3 * (size_t)round8(nc); }
 
-template <int MB, bool DEEP = false>
-__device__ SolveSmem carve(double2* base, int nc) {
+__device__ __forceinline__ SolveSmem carve(double2* base, int nc) {
     SolveSmem s;
-    const int b = round8(nc);
-    double2* p = base;
-    for (int i = 0; i < MB; ++i) {
-        s.pf[i] = p; p += b;
-        s.pw[i] = p; p += b;
-        s.px[i] = p; p += b;
-        s.pd[i] = p; p += b;
-        s.tf[i] = p; p += b;
-        if (DEEP) {
-            s.tw[i] = nullptr;
-        } else {
-            s.tw[i] = p; p += b;
-        }
-        s.tx[i] = p; p += b;
-    }
-    double* d = reinterpret_cast<double*>(p);
-    s.uf = d; d += b;
-    s.ux = d; d += b;
-    float2* f = reinterpret_cast<float2*>(d);
-    s.tr = f; f += b;
-    s.tq = f; f += b;
-    s.td = f; f += b;
-    s.fp = reinterpret_cast<double2*>(f);
-    s.fu = reinterpret_cast<double*>(s.fp + b);
+    const int b = chain_rows(nc);
+    s.pf = base;
+    s.px = base + b;
+    s.pd = base + 2 * b;
+    s.tf = base + 3 * b;
+    s.tx = base + 4 * b;
+    s.uf = reinterpret_cast<double*>(base + 5 * b);
+    s.ux = s.uf + b;
+    s.tr = reinterpret_cast<float2*>(s.ux + b);
+    s.td = s.tr + b;
+    s.ring_p = reinterpret_cast<char*>(s.td + b);
+    s.ring_t = s.ring_p + 4 * ring_bytes<double2>(RD);
+    s.ring_u = s.ring_p;
+    s.fp = reinterpret_cast<double2*>(s.ring_t + 2 * ring_bytes<double>(RD));
+    s.fu = reinterpret_cast<double*>(s.fp + round8(nc));
     return s;
+}
+
+// The zonal flow's chain (the CTA of m = 0) by warps 4-5
+__device__ void zonal_chains(const DevFactors& F, SolveSmem& s, double* b, double* x, int nt) {
+    run_chains<RD, 2>(no_job<double, 1>(), no_job<double, 1>(), no_job<float, 2>(),
+                      ChainJob<double, 1>{b, x, x, nt, F.uBlk, 4, s.ring_u}, s.prevs);
 }
 
 // One FP64 refinement step of the zonal-flow solve (the CTA of m = 0, large N_c):
 // r = f - L u over the assembled rows and the tau rows, solved with the same
 // factors, u += correction.  The residual replaces the right-hand side; the
-// correction and its chain scratch use streamfunction arrays, which mode 0 leaves
-// unused.
+// correction uses a streamfunction array, which mode 0 leaves unused.
 __device__ void refine_zonal_flow(const StepParams& P, const DevFactors& F, SolveSmem& s) {
     const int nc = P.nc, nt = nc - 2;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
@@ -1137,9 +1197,9 @@ __device__ void refine_zonal_flow(const StepParams& P, const DevFactors& F, Solv
         if (lane < 2) s.uf[lane] = -(lane ? t1 : t0);
     }
     __syncthreads();
-    double* du = reinterpret_cast<double*>(s.pw[0]);
-    if (warp == 4 || warp == 5) {
-        pair_block_solve<8, PFB>(s.uf + 2, reinterpret_cast<double*>(s.pf[0]), du + 2, nt, F.uBlk, true, warp - 4, 3);
+    double* du = reinterpret_cast<double*>(s.pd);
+    zonal_chains(F, s, s.uf + 2, du + 2, nt);
+    {
         if (warp == 4) {
             double t0 = 0.0, t1 = 0.0;
             for (int j = lane; j < nt; j += 32) {
@@ -1167,7 +1227,7 @@ __device__ void refine_zonal_flow(const StepParams& P, const DevFactors& F, Solv
     __syncthreads();
 }
 
-// FP64 residual r = f - L x of the temperature system of mode m0 (MB == 1),
+// FP64 residual r = f - L x of the temperature system of mode m0,
 // rounded to FP32 into s.tr: the assembled rows by the whole CTA, the two tau
 // rows (r = 0 - tau x) by warp tw.  The caller synchronises.
 __device__ void temperature_residual(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0, int tw) {
@@ -1175,18 +1235,18 @@ __device__ void temperature_residual(const StepParams& P, const DevFactors& F, S
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
     for (int k = 2 + tid; k < nc; k += nth) {
         const double* row = F.tBand + ((size_t)m0 * nt + (k - 2)) * 9;
-        double2 acc = s.tf[0][k];
+        double2 acc = s.tf[k];
 #pragma unroll
         for (int d = 0; d < 9; ++d) {
             const int n = k - 4 + d;
-            if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), s.tx[0][n]);
+            if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), s.tx[n]);
         }
         s.tr[k] = to_f2(acc);
     }
     if (warp == tw) {
         double2 t0 = make_double2(0.0, 0.0), t1 = t0;
         for (int j = lane; j < nc; j += 32) {
-            const double2 xv = s.tx[0][j];
+            const double2 xv = s.tx[j];
             const double b0 = __ldg(&P.ops.tau_dir[j]), b1 = __ldg(&P.ops.tau_dir[nc + j]);
             t0.x = fma(b0, xv.x, t0.x);
             t0.y = fma(b0, xv.y, t0.y);
@@ -1204,16 +1264,13 @@ __device__ void temperature_residual(const StepParams& P, const DevFactors& F, S
 // joined through the spikes.  Whole CTA; ends with a barrier.
 __device__ void theta32_chains(const DevFactors& F, SolveSmem& s, int m, int nt, int nbt) {
     const float* tb = (F.tsplit ? F.tBlk32S : F.tBlk32) + (size_t)m * nbt * 192;
-    if (F.tsplit) {
-        const int ntA = 8 * (nbt / 2);
-        cta_chain_solve<RD_32, float, float2, float2>(s.tr + 2, s.tq, s.td + 2, ntA, tb, 2, s.tr + 2 + ntA, s.tq + ntA,
-                                                      s.td + 2 + ntA, nt - ntA, tb + (size_t)(nbt / 2) * 192, 4,
-                                                      s.ring32);
-        split_join32(s.td + 2, nt, ntA, F.tSpk32 + (size_t)m * nt * 8, F.tRj32 + (size_t)m * 256);
-    } else {
-        cta_chain_solve<RD_32, float, float2, float2>(s.tr + 2, s.tq, s.td + 2, nt, tb, 2, nullptr, nullptr, nullptr, 0,
-                                                      nullptr, 0, s.ring32);
-    }
+    float *b = reinterpret_cast<float*>(s.tr + 2), *x = reinterpret_cast<float*>(s.td + 2);
+    const int ntA = F.tsplit ? 8 * (nbt / 2) : nt;
+    run_chains<RD, 4>(ChainJob<float, 2>{b, x, x, ntA, tb, 2, s.ring_t},
+                      ChainJob<float, 2>{b + 2 * ntA, x + 2 * ntA, x + 2 * ntA, nt - ntA, tb + (size_t)(nbt / 2) * 192, 4,
+                                         s.ring_t + 2 * ring_bytes<float>(RD)},
+                      no_job<double, 1>(), no_job<double, 1>(), s.prevs);
+    if (F.tsplit) split_join32(s.td + 2, nt, ntA, F.tSpk32 + (size_t)m * nt * 8, F.tRj32 + (size_t)m * 256);
 }
 
 // The same residual with the tau rows summed by the whole CTA (kernel with one
@@ -1224,15 +1281,15 @@ __device__ void temperature_residual_block(const StepParams& P, const DevFactors
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
     for (int k = 2 + tid; k < nc; k += nth) {
         const double* row = F.tBand + ((size_t)m0 * nt + (k - 2)) * 9;
-        double2 acc = s.tf[0][k];
+        double2 acc = s.tf[k];
 #pragma unroll
         for (int d = 0; d < 9; ++d) {
             const int n = k - 4 + d;
-            if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), s.tx[0][n]);
+            if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), s.tx[n]);
         }
         s.tr[k] = to_f2(acc);
     }
-    const double2 t = block_rows_dot<2>(s.tx[0], nc, P.ops.tau_dir);
+    const double2 t = block_rows_dot<2>(s.tx, nc, P.ops.tau_dir);
     if (warp == 0 && lane < 2) s.tr[lane] = to_f2(make_double2(-t.x, -t.y));
 }
 
@@ -1240,7 +1297,7 @@ __device__ void temperature_residual_block(const StepParams& P, const DevFactors
 // ir_t corrections x += S32^{-1}(f - L x), every reduction by the whole CTA.
 __device__ void temperature_corrections_roles(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0) {
     const int nc = P.nc, nt = nc - 2, nbt = (nt + 7) / 8;
-    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
+    const int tid = threadIdx.x, nth = blockDim.x;
     for (int it = 0; it < F.ir_t; ++it) {
         temperature_residual_block(P, F, s, m0);
         __syncthreads();
@@ -1248,80 +1305,121 @@ __device__ void temperature_corrections_roles(const StepParams& P, const DevFact
         block_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
         schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
         __syncthreads();
-        for (int n = tid; n < nc; n += nth) s.tx[0][n] = cadd(s.tx[0][n], to_d2_bits(s.td[n]));
+        for (int n = tid; n < nc; n += nth) s.tx[n] = cadd(s.tx[n], to_d2_bits(s.td[n]));
         __syncthreads();
     }
+}
+
+// the whole FP32 temperature block, walked by warps w, w + 1
+__device__ __forceinline__ ChainJob<float, 2> theta32_job(const DevFactors& F, const SolveSmem& s, int m0, int nt, int nbt, int w) {
+    return ChainJob<float, 2>{reinterpret_cast<float*>(s.tr + 2), reinterpret_cast<float*>(s.td + 2),
+                              reinterpret_cast<float*>(s.td + 2), nt, F.tBlk32 + (size_t)m0 * nbt * 192, w, s.ring_t};
 }
 
 // The FP32-refined temperature solve (F.ir_t > 0, MB == 1): x += S32^{-1}(f - L x)
 // for the passes it0 .. ir_t - 1 (pass 0 may have run beside the streamfunction
 // refinement), then the FP64 refinement of the zonal flow (mode 0).
-template <int MB, bool DEEP>
 __device__ void temperature_corrections(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0, bool has_u,
                                         int it0) {
     const int nc = P.nc, nt = nc - 2, nbt = (nt + 7) / 8;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
-    constexpr int PT = DEEP ? PFB_DEEP_T : PFB;
     if (F.ir_t) {
         for (int it = it0; it < F.ir_t; ++it) {
             temperature_residual(P, F, s, m0, 0);
             __syncthreads();
-            if (warp == 2 || warp == 3)
-                pair_block_solve<8, PT>(s.tr + 2, s.tq, s.td + 2, nt, F.tBlk32 + (size_t)m0 * nbt * 192, true, warp - 2, 2);
-            __syncthreads();
+            run_chains<RD, 4>(no_job<float, 2>(), no_job<float, 2>(), theta32_job(F, s, m0, nt, nbt, 2), no_job<double, 1>(), s.prevs);
             if (warp == 2) warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
             __syncthreads();
             schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
             __syncthreads();
-            for (int n = tid; n < nc; n += nth) s.tx[0][n] = cadd(s.tx[0][n], to_d2_bits(s.td[n]));
+            for (int n = tid; n < nc; n += nth) s.tx[n] = cadd(s.tx[n], to_d2_bits(s.td[n]));
             __syncthreads();
         }
         if (has_u) refine_zonal_flow(P, F, s);  // FP64
     }
 }
 
-template <int MB, bool DEEP, bool DDP = false>
-__global__ void __launch_bounds__(NTHREADS_S) k_solve(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
+// T32: the temperature by FP32 chains refined from FP64 residuals (F.ir_t); DDP:
+// double-float streamfunction chains (explicit buoyancy)
+template <bool T32, bool DDP>
+__global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                       VecSet mass_out, VecSet imp_out, int want_mass,
                                                       int want_imp, int keep_f) {
     extern __shared__ double2 sm[];
-    const int nc = P.nc, M = P.M;
-    const int m0 = P.m_lo + blockIdx.x * MB;
+    __shared__ double part_p[NTHREADS_S / 32][8], part_t[NTHREADS_S / 32][8];
+    const int nc = P.nc;
+    const int m0 = P.m_lo + blockIdx.x;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const int part = tid & 1;  // the component of this thread's tasks
     const int np = nc - 4, nt = nc - 2;
     const int nbp = (np + 7) / 8, nbt = (nt + 7) / 8;
     const int nA = 8 * (nbp / 2);  // first half of a split streamfunction block (F.psplit)
-    SolveSmem s = carve<MB, DEEP>(sm, nc);
+    SolveSmem s = carve(sm, nc);
+    __shared__ __align__(16) double prevs[NTHREADS_S / 32][32];
+    s.prevs = prevs;
     const bool has_u = (m0 == 0);
-    constexpr int PP = DEEP ? PFB_DEEP_P : PFB, PT = DEEP ? PFB_DEEP_T : PFB;
+    // Warps w, w + 4 of a CTA run on the same sub-partition, and so do the same warps of
+    // the two CTAs of an SM, whose chains then wait for one FP64 pipe: the CTA in the
+    // odd slot swaps its warp pairs (a hint only; any value gives the same results).
+    __shared__ int flip_s;
+    if (tid == 0) {
+        unsigned w;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
+        flip_s = (w >> 3) & 1 ? 2 : 0;
+    }
+    __syncthreads();
+    const int flip = flip_s;
+    using CP = std::conditional_t<DDP, ddc, double2>;  // the streamfunction chain's coefficients and components
+    using VP = typename Chain<CP>::V;
+    const CP* blk_p = DDP ? reinterpret_cast<const CP*>(F.pBlkDD) : reinterpret_cast<const CP*>(F.pBlk);
+    blk_p += (size_t)m0 * nbp * 192;
+    const ddc* spk_dd = reinterpret_cast<const ddc*>(F.pSpkDD) + (size_t)m0 * np * 8;
+    const ddc* rj_dd = reinterpret_cast<const ddc*>(F.pRjDD) + (size_t)m0 * 256;
+    // the streamfunction block, one or (psplit) two halves: right-hand side b to x
+    auto job_p = [&](double2* b, double2* x, bool second) {
+        const int n0 = second ? nA : 0, n = m0 == 0 ? 0 : second ? (F.psplit ? np - nA : 0) : F.psplit ? nA : np;
+        return ChainJob<CP, 2>{reinterpret_cast<VP*>(b + 4 + n0), reinterpret_cast<VP*>(x + 4 + n0), reinterpret_cast<VP*>(x + 4 + n0), n,
+                               blk_p + (second ? (size_t)(nbp / 2) * 192 : 0), (second ? 6 : 0) ^ flip,
+                               s.ring_p + (second ? 2 * ring_bytes<CP>(RD) : 0)};
+    };
+    // the temperature: FP32, or FP64
+    using CT = std::conditional_t<T32, float, double>;
+    auto job_t = [&]() {
+        if constexpr (T32)
+            return theta32_job(F, s, m0, nt, nbt, 2 ^ flip);
+        else
+            return ChainJob<double, 2>{reinterpret_cast<double*>(s.tf + 2), reinterpret_cast<double*>(s.tx + 2),
+                                       reinterpret_cast<double*>(s.tx + 2), nt, F.tBlk + (size_t)m0 * nbt * 192, 2 ^ flip, s.ring_t};
+    };
+    auto job_u = [&]() {
+        return ChainJob<double, 1>{s.uf + 2, s.ux + 2, s.ux + 2, nt, F.uBlk, 4 ^ flip, s.ring_u};
+    };
+    auto flat = [](double2* v) { return reinterpret_cast<double*>(v); };
 
     // 1. right-hand side sum_t c_t V_t (tau rows zero)
-    for (int idx = tid; idx < MB * nc; idx += nth) {
-        const int mi = idx / nc, n = idx - mi * nc, m = m0 + mi;
-        if (m >= M) continue;
-        double2 ap = make_double2(0.0, 0.0), at = make_double2(0.0, 0.0);
-        double au = 0.0;
+    for (int q = tid; q < 2 * nc; q += nth) {
+        const int n = q >> 1;
+        const size_t idx = (size_t)m0 * 2 * nc + q;
+        double ap = 0.0, at = 0.0, au = 0.0;
 #pragma unroll 4
         for (int t = 0; t < R.nterms; ++t) {
             const double c = R.t[t].c;
-            const double2 vp = R.t[t].v.psi[(size_t)m * nc + n];
-            const double2 vt = R.t[t].v.th[(size_t)m * nc + n];
-            ap.x = fma(c, vp.x, ap.x);
-            ap.y = fma(c, vp.y, ap.y);
-            at.x = fma(c, vt.x, at.x);
-            at.y = fma(c, vt.y, at.y);
-            if (m == 0) au = fma(c, R.t[t].v.u[n], au);
+            ap = fma(c, reinterpret_cast<const double*>(R.t[t].v.psi)[idx], ap);
+            at = fma(c, reinterpret_cast<const double*>(R.t[t].v.th)[idx], at);
+            if (has_u) au = fma(c, R.t[t].v.u[n], au);
         }
-        s.pf[mi][n] = (n < 4 || m == 0) ? make_double2(0.0, 0.0) : ap;
-        // double-float streamfunction chains (explicit buoyancy, MB = 1): the
-        // right-hand side as double-floats in pd, which the correction fills later
-        if (DDP && m > 0) reinterpret_cast<ddc*>(s.pd[0])[n] = dd_from_bits(s.pf[0][n]);
-        s.tf[mi][n] = (n < 2) ? make_double2(0.0, 0.0) : at;
-        if (F.ir_t) s.tr[n] = to_f2(s.tf[mi][n]);  // MB == 1 with ir_t
-        if (m == 0) s.uf[n] = (n < 2) ? 0.0 : au;
-        if (MB == 1 && keep_f) {  // for the epilogue: pf and uf become residuals
-            s.fp[n] = s.pf[mi][n];
-            if (m == 0) s.fu[n] = s.uf[n];
+        if (n < 4 || m0 == 0) ap = 0.0;
+        if (n < 2) at = 0.0;
+        flat(s.pf)[q] = ap;
+        // double-float streamfunction chains (explicit buoyancy): the right-hand side
+        // as double-floats in pd, which the correction fills later
+        if (DDP && m0 > 0) reinterpret_cast<ddf*>(s.pd)[q] = dd_from_bits(ap);
+        flat(s.tf)[q] = at;
+        if (T32) reinterpret_cast<float*>(s.tr)[q] = f32_from_bits(at);
+        if (has_u && part == 0) s.uf[n] = (n < 2) ? 0.0 : au;
+        if (keep_f) {  // for the epilogue: pf and uf become residuals
+            flat(s.fp)[q] = ap;
+            if (has_u && part == 0) s.fu[n] = s.uf[n];
         }
     }
     __syncthreads();
@@ -1337,72 +1435,41 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve(StepParams P, RhsSpec R, D
         if (P.buoy_imp && pass == 1) {
             if (m0 > 0) {
                 const double cb = F.gdt * P.Ra / P.Pr * (double)m0 / P.s_o;
-                for (int k = 4 + tid; k < nc; k += nth)
-                    s.pf[0][k] = cadd(s.pf[0][k], cmul_i(band_row_c<8>(P.ops.band[OP_C], s.tx[0], k, nc), cb));
+                for (int q = 8 + tid; q < 2 * nc; q += nth) {
+                    const double v = band_part<8>(P.ops.band[OP_C], flat(s.tx) + (part ^ 1), q >> 1, nc);
+                    flat(s.pf)[q] = fma(part ? cb : -cb, v, flat(s.pf)[q]);
+                }
             }
             __syncthreads();
         }
-        // 2. banded solves by warp pairs meeting at their middle blocks: warps 0-1
-        //    streamfunction, 2-3 temperature, 4-5 zonal flow (m = 0 only; its chain
-        //    scratch is the streamfunction correction array, unused until step 5)
-        if (warp < 2) {
-            if (do_p) {
-                const bool act = m0 > 0;
-                if constexpr (DDP)
-                    pair_block_solve<8, PP, ddc, ddc, dacc>(
-                        reinterpret_cast<ddc*>(s.pd[0]) + 4, reinterpret_cast<ddc*>(s.pw[0]),
-                        reinterpret_cast<ddc*>(s.px[0]) + 4, F.psplit ? nA : np,
-                        reinterpret_cast<const ddc*>(F.pBlkDD) + (size_t)(act ? m0 : 0) * nbp * 192, act, warp, 1);
-                else
-                    pair_block_solve<8, PP>(s.pf[0] + 4, s.pw[0], s.px[0] + 4, F.psplit ? nA : np,
-                                            F.pBlk + (size_t)(act ? m0 : 0) * nbp * 192, act, warp, 1);
-            }
-        } else if (warp >= 6) {
-            if (do_p && F.psplit) {  // the second half of the streamfunction block
-                const bool act = m0 > 0;
-                if constexpr (DDP)
-                    pair_block_solve<8, PP, ddc, ddc, dacc>(
-                        reinterpret_cast<ddc*>(s.pd[0]) + 4 + nA, reinterpret_cast<ddc*>(s.pw[0]) + nA,
-                        reinterpret_cast<ddc*>(s.px[0]) + 4 + nA, np - nA,
-                        reinterpret_cast<const ddc*>(F.pBlkDD) + ((size_t)(act ? m0 : 0) * nbp + nbp / 2) * 192, act,
-                        warp - 6, 4);
-                else
-                    pair_block_solve<8, PP>(s.pf[0] + 4 + nA, s.pw[0] + nA, s.px[0] + 4 + nA, np - nA,
-                                            F.pBlk + ((size_t)(act ? m0 : 0) * nbp + nbp / 2) * 192, act, warp - 6, 4);
-            }
-        } else if (warp < 4) {
-            if (do_t) {
-                if (F.ir_t)
-                    pair_block_solve<8, PT>(s.tr + 2, s.tq, s.td + 2, nt, F.tBlk32 + (size_t)m0 * nbt * 192, true, warp - 2,
-                                        2);
-                else
-                    pair_block_solve<8, PP>(s.tf[0] + 2, s.tw[0], s.tx[0] + 2, nt, F.tBlk + (size_t)m0 * nbt * 192, true,
-                                        warp - 2, 2);
-            }
-        } else if (warp < 6 && has_u) {
-            if (do_t)
-                pair_block_solve<8, PFB>(s.uf + 2, reinterpret_cast<double*>(s.pd[0]), s.ux + 2, nt, F.uBlk, true, warp - 4,
-                                    3);
-        }
-        __syncthreads();
+        // 2. banded solves by warp pairs: warps 0-1 the streamfunction (6-7 its second
+        //    half), 2-3 the temperature, 4-5 the zonal flow (m = 0 only)
+        run_chains<RD, 2>(do_p ? job_p(DDP ? s.pd : s.pf, s.px, false) : no_job<CP, 2>(),
+                          do_p ? job_p(DDP ? s.pd : s.pf, s.px, true) : no_job<CP, 2>(),
+                          do_t ? job_t() : no_job<CT, 2>(), do_t && has_u ? job_u() : no_job<double, 1>(), s.prevs);
         if (DDP && do_p && m0 > 0) {  // the solution back from double-floats
-            const ddc* xd = reinterpret_cast<const ddc*>(s.px[0]);
-            for (int n = 4 + tid; n < nc; n += nth) s.px[0][n] = dd_compose(xd[n]);
+            if (F.psplit) split_join_dd(reinterpret_cast<ddc*>(s.px) + 4, np, nA, spk_dd, rj_dd, true);
+            const ddf* xd = reinterpret_cast<const ddf*>(s.px);
+            for (int q = 8 + tid; q < 2 * nc; q += nth) flat(s.px)[q] = dd_compose(xd[q]);
             __syncthreads();
         }
-        if (do_p && F.psplit)
-            split_join(s.px[0] + 4, np, nA, F.pSpk + (size_t)(m0 > 0 ? m0 : 0) * np * 8,
+        if (!DDP && do_p && F.psplit)
+            split_join(s.px + 4, np, nA, F.pSpk + (size_t)(m0 > 0 ? m0 : 0) * np * 8,
                        F.pRj + (size_t)(m0 > 0 ? m0 : 0) * 256, m0 > 0);
 
-        // 3. Schur steps: warp 0 streamfunction, 2 temperature, 4 zonal flow
+        // 3. Schur steps: the tau rows' sums by the CTA, then warp 0 the streamfunction,
+        //    2 the temperature, 4 the zonal flow
+        if (do_p && m0 > 0) rows_dot_part<4>(s.px + 4, np, P.ops.tau_psi_B, part_p);
+        if (do_t && !T32) rows_dot_part<2>(s.tx + 2, nt, P.ops.tau_dir_B, part_t);
+        __syncthreads();
         if (warp == 0) {
-            if (do_p && m0 > 0) warp_schur<4>(s.px[0], nullptr, nc, P.ops.tau_psi_B, F.pSinv + (size_t)m0 * 16);
+            if (do_p && m0 > 0) schur_apply<4>(s.px, nullptr, rows_dot_sum(part_p, 8), F.pSinv + (size_t)m0 * 16);
         } else if (warp == 2) {
             if (do_t) {
-                if (F.ir_t)
+                if (T32)
                     warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
                 else
-                    warp_schur<2>(s.tx[0], nullptr, nc, P.ops.tau_dir_B, F.tSinv + (size_t)m0 * 4);
+                    schur_apply<2>(s.tx, nullptr, rows_dot_sum(part_t, 4), F.tSinv + (size_t)m0 * 4);
             }
         } else if (warp == 4 && has_u && do_t) {
             double t0 = 0.0, t1 = 0.0;
@@ -1419,35 +1486,25 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve(StepParams P, RhsSpec R, D
             __syncwarp();
         }
         __syncthreads();
-        // 4. y2 -= Y y1 (threads split evenly over the systems of the CTA)
-        {
-            const int per = nth / (2 * MB);
-            const int sys = tid / per, t0 = sys * per;
-            if (sys < MB) {
-                const int m = m0 + sys;
-                if (do_p && m < M && m > 0) schur_update<4>(s.px[sys], nc, F.pY + (size_t)m * np * 4, t0, per);
-            } else if (sys < 2 * MB) {
-                const int mi = sys - MB, m = m0 + mi;
-                if (do_t && m < M) {
-                    if (F.ir_t)
-                        schur_update32_dir(s.td, nc, F.tY32 + (size_t)m * nt * 2, t0, per);
-                    else
-                        schur_update<2>(s.tx[mi], nc, F.tY + (size_t)m * nt * 2, t0, per);
-                }
-            }
-            if (has_u && do_t) {
-                __syncthreads();
+        // 4. y2 -= Y y1
+        if (do_p && m0 > 0) schur_update_parts<4>(s.px, nc, F.pY + (size_t)m0 * np * 4);
+        if (do_t) {
+            if (T32)
+                schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
+            else
+                schur_update_parts<2>(s.tx, nc, F.tY + (size_t)m0 * nt * 2);
+            if (has_u) {
                 const double u0 = s.ux[0], u1 = s.ux[1];
                 for (int j = tid; j < nt; j += nth)
                     s.ux[2 + j] -= F.uY[(size_t)j * 2] * u0 + F.uY[(size_t)j * 2 + 1] * u1;
             }
         }
         __syncthreads();
-        if (F.ir_t && do_t) {  // the FP32 temperature solve becomes the FP64 iterate
-            for (int n = tid; n < nc; n += nth) s.tx[0][n] = to_d2_bits(s.td[n]);
+        if (T32 && do_t) {  // the FP32 temperature solve becomes the FP64 iterate
+            for (int n = tid; n < nc; n += nth) s.tx[n] = to_d2_bits(s.td[n]);
             __syncthreads();
         }
-        if (P.buoy_imp && pass == 0) temperature_corrections<MB, DEEP>(P, F, s, m0, has_u, 0);
+        if (P.buoy_imp && pass == 0) temperature_corrections(P, F, s, m0, has_u, 0);
     }
 
     // 5. one refinement step of the streamfunction solve: r = f - L x (a second
@@ -1455,225 +1512,272 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve(StepParams P, RhsSpec R, D
     //    With the FP32-refined temperature solve and explicit buoyancy the first
     //    temperature correction runs beside it: its chain (FP32, warps 2-3) beside
     //    the streamfunction chains (FP64), on disjoint arrays.
-    const bool fuse_t = F.ir_t && !P.buoy_imp;
-    for (int it = 0; it < 1; ++it) {
-    for (int idx = tid; idx < MB * nc; idx += nth) {
-        const int mi = idx / nc, k = idx - mi * nc, m = m0 + mi;
-        if (m >= M || m == 0 || k < 4) continue;
-        const double2* row = F.pBand + ((size_t)m * np + (k - 4)) * 17;
-        // pass 0: r = f - L x; later passes: r <- r - L d (d: the last correction)
-        const double2* x = it ? s.pd[mi] : s.px[mi];
-        double2 acc = s.pf[mi][k];
-#pragma unroll
-        for (int d = 0; d < 17; ++d) {
-            const int n = k - 8 + d;
-            if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), x[n]);
+    const bool fuse_t = T32 && !P.buoy_imp;
+    if (m0 > 0) {
+        for (int q = 8 + tid; q < 2 * nc; q += nth) {
+            const int k = q >> 1;
+            const double acc = residual_part(flat(s.pf)[q], F.pBand + ((size_t)m0 * np + (k - 4)) * 17, s.px, k, nc, part);
+            if (DDP)  // the residual replaces the right-hand side, as double-floats
+                reinterpret_cast<ddf*>(s.pf)[q] = dd_from_bits(acc);
+            else
+                flat(s.pf)[q] = acc;
         }
-        s.pf[mi][k] = acc;  // the residual replaces the right-hand side
-        if (DDP) reinterpret_cast<ddc*>(s.pf[0])[k] = dd_from_bits(acc);  // in place, as double-floats
-    }
-    if (warp < MB) {  // tau rows: r = 0 - tau x
-        const int m = m0 + warp;
-        if (m < M && m > 0) {
-            double2 t[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) t[r] = make_double2(0.0, 0.0);
-            for (int j = lane; j < nc; j += 32) {
-                const double2 xv = it ? s.pd[warp][j] : s.px[warp][j];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const double b = __ldg(&P.ops.tau_psi[(size_t)r * nc + j]);
-                    t[r].x = fma(b, xv.x, t[r].x);
-                    t[r].y = fma(b, xv.y, t[r].y);
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) t[r] = warp_sum(t[r]);
-            if (lane < 4) s.pf[warp][lane] = csub(s.pf[warp][lane], t[lane]);
-        }
+        rows_dot_part<4>(s.px, nc, P.ops.tau_psi, part_p);  // tau rows: r = 0 - tau x
     }
     if (fuse_t) temperature_residual(P, F, s, m0, 1);
     __syncthreads();
-    if (warp < 2) {
-        const bool act = m0 > 0;
-        if constexpr (DDP) {
-            pair_block_solve<8, PP, ddc, ddc, dacc>(
-                reinterpret_cast<ddc*>(s.pf[0]) + 4, reinterpret_cast<ddc*>(s.pw[0]), reinterpret_cast<ddc*>(s.pd[0]) + 4,
-                F.psplit ? nA : np, reinterpret_cast<const ddc*>(F.pBlkDD) + (size_t)(act ? m0 : 0) * nbp * 192, act,
-                warp, 1);
-            if (!F.psplit && act) {  // the pair converts its solution back, then warp 0 takes the Schur step
-                const ddc* xd = reinterpret_cast<const ddc*>(s.pd[0]);
-                for (int n = 4 + (tid & 63); n < nc; n += 64) s.pd[0][n] = dd_compose(xd[n]);
-                pair_sync(1);
-                if (warp == 0) warp_schur<4>(s.pd[0], s.pf[0], nc, P.ops.tau_psi_B, F.pSinv + (size_t)m0 * 16);
-            }
-        } else {
-            pair_block_solve<8, PP>(s.pf[0] + 4, s.pw[0], s.pd[0] + 4, F.psplit ? nA : np,
-                                    F.pBlk + (size_t)(act ? m0 : 0) * nbp * 192, act, warp, 1);
-            if (!F.psplit && act && warp == 0)
-                warp_schur<4>(s.pd[0], s.pf[0], nc, P.ops.tau_psi_B, F.pSinv + (size_t)m0 * 16);
-        }
-    } else if (warp >= 6 && F.psplit) {
-        const bool act = m0 > 0;
-        if constexpr (DDP)
-            pair_block_solve<8, PP, ddc, ddc, dacc>(
-                reinterpret_cast<ddc*>(s.pf[0]) + 4 + nA, reinterpret_cast<ddc*>(s.pw[0]) + nA,
-                reinterpret_cast<ddc*>(s.pd[0]) + 4 + nA, np - nA,
-                reinterpret_cast<const ddc*>(F.pBlkDD) + ((size_t)(act ? m0 : 0) * nbp + nbp / 2) * 192, act, warp - 6, 4);
-        else
-            pair_block_solve<8, PP>(s.pf[0] + 4 + nA, s.pw[0] + nA, s.pd[0] + 4 + nA, np - nA,
-                                    F.pBlk + ((size_t)(act ? m0 : 0) * nbp + nbp / 2) * 192, act, warp - 6, 4);
-    } else if (fuse_t && warp < 4) {
-        pair_block_solve<8, PT>(s.tr + 2, s.tq, s.td + 2, nt, F.tBlk32 + (size_t)m0 * nbt * 192, true, warp - 2, 2);
+    if (warp == 2 && m0 > 0) {
+        const double t = rows_dot_sum(part_p, 8);
+        if (lane < 8) flat(s.pf)[lane] = -t;  // read by the Schur step below, past the next barrier
+    }
+    if (fuse_t)
+        run_chains<RD, 2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), job_t(), no_job<double, 1>(), s.prevs);
+    else if (m0 > 0)
+        run_chains<RD, 2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), no_job<CT, 2>(), no_job<double, 1>(),
+                          s.prevs);
+    if (fuse_t) {
         if (warp == 2) warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
-    }
-    __syncthreads();
-    if (DDP && F.psplit && m0 > 0) {  // the split solution back from double-floats before the join
-        const ddc* xd = reinterpret_cast<const ddc*>(s.pd[0]);
-        for (int n = 4 + tid; n < nc; n += nth) s.pd[0][n] = dd_compose(xd[n]);
         __syncthreads();
     }
-    if (F.psplit) {
-        split_join(s.pd[0] + 4, np, nA, F.pSpk + (size_t)(m0 > 0 ? m0 : 0) * np * 8,
-                   F.pRj + (size_t)(m0 > 0 ? m0 : 0) * 256, m0 > 0);
-        if (m0 > 0 && warp == 0) warp_schur<4>(s.pd[0], s.pf[0], nc, P.ops.tau_psi_B, F.pSinv + (size_t)m0 * 16);
+    if (m0 > 0) {
+        if (DDP) {  // the correction back from double-floats
+            if (F.psplit) split_join_dd(reinterpret_cast<ddc*>(s.pd) + 4, np, nA, spk_dd, rj_dd, true);
+            const ddf* xd = reinterpret_cast<const ddf*>(s.pd);
+            for (int q = 8 + tid; q < 2 * nc; q += nth) flat(s.pd)[q] = dd_compose(xd[q]);
+            __syncthreads();
+        }
+        if (!DDP && F.psplit) split_join(s.pd + 4, np, nA, F.pSpk + (size_t)m0 * np * 8, F.pRj + (size_t)m0 * 256, true);
+        rows_dot_part<4>(s.pd + 4, np, P.ops.tau_psi_B, part_p);
         __syncthreads();
+        if (warp == 0) schur_apply<4>(s.pd, s.pf, rows_dot_sum(part_p, 8), F.pSinv + (size_t)m0 * 16);
+        __syncthreads();
+        schur_update_parts<4>(s.pd, nc, F.pY + (size_t)m0 * np * 4);
     }
-    {
-        const int per = nth / MB;
-        const int sys = tid / per, t0 = sys * per;
-        const int m = m0 + sys;
-        if (sys < MB && m < M && m > 0) schur_update<4>(s.pd[sys], nc, F.pY + (size_t)m * np * 4, t0, per);
-        if (fuse_t) schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
-    }
+    if (fuse_t) schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
     __syncthreads();
-    for (int idx = tid; idx < MB * nc; idx += nth) {
-        const int mi = idx / nc, n = idx - mi * nc, m = m0 + mi;
-        if (m >= M) continue;
-        s.px[mi][n] = (m == 0) ? make_double2(0.0, 0.0) : cadd(s.px[mi][n], s.pd[mi][n]);
-        if (fuse_t) s.tx[0][n] = cadd(s.tx[0][n], to_d2_bits(s.td[n]));
-    }
+    for (int q = tid; q < 2 * nc; q += nth) flat(s.px)[q] = m0 ? flat(s.px)[q] + flat(s.pd)[q] : 0.0;
+    if (fuse_t)
+        for (int n = tid; n < nc; n += nth) s.tx[n] = cadd(s.tx[n], to_d2_bits(s.td[n]));
     __syncthreads();
-    }
-    if (!P.buoy_imp) temperature_corrections<MB, DEEP>(P, F, s, m0, has_u, fuse_t ? 1 : 0);
+    if (!P.buoy_imp) temperature_corrections(P, F, s, m0, has_u, fuse_t ? 1 : 0);
 
     // 6. store, then mass / implicit operators for later stages
-    for (int idx = tid; idx < MB * nc; idx += nth) {
-        const int mi = idx / nc, n = idx - mi * nc, m = m0 + mi;
-        if (m >= M) continue;
-        y_out.psi[(size_t)m * nc + n] = s.px[mi][n];
-        y_out.th[(size_t)m * nc + n] = s.tx[mi][n];
-        if (m == 0) y_out.u[n] = s.ux[n];
-        if (want_mass || want_imp)
-            epilogue_row(P, R, F.gdt, m, n, s.px[mi], s.tx[mi], s.ux, mass_out, imp_out, want_mass, want_imp,
-                         (MB == 1 && keep_f) ? s.fp : nullptr, s.tf[mi], s.fu);
+    for (int q = tid; q < 2 * nc; q += nth) {
+        reinterpret_cast<double*>(y_out.psi)[(size_t)m0 * 2 * nc + q] = flat(s.px)[q];
+        reinterpret_cast<double*>(y_out.th)[(size_t)m0 * 2 * nc + q] = flat(s.tx)[q];
+        if (has_u && part == 0) y_out.u[q >> 1] = s.ux[q >> 1];
     }
+    if (want_mass || want_imp)
+        for (int q = tid; q < 4 * nc; q += nth) {
+            if (q < 2 * nc)
+                epilogue_psi_part(P, R, F.gdt, m0, q >> 1, part, s.px, mass_out, imp_out, want_mass, want_imp,
+                                  keep_f ? s.fp : nullptr);
+            else
+                epilogue_theta_part(P, R, F.gdt, m0, (q - 2 * nc) >> 1, part, s.tx, s.ux, mass_out, imp_out, want_mass,
+                                    want_imp, s.tf, keep_f ? s.fu : nullptr);
+        }
 }
 
 // ---------------------------------------------------------------------------
-// The same solve split by system over two CTAs per mode (large N_c, FP32-refined
-// temperature, explicit buoyancy): role 0 the streamfunction system, role 1 the
-// temperature system (and, for m = 0, the zonal flow after it).  The systems are
-// independent when the buoyancy is explicit; each role holds only its own arrays
-// in shared memory (at N_c = 1365: 109 KB and 98 KB instead of 219 KB) and the
-// kernel is capped at 128 registers, so two CTAs share an SM and one's block
-// chains overlap the other's residual, Schur and epilogue phases.  Interleaved
-// roles (block 2m + role) give every SM a mix.  The same arithmetic as k_solve
-// with fuse_t = 0; chain prefetch depth 2.
+// The tau solve at small N_c (up to DENSE_NC) with the dense inverses of the whole
+// systems: x = G f, one refinement of the streamfunction from the FP64 residual of
+// the assembled band and the tau rows.  At this size a block chain is a handful of
+// steps, each a string of dependent FP64 instructions on one warp (35 us a solve at
+// N_c = 21, of which the chains, Schur sums and single-warp phases were 25); a
+// dense apply has 2 N_c independent sums, cut into up to 6 pieces each, on every
+// warp.  Column-major inverses (pInv [M][N_c][N_c] complex, tInv real, uInv): lanes of
+// consecutive rows read consecutive entries.
 // ---------------------------------------------------------------------------
-__device__ void epilogue_row_psi(const StepParams& P, const RhsSpec& R, double gdt, int m, int k, const double2* xp,
-                                 VecSet mass_out, VecSet imp_out, bool want_mass, bool want_imp,
-                                 const double2* fps) {
-    const int nc = P.nc;
-    const double mu = (double)m * m;
-    double2 mp = make_double2(0.0, 0.0);
-    if (m > 0 && k >= 4) {
-        // A^I_m = A0 + m^2 A2 assembled tap by tap: three FMAs a tap instead of four
-        const double* r0 = P.ops.band[OP_A0] + (size_t)k * 17;
-        const double* r2 = P.ops.band[OP_A2] + (size_t)k * 17;
-#pragma unroll
-        for (int d = 0; d < 17; ++d) {
-            const int n = k - 8 + d;
-            if (n >= 0 && n < nc) {
-                const double c = fma(mu, __ldg(&r2[d]), __ldg(&r0[d]));
-                mp.x = fma(c, xp[n].x, mp.x);
-                mp.y = fma(c, xp[n].y, mp.y);
-            }
+constexpr int DENSE_GROUPS = 6;
+__host__ __device__ inline int dense_groups(int nc) {
+    const int g = NTHREADS_S / (2 * nc);
+    return g < 1 ? 1 : g > DENSE_GROUPS ? DENSE_GROUPS : g;
+}
+__host__ __device__ inline size_t dense_smem_doubles(int nc) { return (size_t)nc * (12 + 4 * dense_groups(nc)); }
+
+__global__ void __launch_bounds__(NTHREADS_S) k_solve_dense(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
+                                                            VecSet mass_out, VecSet imp_out, int want_mass,
+                                                            int want_imp) {
+    extern __shared__ double2 sm[];
+    const int nc = P.nc, n2 = 2 * nc, np = nc - 4;
+    const int m = P.m_lo + blockIdx.x;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int ng = dense_groups(nc);
+    double* fp = reinterpret_cast<double*>(sm);  // assembled right-hand sides (f of the zonal flow in fp for m = 0)
+    double* ft = fp + n2;
+    double* xp = ft + n2;  // solutions (the zonal flow's in xp for m = 0)
+    double* xt = xp + n2;
+    double* rp = xt + n2;  // residual, then correction
+    double* xu = rp + n2;  // (m = 0) the zonal flow
+    double* fu = xu + nc;
+    double* red_p = fu + nc;  // [group][2 N_c] pieces of the sums
+    double* red_t = red_p + ng * n2;
+    const double dm = (double)m;
+
+    // right-hand sides sum_t c_t V_t (tau rows zero)
+    for (int t = tid; t < 2 * n2 + (m == 0 ? nc : 0); t += nth) {
+        double acc = 0.0;
+        if (t < n2) {
+            if (t >= 8 && m > 0)
+                for (int i = 0; i < R.nterms; ++i)
+                    acc = fma(R.t[i].c, reinterpret_cast<const double*>(R.t[i].v.psi)[(size_t)m * n2 + t], acc);
+            fp[t] = acc;
+        } else if (t < 2 * n2) {
+            const int q = t - n2;
+            if (q >= 4)
+                for (int i = 0; i < R.nterms; ++i)
+                    acc = fma(R.t[i].c, reinterpret_cast<const double*>(R.t[i].v.th)[(size_t)m * n2 + q], acc);
+            ft[q] = acc;
+        } else {
+            const int n = t - 2 * n2;
+            if (n >= 2)
+                for (int i = 0; i < R.nterms; ++i) acc = fma(R.t[i].c, R.t[i].v.u[n], acc);
+            fu[n] = acc;
         }
     }
-    const size_t idx = (size_t)m * nc + k;
-    if (want_imp) {  // before any store: an output may be one of the terms of f
-        const double2 fp = fps[k];
-        imp_out.psi[idx] = (m > 0 && k >= 4) ? cscale(csub(mp, fp), 1.0 / gdt) : make_double2(0.0, 0.0);
-    }
-    if (want_mass) mass_out.psi[idx] = mp;
-}
-
-__device__ void epilogue_row_theta(const StepParams& P, const RhsSpec& R, double gdt, int m, int k, const double2* xt,
-                                   const double* xu, VecSet mass_out, VecSet imp_out, bool want_mass, bool want_imp,
-                                   const double2* fts) {
-    const int nc = P.nc;
-    double2 mt = make_double2(0.0, 0.0);
-    double muu = 0.0;
-    if (k >= 2) {
-        mt = band_row_c<4>(P.ops.band[OP_D], xt, k, nc);
-        if (m == 0) {
-            const double* rd = P.ops.band[OP_D] + (size_t)k * 9;
-            for (int d = 0; d < 9; ++d) {
-                const int n = k - 4 + d;
-                if (n >= 0 && n < nc) muu = fma(__ldg(&rd[d]), xu[n], muu);
+    __syncthreads();
+    // pieces of G r: group g takes the columns n0 + g, n0 + g + ng, ...
+    auto pieces = [&](auto&& term, int n0, double* red) {
+        for (int t = tid; t < ng * n2; t += nth) {
+            const int g = t / n2, q = t - g * n2;
+            double acc = 0.0;
+            for (int n = n0 + g; n < nc; n += ng) acc = term(q, n, acc);
+            red[t] = acc;
+        }
+    };
+    auto joined = [&](const double* red, int q) {
+        double v = red[q];
+        for (int g = 1; g < ng; ++g) v += red[g * n2 + q];
+        return v;
+    };
+    const double2* gp = F.pInv + (size_t)m * nc * nc;
+    const double* gt = F.tInv + (size_t)m * nc * nc;
+    auto psi_term = [&](const double* r) {
+        return [=](int q, int n, double acc) {
+            const double2 a = __ldg(&gp[(size_t)n * nc + (q >> 1)]);
+            const double o = r[2 * n + 1 - (q & 1)];
+            return fma(a.x, r[2 * n + (q & 1)], fma(a.y, (q & 1) ? o : -o, acc));
+        };
+    };
+    auto theta_term = [&](int q, int n, double acc) { return fma(__ldg(&gt[(size_t)n * nc + (q >> 1)]), ft[2 * n + (q & 1)], acc); };
+    auto zonal_term = [&](int q, int n, double acc) { return q < nc ? fma(__ldg(&F.uInv[(size_t)n * nc + q]), fu[n], acc) : acc; };
+    // temperature (and zonal flow); with implicit buoyancy (Section 4) its
+    // g (Ra/Pr)(i m/s_o) C^I theta_new then joins the streamfunction rows
+    pieces(theta_term, 2, red_t);
+    if (m == 0)
+        pieces(zonal_term, 2, red_p);
+    else if (!P.buoy_imp)
+        pieces(psi_term(fp), 4, red_p);
+    __syncthreads();
+    for (int q = tid; q < 2 * n2; q += nth) {
+        if (q < n2) {
+            if (m == 0) {
+                xp[q] = 0.0;
+                if (q < nc) xu[q] = joined(red_p, q);
+            } else if (!P.buoy_imp) {
+                xp[q] = joined(red_p, q);
             }
+        } else {
+            xt[q - n2] = joined(red_t, q - n2);
         }
     }
-    const size_t idx = (size_t)m * nc + k;
-    if (want_imp) {  // before any store: an output may be one of the terms of f
-        const double2 ft = fts[k];
-        double fu = 0.0;
-        if (m == 0)
-            for (int t = 0; t < R.nterms; ++t) fu = fma(R.t[t].c, R.t[t].v.u[k], fu);
-        const double ig = 1.0 / gdt;
-        imp_out.th[idx] = (k >= 2) ? cscale(csub(mt, ft), ig) : make_double2(0.0, 0.0);
-        if (m == 0) imp_out.u[k] = (k >= 2) ? (muu - fu) * ig : 0.0;
+    __syncthreads();
+    if (m > 0) {
+        if (P.buoy_imp) {
+            const double cb = F.gdt * P.Ra / P.Pr * dm / P.s_o;
+            for (int q = 8 + tid; q < n2; q += nth) {
+                const double v = band_part<8>(P.ops.band[OP_C], xt + ((q & 1) ^ 1), q >> 1, nc);
+                fp[q] = fma((q & 1) ? cb : -cb, v, fp[q]);
+            }
+            __syncthreads();
+            pieces(psi_term(fp), 4, red_p);
+            __syncthreads();
+            for (int q = tid; q < n2; q += nth) xp[q] = joined(red_p, q);
+            __syncthreads();
+        }
+        // residual r = f - L x: the band's 17 taps in pieces; tau rows r = -tau x
+        const double2* band = F.pBand + (size_t)m * np * 17;
+        for (int t = tid; t < ng * n2; t += nth) {
+            const int g = t / n2, q = t - g * n2, k = q >> 1;
+            double acc = 0.0;
+            if (k < 4) {
+                for (int n = g; n < nc; n += ng) acc = fma(-__ldg(&P.ops.tau_psi[k * nc + n]), xp[2 * n + (q & 1)], acc);
+            } else {
+                if (g == 0) acc = fp[q];
+                for (int d = g; d < 17; d += ng) {
+                    const int n = k - 8 + d;
+                    if (n >= 0 && n < nc)
+                        acc = fms_part(acc, __ldg(&band[(size_t)(k - 4) * 17 + d]), make_double2(xp[2 * n], xp[2 * n + 1]), q & 1);
+                }
+            }
+            red_p[t] = acc;
+        }
+        __syncthreads();
+        for (int q = tid; q < n2; q += nth) rp[q] = joined(red_p, q);
+        __syncthreads();
+        pieces(psi_term(rp), 0, red_p);
+        __syncthreads();
+        for (int q = tid; q < n2; q += nth) xp[q] += joined(red_p, q);
+        __syncthreads();
     }
-    if (want_mass) {
-        mass_out.th[idx] = mt;
-        if (m == 0) mass_out.u[k] = muu;
+    // store, then mass / implicit terms for later stages (epilogue_psi_part, epilogue_theta_part)
+    for (int q = tid; q < n2; q += nth) {
+        reinterpret_cast<double*>(y_out.psi)[(size_t)m * n2 + q] = xp[q];
+        reinterpret_cast<double*>(y_out.th)[(size_t)m * n2 + q] = xt[q];
+        if (m == 0 && q < nc) y_out.u[q] = xu[q];
     }
+    if (want_mass || want_imp)
+        for (int q = tid; q < 2 * n2; q += nth) {
+            if (q < n2)
+                epilogue_psi_part(P, R, F.gdt, m, q >> 1, q & 1, reinterpret_cast<const double2*>(xp), mass_out, imp_out,
+                                  want_mass, want_imp, P.buoy_imp ? nullptr : reinterpret_cast<const double2*>(fp));
+            else
+                epilogue_theta_part(P, R, F.gdt, m, (q - n2) >> 1, q & 1, reinterpret_cast<const double2*>(xt), xu, mass_out,
+                                    imp_out, want_mass, want_imp, reinterpret_cast<const double2*>(ft), fu);
+        }
 }
 
-// Shared memory of the kernel with one CTA per system, bytes: the larger role.
-// Role 0 with double-float chains: pf, pw, px, fp (double2) and the rings of its
-// four walking warps (RD_DD matrices of complex double-floats each); with FP64
-// chains pf, pw, px, pd, fp.  Role 1: tf, tx (double2), tr, tq, td (float2), uf,
-// ux (double) and the rings of its (up to four) walking warps (RD_32 FP32 matrices).
-__host__ __device__ inline size_t solve_roles_smem_bytes(int nc, bool ddp) {
-    const size_t b = (size_t)round8(nc);
-    const size_t psi = ddp ? 4 * b * 16 + 4 * (size_t)RD_DD * 64 * 16 : 5 * b * 16;
-    const size_t th = 2 * b * 16 + 3 * b * 8 + 2 * b * 8 + 4 * (size_t)RD_32 * 64 * 4;
+// ---------------------------------------------------------------------------
+// The same solve split by system over two CTAs per mode (large N_c, explicit
+// buoyancy): role 0 the streamfunction system, role 1 the temperature system (and,
+// for m = 0, the zonal flow after it).  Interleaved roles (block 2m + role) give
+// every SM a mix.  The same arithmetic as k_solve with fuse_t = 0.
+//
+// A CTA alternates between block chains (two to four walking warps, latency) and
+// phases of the whole CTA (FP64 and the factors' HBM reads), so it takes several on
+// an SM to keep either busy: three, by holding two vectors a system.  Chains run in
+// place and the assembled right-hand side f waits in y_out, which the solution
+// replaces in the end: each element of y_out is written, read and written by this
+// CTA alone, first after the terms of f at that element have been read.  60 KB at
+// N_c = 1365 where five vectors a system took 109 KB (two CTAs).  Bound by FP64 (43%
+// of its rate) and the latency of the chains; solve 3231 -> 2970 us at n_r x n_phi =
+// 2049 x 6144, 1005 -> 879 us at 1025 x 3072.
+// ---------------------------------------------------------------------------
+__host__ __device__ inline size_t solve_roles_smem_bytes(int nc) {
+    const size_t b = (size_t)chain_rows(nc);
+    const size_t psi = 2 * b * 16 + 4 * (size_t)ring_bytes<ddc>(RD);          // work vector, solution
+    const size_t th = 5 * b * 8 + 4 * (size_t)ring_bytes<double>(RD);         // solution, FP32 work vector, uf, ux
     return psi > th ? psi : th;
 }
 
 template <bool DDP>
-__global__ void __launch_bounds__(NTHREADS_S, 2) k_solve_roles(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
+__global__ void __launch_bounds__(NTHREADS_S, 3) k_solve_roles(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                                 VecSet mass_out, VecSet imp_out, int want_mass,
                                                                 int want_imp) {
     extern __shared__ double2 sm[];
+    __shared__ double part_s[NTHREADS_S / 32][8];
+    __shared__ __align__(16) double prevs[NTHREADS_S / 32][32];
     const int nc = P.nc;
     const int m = P.m_lo + (int)(blockIdx.x >> 1), role = blockIdx.x & 1;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const int part = tid & 1;  // the component of this thread's tasks
     const int np = nc - 4, nt = nc - 2;
-    const int nbp = (np + 7) / 8;
-    const int nA = 8 * (nbp / 2);
-    const int b = round8(nc);
+    const int b = chain_rows(nc);
+    auto flat = [](double2* v) { return reinterpret_cast<double*>(v); };
     SolveSmem s{};
+    s.prevs = prevs;
     if (role == 0) {
         // ---------------------------------------------------- streamfunction
-        s.pf[0] = sm;
-        s.pw[0] = sm + b;
-        s.px[0] = sm + 2 * b;
-        s.pd[0] = DDP ? nullptr : sm + 3 * b;  // double-float chains: the correction in place of the residual
-        s.fp = DDP ? sm + 3 * b : sm + 4 * b;
-        ddc* ring = reinterpret_cast<ddc*>(sm + 4 * b);  // double-float chains only
         if (m == 0) {  // Psi_0 = 0
             for (int n = tid; n < nc; n += nth) {
                 y_out.psi[n] = make_double2(0.0, 0.0);
@@ -1682,137 +1786,102 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve_roles(StepParams P, Rhs
             }
             return;
         }
-        // two rows per thread and pass: twice the loads in flight
-        for (int n0 = tid; n0 < nc; n0 += 2 * nth) {
-            const int n1 = n0 + nth;
-            double2 a0 = make_double2(0.0, 0.0), a1 = a0;
+        const int nbp = (np + 7) / 8, nA = 8 * (nbp / 2);
+        using C = std::conditional_t<DDP, ddc, double2>;
+        using V = typename Chain<C>::V;
+        double2 *work = sm, *x = sm + b, *f = y_out.psi + (size_t)m * nc;
+        char* ring = reinterpret_cast<char*>(sm + 2 * b);
+        const C* blk = (DDP ? reinterpret_cast<const C*>(F.pBlkDD) : reinterpret_cast<const C*>(F.pBlk)) + (size_t)m * nbp * 192;
+        const ddc* spk_dd = reinterpret_cast<const ddc*>(F.pSpkDD) + (size_t)m * np * 8;
+        for (int q = tid; q < 2 * nc; q += nth) {
+            double acc = 0.0;
 #pragma unroll 4
-            for (int t = 0; t < R.nterms; ++t) {
-                const double c = R.t[t].c;
-                const double2 v0 = R.t[t].v.psi[(size_t)m * nc + n0];
-                const double2 v1 = (n1 < nc) ? R.t[t].v.psi[(size_t)m * nc + n1] : make_double2(0.0, 0.0);
-                a0.x = fma(c, v0.x, a0.x);
-                a0.y = fma(c, v0.y, a0.y);
-                a1.x = fma(c, v1.x, a1.x);
-                a1.y = fma(c, v1.y, a1.y);
-            }
-            s.pf[0][n0] = (n0 < 4) ? make_double2(0.0, 0.0) : a0;
-            s.fp[n0] = s.pf[0][n0];
-            if (n1 < nc) {
-                s.pf[0][n1] = (n1 < 4) ? make_double2(0.0, 0.0) : a1;
-                s.fp[n1] = s.pf[0][n1];
-            }
+            for (int t = 0; t < R.nterms; ++t)
+                acc = fma(R.t[t].c, reinterpret_cast<const double*>(R.t[t].v.psi)[(size_t)m * 2 * nc + q], acc);
+            if (q < 8) acc = 0.0;
+            flat(f)[q] = acc;
+            if constexpr (DDP)
+                reinterpret_cast<ddf*>(work)[q] = dd_from_bits(acc);
+            else
+                flat(work)[q] = acc;
         }
         __syncthreads();
-        const double2* blk = F.pBlk + (size_t)m * nbp * 192;
-        const ddc* blkd = reinterpret_cast<const ddc*>(F.pBlkDD) + (size_t)m * nbp * 192;
-        ddc* zd = reinterpret_cast<ddc*>(s.pw[0]);
+        // the block in place, one or (psplit) two halves by warps 0-1 and 6-7
+        auto job = [&](bool second) {
+            const int n0 = second ? nA : 0, n = second ? (F.psplit ? np - nA : 0) : F.psplit ? nA : np;
+            V* v = reinterpret_cast<V*>(work + 4 + n0);
+            return ChainJob<C, 2>{v, v, v, n, blk + (second ? (size_t)(nbp / 2) * 192 : 0), second ? 6 : 0,
+                                  ring + (second ? 2 * ring_bytes<C>(RD) : 0)};
+        };
         for (int it = 0; it < 2; ++it) {  // solve, then one refinement step
-            // double-float chains: pass 0 solves into px, pass 1 (the correction)
-            // into pf, over its own right-hand side (the residual): the walks read
-            // a block's right-hand side before they write its solution
-            double2* x = it ? (DDP ? s.pf[0] : s.pd[0]) : s.px[0];
+            double2* sol = it ? work : x;
+            run_chains<RD, 2>(job(false), job(true), no_job<float, 2>(), no_job<double, 1>(), prevs);
             if constexpr (DDP) {
-                // The conversions between FP64 and double-float run on the FP64
-                // pipe, so they happen here for the whole vector at once, off the
-                // chains' dependent path: the right-hand side in place (f stays in
-                // fp for the residual and the epilogue), the solution back from
-                // double-floats in place.
-                ddc* bd = reinterpret_cast<ddc*>(s.pf[0]);
-                ddc* xd = reinterpret_cast<ddc*>(x);
-                for (int n = 4 + tid; n < nc; n += nth) bd[n] = dd_from(s.pf[0][n]);
-                __syncthreads();
-                cta_chain_solve<RD_DD, ddc, ddc, dacc>(bd + 4, zd, xd + 4, F.psplit ? nA : np, blkd, 0, bd + 4 + nA, zd + nA,
-                                                       xd + 4 + nA, F.psplit ? np - nA : 0,
-                                                       blkd + (size_t)(nbp / 2) * 192, 6, ring);
                 if (F.psplit)
-                    split_join_dd(xd + 4, np, nA, reinterpret_cast<const ddc*>(F.pSpkDD) + (size_t)m * np * 8,
+                    split_join_dd(reinterpret_cast<ddc*>(work) + 4, np, nA, spk_dd,
                                   reinterpret_cast<const ddc*>(F.pRjDD) + (size_t)m * 256, true);
-                for (int n = 4 + tid; n < nc; n += nth) x[n] = dd_compose(xd[n]);
+                for (int q = 8 + tid; q < 2 * nc; q += nth) flat(sol)[q] = dd_compose(reinterpret_cast<const ddf*>(work)[q]);
             } else {
-                if (warp < 2)
-                    pair_block_solve<8, PFB>(s.pf[0] + 4, s.pw[0], x + 4, F.psplit ? nA : np, blk, true, warp, 1);
-                else if (warp >= 6 && F.psplit)
-                    pair_block_solve<8, PFB>(s.pf[0] + 4 + nA, s.pw[0] + nA, x + 4 + nA, np - nA,
-                                             blk + (size_t)(nbp / 2) * 192, true, warp - 6, 4);
+                if (F.psplit) split_join(work + 4, np, nA, F.pSpk + (size_t)m * np * 8, F.pRj + (size_t)m * 256, true);
+                if (!it)
+                    for (int q = 8 + tid; q < 2 * nc; q += nth) flat(x)[q] = flat(work)[q];
             }
             __syncthreads();
-            if (!DDP && F.psplit)
-                split_join(x + 4, np, nA, F.pSpk + (size_t)m * np * 8, F.pRj + (size_t)m * 256, true);
-            block_schur<4>(x, it ? s.pf[0] : nullptr, nc, P.ops.tau_psi_B, F.pSinv + (size_t)m * 16);
-            schur_update<4>(x, nc, F.pY + (size_t)m * np * 4, 0, nth);
+            rows_dot_part<4>(sol + 4, np, P.ops.tau_psi_B, part_s);
             __syncthreads();
-            if (it == 0) {
-                // residual r = f - L x over the assembled rows, and the tau rows
-                // (whose f is zero)
-                for (int k = 4 + tid; k < nc; k += nth) {
-                    const double2* row = F.pBand + ((size_t)m * np + (k - 4)) * 17;
-                    double2 acc = s.fp[k];
-#pragma unroll
-                    for (int d = 0; d < 17; ++d) {
-                        const int n = k - 8 + d;
-                        if (n >= 0 && n < nc) acc = fms(acc, __ldg(&row[d]), s.px[0][n]);
-                    }
-                    s.pf[0][k] = acc;
+            if (warp == 0) schur_apply<4>(sol, it ? work : nullptr, rows_dot_sum(part_s, 8), F.pSinv + (size_t)m * 16);
+            __syncthreads();
+            schur_update_parts<4>(sol, nc, F.pY + (size_t)m * np * 4);
+            __syncthreads();
+            if (it == 0) {  // residual r = f - L x over the assembled rows, and the tau rows (f = 0)
+                for (int q = 8 + tid; q < 2 * nc; q += nth) {
+                    const int k = q >> 1;
+                    const double acc = residual_part(flat(f)[q], F.pBand + ((size_t)m * np + (k - 4)) * 17, x, k, nc, part);
+                    if constexpr (DDP)
+                        reinterpret_cast<ddf*>(work)[q] = dd_from_bits(acc);
+                    else
+                        flat(work)[q] = acc;
                 }
-                const double2 t = block_rows_dot<4>(s.px[0], nc, P.ops.tau_psi);
-                if (warp == 0 && lane < 4) s.pf[0][lane] = make_double2(-t.x, -t.y);
+                rows_dot_part<4>(x, nc, P.ops.tau_psi, part_s);
                 __syncthreads();
+                if (warp == 2) {
+                    const double t = rows_dot_sum(part_s, 8);
+                    if (lane < 8) flat(work)[lane] = -t;  // read by the Schur step, past the chains' barriers
+                }
             }
         }
-        {
-            const double2* d = DDP ? s.pf[0] : s.pd[0];
-            for (int n = tid; n < nc; n += nth) s.px[0][n] = cadd(s.px[0][n], d[n]);
-        }
+        for (int q = tid; q < 2 * nc; q += nth) flat(x)[q] += flat(work)[q];
         __syncthreads();
-        for (int n = tid; n < nc; n += nth) {
-            y_out.psi[(size_t)m * nc + n] = s.px[0][n];
+        for (int q = tid; q < 2 * nc; q += nth) {
             if (want_mass || want_imp)
-                epilogue_row_psi(P, R, F.gdt, m, n, s.px[0], mass_out, imp_out, want_mass, want_imp, s.fp);
+                epilogue_psi_part(P, R, F.gdt, m, q >> 1, part, x, mass_out, imp_out, want_mass, want_imp, f);
+            flat(f)[q] = flat(x)[q];
         }
         return;
     }
     // ------------------------------------------- temperature (and zonal flow)
-    // FP32-refined (ir_t): tf, tx, then the FP32 tr, tq, td; otherwise FP64 blocks
-    // with tw as chain scratch in the place of tr
-    s.tf[0] = sm;
-    s.tx[0] = sm + b;
-    float2* f32 = reinterpret_cast<float2*>(sm + 2 * b);
-    s.tr = f32;
-    s.tq = f32 + b;
-    s.td = f32 + 2 * b;
-    s.tw[0] = reinterpret_cast<double2*>(f32);  // FP64 path: b double2 over tr and tq
-    double* d64 = reinterpret_cast<double*>(f32 + 3 * b);
-    s.uf = d64;
-    s.ux = d64 + b;
-    s.ring32 = reinterpret_cast<float*>(d64 + 2 * b);
+    s.tx = sm;
+    s.tr = s.td = reinterpret_cast<float2*>(sm + b);  // FP32 residual, then (in place) correction
+    s.uf = reinterpret_cast<double*>(s.tr + b);
+    s.ux = s.uf + b;
+    s.ring_t = s.ring_u = reinterpret_cast<char*>(s.ux + b);
+    s.tf = y_out.th + (size_t)m * nc;
     const int nbt = (nt + 7) / 8;
-    for (int n0 = tid; n0 < nc; n0 += 2 * nth) {  // two rows per thread and pass
-        const int n1 = n0 + nth;
-        double2 a0 = make_double2(0.0, 0.0), a1 = a0;
-        double u0 = 0.0, u1 = 0.0;
+    for (int q = tid; q < 2 * nc; q += nth) {
+        const int n = q >> 1;
+        double acc = 0.0, au = 0.0;
 #pragma unroll 4
         for (int t = 0; t < R.nterms; ++t) {
-            const double c = R.t[t].c;
-            const double2 v0 = R.t[t].v.th[(size_t)m * nc + n0];
-            const double2 v1 = (n1 < nc) ? R.t[t].v.th[(size_t)m * nc + n1] : make_double2(0.0, 0.0);
-            a0.x = fma(c, v0.x, a0.x);
-            a0.y = fma(c, v0.y, a0.y);
-            a1.x = fma(c, v1.x, a1.x);
-            a1.y = fma(c, v1.y, a1.y);
-            if (m == 0) {
-                u0 = fma(c, R.t[t].v.u[n0], u0);
-                if (n1 < nc) u1 = fma(c, R.t[t].v.u[n1], u1);
-            }
+            acc = fma(R.t[t].c, reinterpret_cast<const double*>(R.t[t].v.th)[(size_t)m * 2 * nc + q], acc);
+            if (m == 0) au = fma(R.t[t].c, R.t[t].v.u[n], au);
         }
-        s.tf[0][n0] = (n0 < 2) ? make_double2(0.0, 0.0) : a0;
-        if (F.ir_t) s.tr[n0] = to_f2(s.tf[0][n0]);
-        if (m == 0) s.uf[n0] = (n0 < 2) ? 0.0 : u0;
-        if (n1 < nc) {
-            s.tf[0][n1] = (n1 < 2) ? make_double2(0.0, 0.0) : a1;
-            if (F.ir_t) s.tr[n1] = to_f2(s.tf[0][n1]);
-            if (m == 0) s.uf[n1] = (n1 < 2) ? 0.0 : u1;
-        }
+        if (n < 2) acc = au = 0.0;
+        flat(s.tf)[q] = acc;
+        if (F.ir_t)
+            reinterpret_cast<float*>(s.tr)[q] = f32_from_bits(acc);
+        else
+            flat(s.tx)[q] = acc;
+        if (m == 0 && part == 0) s.uf[n] = au;
     }
     __syncthreads();
     if (F.ir_t) {
@@ -1820,28 +1889,26 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve_roles(StepParams P, Rhs
         block_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m * 4);
         schur_update32_dir(s.td, nc, F.tY32 + (size_t)m * nt * 2, 0, nth);
         __syncthreads();
-        for (int n = tid; n < nc; n += nth) s.tx[0][n] = to_d2_bits(s.td[n]);
+        for (int n = tid; n < nc; n += nth) s.tx[n] = to_d2_bits(s.td[n]);
         __syncthreads();
         temperature_corrections_roles(P, F, s, m);
     } else {
-        if (warp == 2 || warp == 3)
-            pair_block_solve<8, PFB>(s.tf[0] + 2, s.tw[0], s.tx[0] + 2, nt, F.tBlk + (size_t)m * nbt * 192, true,
-                                     warp - 2, 2);
+        double* v = flat(s.tx + 2);
+        run_chains<RD, 2>(no_job<double, 1>(), no_job<double, 1>(),
+                          ChainJob<double, 2>{v, v, v, nt, F.tBlk + (size_t)m * nbt * 192, 2, s.ring_t}, no_job<double, 1>(),
+                          prevs);
+        rows_dot_part<2>(s.tx + 2, nt, P.ops.tau_dir_B, part_s);
         __syncthreads();
-        block_schur<2>(s.tx[0], nullptr, nc, P.ops.tau_dir_B, F.tSinv + (size_t)m * 4);
-        schur_update<2>(s.tx[0], nc, F.tY + (size_t)m * nt * 2, 0, nth);
+        if (warp == 0) schur_apply<2>(s.tx, nullptr, rows_dot_sum(part_s, 4), F.tSinv + (size_t)m * 4);
+        __syncthreads();
+        schur_update_parts<2>(s.tx, nc, F.tY + (size_t)m * nt * 2);
         __syncthreads();
     }
     if (m == 0) {
-        // the zonal flow after the temperature, in its freed FP32 arrays (the
-        // same footprint in doubles): chain scratch in tq, correction in td, the
-        // refinement's chain scratch in tr
-        s.pd[0] = reinterpret_cast<double2*>(s.tq);
-        s.pw[0] = reinterpret_cast<double2*>(s.td);
-        s.pf[0] = reinterpret_cast<double2*>(s.tr);
-        if (warp == 4 || warp == 5)
-            pair_block_solve<8, PFB>(s.uf + 2, reinterpret_cast<double*>(s.pd[0]), s.ux + 2, nt, F.uBlk, true, warp - 4, 3);
-        __syncthreads();
+        // the zonal flow after the temperature, whose FP32 array takes the
+        // refinement's correction
+        s.pd = reinterpret_cast<double2*>(s.td);
+        zonal_chains(F, s, s.uf + 2, s.ux + 2, nt);
         if (warp == 4) {
             double t0 = 0.0, t1 = 0.0;
             for (int j = lane; j < nt; j += 32) {
@@ -1864,11 +1931,12 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve_roles(StepParams P, Rhs
         __syncthreads();
         if (F.ir_t) refine_zonal_flow(P, F, s);
     }
-    for (int n = tid; n < nc; n += nth) {
-        y_out.th[(size_t)m * nc + n] = s.tx[0][n];
-        if (m == 0) y_out.u[n] = s.ux[n];
+    for (int q = tid; q < 2 * nc; q += nth) {
+        const int n = q >> 1;
         if (want_mass || want_imp)
-            epilogue_row_theta(P, R, F.gdt, m, n, s.tx[0], s.ux, mass_out, imp_out, want_mass, want_imp, s.tf[0]);
+            epilogue_theta_part(P, R, F.gdt, m, n, part, s.tx, s.ux, mass_out, imp_out, want_mass, want_imp, s.tf, nullptr);
+        flat(s.tf)[q] = flat(s.tx)[q];
+        if (m == 0 && part == 0) y_out.u[n] = s.ux[n];
     }
 }
 
@@ -1893,7 +1961,6 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve_roles(StepParams P, Rhs
 // staged through shared memory in chunks of GCH rows by asynchronous copies, the
 // next chunk in flight while the current one is used.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double mul(double a, double b) { return a * b; }
 __device__ __forceinline__ double shfl_down_x(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ double2 shfl_down_x(double2 v) {
     return make_double2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
@@ -1983,10 +2050,13 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve_galerkin(StepParams P, Rhs
     const int nc = P.nc, m = P.m_lo + blockIdx.x;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
     const int np = nc - 4, nt = nc - 2;
-    SolveSmem s = carve<1>(sm, nc);
     const bool has_u = (m == 0);
-    double2 *pf = s.pf[0], *tf = s.tf[0], *px = s.px[0], *tx = s.tx[0], *xp = s.pw[0], *xt = s.tw[0];
-    double* xu = reinterpret_cast<double*>(s.pd[0]);
+    const int b = round8(nc);
+    double2 *pf = sm, *xp = sm + b, *px = sm + 2 * b, *tf = sm + 4 * b, *xt = sm + 5 * b, *tx = sm + 6 * b;
+    double* xu = reinterpret_cast<double*>(sm + 3 * b);
+    SolveSmem s{};
+    s.uf = reinterpret_cast<double*>(sm + 7 * b);
+    s.ux = s.uf + b;
     // after the FP64 solve arrays (over the FP32 refinement arrays of the tau
     // path, unused here): factor staging (2 GCH rows per system) and pivots
     double2* stp = sm + 8 * round8(nc);
@@ -2130,10 +2200,6 @@ __global__ void k_check_finite(VecSet y, size_t n2, int nu, int* __restrict__ fl
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
 }
 
-size_t smem_solve_mb(const StepParams& P, int MB, bool deep = false) {
-    return sizeof(double) * solve_smem_doubles(P.nc, MB, deep);
-}
-
 }  // namespace
 
 
@@ -2150,15 +2216,24 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
                                                       want_imp ? 1 : 0);
         return cudaGetLastError();
     }
+    // small systems (N_c <= DENSE_NC): the dense inverses, 35 -> 16 us at N_c = 21.
+    // Their operations and bytes grow as N_c^2: at N_c = 85 (n_r = 129) the applies
+    // alone are 2300 FP64 instructions a warp and mode, 19 us of an SM's FP64 units for
+    // each mode on it, where the chains take 39 us for two.  The options that pick a
+    // form of the chains keep them.
+    if (F.pInv && P.psi_dd < 0 && P.solve_roles <= 0 && !F.ir_t) {
+        k_solve_dense<<<slab_modes(P), NTHREADS_S, sizeof(double) * dense_smem_doubles(P.nc), st>>>(
+            P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
+        return cudaGetLastError();
+    }
     // the systems with FP32-refined temperature solves (N_c > 600): with explicit
-    // buoyancy one CTA per system (two per mode, two per SM), else the deep chain
-    // prefetch (one CTA per SM by shared memory)
+    // buoyancy one CTA per system (two per mode, three per SM)
     const bool large = P.nc > 600;
     if (!P.buoy_imp && (P.solve_roles > 0 || (P.solve_roles < 0 && large))) {
         // double-float streamfunction chains: option psi_chain_dd, by default
         // from N_c > 600 (where the roles kernel is the default)
         const bool ddp = F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && large));
-        const size_t smr = solve_roles_smem_bytes(P.nc, ddp);
+        const size_t smr = solve_roles_smem_bytes(P.nc);
         auto kern = ddp ? k_solve_roles<true> : k_solve_roles<false>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
         // two CTAs per SM need the largest shared-memory carveout
@@ -2170,14 +2245,13 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
                                                          want_imp ? 1 : 0);
         return cudaGetLastError();
     }
-    // one CTA per mode: the deep chain prefetch for the large systems (one CTA per
-    // SM); below N_c = 600 double-float streamfunction chains (option
-    // psi_chain_dd, by default from N_c > 64 with explicit buoyancy: n_r = 129,
-    // 257, 513 solve 47.6 -> 45.4, 87.8 -> 74.2, 335.5 -> 279.3 us; at n_r = 33
-    // the conversions cost more than the chains save, 34.5 -> 36.5 us)
+    // one CTA per mode; below N_c = 600 double-float streamfunction chains (option
+    // psi_chain_dd, by default from N_c > 64 with explicit buoyancy: with FP64 ones
+    // n_r = 129, 257, 513 took 47.6, 87.8, 335.5 us where these took 45.4, 74.2, 279.3;
+    // below, the conversions cost more than the chains save)
     const bool ddp = !large && !P.buoy_imp && F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && P.nc > 64));
-    auto kern = large ? k_solve<1, true> : (ddp ? k_solve<1, false, true> : k_solve<1, false>);
-    const size_t sm = smem_solve_mb(P, 1, large);
+    auto kern = F.ir_t ? (ddp ? k_solve<true, true> : k_solve<true, false>) : (ddp ? k_solve<false, true> : k_solve<false, false>);
+    const size_t sm = sizeof(double) * solve_smem_doubles(P.nc);
     // the epilogue reads the assembled right-hand sides from shared memory where
     // they fit (up to N_c ~ 1300), else sums the terms again
     int dev = 0, smax = 0;

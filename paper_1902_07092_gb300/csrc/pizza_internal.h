@@ -11,6 +11,8 @@ namespace pz {
 
 constexpr int MAX_PASSES = 16;
 constexpr int MAX_RHS_TERMS = 10;
+// largest N_c whose tau systems are solved by dense inverses (k_solve_dense)
+constexpr int DENSE_NC = 42;
 
 // Mixed-radix (3 * 2^j) Stockham plan for one transform length.
 struct FftPlan {
@@ -81,6 +83,10 @@ struct DevFactors {
     // interface inverse, as for the streamfunction
     int tsplit;
     float *tBlk32S, *tSpk32, *tRj32;
+    // dense inverses of the whole tau systems for small N_c (<= DENSE_NC), else null:
+    // column-major pInv [M][N_c][N_c] complex, tInv [M][N_c][N_c] and uInv [N_c][N_c] real
+    double2* pInv;
+    double *tInv, *uInv;
     // Galerkin bases (option "radial" = 2, Appendix B): banded LU with partial
     // pivoting of the square integrated systems (host_ops.h, band_lu_pivot).
     // Streamfunction, complex, 8 diagonals below / 12 above: gpL [M][n_p][8],
