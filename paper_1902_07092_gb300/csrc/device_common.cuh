@@ -654,4 +654,34 @@ __device__ __forceinline__ void cheb_derivative_adjoint_scan2(T* e0, T* t0, T* e
     __syncthreads();
 }
 
+// Chained launches.  A kernel launched by launch_chained may start once every CTA of
+// its predecessor in the stream has exited, without waiting for the launch that a
+// complete dependency costs; it begins with chain_wait(), which returns when the
+// predecessor has completed (after its own predecessors) and its writes are visible.
+// Nothing that another kernel writes may reach such a kernel through __ldg or a const
+// __restrict__ parameter: those loads may be moved above the wait.  A step of
+// n_r x n_phi = 33 x 96, 129 x 384, 257 x 768 (four kernels): 53.2 -> 42.8, 86.0 -> 75.8,
+// 156.1 -> 147.8 us.  (With griddepcontrol.launch_dependents at the start the waiting
+// CTAs crowd on the SMs that are free first: 129 x 384 99.9 us.)
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... K, class... A>
+inline cudaError_t launch_chained(void (*kern)(K...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    // in a stream capture plain launches: the graph's edges stay complete dependencies
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    cudaError_t err = cudaStreamIsCapturing(st, &cap);
+    cfg.attrs = at;
+    cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    if (err == cudaSuccess) err = cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+    const cudaError_t last = cudaGetLastError();
+    return err != cudaSuccess ? err : last;
+}
+
 }  // namespace pz

@@ -99,6 +99,7 @@ __device__ void cos_sums(const double2* src, double2* dst, int nb, double2* bufA
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NTA) k_adj_grid_to_spec(StepParams P, VecSet w, VecSet y, VecSet lam,
                                                           double2* __restrict__ Gb2, double* __restrict__ ra) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(NTA) k_adj_grid_to_spec(StepParams P, VecSet w
 // f_bar_j e^{-i m phi_j} (m >= 1).  smem: two work buffers and the two packed
 // forward fields (4 n_phi complex).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void load_hermitian_pair(double2* Z, const double2* __restrict__ src, int M, int Pn,
+__device__ __forceinline__ void load_hermitian_pair(double2* Z, const double2* src, int M, int Pn,
                                                     int n_m, double s0, double s1) {
     // z = a + i b from one-sided spectra a = src[0..M), b = src[M..2M): a_0, b_0
     // real parts scaled by s0; m >= 1 scaled by s1 with the conjugate images
@@ -241,9 +242,10 @@ __device__ __forceinline__ void store_split_adjoint(const double2* Y, double2* _
     }
 }
 
-__global__ void __launch_bounds__(NTA, 1) k_adj_phi(StepParams P, const double2* __restrict__ G1,
-                                                    const double2* __restrict__ Gb2, double2* __restrict__ Gb1,
+__global__ void __launch_bounds__(NTA, 1) k_adj_phi(StepParams P, const double2* G1,
+                                                    const double2* Gb2, double2* __restrict__ Gb1,
                                                     int pair) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int k = blockIdx.x;
     const int Pn = P.n_phi, M = P.M, n_m = P.n_m;
@@ -348,8 +350,9 @@ __global__ void __launch_bounds__(NTA, 1) k_adj_phi(StepParams P, const double2*
 //   theta_bar_n += C w_n [Syn^T t_bar]_n
 // m = 0 (real parts): u_bar_n += C w_n [Syn^T (u_bar + w_bar/s) + Dc^T Syn^T w_bar]_n.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NTA) k_adj_spec_to_grid(StepParams P, const double2* __restrict__ Gb1,
+__global__ void __launch_bounds__(NTA) k_adj_spec_to_grid(StepParams P, const double2* Gb1,
                                                           VecSet lam) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
@@ -419,6 +422,7 @@ __global__ void __launch_bounds__(NTA) k_adj_spec_to_grid(StepParams P, const do
 constexpr int ASR = 32, ASS = 8;
 
 __global__ void __launch_bounds__(ASR * ASS) k_adj_solve(StepParams P, AdjFactors A, VecSet lam, VecSet rho) {
+    chain_wait();
     extern __shared__ double2 sm[];  // the input vector, nc entries
     __shared__ double2 part[ASS][ASR];
     const int m = blockIdx.x, nc = P.nc, np = nc - 4, nt = nc - 2;
@@ -494,6 +498,7 @@ __global__ void __launch_bounds__(ASR * ASS) k_adj_solve(StepParams P, AdjFactor
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NTA) k_adj_apply(StepParams P, VecSet g, VecSet rho, VecSet rho_next, VecSet lam,
                                                    VecSet w, double dt, double c, double c2) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x, nc = P.nc;
     double2* rp = sm;
@@ -546,6 +551,7 @@ __global__ void __launch_bounds__(NTA) k_adj_apply(StepParams P, VecSet g, VecSe
 
 // a += b over the three fields (b's null fields are skipped)
 __global__ void k_vec_add(int M, int nc, VecSet a, VecSet b) {
+    chain_wait();
     const size_t n = (size_t)M * nc;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         if (b.psi) a.psi[i] = cadd(a.psi[i], b.psi[i]);
@@ -554,7 +560,8 @@ __global__ void k_vec_add(int M, int nc, VecSet a, VecSet b) {
     }
 }
 
-__global__ void k_ra_accumulate(const double* __restrict__ ra, int M, double* __restrict__ acc) {
+__global__ void k_ra_accumulate(const double* ra, int M, double* __restrict__ acc) {
+    chain_wait();
     double t = 0.0;
     for (int m = threadIdx.x; m < M; m += 32) t += ra[m];
 #pragma unroll
@@ -565,13 +572,11 @@ __global__ void k_ra_accumulate(const double* __restrict__ ra, int M, double* __
 }  // namespace
 
 cudaError_t launch_ra_accumulate(const double* ra, int M, double* acc, cudaStream_t st) {
-    k_ra_accumulate<<<1, 32, 0, st>>>(ra, M, acc);
-    return cudaGetLastError();
+    return launch_chained(k_ra_accumulate, 1, 32, 0, st, ra, M, acc);
 }
 
 cudaError_t launch_vec_add(const StepParams& P, VecSet a, VecSet b, cudaStream_t st) {
-    k_vec_add<<<P.M, NTA, 0, st>>>(P.M, P.nc, a, b);
-    return cudaGetLastError();
+    return launch_chained(k_vec_add, P.M, NTA, 0, st, P.M, P.nc, a, b);
 }
 
 size_t smem_adj_grid_to_spec(const StepParams& P) {
@@ -589,8 +594,7 @@ cudaError_t launch_adj_explicit(const StepParams& P, VecSet w, VecSet y, VecSet 
     size_t sm = smem_adj_grid_to_spec(P);
     cudaError_t err = cudaFuncSetAttribute(k_adj_grid_to_spec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_adj_grid_to_spec<<<P.M, NTA, sm, st>>>(P, w, y, lam, Gb2, ra);
-    err = cudaGetLastError();
+    err = launch_chained(k_adj_grid_to_spec, P.M, NTA, sm, st, P, w, y, lam, Gb2, ra);
     if (err != cudaSuccess) return err;
     // the batched pairs need 6 n_phi entries (n_phi <= 2048), else 4 n_phi
     int dev = 0, smax = 0;
@@ -601,29 +605,25 @@ cudaError_t launch_adj_explicit(const StepParams& P, VecSet w, VecSet y, VecSet 
     sm = sizeof(double2) * (pair ? 6 : 4) * P.n_phi;
     err = cudaFuncSetAttribute(k_adj_phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_adj_phi<<<P.n_r, NTA, sm, st>>>(P, G1, Gb2, Gb1, pair);
-    err = cudaGetLastError();
+    err = launch_chained(k_adj_phi, P.n_r, NTA, sm, st, P, G1, Gb2, Gb1, pair);
     if (err != cudaSuccess) return err;
     sm = smem_adj_spec_to_grid(P);
     err = cudaFuncSetAttribute(k_adj_spec_to_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_adj_spec_to_grid<<<P.M, NTA, sm, st>>>(P, Gb1, lam);
-    return cudaGetLastError();
+    return launch_chained(k_adj_spec_to_grid, P.M, NTA, sm, st, P, Gb1, lam);
 }
 
 cudaError_t launch_adj_solve(const StepParams& P, const AdjFactors& A, VecSet lam, VecSet rho, cudaStream_t st) {
     const size_t sm = sizeof(double2) * P.nc;
     const int tp = (P.nc - 4 + ASR - 1) / ASR, tt = (P.nc - 2 + ASR - 1) / ASR;
     dim3 grid(P.M, tp + 2 * tt);
-    k_adj_solve<<<grid, ASR * ASS, sm, st>>>(P, A, lam, rho);
-    return cudaGetLastError();
+    return launch_chained(k_adj_solve, grid, ASR * ASS, sm, st, P, A, lam, rho);
 }
 
 cudaError_t launch_adj_apply(const StepParams& P, VecSet g, VecSet rho, VecSet rho_next, VecSet lam, VecSet w,
                              double dt, double c, double c2, cudaStream_t st) {
     const size_t sm = sizeof(double2) * 2 * P.nc + sizeof(double) * P.nc;
-    k_adj_apply<<<P.M, NTA, sm, st>>>(P, g, rho, rho_next, lam, w, dt, c, c2);
-    return cudaGetLastError();
+    return launch_chained(k_adj_apply, P.M, NTA, sm, st, P, g, rho, rho_next, lam, w, dt, c, c2);
 }
 
 }  // namespace pz

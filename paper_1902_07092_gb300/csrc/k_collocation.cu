@@ -51,6 +51,7 @@ __device__ __forceinline__ void load_plain_for_synthesis(double2* z, const doubl
 // the DCT-I, the derivative recurrence, Eq. cheb.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_coll_spec_to_grid(StepParams P, VecSet y, double2* __restrict__ G1) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, M = P.M;
@@ -101,8 +102,9 @@ __global__ void __launch_bounds__(NT) k_coll_spec_to_grid(StepParams P, VecSet y
 // (Eqs. psiomcoll, tempcoll, uphicoll; dT_c/ds = tc/s with tc = alpha/ln eta; the
 // conduction term is -u_s dT_c/ds as in Eq. temp.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) k_coll_grid_rows(StepParams P, const double2* __restrict__ G1,
-                                                       const double2* __restrict__ G2, VecSet e) {
+__global__ void __launch_bounds__(NT) k_coll_grid_rows(StepParams P, const double2* G1,
+                                                       const double2* G2, VecSet e) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, M = P.M;
@@ -190,6 +192,7 @@ __global__ void __launch_bounds__(NT) k_coll_grid_rows(StepParams P, const doubl
 // phase 0: all rows at once (explicit buoyancy).
 __global__ void __launch_bounds__(NT) k_coll_solve(StepParams P, RhsSpec R, DevFactors F, VecSet yo, VecSet mo,
                                                    VecSet io, int want_mass, int want_imp, int phase) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x;
     const int N = P.n_r, ni = N - 2;
@@ -299,6 +302,7 @@ __global__ void __launch_bounds__(NT) k_coll_solve(StepParams P, RhsSpec R, DevF
 // and the u rows -U u  (U = Upsilon, c5 = 5 s_o beta/(2 h s)).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_coll_apply(StepParams P, VecSet y, VecSet io) {
+    chain_wait();
     const int m = blockIdx.x, N = P.n_r;
     const double mu = (double)m * m;
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
@@ -362,6 +366,7 @@ __global__ void __launch_bounds__(NT) k_coll_apply(StepParams P, VecSet y, VecSe
 // s_o, where psi = dpsi/ds = 0.  In: hat.psi, hat.th [M][n_r], hat.u [n_r].
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_coll_from_hat(StepParams P, VecSet hat, VecSet y) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = blockIdx.x, N = P.n_r;
     double2* pg = sm;  // psi grid values
@@ -416,6 +421,7 @@ __global__ void __launch_bounds__(NT) k_coll_from_hat(StepParams P, VecSet hat, 
 // matrix T is an involution, f_hat_n = sum_k T_nk f_k):
 // out.psi, out.th, out.w [M][n_r], out.u [n_r]
 __global__ void __launch_bounds__(NT) k_coll_to_hat(StepParams P, VecSet y, VecSet out) {
+    chain_wait();
     const int m = blockIdx.x, N = P.n_r;
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
         const double* t = P.cTm + (size_t)n * N;
@@ -454,8 +460,7 @@ cudaError_t launch_coll_spec_to_grid(const StepParams& P, VecSet y, double2* G1,
     const size_t sm = smem_coll_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_coll_spec_to_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_coll_spec_to_grid<<<P.M, NT, sm, st>>>(P, y, G1);
-    return cudaGetLastError();
+    return launch_chained(k_coll_spec_to_grid, P.M, NT, sm, st, P, y, G1);
 }
 
 cudaError_t launch_coll_grid_rows(const StepParams& P, const double2* G1, const double2* G2, VecSet e,
@@ -463,8 +468,7 @@ cudaError_t launch_coll_grid_rows(const StepParams& P, const double2* G1, const 
     const size_t sm = smem_coll_grid_rows(P);
     cudaError_t err = cudaFuncSetAttribute(k_coll_grid_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_coll_grid_rows<<<P.M, NT, sm, st>>>(P, G1, G2, e);
-    return cudaGetLastError();
+    return launch_chained(k_coll_grid_rows, P.M, NT, sm, st, P, G1, G2, e);
 }
 
 cudaError_t launch_coll_solve(const StepParams& P, const RhsSpec& R, const DevFactors& F, VecSet y_out,
@@ -472,28 +476,24 @@ cudaError_t launch_coll_solve(const StepParams& P, const RhsSpec& R, const DevFa
     const size_t sm = sizeof(double2) * 3 * (P.n_r - 2);
     dim3 grid(P.M, (3 * P.n_r + NT - 1) / NT);
     for (int phase = P.buoy_imp ? 1 : 0; phase <= (P.buoy_imp ? 2 : 0); ++phase) {
-        k_coll_solve<<<grid, NT, sm, st>>>(P, R, F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0,
-                                           phase);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_chained(k_coll_solve, grid, NT, sm, st, P, R, F, y_out, mass_out, imp_out,
+                                             want_mass ? 1 : 0, want_imp ? 1 : 0, phase);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 cudaError_t launch_coll_apply(const StepParams& P, VecSet y, VecSet imp_out, cudaStream_t st) {
-    k_coll_apply<<<P.M, NT, 0, st>>>(P, y, imp_out);
-    return cudaGetLastError();
+    return launch_chained(k_coll_apply, P.M, NT, 0, st, P, y, imp_out);
 }
 
 cudaError_t launch_coll_from_hat(const StepParams& P, VecSet hat, VecSet y, cudaStream_t st) {
     const size_t sm = sizeof(double2) * P.n_r;
-    k_coll_from_hat<<<P.M, NT, sm, st>>>(P, hat, y);
-    return cudaGetLastError();
+    return launch_chained(k_coll_from_hat, P.M, NT, sm, st, P, hat, y);
 }
 
 cudaError_t launch_coll_to_hat(const StepParams& P, VecSet y, VecSet out, cudaStream_t st) {
-    k_coll_to_hat<<<P.M, NT, 0, st>>>(P, y, out);
-    return cudaGetLastError();
+    return launch_chained(k_coll_to_hat, P.M, NT, 0, st, P, y, out);
 }
 
 }  // namespace pz

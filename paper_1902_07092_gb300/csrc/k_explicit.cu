@@ -41,10 +41,11 @@ inline int phi_threads(const StepParams& P) {
 }
 
 // of the fixed-point one: a divisor of the n_phi/2 radix-4 butterflies of a pass over
-// both pairs (96 2^j of them), at most 384 (two CTAs share an SM's registers)
+// both pairs (96 2^j of them), at most 384 (two CTAs share an SM's registers); 512 where
+// shared memory leaves one CTA an SM (1025 x 3072: 336 -> 327 us)
 inline int phi_threads_fx(const StepParams& P) {
     if (P.phi_threads > 0 || P.n_phi > 256 * MAXPER) return phi_threads(P);
-    return P.n_phi >= 768 ? 384 : 192;
+    return P.n_phi >= 3072 ? 512 : P.n_phi >= 768 ? 384 : 192;
 }
 
 // ---------------------------------------------------------------------------
@@ -67,6 +68,7 @@ inline int phi_threads_fx(const StepParams& P) {
 // ---------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSet y, T* __restrict__ G1, T* __restrict__ W) {
+    chain_wait();
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(NTHREADS_R) k_spec_to_grid(StepParams P, VecSe
 //   g1 * Re(g2) = v omega + i u_phi omega,  g1 * Im(g2) = v theta + i u_phi theta.
 // ---------------------------------------------------------------------------
 template <class T>
-__device__ __forceinline__ void load_packed_spectrum(T* Z, const T* __restrict__ src, int M, int Pn, int n_m,
+__device__ __forceinline__ void load_packed_spectrum(T* Z, const T* src, int M, int Pn, int n_m,
                                                      typename Cx<T>::R sa, typename Cx<T>::R sb) {
     // src points at G1/G2 row (k, f): field a = src[0..M), field b = src[M..2M);
     // packed as sa a + i sb b
@@ -319,8 +321,9 @@ __device__ void cfl_rates(const StepParams& P, const T* R, int Pn, double l1, in
 }
 
 template <class T>
-__global__ void __launch_bounds__(512, 1) k_phi_products(StepParams P, const T* __restrict__ G1,
+__global__ void __launch_bounds__(512, 1) k_phi_products(StepParams P, const T* G1,
                                                          T* __restrict__ G2, int pair) {
+    chain_wait();
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
@@ -422,8 +425,9 @@ __device__ __forceinline__ double2 band_row(const double* __restrict__ band, con
 }
 
 template <class T>
-__global__ void __launch_bounds__(NTHREADS_R) k_grid_to_spec(StepParams P, const T* __restrict__ G2, VecSet y,
+__global__ void __launch_bounds__(NTHREADS_R) k_grid_to_spec(StepParams P, const T* G2, VecSet y,
                                                              VecSet e) {
+    chain_wait();
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
@@ -698,6 +702,7 @@ __device__ __forceinline__ void cheb_derivative_part(const double2* c, double2* 
 // at 513 x 384 (against the double-float lean layout it replaces at that size).
 __global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P, VecSet y, double2* __restrict__ G1,
                                                                    double2* __restrict__ W) {
+    chain_wait();
     __shared__ FxScale sc;
     const int m = P.m_lo + blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
@@ -829,8 +834,9 @@ __device__ __forceinline__ double band_part(const double* __restrict__ band, con
 // (from the double-float lean layout).
 // Vectors 0, 1: F1, F2 (to coefficients); 2, 3: their derivatives (to the grid);
 // 4, 5: N_omega (N_u), N_theta (to coefficients).
-__global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P, const double2* __restrict__ G2,
+__global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P, const double2* G2,
                                                                     VecSet y, VecSet e) {
+    chain_wait();
     __shared__ FxScale sc;
     const int m = P.m_lo + blockIdx.x;
     const int K = P.K, L = 2 * K, N = P.n_r, nc = P.nc, M = P.M;
@@ -1087,8 +1093,9 @@ __device__ void cfl_rates_fx(const StepParams& P, const fxc* R, int k, int sv, i
 // points each); else one after the other, the first pair's physical values
 // and the second products waiting in registers.
 template <bool PAIR>
-__global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParams P, const double2* __restrict__ G1,
+__global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParams P, const double2* G1,
                                                             double2* __restrict__ G2) {
+    chain_wait();
     __shared__ PhiScale sc;
     const int k = P.k_lo + blockIdx.x;
     const int Pn = P.n_phi, M = P.M, n_m = P.n_m;
@@ -1632,6 +1639,7 @@ constexpr int lean_ctas() { return sizeof(T) == sizeof(double2) ? 2 : 3; }
 template <class T>
 __global__ void __launch_bounds__(NTHREADS_R, lean_ctas<T>()) k_spec_to_grid_lean(StepParams P, VecSet y,
                                                                                   T* __restrict__ G1) {
+    chain_wait();
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int m = P.m_lo + blockIdx.x;
@@ -1727,8 +1735,9 @@ __host__ __device__ inline size_t lean_cd_offset(int n_r) {
 }
 
 template <class T>
-__global__ void __launch_bounds__(NTHREADS_R, lean_ctas<T>()) k_grid_to_spec_lean(StepParams P, const T* __restrict__ G2,
+__global__ void __launch_bounds__(NTHREADS_R, lean_ctas<T>()) k_grid_to_spec_lean(StepParams P, const T* G2,
                                                                                   VecSet y, VecSet e) {
+    chain_wait();
     using RT = typename Cx<T>::R;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int m = P.m_lo + blockIdx.x;
@@ -2020,6 +2029,7 @@ __device__ __forceinline__ void cheb_derivative_cta(const double2* c, double2* d
 __global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepParams P, VecSet y,
                                                                          double2* __restrict__ G1,
                                                                          double2* __restrict__ W) {
+    chain_wait();
     __shared__ FxScale sc;
     __shared__ DctHalf dh;
     const int m = P.m_lo + blockIdx.x;
@@ -2110,8 +2120,9 @@ __global__ void __launch_bounds__(NTHREADS_LX, 2) k_spec_to_grid_lean_fx(StepPar
     }
 }
 
-__global__ void __launch_bounds__(NTHREADS_LX, 2) k_grid_to_spec_lean_fx(StepParams P, const double2* __restrict__ G2,
+__global__ void __launch_bounds__(NTHREADS_LX, 2) k_grid_to_spec_lean_fx(StepParams P, const double2* G2,
                                                                          VecSet y, VecSet e) {
+    chain_wait();
     __shared__ FxScale sc;
     __shared__ DctHalf dh;
     const int m = P.m_lo + blockIdx.x;
@@ -2226,8 +2237,8 @@ static cudaError_t spec_to_grid_t(const StepParams& P, VecSet y, void* G1, void*
     const size_t sm = smem_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_spec_to_grid<T><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, static_cast<T*>(G1), static_cast<T*>(W));
-    return cudaGetLastError();
+    return launch_chained(k_spec_to_grid<T>, slab_modes(P), NTHREADS_R, sm, st, P, y, static_cast<T*>(G1),
+                          static_cast<T*>(W));
 }
 
 // 1 when the azimuthal kernels can hold both packed pairs at once (twice
@@ -2249,8 +2260,8 @@ static cudaError_t phi_products_t(const StepParams& P, const void* G1, void* G2,
     const size_t sm = (pair ? 2 : 1) * smem_phi_products(P);
     err = cudaFuncSetAttribute(k_phi_products<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_phi_products<T><<<slab_radii(P), nth, sm, st>>>(P, static_cast<const T*>(G1), static_cast<T*>(G2), pair);
-    return cudaGetLastError();
+    return launch_chained(k_phi_products<T>, slab_radii(P), nth, sm, st, P, static_cast<const T*>(G1),
+                          static_cast<T*>(G2), pair);
 }
 
 template <class T>
@@ -2258,8 +2269,7 @@ static cudaError_t grid_to_spec_t(const StepParams& P, const void* G2, VecSet y,
     const size_t sm = smem_grid_to_spec(P);
     cudaError_t err = cudaFuncSetAttribute(k_grid_to_spec<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_grid_to_spec<T><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, static_cast<const T*>(G2), y, e);
-    return cudaGetLastError();
+    return launch_chained(k_grid_to_spec<T>, slab_modes(P), NTHREADS_R, sm, st, P, static_cast<const T*>(G2), y, e);
 }
 
 cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, double2* W, cudaStream_t st) {
@@ -2268,8 +2278,8 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, doub
         cudaError_t err =
             cudaFuncSetAttribute(k_spec_to_grid_lean<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        k_spec_to_grid_lean<float2><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, reinterpret_cast<float2*>(G1));
-        return cudaGetLastError();
+        return launch_chained(k_spec_to_grid_lean<float2>, slab_modes(P), NTHREADS_R, sm, st, P, y,
+                              reinterpret_cast<float2*>(G1));
     }
     if (lean_radial(P)) {
         const size_t sm = smem_radial_lean(P);
@@ -2278,18 +2288,14 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, doub
                              : cudaFuncSetAttribute(k_spec_to_grid_lean<double2>,
                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        if (fx)
-            k_spec_to_grid_lean_fx<<<slab_modes(P), NTHREADS_LX, sm, st>>>(P, y, G1, W);
-        else
-            k_spec_to_grid_lean<double2><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, y, G1);
-        return cudaGetLastError();
+        if (fx) return launch_chained(k_spec_to_grid_lean_fx, slab_modes(P), NTHREADS_LX, sm, st, P, y, G1, W);
+        return launch_chained(k_spec_to_grid_lean<double2>, slab_modes(P), NTHREADS_R, sm, st, P, y, G1);
     }
     if (P.fp32) return spec_to_grid_t<float2>(P, y, G1, W, st);
     const size_t sm = smem_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_spec_to_grid_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, y, G1, W);
-    return cudaGetLastError();
+    return launch_chained(k_spec_to_grid_fx, slab_modes(P), fx_threads(P), sm, st, P, y, G1, W);
 }
 
 cudaError_t launch_phi_products(const StepParams& P, const double2* G1, double2* G2, cudaStream_t st) {
@@ -2305,8 +2311,7 @@ cudaError_t launch_phi_products(const StepParams& P, const double2* G1, double2*
         auto kern = pair ? k_phi_products_fx<true> : k_phi_products_fx<false>;
         err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        kern<<<slab_radii(P), nth, sm, st>>>(P, G1, G2);
-        return cudaGetLastError();
+        return launch_chained(kern, slab_radii(P), nth, sm, st, P, G1, G2);
     }
     return phi_products_t<double2>(P, G1, G2, st);
 }
@@ -2317,8 +2322,8 @@ cudaError_t launch_grid_to_spec(const StepParams& P, const double2* G2, VecSet y
         cudaError_t err =
             cudaFuncSetAttribute(k_grid_to_spec_lean<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        k_grid_to_spec_lean<float2><<<slab_modes(P), NTHREADS_R, sm, st>>>(P, reinterpret_cast<const float2*>(G2), y, e);
-        return cudaGetLastError();
+        return launch_chained(k_grid_to_spec_lean<float2>, slab_modes(P), NTHREADS_R, sm, st, P,
+                              reinterpret_cast<const float2*>(G2), y, e);
     }
     if (lean_radial(P)) {
         const size_t sm = smem_radial_lean(P);
@@ -2326,15 +2331,13 @@ cudaError_t launch_grid_to_spec(const StepParams& P, const double2* G2, VecSet y
         auto kern = fx ? k_grid_to_spec_lean_fx : k_grid_to_spec_lean<double2>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
-        kern<<<slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st>>>(P, G2, y, e);
-        return cudaGetLastError();
+        return launch_chained(kern, slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st, P, G2, y, e);
     }
     if (P.fp32) return grid_to_spec_t<float2>(P, G2, y, e, st);
     const size_t sm = smem_grid_to_spec(P);
     cudaError_t err = cudaFuncSetAttribute(k_grid_to_spec_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_grid_to_spec_fx<<<slab_modes(P), fx_threads(P), sm, st>>>(P, G2, y, e);
-    return cudaGetLastError();
+    return launch_chained(k_grid_to_spec_fx, slab_modes(P), fx_threads(P), sm, st, P, G2, y, e);
 }
 
 }  // namespace pz

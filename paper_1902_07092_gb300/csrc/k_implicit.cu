@@ -1345,6 +1345,7 @@ template <bool T32, bool DDP>
 __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                       VecSet mass_out, VecSet imp_out, int want_mass,
                                                       int want_imp, int keep_f) {
+    chain_wait();
     extern __shared__ double2 sm[];
     __shared__ double part_p[NTHREADS_S / 32][8], part_t[NTHREADS_S / 32][8];
     const int nc = P.nc;
@@ -1598,6 +1599,7 @@ __host__ __device__ inline size_t dense_smem_doubles(int nc) { return (size_t)nc
 __global__ void __launch_bounds__(NTHREADS_S) k_solve_dense(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                             VecSet mass_out, VecSet imp_out, int want_mass,
                                                             int want_imp) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int nc = P.nc, n2 = 2 * nc, np = nc - 4;
     const int m = P.m_lo + blockIdx.x;
@@ -1764,6 +1766,7 @@ template <bool DDP>
 __global__ void __launch_bounds__(NTHREADS_S, 3) k_solve_roles(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                                 VecSet mass_out, VecSet imp_out, int want_mass,
                                                                 int want_imp) {
+    chain_wait();
     extern __shared__ double2 sm[];
     __shared__ double part_s[NTHREADS_S / 32][8];
     __shared__ __align__(16) double prevs[NTHREADS_S / 32][32];
@@ -2046,6 +2049,7 @@ __device__ void warp_band_solve(TX* b, TX* x, int n, const TF* __restrict__ Lm, 
 __global__ void __launch_bounds__(NTHREADS_S) k_solve_galerkin(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                                VecSet mass_out, VecSet imp_out, int want_mass,
                                                                int want_imp) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int nc = P.nc, m = P.m_lo + blockIdx.x;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
@@ -2169,6 +2173,7 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve_galerkin(StepParams P, Rhs
 
 __global__ void __launch_bounds__(NTHREADS_S) k_apply(StepParams P, VecSet y, VecSet mass_out, VecSet imp_out,
                                                       int want_mass, int want_imp) {
+    chain_wait();
     extern __shared__ double2 sm[];
     const int m = P.m_lo + blockIdx.x;
     const int nc = P.nc;
@@ -2187,6 +2192,7 @@ __global__ void __launch_bounds__(NTHREADS_S) k_apply(StepParams P, VecSet y, Ve
 // Sets *flag when any entry of the state (Psi, theta, u_bar and, for
 // collocation, omega) is NaN or infinite.
 __global__ void k_check_finite(VecSet y, size_t n2, int nu, int* __restrict__ flag) {
+    chain_wait();
     bool bad = false;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
         const double2 a = y.psi[i], b = y.th[i];
@@ -2212,9 +2218,8 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
                            sizeof(double) * 2 * 2 * GCH * 12 + 3 * round8(P.nc);
         cudaError_t err = cudaFuncSetAttribute(k_solve_galerkin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smg);
         if (err != cudaSuccess) return err;
-        k_solve_galerkin<<<slab_modes(P), NTHREADS_S, smg, st>>>(P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0,
-                                                      want_imp ? 1 : 0);
-        return cudaGetLastError();
+        return launch_chained(k_solve_galerkin, slab_modes(P), NTHREADS_S, smg, st, P, rhs, F, y_out, mass_out, imp_out,
+                              want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
     // small systems (N_c <= DENSE_NC): the dense inverses, 35 -> 16 us at N_c = 21.
     // Their operations and bytes grow as N_c^2: at N_c = 85 (n_r = 129) the applies
@@ -2222,9 +2227,8 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
     // each mode on it, where the chains take 39 us for two.  The options that pick a
     // form of the chains keep them.
     if (F.pInv && P.psi_dd < 0 && P.solve_roles <= 0 && !F.ir_t) {
-        k_solve_dense<<<slab_modes(P), NTHREADS_S, sizeof(double) * dense_smem_doubles(P.nc), st>>>(
-            P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
-        return cudaGetLastError();
+        return launch_chained(k_solve_dense, slab_modes(P), NTHREADS_S, sizeof(double) * dense_smem_doubles(P.nc), st, P, rhs,
+                              F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
     // the systems with FP32-refined temperature solves (N_c > 600): with explicit
     // buoyancy one CTA per system (two per mode, three per SM)
@@ -2236,14 +2240,13 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
         const size_t smr = solve_roles_smem_bytes(P.nc);
         auto kern = ddp ? k_solve_roles<true> : k_solve_roles<false>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
-        // two CTAs per SM need the largest shared-memory carveout
+        // three CTAs per SM need the largest shared-memory carveout
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        (int)cudaSharedmemCarveoutMaxShared);
         if (err != cudaSuccess) return err;
-        kern<<<2 * slab_modes(P), NTHREADS_S, smr, st>>>(P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0,
-                                                         want_imp ? 1 : 0);
-        return cudaGetLastError();
+        return launch_chained(kern, 2 * slab_modes(P), NTHREADS_S, smr, st, P, rhs, F, y_out, mass_out, imp_out,
+                              want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
     // one CTA per mode; below N_c = 600 double-float streamfunction chains (option
     // psi_chain_dd, by default from N_c > 64 with explicit buoyancy: with FP64 ones
@@ -2265,15 +2268,15 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
     const int keep = smk + fa.sharedSizeBytes <= (size_t)smax ? 1 : 0;
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(keep ? smk : sm));
     if (err != cudaSuccess) return err;
-    kern<<<slab_modes(P), NTHREADS_S, keep ? smk : sm, st>>>(P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0,
-                                                   want_imp ? 1 : 0, keep);
-    return cudaGetLastError();
+    return launch_chained(kern, slab_modes(P), NTHREADS_S, keep ? smk : sm, st, P, rhs, F, y_out, mass_out, imp_out,
+                          want_mass ? 1 : 0, want_imp ? 1 : 0, keep);
 }
 
 // acc[0] += sum_n w_n Re theta_hat_0n = Nu - 1 of the state (one warp, a fixed
 // summation order: the lane sums, then a butterfly of shuffles)
-__global__ void k_nusselt_accumulate(const double2* __restrict__ th0, const double* __restrict__ w, int nc,
+__global__ void k_nusselt_accumulate(const double2* th0, const double* __restrict__ w, int nc,
                                      double* acc) {
+    chain_wait();
     double t = 0.0;
     for (int n = threadIdx.x; n < nc; n += 32) t = fma(w[n], th0[n].x, t);
 #pragma unroll
@@ -2283,13 +2286,11 @@ __global__ void k_nusselt_accumulate(const double2* __restrict__ th0, const doub
 
 cudaError_t launch_nusselt_accumulate(const StepParams& P, VecSet y, const double* w, double* acc,
                                       cudaStream_t st) {
-    k_nusselt_accumulate<<<1, 32, 0, st>>>(y.th, w, P.nc, acc);
-    return cudaGetLastError();
+    return launch_chained(k_nusselt_accumulate, 1, 32, 0, st, y.th, w, P.nc, acc);
 }
 
 cudaError_t launch_check_finite(const StepParams& P, VecSet y, int* flag, cudaStream_t st) {
-    k_check_finite<<<152, 256, 0, st>>>(y, (size_t)P.M * P.nc, P.nc, flag);
-    return cudaGetLastError();
+    return launch_chained(k_check_finite, 152, 256, 0, st, y, (size_t)P.M * P.nc, P.nc, flag);
 }
 
 cudaError_t launch_apply(const StepParams& P, VecSet y, VecSet mass_out, VecSet imp_out, bool want_mass,
@@ -2297,8 +2298,7 @@ cudaError_t launch_apply(const StepParams& P, VecSet y, VecSet mass_out, VecSet 
     const size_t sm = sizeof(double2) * 2 * P.nc + sizeof(double) * P.nc;
     cudaError_t err = cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    k_apply<<<slab_modes(P), NTHREADS_S, sm, st>>>(P, y, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chained(k_apply, slab_modes(P), NTHREADS_S, sm, st, P, y, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
 }
 
 }  // namespace pz
