@@ -1742,8 +1742,12 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve_dense(StepParams P, RhsSpe
 // ---------------------------------------------------------------------------
 // The same solve split by system over two CTAs per mode (large N_c, explicit
 // buoyancy): role 0 the streamfunction system, role 1 the temperature system (and,
-// for m = 0, the zonal flow after it).  Interleaved roles (block 2m + role) give
-// every SM a mix.  The same arithmetic as k_solve with fuse_t = 0.
+// for m = 0, the zonal flow after it).  The streamfunctions' CTAs come first: they
+// take twice as long, so the short ones fill the end of the launch.  (Interleaved,
+// block 2m + role, the 152 SMs got only one role each per pass over them: 875 and 2949
+// us against 780 and 2786 at 1025 x 3072 and 2049 x 6144; interleaved with the roles
+// exchanged from pass to pass 858 and 2906.)  The same arithmetic as k_solve with
+// fuse_t = 0.
 //
 // A CTA alternates between block chains (two to four walking warps, latency) and
 // phases of the whole CTA (FP64 and the factors' HBM reads), so it takes several on
@@ -1752,8 +1756,8 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve_dense(StepParams P, RhsSpe
 // replaces in the end: each element of y_out is written, read and written by this
 // CTA alone, first after the terms of f at that element have been read.  60 KB at
 // N_c = 1365 where five vectors a system took 109 KB (two CTAs).  Bound by FP64 (43%
-// of its rate) and the latency of the chains; solve 3231 -> 2970 us at n_r x n_phi =
-// 2049 x 6144, 1005 -> 879 us at 1025 x 3072.
+// of its rate) and the latency of the chains; with two CTAs an SM 3231 and 1005 us at
+// n_r x n_phi = 2049 x 6144 and 1025 x 3072, with three 2949 and 875.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t solve_roles_smem_bytes(int nc) {
     const size_t b = (size_t)chain_rows(nc);
@@ -1771,7 +1775,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 3) k_solve_roles(StepParams P, Rhs
     __shared__ double part_s[NTHREADS_S / 32][8];
     __shared__ __align__(16) double prevs[NTHREADS_S / 32][32];
     const int nc = P.nc;
-    const int m = P.m_lo + (int)(blockIdx.x >> 1), role = blockIdx.x & 1;
+    const int nm = gridDim.x >> 1, role = (int)blockIdx.x >= nm, m = P.m_lo + (int)blockIdx.x - role * nm;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
     const int part = tid & 1;  // the component of this thread's tasks
     const int np = nc - 4, nt = nc - 2;
