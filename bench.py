@@ -106,11 +106,6 @@ def algorithmic_flops(n_r, n_phi, scheme, radial="integration"):
 # DRAM bytes (read + write) per launch of the roofline kernel from one ncu capture
 # of this workload (summaries under profiles/); null for kernels not captured.
 NCU_TRAFFIC = {
-    ("sparse_n257_p768", "solve"): (44.36e6 + 0.03e6, "profiles/imex_step_kernels_n257_p768.md"),
-    ("large_n2049_p6144", "solve"): (5672.7e6 + 171.6e6, "profiles/imex_step_kernels_n2049_p6144.md"),
-    ("large_n2049_p6144", "spec_to_grid"): (106.3e6 + 226.2e6, "profiles/imex_step_kernels_n2049_p6144.md"),
-    ("large_n2049_p6144", "phi_products"): (269.1e6 + 216.3e6, "profiles/imex_step_kernels_n2049_p6144.md"),
-    ("large_n2049_p6144", "grid_to_spec"): (360.1e6 + 71.0e6, "profiles/imex_step_kernels_n2049_p6144.md"),
     ("coll_n257_p768", "solve"): (735.4e6 + 6.9e6, "profiles/collocation_step_kernels_n257_p768.md"),
     ("galerkin_n257_p768", "solve"): (34.58e6 + 0.003e6, "profiles/galerkin_step_kernels_n257_p768.md"),
 }
@@ -282,17 +277,14 @@ def config_of(args, wl, Ra):
 
 
 def precision_label(wl):
-    """What the FP64 path computes in which arithmetic (double-float: pairs of
-    FP32 words, ~48-bit significands, on the FP32 pipe)."""
-    big = wl["n_r"] >= 513 and wl.get("radial", "integration") == "integration"
+    """What the FP64 path computes in which arithmetic (fixed point: 64-bit integers
+    with 60 significant bits; double-float: pairs of FP32 words, ~48-bit significands)."""
     nc = inputs.n_c_of(wl)
-    parts = ["fp64: state, history, stored grid values, linear couplings, banded applies, "
-             "Schur steps, residuals and refinements in FP64" + ("" if big else "; field arithmetic at each "
-                                                                 "radius in FP64"),
-             "azimuthal FFTs and products in double-float with the m = 0 means of the products in FP64"]
-    if big:
-        parts.append("radial DCT-I, derivative scans and field arithmetic at each radius in double-float "
-                     "(lean layout, n_r >= 513)")
+    parts = ["fp64: state, history, stored grid values, field arithmetic at each radius, linear couplings, banded "
+             "applies, Schur steps, residuals and refinements in FP64",
+             "azimuthal FFTs and products in fixed point with the m = 0 means of the products in FP64"]
+    if wl.get("radial", "integration") == "integration":
+        parts.append("radial DCT-I in fixed point")
     if wl.get("radial", "integration") == "integration" and nc > 64:
         parts.append("block chains of the streamfunction solve in double-float (N_c > 64)")
     if nc > 600:
@@ -517,7 +509,7 @@ def kernel_table(kt, kn, flops, nbytes, hbm_peak):
         us = 1e3 * float(kt[i]) / max(int(kn[i]), 1)
         out[k] = {"launches": int(kn[i]), "avg_us": us, "share": share[k], "gflop_per_launch": flops[k] / 1e9,
                   # FP64-grade algorithmic flops per second, whichever pipe ran them
-                  # (the double-float transforms and chains run on the FP32 pipe)
+                  # (the transforms run on the integer pipes, double-float chains on the FP32 pipe)
                   "tflops_algorithmic": flops[k] / (us * 1e-6) / 1e12 if us > 0 else None,
                   "mb_per_launch": nbytes[k] / 1e6,
                   "hbm_frac": nbytes[k] / (us * 1e-6) / 1e9 / hbm_peak if us > 0 else None}

@@ -123,10 +123,11 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *            its buoyancy into the streamfunction (vorticity) system.  The adjoint
  *            refuses it.  Set before stepping;
  *   "azimuthal_dd" 1 (default) = the azimuthal transforms and grid products of
- *            the FP64 explicit stage in double-float arithmetic (pairs of floats,
- *            ~48-bit significands, on the FP32 pipe), their m = 0 modes in FP64;
- *            0 = in FP64.  Both meet the FP64 parity bars of the explicit terms.
- *            The adjoint's azimuthal stage is FP64 either way;
+ *            the FP64 explicit stage in fixed point (64-bit integers with 60
+ *            significant bits under each vector's maximum, on the integer pipes),
+ *            the m = 0 modes of the products in FP64; 0 = in FP64.  Both meet the
+ *            FP64 parity bars of the explicit terms.  The adjoint's azimuthal stage
+ *            is FP64 either way;
  *   "check_finite" 1 = after every step a small kernel scans the state for NaN
  *            or infinite values and sets a device flag; pizza_synchronize then
  *            returns PIZZA_ENONFINITE (cleared by pizza_set_state).  0 (default) =
@@ -143,33 +144,33 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *   "radial_lean" the FP64 synthesis and analysis kernels in the layout of
  *            three shared arrays of n_r values, the fields one after another (two
  *            CTAs per SM at n_r = 2049) instead of the batched layout: 1 from
- *            n_r = 129, 0 never, -1 (default) from n_r = 513.  Results agree to
+ *            n_r = 129, 0 never, -1 (default) from n_r = 1025.  Results agree to
  *            rounding (the DCT-I sums in another order).  In mixed precision
  *            ("precision" = 1) the FP32 kernels take this layout only with 1
  *            (three CTAs per SM; faster at n_r = 2049, but the half-length DCT-I
  *            accumulates the FP32 rounding of its outputs: about 20x the
  *            batched layout's distance from FP64, still within the mixed bar);
- *   "radial_dd" the DCT-I, the Chebyshev derivative scans and the field
- *            arithmetic at each radius of the lean radial kernels in
- *            double-float arithmetic on the FP32 pipe (about 48 significant bits;
- *            stored values, banded applies and couplings in FP64): 1 always
- *            (with the lean layout), 0 never, -1
- *            (default) with the lean layout's default, from n_r = 513.  Results
- *            agree with the FP64 transforms to well within the explicit terms'
- *            FP64 bar, not bitwise;
+ *   "radial_dd" the DCT-I of the lean radial kernels in fixed point (as
+ *            "azimuthal_dd"; the batched layout's FP64 stage always is; stored
+ *            values, field arithmetic, derivatives, banded applies and couplings in
+ *            FP64): 1 always (with the lean layout), 0 never, -1 (default) with the
+ *            lean layout's default, from n_r = 1025.  Results agree with the FP64
+ *            transforms to well within the explicit terms' FP64 bar, not bitwise;
  *   "solve_roles" with explicit buoyancy, the implicit solve in one CTA per
  *            system (streamfunction; temperature, then the zonal flow for m = 0)
  *            instead of one per mode: 1 always, 0 never, -1 (default) from
- *            N_c > 600, where it fits two CTAs per SM.  The same operations
- *            but for the order of the Schur steps' sums (the whole CTA against
- *            one warp): results agree to the accuracy of the refined solve;
+ *            N_c > 600, where three CTAs share an SM.  The same operations but
+ *            for the order of some sums: results agree to the accuracy of the
+ *            refined solve.  1 also keeps the block chains where N_c <= 42, whose
+ *            default is a dense inverse of each system with one refinement;
  *   "psi_chain_dd" the block chains of the streamfunction solve (Appendix
  *            A's banded block) in double-float arithmetic on the FP32 pipe
  *            (about 48 significant bits; the Schur step, residual and refinement
  *            stay FP64), explicit buoyancy: 1 always, 0 never (FP64 chains), -1
  *            (default) from N_c > 64 (at N_c <= 64 the conversions cost more
  *            than the shorter chains save).  Results agree with the FP64 chains
- *            to the accuracy of the refined solve, not bitwise;
+ *            to the accuracy of the refined solve, not bitwise.  0 and 1 keep the
+ *            chains where N_c <= 42 (see "solve_roles");
  *   "theta_fp32" the temperature systems solved by FP32 block chains and two
  *            corrections from FP64 residuals (the zonal flow then refined once
  *            in FP64): 1 always, 0 never (one FP64 solve), -1 (default) from
@@ -177,7 +178,7 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *            drops the factored operators (rebuilt at the next step);
  *   "radial_batch" radial transforms batched per shared-memory pass in the
  *            per-mode explicit kernels: 1, 2 or 4, 0 = the default rule (up to
- *            n_r = 513: 4 in FP64, 2 in mixed precision; else 1); "phi_threads" threads of the per-radius azimuthal
+ *            n_r = 257: 4 in FP64, 2 in mixed precision; 2 at 513; else 1); "phi_threads" threads of the per-radius azimuthal
  *            kernel: 128, 256 or 512 (at most 12 points per thread), 0 = default.
  *            Launch shapes only (pizza_autotune picks them by timing): results
  *            are bitwise the same.
