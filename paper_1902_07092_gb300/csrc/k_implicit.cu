@@ -2234,13 +2234,23 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
         return launch_chained(k_solve_dense, slab_modes(P), NTHREADS_S, sizeof(double) * dense_smem_doubles(P.nc), st, P, rhs,
                               F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
-    // the systems with FP32-refined temperature solves (N_c > 600): with explicit
-    // buoyancy one CTA per system (two per mode, three per SM)
-    const bool large = P.nc > 600;
-    if (!P.buoy_imp && (P.solve_roles > 0 || (P.solve_roles < 0 && large))) {
-        // double-float streamfunction chains: option psi_chain_dd, by default
-        // from N_c > 600 (where the roles kernel is the default)
-        const bool ddp = F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && large));
+    // double-float streamfunction chains with explicit buoyancy (option psi_chain_dd),
+    // by default from N_c > 64: with FP64 ones n_r = 129, 257, 513 took 47.6, 87.8, 335.5
+    // us where these took 45.4, 74.2, 279.3; below, the conversions cost more than the
+    // chains save
+    const bool ddp = !P.buoy_imp && F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && P.nc > 64));
+    // With explicit buoyancy one CTA per system or one per mode.  N_c > 600 (an
+    // FP32-refined temperature): per system.  Below, per system for up to a mode an SM,
+    // whose two systems then run on two SMs, and from four modes an SM on, where three
+    // CTAs of two vectors an SM beat two of seven; between, the modes fit one or two
+    // passes of two CTAs an SM, the systems need part of another.  Solve, us, per mode /
+    // per system: n_r = 129, 257, 513 with 129 modes 38.5 / 35.9, 55.2 / 53.1, 88.0 / 76.3; with
+    // 257 modes 45.2 / 53.1, 69.9 / 79.9, 124.8 / 140.0; with 513 modes 92.3 / 98.2, 153.0 /
+    // 154.1, 257.1 / 248.4; with 1025 modes 186.8 / 151.9, 294.9 / 241.3, 520.7 / 404.6.  (By
+    // the whole number of modes: a slab solves as the whole step does.)
+    const int sms = 152;
+    const bool per_system = P.nc > 600 || (P.nc > 64 && (P.M <= sms || P.M > 4 * sms));
+    if (!P.buoy_imp && (P.solve_roles > 0 || (P.solve_roles < 0 && per_system))) {
         const size_t smr = solve_roles_smem_bytes(P.nc);
         auto kern = ddp ? k_solve_roles<true> : k_solve_roles<false>;
         cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
@@ -2252,11 +2262,6 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
         return launch_chained(kern, 2 * slab_modes(P), NTHREADS_S, smr, st, P, rhs, F, y_out, mass_out, imp_out,
                               want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
-    // one CTA per mode; below N_c = 600 double-float streamfunction chains (option
-    // psi_chain_dd, by default from N_c > 64 with explicit buoyancy: with FP64 ones
-    // n_r = 129, 257, 513 took 47.6, 87.8, 335.5 us where these took 45.4, 74.2, 279.3;
-    // below, the conversions cost more than the chains save)
-    const bool ddp = !large && !P.buoy_imp && F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && P.nc > 64));
     auto kern = F.ir_t ? (ddp ? k_solve<true, true> : k_solve<true, false>) : (ddp ? k_solve<false, true> : k_solve<false, false>);
     const size_t sm = sizeof(double) * solve_smem_doubles(P.nc);
     // the epilogue reads the assembled right-hand sides from shared memory where

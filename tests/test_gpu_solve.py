@@ -57,3 +57,15 @@ def test_chains_below_the_dense_size(n_r, implicit, options):
     dense, _ = run(n_r, 24, "ARS443", implicit, ora=ora)
     flat = [np.concatenate([np.ravel(x) for x in y]) for y in (got, dense)]
     assert rel_l2(*flat) <= bar(n_r)
+
+
+@pytest.mark.parametrize("n_r,n_phi,scheme", [(65, 384, "SBDF2"), (129, 24, "SBDF3"), (129, 384, "ARS443"),
+                                              (129, 768, "CNAB2"), (257, 12, "BPR353"), (129, 3072, "CNAB2")])
+def test_one_cta_per_system_or_per_mode_by_default(n_r, n_phi, scheme):
+    """Either side of the default rule's lines (N_c 64, 152 and 608 modes): the default
+    is one of the two arrangements bit by bit, and the two agree."""
+    got = [run(n_r, n_phi, scheme, False, o, ora=0)[0] for o in ((), (("solve_roles", 0),), (("solve_roles", 1),))]
+    flat = [np.concatenate([np.ravel(x) for x in y]) for y in got]
+    per_system = inputs.n_c_integration(n_r) > 64 and not 152 < n_phi // 3 + 1 <= 608
+    assert np.array_equal(flat[0], flat[2 if per_system else 1])
+    assert rel_l2(flat[1], flat[2]) <= bar(n_r)
