@@ -1055,8 +1055,12 @@ __device__ __forceinline__ void phi_split(const fxc* Y, double2* __restrict__ ds
     }
 }
 
-// Courant rates (cfl_rates) from the packed physical pair (u_phi, v) in R
+// Courant rates (cfl_rates) from the packed physical pair (u_phi, v) in R.  A radius
+// whose fields hold an infinity or NaN (bad) adds no rate, as in cfl_rates, whose
+// maxima pass over NaNs: the rates of the radii and states before it stay to be
+// reported (a NaN, above every number as a bit pattern, would replace them).
 __device__ void cfl_rates_fx(const StepParams& P, const fxc* R, int k, int sv, int su, bool bad, double* red) {
+    if (bad) return;
     fx64 a = 0, b = 0;
     for (int j = threadIdx.x; j < P.n_phi; j += blockDim.x) {
         const fxc g = R[j];
@@ -1070,8 +1074,8 @@ __device__ void cfl_rates_fx(const StepParams& P, const fxc* R, int k, int sv, i
     }
     const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
-        red[2 * w] = fx_to(a, sv, bad);
-        red[2 * w + 1] = fx_to(b, su, bad);
+        red[2 * w] = fx_to(a, sv, false);
+        red[2 * w + 1] = fx_to(b, su, false);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
