@@ -8,18 +8,18 @@
 // butterfly costs ~120 integer instructions where FP64 needs 34 instructions of
 // 64 cycles and double-floats ~400; the code is also short enough to stay in the
 // instruction cache.  One rounding of a value x with block maximum 2^e is
-// 2^(e - 60) or finer: no worse than the rounding of an FP64 transform (host
-// comparison with long double sums: flat and decaying inputs, lengths 16 to 8192).
+// 2^(e - 60) or finer, so a transform is no worse than an FP64 one (compared with
+// long double in the tests, as it is and through a Chebyshev derivative).
 //
 // Scaling.  Each real component of a vector is normalised by the power of two
-// above its largest magnitude (|x| < 2^60 on entry).  The first pass grows the
+// above its largest magnitude (|x| <= 2^60 on entry).  The first pass grows the
 // magnitude by at most its radix and is not scaled.  A later radix-4 or radix-3
 // pass is either scaled by 1/4 -- a twiddle product comes out as a w / 4 without
 // a shift, so this costs one shift of the untwiddled point -- or, where the
-// 1-norm of the vector shows that no intermediate can leave 62 bits, scaled back
-// by a left shift (fx_schedule).  A vector whose 1-norm is close to its maximum
-// (a decaying spectrum) so keeps almost all 60 bits; a flat one loses only the
-// bits its transform can grow by.
+// 1-norm of the vector shows that no intermediate can leave 62 bits, not scaled:
+// the products are shifted back (fx_schedule).  A vector whose 1-norm is close to its
+// maximum (a decaying spectrum) so keeps almost all 60 bits; a flat one loses only
+// the bits its transform can grow by.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -37,7 +37,7 @@ struct __align__(16) fxw {
     int x1, x0, y1, y0;
 };
 
-constexpr int FX_BITS = 60;  // |component| < 2^FX_BITS on entry to a transform
+constexpr int FX_BITS = 60;  // |component| <= 2^FX_BITS on entry to a transform
 
 // The widening multiply-adds and the word accesses are written out: from plain C
 // the compiler spends 40 instructions on a complex product instead of 29.
@@ -76,7 +76,28 @@ FX_HD fx64 fx_round32(fx64 a) {
 }
 FX_HD fxc fx_add(fxc a, fxc b) { return fxc{a.x + b.x, a.y + b.y}; }
 FX_HD fxc fx_sub(fxc a, fxc b) { return fxc{a.x - b.x, a.y - b.y}; }
-FX_HD fxc fx_shr(fxc a, int s) { return fxc{a.x >> s, a.y >> s}; }
+// Shifts to the right without a preferred direction.  One that rounds down moves every
+// butterfly of a pass the same way, by 3/8 of a unit (1/8 rounding halves up), and such
+// a constant survives the sums of a transform and of a Chebyshev derivative, where
+// unbiased roundings cancel: a derivative from 2049 grid values comes out 2.7e-11 wrong
+// rounding down, 7.2e-12 with halves up, 2.3e-12 unbiased (7.0e-12 in FP64).  The radial
+// transforms round so (RND); the azimuthal ones, whose spectra no sum differentiates,
+// shift down (1 % of a step less; no worse than FP64 either).
+// a 2^-s to nearest, halves to even (s >= 1)
+FX_HD fx64 fx_shr(fx64 a, int s) { return (a + ((((fx64)1 << (s - 1)) - 1) + ((a >> s) & 1))) >> s; }
+// a/2 and (a + b)/2, a half to the odd neighbour: one instruction beside the shift
+FX_HD fx64 fx_half(fx64 a) { return (a >> 1) | (a & 1); }
+FX_HD fxc fx_half(fxc a) { return fxc{fx_half(a.x), fx_half(a.y)}; }
+FX_HD fx64 fx_avg(fx64 a, fx64 b) { return ((a >> 1) + (b >> 1) + (a & b & 1)) | ((a ^ b) & 1); }
+// a/2 and a/4 of the passes
+template <bool RND>
+FX_HD fxc fx_scale2(fxc a) {
+    return RND ? fx_half(a) : fxc{a.x >> 1, a.y >> 1};
+}
+template <bool RND>
+FX_HD fxc fx_scale4(fxc a) {
+    return RND ? fxc{fx_shr(a.x, 2), fx_shr(a.y, 2)} : fxc{a.x >> 2, a.y >> 2};
+}
 FX_HD fxc fx_shl2(fxc a) {
     return fxc{(fx64)((unsigned long long)a.x << 2), (fx64)((unsigned long long)a.y << 2)};
 }
@@ -135,18 +156,19 @@ FX_HD void fx_first4(const fxc* src, fxc* dst, int quarter, int t) {
 }
 // radix 8 as the first pass (L = 8^a 4^b with an odd log2): two 4-point transforms of
 // the even and the odd points, halved, and one radix-2 level.  Scaled by 1/2.
+template <bool RND>
 FX_HD void fx_first8(const fxc* src, fxc* dst, int eighth, int t) {
     fxc e0, e1, e2, e3, o0, o1, o2, o3;
     fx_bfly4(src[t], src[t + 2 * eighth], src[t + 4 * eighth], src[t + 6 * eighth], e0, e1, e2, e3);
     fx_bfly4(src[t + eighth], src[t + 3 * eighth], src[t + 5 * eighth], src[t + 7 * eighth], o0, o1, o2, o3);
-    e0 = fx_shr(e0, 1);
-    e1 = fx_shr(e1, 1);
-    e2 = fx_shr(e2, 1);
-    e3 = fx_shr(e3, 1);
-    o0 = fx_shr(o0, 1);
-    o1 = fx_shr(o1, 1);
-    o2 = fx_shr(o2, 1);
-    o3 = fx_shr(o3, 1);
+    e0 = fx_scale2<RND>(e0);
+    e1 = fx_scale2<RND>(e1);
+    e2 = fx_scale2<RND>(e2);
+    e3 = fx_scale2<RND>(e3);
+    o0 = fx_scale2<RND>(o0);
+    o1 = fx_scale2<RND>(o1);
+    o2 = fx_scale2<RND>(o2);
+    o3 = fx_scale2<RND>(o3);
     // o1 (1 - i)/sqrt 2, o2 (-i), o3 (-1 - i)/sqrt 2
     o1 = fxc{fx_mulc(o1.x + o1.y, FX_R2_1, FX_R2_0), fx_mulc(o1.y - o1.x, FX_R2_1, FX_R2_0)};
     o2 = fxc{o2.y, -o2.x};
@@ -171,55 +193,57 @@ FX_HD fxw fx_ldw(const fxw* p) {
 FX_HD fxw fx_ldw(const fxw* p) { return *p; }
 #endif
 // twstep: stride of the twiddle table times L / (4 Ns)
+template <bool RND>
 FX_HD void fx_pass4(const fxc* src, fxc* dst, int quarter, int q, const fxw* tw, int twstep, bool back, bool swz, int t) {
     const int k = t & ((1 << q) - 1);
     const int i0 = k * twstep;
     const int p0 = swz ? fx_swz(t) : t, p1 = swz ? fx_swz(t + quarter) : t + quarter;
     const int p2 = swz ? fx_swz(t + 2 * quarter) : t + 2 * quarter, p3 = swz ? fx_swz(t + 3 * quarter) : t + 3 * quarter;
-    const fxc v0 = fx_shr(src[p0], 2);
-    const fxc v1 = fx_mul4(src[p1], fx_ldw(tw + i0));
-    const fxc v2 = fx_mul4(src[p2], fx_ldw(tw + 2 * i0));
-    const fxc v3 = fx_mul4(src[p3], fx_ldw(tw + 3 * i0));
+    fxc v0 = src[p0];
+    fxc v1 = fx_mul4(src[p1], fx_ldw(tw + i0));
+    fxc v2 = fx_mul4(src[p2], fx_ldw(tw + 2 * i0));
+    fxc v3 = fx_mul4(src[p3], fx_ldw(tw + 3 * i0));
+    if (back) {
+        v1 = fx_shl2(v1);
+        v2 = fx_shl2(v2);
+        v3 = fx_shl2(v3);
+    } else {
+        v0 = fx_scale4<RND>(v0);
+    }
     fxc o0, o1, o2, o3;
     fx_bfly4(v0, v1, v2, v3, o0, o1, o2, o3);
-    if (back) {
-        o0 = fx_shl2(o0);
-        o1 = fx_shl2(o1);
-        o2 = fx_shl2(o2);
-        o3 = fx_shl2(o3);
-    }
     fxc* d = dst + (((t >> q) << (q + 2)) + k);
     d[0] = o0;
     d[1 << q] = o1;
     d[2 << q] = o2;
     d[3 << q] = o3;
 }
-// the last pass of a length 3 * 2^p: sub-transforms of length third = L/3
+// the last pass of a length 3 * 2^p (azimuthal): sub-transforms of length third = L/3
 FX_HD void fx_pass3(const fxc* src, fxc* dst, int third, const fxw* tw, int tws, bool back, bool swz, int t) {
     const int p1 = t + third, p2 = t + 2 * third;
-    const fxc v0 = fx_shr(src[swz ? fx_swz(t) : t], 2);
-    const fxc v1 = fx_mul4(src[swz ? fx_swz(p1) : p1], fx_ldw(tw + t * tws));
-    const fxc v2 = fx_mul4(src[swz ? fx_swz(p2) : p2], fx_ldw(tw + 2 * t * tws));
-    const fxc s = fx_add(v1, v2), e = fx_sub(v1, v2);
-    const fxc m = fxc{v0.x - (s.x >> 1), v0.y - (s.y >> 1)};
-    const fxc r = fxc{fx_mulc(e.y, FX_H3_1, FX_H3_0), -fx_mulc(e.x, FX_H3_1, FX_H3_0)};  // -i (sqrt 3/2) e
-    fxc o0 = fx_add(v0, s), o1 = fx_add(m, r), o2 = fx_sub(m, r);
+    fxc v0 = src[swz ? fx_swz(t) : t];
+    fxc v1 = fx_mul4(src[swz ? fx_swz(p1) : p1], fx_ldw(tw + t * tws));
+    fxc v2 = fx_mul4(src[swz ? fx_swz(p2) : p2], fx_ldw(tw + 2 * t * tws));
     if (back) {
-        o0 = fx_shl2(o0);
-        o1 = fx_shl2(o1);
-        o2 = fx_shl2(o2);
+        v1 = fx_shl2(v1);
+        v2 = fx_shl2(v2);
+    } else {
+        v0 = fx_scale4<false>(v0);
     }
-    dst[t] = o0;
-    dst[t + third] = o1;
-    dst[t + 2 * third] = o2;
+    const fxc s = fx_add(v1, v2), e = fx_sub(v1, v2);
+    const fxc m = fx_sub(v0, fx_scale2<false>(s));
+    const fxc r = fxc{fx_mulc(e.y, FX_H3_1, FX_H3_0), -fx_mulc(e.x, FX_H3_1, FX_H3_0)};  // -i (sqrt 3/2) e
+    dst[t] = fx_add(v0, s);
+    dst[t + third] = fx_add(m, r);
+    dst[t + 2 * third] = fx_sub(m, r);
 }
 
 // Passes of a transform of length (three ? 3 : 1) << lg (lg >= 2): radix 8 first when
 // lg is odd, else radix 4; radix 4; then radix 3.
 FX_HD int fx_passes(int lg, bool three) { return lg / 2 + (three ? 1 : 0); }
 
-// Which passes scale back (bit p of the result) and the bits S lost by the whole
-// transform (the outputs hold X 2^-S), for inputs with components below
+// Which passes are not scaled (bit p of the result) and the bits S lost by the whole
+// transform (the outputs hold X 2^-S), for inputs with components up to
 // 2^FX_BITS and 1-norm (sum of |re| + |im|) below 2^l1.  Every intermediate of
 // the transform is at most the 1-norm and at most the growth of its passes times
 // the largest input.
@@ -303,11 +327,12 @@ __device__ __forceinline__ unsigned fx_exponent(double v) { return ((unsigned)__
 // that they are read and written as such): one copy of the passes serves every
 // transform of a kernel and stays in the instruction cache.
 extern __shared__ __align__(16) fxc fx_shared[];
+template <bool RND>
 __device__ __noinline__ int fx_fft_off(int a, int b, const fxw* __restrict__ tw, int tws, int lg, bool three, int nb,
                                        const unsigned* back) {
     const int L = (three ? 3 : 1) << lg;
     const int tid = threadIdx.x, nth = blockDim.x;
-    // bit 8 i + p: pass p of vector i scales back (at most four vectors of eight passes)
+    // bit 8 i + p: pass p of vector i is not scaled (at most four vectors of eight passes)
     unsigned bk = 0u;
     __syncthreads();
     for (int i = 0; i < nb; ++i) bk |= back[i] << (8 * i);
@@ -318,7 +343,7 @@ __device__ __noinline__ int fx_fft_off(int a, int b, const fxw* __restrict__ tw,
             const fxc* s = fx_shared + (a + i * L);
             fxc* d = fx_shared + (b + i * L);
             if (lg & 1)
-                fx_first8(s, d, n, u - i * n);
+                fx_first8<RND>(s, d, n, u - i * n);
             else
                 fx_first4(s, d, n, u - i * n);
         }
@@ -333,8 +358,8 @@ __device__ __noinline__ int fx_fft_off(int a, int b, const fxw* __restrict__ tw,
         const int twstep = (L >> (q + 2)) * tws;
         for (int u = tid; u < nb * n; u += nth) {
             const int i = three ? (u >= n) : u >> (lg - 2);
-            fx_pass4(fx_shared + (a + i * L), fx_shared + (b + i * L), n, q, tw, twstep, (bk >> (8 * i + p)) & 1u, p == 1,
-                     u - i * n);
+            fx_pass4<RND>(fx_shared + (a + i * L), fx_shared + (b + i * L), n, q, tw, twstep, (bk >> (8 * i + p)) & 1u, p == 1,
+                          u - i * n);
         }
     }
     if (three) {
@@ -351,9 +376,10 @@ __device__ __noinline__ int fx_fft_off(int a, int b, const fxw* __restrict__ tw,
     __syncthreads();
     return b;
 }
+template <bool RND>
 __device__ __forceinline__ fxc* fx_fft(fxc* a, fxc* b, const fxw* __restrict__ tw, int tws, int lg, bool three, int nb,
                                        const unsigned* back) {
-    return fx_shared + fx_fft_off((int)(a - fx_shared), (int)(b - fx_shared), tw, tws, lg, three, nb, back);
+    return fx_shared + fx_fft_off<RND>((int)(a - fx_shared), (int)(b - fx_shared), tw, tws, lg, three, nb, back);
 }
 #endif
 

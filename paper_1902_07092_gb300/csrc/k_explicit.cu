@@ -644,7 +644,7 @@ __device__ __forceinline__ fxc* dct1_fx(const StepParams& P, FxScale& sc, int v0
         sc.back[v] = fx_schedule(lg, false, fx_l1_bits(sc.l1[v]), S);
         sc.S[v] = S;
     }
-    return fx_fft(a, b, reinterpret_cast<const fxw*>(P.fx_r), 1, lg, false, nb, sc.back + v0);
+    return fx_fft<true>(a, b, reinterpret_cast<const fxw*>(P.fx_r), 1, lg, false, nb, sc.back + v0);
 }
 // 2^p times part of an output of vector v
 __device__ __forceinline__ double dct_part(const FxScale& sc, int v, const fxc* z, int part, int p) {
@@ -1018,16 +1018,16 @@ __device__ __forceinline__ fx64 fx_mul62(fx64 a, fx64 b) {
 }
 __device__ __forceinline__ unsigned fx_top(fx64 a) { return (unsigned)((a < 0 ? ~a : a) >> 32); }
 
-// a field's coefficient in fixed point, components below 2^FX_BITS
+// a field's coefficient in fixed point, components up to 2^FX_BITS
 __device__ __forceinline__ fxc phi_coef(double2 v, unsigned e) {
     return (e == 0x7ff) ? fxc{0, 0} : fxc{fx_from(v.x, (int)e), fx_from(v.y, (int)e)};
 }
 // mode m of the fields a and b packed as a + i b into Z, halved (the packed values
-// stay below 2^FX_BITS) and with the components exchanged (fx_fft then runs the
+// stay within 2^FX_BITS) and with the components exchanged (fx_fft then runs the
 // backward transform); returns the 1-norm written
 __device__ __forceinline__ unsigned phi_pack(fxc a, fxc b, int m, int Pn, fxc* Z) {
-    a = fx_shr(a, 1);
-    b = fx_shr(b, 1);
+    a = fx_half(a);
+    b = fx_half(b);
     if (m == 0) {
         Z[0] = fxc{b.x, a.x};
         return fx_l1_part(a.x) + fx_l1_part(b.x);
@@ -1044,8 +1044,7 @@ __device__ __forceinline__ void phi_split(const fxc* Y, double2* __restrict__ ds
     for (int m = threadIdx.x; m <= n_m; m += blockDim.x) {
         const fxc y1 = Y[m], y2 = Y[m ? Pn - m : 0];
         // a = (y1 + conj(y2))/2,  b = (y1 - conj(y2))/(2i)
-        fx64 v[4] = {(y1.x >> 1) + (y2.x >> 1), (y1.y >> 1) - (y2.y >> 1), (y1.y >> 1) + (y2.y >> 1),
-                     (y2.x >> 1) - (y1.x >> 1)};
+        const fx64 v[4] = {fx_avg(y1.x, y2.x), fx_avg(y1.y, -y2.y), fx_avg(y1.y, y2.y), fx_avg(y2.x, -y1.x)};
         double d[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -1202,7 +1201,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
     }
     if (PAIR) {
         schedule(0, 2);
-        R1 = fx_fft(X, Y, tw, 1, lg, three, 2, sc.back);
+        R1 = fx_fft<false>(X, Y, tw, 1, lg, three, 2, sc.back);
         R2 = R1 + Pn;
         for (int i = 0; i < 2; ++i) {
             unsigned x = 0u, yv = 0u;
@@ -1223,7 +1222,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
                 if ((tid & 31) == 0) atomicAdd(&sc.l1[1], w1);
             }
             schedule(i, 1);
-            R2 = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + i);
+            R2 = fx_fft<false>(X, Y, tw, 1, lg, three, 1, sc.back + i);
             unsigned x = 0u, yv = 0u;
             for (int j = tid; j < Pn; j += nth) {
                 x |= fx_top(R2[j].x);
@@ -1255,7 +1254,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
     const int xv = sc.S[0] + (int)ev - 1022 - FX_BITS + 1 - sh[0], xu = sc.S[0] + (int)eu - 1022 - FX_BITS + 1 - sh[1];
     const int xw = sc.S[1] + (int)ew - 1022 - FX_BITS + 1 - sh[2], xt = sc.S[1] + (int)et - 1022 - FX_BITS + 1 - sh[3];
     unsigned l0 = 0u, l1 = 0u;
-    auto up = [](fx64 a, int s) { return s >= 0 ? (fx64)((unsigned long long)a << s) : a >> -s; };
+    auto up = [](fx64 a, int s) { return s >= 0 ? (fx64)((unsigned long long)a << s) : fx_shr(a, -s); };
     // (v omega, u_phi omega) and (v theta, u_phi theta), each 2^-62 of the integers' product
     auto prods = [&](fxc g1, fxc g2, fxc& p, fxc& r) {
         const fx64 v = up(g1.y, sh[0]), u = up(g1.x, sh[1]), w = up(g2.y, sh[2]), t = up(g2.x, sh[3]);
@@ -1289,7 +1288,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         }
         norms();
         schedule(2, 2);
-        const fxc* Z = fx_fft(O, const_cast<fxc*>(R1), tw, 1, lg, three, 2, sc.back + 2);
+        const fxc* Z = fx_fft<false>(O, const_cast<fxc*>(R1), tw, 1, lg, three, 2, sc.back + 2);
         phi_split(Z, dst, M, Pn, n_m, three, xv + xw + 62 + sc.S[2] + ln, xu + xw + 62 + sc.S[2] + ln, bv || bw, bu || bw);
         phi_split(Z + Pn, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln,
                   bv || bt, bu || bt);
@@ -1307,7 +1306,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         }
         norms();
         schedule(2, 2);
-        const fxc* Z = fx_fft(O, const_cast<fxc*>(R2), tw, 1, lg, three, 1, sc.back + 2);
+        const fxc* Z = fx_fft<false>(O, const_cast<fxc*>(R2), tw, 1, lg, three, 1, sc.back + 2);
         phi_split(Z, dst, M, Pn, n_m, three, xv + xw + 62 + sc.S[2] + ln, xu + xw + 62 + sc.S[2] + ln, bv || bw, bu || bw);
         __syncthreads();
 #pragma unroll
@@ -1315,7 +1314,7 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
             const int j = tid + n * nth;
             if (j < Pn) X[j] = reg[n];
         }
-        Z = fx_fft(X, Y, tw, 1, lg, three, 1, sc.back + 3);
+        Z = fx_fft<false>(X, Y, tw, 1, lg, three, 1, sc.back + 3);
         phi_split(Z, dst + 2 * M, M, Pn, n_m, three, xv + xt + 62 + sc.S[3] + ln, xu + xt + 62 + sc.S[3] + ln, bv || bt,
                   bu || bt);
         means();
@@ -1872,7 +1871,7 @@ __device__ __forceinline__ void dct1_half_fx(const StepParams& P, FxScale& sc, D
         fx64 ch = 0, cl = 0;
         auto get = [&](int j) -> fx64 {
             if (j >= n || e == 0x7ff) return 0;
-            const fx64 q = fx_from(val(2 * j + part), e) >> 2;  // pairs grow by less than four
+            const fx64 q = fx_shr(fx_from(val(2 * j + part), e), 2);  // pairs grow by less than four
             return (twice && (j == 0 || j == K)) ? 2 * q : q;
         };
         for (int j = tid >> 1; j <= H; j += nth >> 1) {
@@ -1884,7 +1883,7 @@ __device__ __forceinline__ void dct1_half_fx(const StepParams& P, FxScale& sc, D
             }
             const fx64 b = get(K - j);
             l1 += fx_l1_part(b);
-            const fx64 hs = (a + b) >> 1, dif = a - b;
+            const fx64 hs = fx_half(a + b), dif = a - b;
             fx64 c;
             if (j == 0) {
                 x[0] = hs;
@@ -1928,14 +1927,14 @@ __device__ __forceinline__ void dct1_half_fx(const StepParams& P, FxScale& sc, D
         }
         h += l >> 32;
         l &= 0xffffffffll;
-        dh.c1[tid] = (fx64)((unsigned long long)h << (31 - S)) + (l >> (S + 1));  // rounded down (S < 31)
+        dh.c1[tid] = (fx64)((unsigned long long)h << (31 - S)) + fx_shr(l, S + 1);  // (S < 31)
     }
-    F = fx_fft(X, Y, tw, 2, lg, false, 1, sc.back + v);
+    F = fx_fft<true>(X, Y, tw, 2, lg, false, 1, sc.back + v);
     O = (F == X) ? Y : X;
     // odd outputs: each thread a run of k, its increments, a scan over the CTA
     const int chunk = (H + nth - 1) / nth;
     const int lo = min(tid * chunk, H), hi = min(lo + chunk, H);
-    auto inc = [&](int k) {
+    auto inc = [&](int k) {  // (the roundings of the two halves cancel on average)
         const fxc p = F[k], q = F[K - k];
         return fxc{(q.y >> 1) - (p.y >> 1), (p.x >> 1) - (q.x >> 1)};
     };
@@ -1977,7 +1976,7 @@ __device__ __forceinline__ double half_part(const FxScale& sc, int v, const fxc*
     } else {
         const fxc* f0 = F + kk;
         const fxc* f1 = F + (kk ? K - kk : 0);
-        c = part ? (f0->y >> 1) + (f1->y >> 1) : (f0->x >> 1) + (f1->x >> 1);
+        c = part ? fx_avg(f0->y, f1->y) : fx_avg(f0->x, f1->x);
     }
     const int ex = (int)sc.e[v][part];
     return fx_to(c, sc.S[v] + 1 - 1022 - (FX_BITS - 2) + p + ex, ex == 0x7ff);
