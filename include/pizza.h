@@ -150,11 +150,11 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *            (three CTAs per SM; faster at n_r = 2049, but the half-length DCT-I
  *            accumulates the FP32 rounding of its outputs: about 20x the
  *            batched layout's distance from FP64, still within the mixed bar);
- *   "radial_dd" the DCT-I of the lean radial kernels in fixed point (as
- *            "azimuthal_dd"; the batched layout's FP64 stage always is; stored
- *            values, field arithmetic, derivatives, banded applies and couplings in
- *            FP64): 1 always (with the lean layout), 0 never, -1 (default) with the
- *            lean layout's default, from n_r = 1025.  Results agree with the FP64
+ *   "radial_dd" the DCT-I of the FP64 stage's radial kernels in fixed point (as
+ *            "azimuthal_dd"; stored values, field arithmetic, derivatives, banded
+ *            applies and couplings in FP64): 1 always, 0 never (FP64 transforms in
+ *            either layout of "radial_lean"), -1 (default) always in the batched
+ *            layout and from n_r = 1025 in the lean one.  Results agree with the FP64
  *            transforms to well within the explicit terms' FP64 bar, not bitwise;
  *   "solve_roles" with explicit buoyancy, the implicit solve in one CTA per
  *            system (streamfunction; temperature, then the zonal flow for m = 0)

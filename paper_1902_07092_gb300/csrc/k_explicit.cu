@@ -1506,11 +1506,12 @@ __host__ __device__ inline bool lean_radial(const StepParams& P) {
     return P.radial_lean > 0 || P.K >= LEAN_K;
 }
 
-// fixed-point radial transforms in the lean kernels (option "radial_dd"):
-// 1 always, 0 never, -1 (default) as the lean layout's own default
-__host__ __device__ inline bool radial_fx(const StepParams& P) {
+// fixed-point radial transforms of the FP64 stage (option "radial_dd"): 1 always, 0
+// never (FP64 transforms in either layout), -1 (default) in the batched layout and, in
+// the lean one, from its own default size
+inline bool radial_fx(const StepParams& P) {
     if (!P.fx_r || P.radial_dd == 0) return false;
-    return P.radial_dd > 0 || P.K >= LEAN_K;
+    return P.radial_dd > 0 || !lean_radial(P) || P.K >= LEAN_K;
 }
 
 // The FP64 accumulators of dct1_pair: exact widening of FP32 values by their
@@ -2269,7 +2270,7 @@ static cudaError_t phi_products_t(const StepParams& P, const void* G1, void* G2,
 
 template <class T>
 static cudaError_t grid_to_spec_t(const StepParams& P, const void* G2, VecSet y, VecSet e, cudaStream_t st) {
-    const size_t sm = smem_grid_to_spec(P);
+    const size_t sm = smem_spec_to_grid(P);  // (its buffers are those of the synthesis)
     cudaError_t err = cudaFuncSetAttribute(k_grid_to_spec<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
     return launch_chained(k_grid_to_spec<T>, slab_modes(P), NTHREADS_R, sm, st, P, static_cast<const T*>(G2), y, e);
@@ -2295,6 +2296,7 @@ cudaError_t launch_spec_to_grid(const StepParams& P, VecSet y, double2* G1, doub
         return launch_chained(k_spec_to_grid_lean<double2>, slab_modes(P), NTHREADS_R, sm, st, P, y, G1);
     }
     if (P.fp32) return spec_to_grid_t<float2>(P, y, G1, W, st);
+    if (!radial_fx(P)) return spec_to_grid_t<double2>(P, y, G1, W, st);
     const size_t sm = smem_spec_to_grid(P);
     cudaError_t err = cudaFuncSetAttribute(k_spec_to_grid_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
@@ -2337,6 +2339,7 @@ cudaError_t launch_grid_to_spec(const StepParams& P, const double2* G2, VecSet y
         return launch_chained(kern, slab_modes(P), fx ? NTHREADS_LX : NTHREADS_R, sm, st, P, G2, y, e);
     }
     if (P.fp32) return grid_to_spec_t<float2>(P, G2, y, e, st);
+    if (!radial_fx(P)) return grid_to_spec_t<double2>(P, G2, y, e, st);
     const size_t sm = smem_grid_to_spec(P);
     cudaError_t err = cudaFuncSetAttribute(k_grid_to_spec_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;

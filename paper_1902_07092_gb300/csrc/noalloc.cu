@@ -190,6 +190,7 @@ extern "C" int pizza_explicit_terms_noalloc(int n_r, int n_phi, double Ra, doubl
     }
     const double* fx = sl->tables + NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND;
     P.fx_r = reinterpret_cast<const int4*>(fx);
+    P.radial_dd = -1;  // as by default
     P.fx_p = reinterpret_cast<const int4*>(fx + NA_TAB_TWR);
     P.ops.tau_psi_B = nullptr;  // the explicit stage uses no tau rows
     P.ops.tau_dir_B = nullptr;

@@ -165,8 +165,8 @@ struct StepParams {
     // FP64 radial kernels in the three-array layout (option "radial_lean"):
     // 1 from n_r = 129 (the half-length DCT-I), 0 never, -1 (default) from n_r = 1025
     int radial_lean;
-    // fixed-point DCT-I in the lean radial kernels (option "radial_dd"): 1 always,
-    // 0 never (FP64), -1 (default) from n_r = 1025
+    // fixed-point DCT-I of the FP64 radial kernels (option "radial_dd"): 1 always, 0 never
+    // (FP64), -1 (default) in the batched layout and in the lean one from n_r = 1025
     int radial_dd;
     // streamfunction block chains of the solve in double-float arithmetic
     // (option "psi_chain_dd", explicit buoyancy): 1 always, 0 never, -1
