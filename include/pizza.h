@@ -126,8 +126,9 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *            the FP64 explicit stage in fixed point (64-bit integers with 60
  *            significant bits under each vector's maximum, on the integer pipes),
  *            the m = 0 modes of the products in FP64; 0 = in FP64.  Both meet the
- *            FP64 parity bars of the explicit terms.  The adjoint's azimuthal stage
- *            is FP64 either way;
+ *            FP64 parity bars of the explicit terms.  The fixed-point transforms take
+ *            values below the normal FP64 range (2^-1022) for zeros; the FP64 ones keep
+ *            them.  The adjoint's azimuthal stage is FP64 either way;
  *   "check_finite" 1 = after every step a small kernel scans the state for NaN
  *            or infinite values and sets a device flag; pizza_synchronize then
  *            returns PIZZA_ENONFINITE (cleared by pizza_set_state).  0 (default) =

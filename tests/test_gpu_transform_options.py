@@ -44,3 +44,20 @@ def test_fp64_transforms_with_pumping(n_r):
     ora = IntegrationStepper(n_r, 48, 1e-3, 1.1e5, 1.0, 0.35, "CNAB2", 1e-4, pumping_eps=3e-3)
     for a, b in zip(got, explicit_terms(ora.g, ps, th, u)):
         assert np.linalg.norm(a - b) <= bar(n_r) * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n_r", [33, 257])
+def test_fp64_transforms_keep_subnormal_values(n_r):
+    """A state of 2^-1040: its grid values to the spacing of the subnormal numbers (2^-1074;
+    off the walls, where u_phi is scaled by the vanishing v), against those of the state itself."""
+    from paper_1902_07092_gb300 import binding as B
+    ps, th, u = state(n_r, 24, (1.0, 1.0, 1.0))
+    f = 2.0 ** -1040
+    s = B.Solver(n_r, 24, 1e-3, 1.1e5, 1.0, 0.35, "CNAB2", 1e-4)
+    B.pizza_set_option(s.ctx, "radial_dd", 0)
+    s.set_state(th, ps, u)
+    ref = s.get_grid()
+    s.set_state(th * f, ps * f, u * f)
+    for a, b in zip(s.get_grid(), ref):
+        assert np.abs(a[1:-1] / f - b[1:-1]).max() <= 1e-3 * np.abs(b).max()
+    s.close()
