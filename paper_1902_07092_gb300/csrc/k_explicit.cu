@@ -992,13 +992,14 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P
 // two buffers fill its shared memory).  Against the double-float kernel: 257 x 768 37 -> 24.4 us, 33 x 96 22 -> 12.2, 1025 x 3072
 // 443 -> 313, 2049 x 6144 1706 -> 1265 us.
 // ---------------------------------------------------------------------------
+constexpr int PHI_SUMS = 12;
 struct PhiScale {
     unsigned e[4];      // biased exponents of v, u_phi, omega, theta
     unsigned top[4];    // OR of the leading words of the fields' physical values
     unsigned l1[4];     // 1-norms of the packed spectra, then of the packed products
     unsigned back[4];
     int S[4];
-    double mean[16][4];  // per warp: sums of the four products over the modes
+    double mean[PHI_SUMS][4];  // partial sums of the four products over the modes
     double mean0[4];     // the products' means
     double cfl[2 * 16];
 };
@@ -1116,47 +1117,56 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         // exponents of the fields and, in FP64 (its pipe is idle here), the means of the
         // products, a_0 b_0 + 2 sum_{m >= 1} Re(a_m conj(b_m)), exact for these band-limited fields:
         // they cancel (the zonal forcing [v omega]_0 down to 1e-7 of its terms), where even a
-        // few units of rounding of the transforms' m = 0 entries show
+        // few units of rounding of the transforms' m = 0 entries show.  In the same order for
+        // any number of threads (a launch shape, which changes no bit of a result): partial
+        // sum w takes the modes of warp w of PHI_SUMS, and a smaller CTA's warps take several.
+        // (Twelve are what the 384 threads of n_phi = 768 and 1536 have: 83.5 us at 513 x
+        // 1536 as with one sum a warp, 85.7 with sixteen.)
         unsigned ex[4] = {0u, 0u, 0u, 0u};
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int m = tid; m <= n_m; m += nth) {
-            double2 f[4];
+        const int lane = tid & 31;
+        for (int w = tid >> 5; w < PHI_SUMS; w += nth >> 5) {
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+            for (int m = 32 * w + lane; m <= n_m; m += 32 * PHI_SUMS) {
+                double2 f[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                f[q] = src[q * M + m];
-                ex[q] = max(ex[q], max(fx_exponent(f[q].x), fx_exponent(f[q].y)));
-            }
+                for (int q = 0; q < 4; ++q) {
+                    f[q] = src[q * M + m];
+                    ex[q] = max(ex[q], max(fx_exponent(f[q].x), fx_exponent(f[q].y)));
+                }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {  // (v, omega), (u_phi, omega), (v, theta), (u_phi, theta)
-                const double2 a = f[q & 1], b = f[2 + (q >> 1)];
-                acc[q] = m ? fma(a.x, b.x, fma(a.y, b.y, acc[q])) : 0.5 * (a.x * b.x);
+                for (int q = 0; q < 4; ++q) {  // (v, omega), (u_phi, omega), (v, theta), (u_phi, theta)
+                    const double2 a = f[q & 1], b = f[2 + (q >> 1)];
+                    acc[q] = m ? fma(a.x, b.x, fma(a.y, b.y, acc[q])) : 0.5 * (a.x * b.x);
+                }
             }
+            if (32 * w <= n_m) {
+                // four sums over the warp: halves exchanged twice, then lanes of equal l >> 3 added up
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const int o = 16 >> s, half = 2 >> s;
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int i = 0; i < half; ++i) {
+                        const double send = up ? acc[i] : acc[i + half];
+                        acc[i] = (up ? acc[i + half] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+            }
+            if ((lane & 7) == 0) sc.mean[w][lane >> 3] = acc[0];
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             ex[q] = __reduce_max_sync(0xffffffffu, ex[q]);
-            if ((tid & 31) == 0) atomicMax(&sc.e[q], ex[q]);
+            if (lane == 0) atomicMax(&sc.e[q], ex[q]);
         }
-        // four sums over the warp: halves exchanged twice, then lanes of equal l >> 3 added up
-        const int lane = tid & 31;
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const int o = 16 >> s, half = 2 >> s;
-            const bool up = lane & o;
-#pragma unroll
-            for (int i = 0; i < half; ++i) {
-                const double send = up ? acc[i] : acc[i + half];
-                acc[i] = (up ? acc[i + half] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-        if ((lane & 7) == 0) sc.mean[tid >> 5][lane >> 3] = acc[0];
     }
     __syncthreads();
-    if (tid >= nth - 32) {  // one warp: lane 4 w + q adds warps w and w + 8 of product q
-        const int q = tid & 3, w = (tid & 31) >> 2, nw = nth >> 5;
-        double v = (w < nw ? sc.mean[w][q] : 0.0) + (w + 8 < nw ? sc.mean[w + 8][q] : 0.0);
+    if (tid >= nth - 32) {  // one warp: lane 4 w + q adds partial sums w and w + 8 of product q
+        const int q = tid & 3, w = (tid & 31) >> 2;
+        double v = sc.mean[w][q] + (w + 8 < PHI_SUMS ? sc.mean[w + 8][q] : 0.0);
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (w == 0) sc.mean0[q] = 2.0 * v;

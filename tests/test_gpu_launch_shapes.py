@@ -1,0 +1,28 @@
+"""Option phi_threads is a launch shape: the explicit terms are the same bits for every
+thread count of the azimuthal kernel and for the default rule's, with fewer modes
+than threads and with several modes a thread, in fixed point, FP64 and FP32."""
+import numpy as np
+import pytest
+
+from tests.test_gpu_fixed_point import state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("options", [(), (("azimuthal_dd", 0),), (("precision", 1),)])
+@pytest.mark.parametrize("n_phi", [12, 96, 384, 768, 1536, 3072, 6144])
+def test_thread_counts_give_the_same_bits(n_phi, options):
+    from paper_1902_07092_gb300 import binding as B
+    ps, th, u = state(33, n_phi, (1.0, 1.0, 1.0))
+    out = {}
+    for threads in (0, 128, 256, 512):
+        if n_phi > 12 * (threads or 512):
+            continue
+        s = B.Solver(33, n_phi, 1e-3, 1.1e5, 1.0, 0.35, "CNAB2", 1e-4)
+        for k, v in options + (("phi_threads", threads),):
+            B.pizza_set_option(s.ctx, k, v)
+        s.set_state(th, ps, u)
+        out[threads] = s.explicit_terms()
+        s.close()
+    for threads, got in out.items():
+        assert all(np.array_equal(a, b) for a, b in zip(got, out[0])), threads
