@@ -308,12 +308,14 @@ int pizza_nusselt_end(pizza_ctx *ctx, double *sum, int *steps);
  * or four per shared-memory pass, 128/256/512 threads in the azimuthal kernel --
  * and, with explicit buoyancy and tau rows, the implicit solve with one CTA per
  * mode and with one per system (option "solve_roles"), and keeps the fastest
- * for later steps.  The launch shapes change the schedule, not the arithmetic
- * (bitwise the same results); the solve arrangement changes the order of the
- * Schur steps' sums, so results agree to the accuracy of the refined solve.
- * *nb_r and *phi_threads (may be NULL) receive the
- * explicit-stage choice.  Integration formulation only; builds the factored
- * operators if the context has not stepped yet. */
+ * for later steps.  The default rule of the launch shapes (both options 0), which
+ * has thread counts of its own, is kept where no listed shape is faster.  The
+ * launch shapes change the schedule, not the arithmetic (bitwise the same results);
+ * the solve arrangement changes the order of the Schur steps' sums, so results
+ * agree to the accuracy of the refined solve.  *nb_r and *phi_threads (may be NULL)
+ * receive the fastest of the listed launch shapes, also where the default rule is
+ * kept.  Integration formulation only; builds the factored operators if the
+ * context has not stepped yet. */
 int pizza_autotune(pizza_ctx *ctx, int *nb_r, int *phi_threads);
 
 /* Batches of independent contexts (any sizes, parameters and schemes) advanced

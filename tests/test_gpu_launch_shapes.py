@@ -26,3 +26,29 @@ def test_thread_counts_give_the_same_bits(n_phi, options):
         s.close()
     for threads, got in out.items():
         assert all(np.array_equal(a, b) for a, b in zip(got, out[0])), threads
+
+
+@pytest.mark.parametrize("n_r,n_phi", [(257, 768), (513, 768)])
+def test_autotuned_azimuthal_kernel_is_no_slower_than_the_default(n_r, n_phi):
+    """Best of twelve averages of ten launches each, contexts in turn; 3 % for their
+    spread (the listed thread counts are 6 % behind the default rule's here)."""
+    from paper_1902_07092_gb300 import binding as B
+    ps, th, u = state(n_r, n_phi, (1e-2, 1e-2, 1e-2))
+    sols = []
+    for tuned in (False, True):
+        s = B.Solver(n_r, n_phi, 1e-4, 1e6, 1.0, 0.35, "CNAB2", 1e-6)
+        s.set_state(th, ps, u)
+        if tuned:
+            s.autotune()
+        sols.append(s)
+    best = [np.inf, np.inf]
+    for _ in range(12):
+        for i, s in enumerate(sols):
+            B.pizza_profile_begin(s.ctx, 2)
+            for _ in range(10):
+                s.explicit_terms()
+            ms, n = B.pizza_profile_end(s.ctx)
+            best[i] = min(best[i], ms[1] / n[1])
+    for s in sols:
+        s.close()
+    assert best[1] <= 1.03 * best[0], best
