@@ -145,13 +145,13 @@ __device__ __forceinline__ void cp_async_wait1() { cp_async_wait<1>(); }
 // value and columns 4 g .. 4 g + 3: a step is four multiply-adds a lane (eight with
 // complex coefficients) and one exchange, the right-hand side being the sum's start.
 // With a lane per (row, two columns) and both components a step took 10 and 18 FP64
-// instructions of 64 cycles where it now takes 5 and 9, and the previous block's
-// values come from shared memory instead of 8 shuffles.  Measured: 800-900 cycles a
-// step of the real FP64 chain alone on its SM, 600-700 of the double-float one.
+// instructions of 64 cycles where it now takes 5 and 9.  The previous block's values
+// come by shuffles (real coefficients) or through shared memory (complex ones, whose
+// lanes need both components of four rows).
 //
-// The matrices of a walk stream through a ring of D slots in shared memory, filled by
-// asynchronous copies D - 1 ahead and kept filled across the phases' barriers:
-// forward, the middle block's three, backward.  (D = 6 measured the same as 4.)
+// The matrices of a walk stream through a ring of slots in shared memory, filled by
+// asynchronous copies one slot short of its length ahead and kept filled across the phases' barriers:
+// forward, the middle block's three, backward.  (Six slots measured the same as four.)
 // ---------------------------------------------------------------------------
 // Component, accumulator and arithmetic of a chain by its coefficient type: double2
 // (complex, FP64), ddc (complex double-float), double and float (real coefficients).
@@ -267,8 +267,11 @@ __device__ __forceinline__ void ch_prev(const typename Chain<C>::V* v, int c0, i
     if constexpr (Chain<C>::cplx) ch_four(v + 8 * (1 - part) + c0, q);
 }
 
+// slots of a walk's ring (a power of two): 4 KB of complex or double-float matrices,
+// 2 KB of real FP64, 1 KB of FP32 ones (eight of these measured the same)
+constexpr int RING = 4;
 template <class C>
-__host__ __device__ constexpr int ring_bytes(int D) { return D * 64 * (int)sizeof(C); }
+__host__ __device__ constexpr int ring_bytes() { return RING * 64 * (int)sizeof(C); }
 
 struct ChainGeom {
     int nb, cm, len, k_fw, k_bw, dir;  // blocks, middle block, blocks of this half, its first blocks, forward direction
@@ -282,85 +285,133 @@ struct ChainGeom {
     }
 };
 
-// One warp's walk (one set of registers whatever its system) and its stream of
-// matrices through a ring of D slots: entry e (issued in order) to slot e % D, src
-// following the entries from block to block.
+// One warp's walk (one set of registers whatever its system) and its stream of matrices
+// through a ring: entry e (issued in order) to slot e % RING.  A walking warp is mostly alone
+// on its sub-partition and pays for every instruction of a step, so its arrays are
+// offsets into shared memory (read and written as such, 32-bit arithmetic), and the
+// loops run on a pointer that moves by a constant for as long as the entries stay in
+// one direction (far), instead of 64-bit pointers of unknown space and a choice of the
+// source in every step.  Solve, us: 257 x 768 67.7 -> 63.1, 513 x 1536 254 -> 233,
+// 1025 x 3072 770 -> 688, 2049 x 6144 2834 -> 2505; implicit buoyancy, whose temperature
+// and streamfunction chains follow one another, 1025 x 384 305 -> 268 (277 with the
+// real coefficients' previous block through shared memory too).  Real matrices straight
+// to registers, 8 ahead, with unrolled steps: 343 (the code no longer fits the
+// instruction cache next to a lone warp).
+extern __shared__ __align__(16) char walk_shared[];
+template <class V>
+__device__ __forceinline__ V* walk_at(int off) {
+    return reinterpret_cast<V*>(walk_shared + off);
+}
+__device__ __forceinline__ int walk_off(const void* p) { return (int)(reinterpret_cast<const char*>(p) - walk_shared); }
 struct Walk {
-    char *b, *Z, *x, *ring;
-    const char *blk, *src;
+    int b, Z, x, ring;  // offsets
+    const char* blk;
     int n, half, e;
     ChainGeom g;
-    template <class C, int D>
-    __device__ __forceinline__ void issue() {
+    template <class C>
+    __device__ __forceinline__ void copy(const char* src) {
         constexpr int MAT = 64 * (int)sizeof(C);
-        if (e < 2 * g.len + 3) {
-            if (e > 0 && e < g.len) {
-                src += g.dir * 3 * MAT;
-            } else if (e > g.len + 3) {
-                src -= g.dir * 3 * MAT;
-            } else {  // the first block, the middle one's three matrices, the first block backward
-                const int i = e - g.len;
-                src = blk + (i < 0 ? g.k_fw * 3 : i < 3 ? g.cm * 3 + (i == 0 ? 0 : i == 1 ? 2 : 1) : g.k_bw * 3 + 2) * MAT;
-            }
-            char* dst = ring + (e % D) * MAT;
-            const int lane = threadIdx.x & 31;
+        const int lane = threadIdx.x & 31;
+        char* dst = walk_at<char>(ring + (e & (RING - 1)) * MAT + 16 * lane);
 #pragma unroll
-            for (int j = 0; j < MAT; j += 512)
-                if (j + 512 <= MAT || lane < 16) cp_async16(dst + j + 16 * lane, src + j + 16 * lane);
-        }
+        for (int j = 0; j < MAT; j += 512)
+            if (j + 512 <= MAT || lane < 16) cp_async16(dst + j, src + j + 16 * lane);
         cp_async_commit();
         ++e;
     }
-    // the four coefficients of this lane of entry e - D + 1, the oldest in flight
-    template <class C, int D>
+    // entry i: the blocks forward, the middle one's three matrices, the blocks backward
+    template <class C>
+    __device__ __forceinline__ const char* entry(int i) const {
+        const int j = i - g.len;
+        const int mat = j < 0    ? (g.k_fw + g.dir * i) * 3
+                        : j < 3  ? g.cm * 3 + (j == 0 ? 0 : j == 1 ? 2 : 1)
+                                 : (g.k_bw - g.dir * (j - 3)) * 3 + 2;
+        return blk + (ptrdiff_t)mat * (64 * (int)sizeof(C));
+    }
+    template <class C>
+    __device__ __forceinline__ void issue() {
+        if (e < 2 * g.len + 3) {
+            copy<C>(entry<C>(e));
+        } else {
+            cp_async_commit();
+            ++e;
+        }
+    }
+    // the four coefficients of this lane of entry e - RING + 1, the oldest in flight
+    template <class C>
     __device__ __forceinline__ void take(C (&a)[4]) {
         const int lane = threadIdx.x & 31;
-        cp_async_wait<D - 2>();
+        cp_async_wait<RING - 2>();
         __syncwarp();  // also: every lane has read the slot before, which issue refills
-        const C* p = reinterpret_cast<const C*>(ring + ((e + 1) % D) * 64 * (int)sizeof(C)) + (lane >> 2) * 8 + (lane & 1) * 4;
-        ch_four(p, a);
+        ch_four(walk_at<C>(ring + ((e + 1) & (RING - 1)) * 64 * (int)sizeof(C)) + (lane >> 2) * 8 + (lane & 1) * 4, a);
     }
 };
+// A walk over the blocks of one direction: step(i, next) for i < len, next() asking for
+// the matrix that takes the slot of the one just read
+template <class C, class Step>
+__device__ __forceinline__ void walk_blocks(Walk& w, int stride, Step step) {
+    const int len = w.g.len, far = len - (RING - 1);
+    int i = 0;
+    if (far > 0) {
+        const char* src = w.entry<C>(w.e);
+        for (; i < far; ++i)
+            step(i, [&]() {
+                w.copy<C>(src);
+                src += stride;
+            });
+    }
+    for (; i < len; ++i) step(i, [&]() { w.issue<C>(); });
+}
 
 // Forward walk of one warp.  b: n rows (NP components each), Z: 8 nb rows.  prev:
 // this warp's 2 x 16 components in shared memory.
-template <class C, int NP, int D>
+template <class C, int NP>
 __device__ __forceinline__ void chain_forward(Walk& w, typename Chain<C>::V* prev) {
     using V = typename Chain<C>::V;
-    const V* b = reinterpret_cast<const V*>(w.b);
-    V* Z = reinterpret_cast<V*>(w.Z);
     const ChainGeom& g = w.g;
     const int n = w.n;
     const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
     const bool own = gcol == 0 && part < NP;
-#pragma unroll
-    for (int e = 0; e < D - 1; ++e) w.issue<C, D>();
+#pragma unroll 1
+    for (int e = 0; e < RING - 1; ++e) w.issue<C>();
     if (lane < 16) ch_zero(prev[lane]);
-    for (int i = 0; i < g.len; ++i) {
-        const int row = (g.k_fw + g.dir * i) * 8 + r;
+    V pv;
+    ch_zero(pv);
+    int row = g.k_fw * 8 + r;
+    const V* b = walk_at<const V>(w.b) + row * NP + part;
+    V* Z = walk_at<V>(w.Z) + row * NP + part;
+    walk_blocks<C>(w, g.dir * 3 * 64 * (int)sizeof(C), [&](int i, auto next) {
         V bv, p[4], q[4];
         C a[4];
-        w.take<C, D>(a);
-        ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        w.take<C>(a);
+        if constexpr (Chain<C>::cplx) ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) p[j] = __shfl_sync(0xffffffffu, pv, (4 * gcol + j) * 4 + 2 * part);
+        }
         ch_zero(bv);
-        if (row < n && own) bv = b[row * NP + part];
-        w.issue<C, D>();
+        if (row < n && own) bv = *b;
+        next();
         typename Chain<C>::A acc;
         ch_start(acc, bv);
         ch_row<true>(acc, a, p, q, part);
         const V z = ch_value<true>(acc, part);
+        if constexpr (!Chain<C>::cplx) pv = z;
         if (own) {
-            prev[((i + 1) & 1) * 16 + 8 * part + r] = z;
-            Z[row * NP + part] = z;
+            if constexpr (Chain<C>::cplx) prev[((i + 1) & 1) * 16 + 8 * part + r] = z;
+            *Z = z;
         }
-    }
+        row += 8 * g.dir;
+        b += 8 * NP * g.dir;
+        Z += 8 * NP * g.dir;
+    });
 }
 // middle block by both warps of the pair; returns the lane's component of it, also
 // left in prev[0 .. 16) for the backward walk.  The caller stores it after a barrier.
-template <class C, int NP, int D>
+template <class C, int NP>
 __device__ __forceinline__ typename Chain<C>::V chain_middle(Walk& w, typename Chain<C>::V* prev) {
     using V = typename Chain<C>::V;
-    const V *b = reinterpret_cast<const V*>(w.b), *Z = reinterpret_cast<const V*>(w.Z);
+    const V *b = walk_at<const V>(w.b), *Z = walk_at<const V>(w.Z);
     const ChainGeom& g = w.g;
     const int n = w.n;
     const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
@@ -373,14 +424,14 @@ __device__ __forceinline__ typename Chain<C>::V chain_middle(Walk& w, typename C
     ch_start(acc, bv);
     C a[4];
     V p[4], q[4];
-    w.take<C, D>(a);
-    w.issue<C, D>();
+    w.take<C>(a);
+    w.issue<C>();
     if (g.cm > 0) {
         ch_values<C, NP>(Z + (g.cm - 1) * 8 * NP, 4 * gcol, part, p, q);
         ch_row<true>(acc, a, p, q, part);
     }
-    w.take<C, D>(a);
-    w.issue<C, D>();
+    w.take<C>(a);
+    w.issue<C>();
     if (g.cm < g.nb - 1) {
         ch_values<C, NP>(Z + (g.cm + 1) * 8 * NP, 4 * gcol, part, p, q);
         ch_row<true>(acc, a, p, q, part);
@@ -388,8 +439,8 @@ __device__ __forceinline__ typename Chain<C>::V chain_middle(Walk& w, typename C
     const V y = ch_value<true>(acc, part);
     __syncwarp();  // the lanes' reads of the last block
     if (own) prev[16 + 8 * part + r] = y;
-    w.take<C, D>(a);  // (synchronises the warp)
-    w.issue<C, D>();
+    w.take<C>(a);  // (synchronises the warp)
+    w.issue<C>();
     ch_prev<C, NP>(prev + 16, 4 * gcol, part, p, q);
     ch_zero(bv);
     ch_start(acc, bv);
@@ -402,7 +453,7 @@ template <int NP, class V>
 __device__ __forceinline__ void chain_middle_store(const Walk& w, V xv) {
     const int lane = threadIdx.x & 31, part = (lane >> 1) & 1;
     const int row = w.g.cm * 8 + (lane >> 2);
-    if (w.half == 0 && (lane & 1) == 0 && part < NP && row < w.n) reinterpret_cast<V*>(w.x)[row * NP + part] = xv;
+    if (w.half == 0 && (lane & 1) == 0 && part < NP && row < w.n) walk_at<V>(w.x)[row * NP + part] = xv;
 }
 // W_k = [1]_k Z_k in place for every block but the middle one, blocks w, w + nw, ...
 // by warp w, DU of them in flight (their loads before any product)
@@ -437,33 +488,42 @@ __device__ __forceinline__ void chain_diag(typename Chain<C>::V* Z, int n, const
     }
 }
 // backward walk away from the middle block (prev[0 .. 16) holds it)
-template <class C, int NP, int D>
-__device__ __forceinline__ void chain_backward(Walk& w, typename Chain<C>::V* prev) {
+template <class C, int NP>
+__device__ __forceinline__ void chain_backward(Walk& w, typename Chain<C>::V* prev, typename Chain<C>::V mid) {
     using V = typename Chain<C>::V;
-    const V* W = reinterpret_cast<const V*>(w.Z);
-    V* x = reinterpret_cast<V*>(w.x);
     const ChainGeom& g = w.g;
     const int n = w.n;
     const int lane = threadIdx.x & 31, r = lane >> 2, part = (lane >> 1) & 1, gcol = lane & 1;
     const bool own = gcol == 0 && part < NP;
-    for (int i = 0; i < g.len; ++i) {
-        const int row = (g.k_bw - g.dir * i) * 8 + r;
+    int row = g.k_bw * 8 + r;
+    V pv = mid;
+    const V* W = walk_at<const V>(w.Z) + row * NP + part;
+    V* x = walk_at<V>(w.x) + row * NP + part;
+    walk_blocks<C>(w, -g.dir * 3 * 64 * (int)sizeof(C), [&](int i, auto next) {
         V wv, p[4], q[4];
         C a[4];
-        w.take<C, D>(a);
-        ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        w.take<C>(a);
+        if constexpr (Chain<C>::cplx) ch_prev<C, NP>(prev + (i & 1) * 16, 4 * gcol, part, p, q);
+        else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) p[j] = __shfl_sync(0xffffffffu, pv, (4 * gcol + j) * 4 + 2 * part);
+        }
         ch_zero(wv);
-        if (row < n && own) wv = W[row * NP + part];
-        w.issue<C, D>();
+        if (row < n && own) wv = *W;
+        next();
         typename Chain<C>::A acc;
         ch_start(acc, wv);
         ch_row<true>(acc, a, p, q, part);
         const V xv = ch_value<true>(acc, part);
+        if constexpr (!Chain<C>::cplx) pv = xv;
         if (own) {
-            prev[((i + 1) & 1) * 16 + 8 * part + r] = xv;
-            if (row < n) x[row * NP + part] = xv;
+            if constexpr (Chain<C>::cplx) prev[((i + 1) & 1) * 16 + 8 * part + r] = xv;
+            if (row < n) *x = xv;
         }
-    }
+        row -= 8 * g.dir;
+        W -= 8 * NP * g.dir;
+        x -= 8 * NP * g.dir;
+    });
     cp_async_wait<0>();
     __syncwarp();
 }
@@ -480,21 +540,21 @@ struct ChainJob {
 // Whole-CTA driver: ja, jb two halves of one system or one alone, jt and ju others, on
 // disjoint warp pairs.  prevs: 16 doubles x 2 a warp in shared memory.  Z may be b
 // and x where it has room for whole blocks; ends with a barrier that publishes x.
-// With the walks, the diagonal products and the phases above: solve at n_r x n_phi =
-// 129 x 384, 257 x 768, 513 x 1536 46 -> 39, 71 -> 69, 270 -> 260 us; 513 x 384 with
-// implicit buoyancy 136 -> 88 us.
-template <int D, int DU, class CP, int NPP, class CT, int NPT, class CU, int NPU>
+// With the walks, the diagonal products and the phases above: solve by mode at n_r x
+// n_phi = 129 x 384, 257 x 768, 513 x 1536 46 -> 35, 71 -> 63, 270 -> 233 us; 513 x 384
+// with implicit buoyancy 136 -> 123 us.
+template <int DU, class CP, int NPP, class CT, int NPT, class CU, int NPU>
 __device__ __forceinline__ void run_chains(const ChainJob<CP, NPP>& ja, const ChainJob<CP, NPP>& jb, const ChainJob<CT, NPT>& jt,
                                            const ChainJob<CU, NPU>& ju, double (*prevs)[32]) {
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    Walk w{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, warp & 1, 0, ChainGeom(0, 0)};
+    Walk w{0, 0, 0, 0, nullptr, 0, warp & 1, 0, ChainGeom(0, 0)};
     auto pick = [&]<class C, int NP>(const ChainJob<C, NP>& j) {
         if (j.n == 0 || (warp & ~1) != j.w) return false;
-        w.b = reinterpret_cast<char*>(j.b);
-        w.Z = reinterpret_cast<char*>(j.Z);
-        w.x = reinterpret_cast<char*>(j.x);
-        w.ring = j.ring + (warp & 1) * ring_bytes<C>(D);
-        w.blk = w.src = reinterpret_cast<const char*>(j.blk);
+        w.b = walk_off(j.b);
+        w.Z = walk_off(j.Z);
+        w.x = walk_off(j.x);
+        w.ring = walk_off(j.ring) + (warp & 1) * ring_bytes<C>();
+        w.blk = reinterpret_cast<const char*>(j.blk);
         w.n = j.n;
         w.g = ChainGeom(j.n, warp & 1);
         return true;
@@ -508,16 +568,16 @@ __device__ __forceinline__ void run_chains(const ChainJob<CP, NPP>& ja, const Ch
     VP* pp = reinterpret_cast<VP*>(prevs[warp]);
     VT* pt = reinterpret_cast<VT*>(prevs[warp]);
     VU* pu = reinterpret_cast<VU*>(prevs[warp]);
-    if (inp) chain_forward<CP, NPP, D>(w, pp);
-    if (in_t) chain_forward<CT, NPT, D>(w, pt);
-    if (in_u) chain_forward<CU, NPU, D>(w, pu);
+    if (inp) chain_forward<CP, NPP>(w, pp);
+    if (in_t) chain_forward<CT, NPT>(w, pt);
+    if (in_u) chain_forward<CU, NPU>(w, pu);
     __syncthreads();
     VP xp;
     VT xt;
     VU xu;
-    if (inp) xp = chain_middle<CP, NPP, D>(w, pp);
-    if (in_t) xt = chain_middle<CT, NPT, D>(w, pt);
-    if (in_u) xu = chain_middle<CU, NPU, D>(w, pu);
+    if (inp) xp = chain_middle<CP, NPP>(w, pp);
+    if (in_t) xt = chain_middle<CT, NPT>(w, pt);
+    if (in_u) xu = chain_middle<CU, NPU>(w, pu);
     __syncthreads();
     if (inp) chain_middle_store<NPP>(w, xp);
     if (in_t) chain_middle_store<NPT>(w, xt);
@@ -529,17 +589,13 @@ __device__ __forceinline__ void run_chains(const ChainJob<CP, NPP>& ja, const Ch
     if (jt.n > 0) chain_diag<CT, NPT, DU>(jt.Z, jt.n, jt.blk, nw - 1 - warp, nw);
     if (ju.n > 0) chain_diag<CU, NPU, DU>(ju.Z, ju.n, ju.blk, warp, nw);
     __syncthreads();
-    if (inp) chain_backward<CP, NPP, D>(w, pp);
-    if (in_t) chain_backward<CT, NPT, D>(w, pt);
-    if (in_u) chain_backward<CU, NPU, D>(w, pu);
+    if (inp) chain_backward<CP, NPP>(w, pp, xp);
+    if (in_t) chain_backward<CT, NPT>(w, pt, xt);
+    if (in_u) chain_backward<CU, NPU>(w, pu, xu);
     __syncthreads();
 }
 template <class C, int NP>
 __device__ __forceinline__ ChainJob<C, NP> no_job() { return ChainJob<C, NP>{nullptr, nullptr, nullptr, 0, nullptr, 0, nullptr}; }
-
-// Ring depths (matrices a walking warp): 1152 bytes a complex or double-float
-// matrix, 640 a real FP64 one, 384 an FP32 one
-constexpr int RD = 4;
 
 // acc - a z, component part
 __device__ __forceinline__ double fms_part(double acc, double2 a, double2 z, int part) {
@@ -1135,35 +1191,38 @@ __host__ __device__ inline int round8(int n) { return (n + 7) / 8 * 8; }
 // rows of an array that a chain solves in place: whole blocks past an offset of up to 4
 __host__ __device__ inline int chain_rows(int nc) { return round8(nc) + 8; }
 
-__host__ __device__ inline size_t solve_smem_doubles(int nc) {
-    return (size_t)14 * chain_rows(nc) + (4 * ring_bytes<double2>(RD) + 2 * ring_bytes<double>(RD)) / 8;
+// shared_d: the streamfunction's correction over the temperature's FP32 arrays, which are
+// done with before it is formed when the buoyancy is implicit: two CTAs on an SM
+// instead of one at N_c = 682 (solve at 1025 x 1536 1100 -> 788 us)
+__host__ __device__ inline size_t solve_smem_doubles(int nc, bool shared_d) {
+    return (size_t)(shared_d ? 12 : 14) * chain_rows(nc) + (4 * ring_bytes<double2>() + 2 * ring_bytes<double>()) / 8;
 }
 
 __host__ __device__ inline size_t keep_f_doubles(int nc) { return 3 * (size_t)round8(nc); }
 
-__device__ __forceinline__ SolveSmem carve(double2* base, int nc) {
+__device__ __forceinline__ SolveSmem carve(double2* base, int nc, bool shared_d) {
     SolveSmem s;
     const int b = chain_rows(nc);
     s.pf = base;
     s.px = base + b;
-    s.pd = base + 2 * b;
-    s.tf = base + 3 * b;
-    s.tx = base + 4 * b;
-    s.uf = reinterpret_cast<double*>(base + 5 * b);
+    s.tf = base + 2 * b;
+    s.tx = base + 3 * b;
+    s.uf = reinterpret_cast<double*>(base + 4 * b);
     s.ux = s.uf + b;
     s.tr = reinterpret_cast<float2*>(s.ux + b);
     s.td = s.tr + b;
-    s.ring_p = reinterpret_cast<char*>(s.td + b);
-    s.ring_t = s.ring_p + 4 * ring_bytes<double2>(RD);
+    s.pd = reinterpret_cast<double2*>(s.tr) + (shared_d ? 0 : b);
+    s.ring_p = reinterpret_cast<char*>(s.pd + b);
+    s.ring_t = s.ring_p + 4 * ring_bytes<double2>();
     s.ring_u = s.ring_p;
-    s.fp = reinterpret_cast<double2*>(s.ring_t + 2 * ring_bytes<double>(RD));
+    s.fp = reinterpret_cast<double2*>(s.ring_t + 2 * ring_bytes<double>());
     s.fu = reinterpret_cast<double*>(s.fp + round8(nc));
     return s;
 }
 
 // The zonal flow's chain (the CTA of m = 0) by warps 4-5
 __device__ void zonal_chains(const DevFactors& F, SolveSmem& s, double* b, double* x, int nt) {
-    run_chains<RD, 2>(no_job<double, 1>(), no_job<double, 1>(), no_job<float, 2>(),
+    run_chains<2>(no_job<double, 1>(), no_job<double, 1>(), no_job<float, 2>(),
                       ChainJob<double, 1>{b, x, x, nt, F.uBlk, 4, s.ring_u}, s.prevs);
 }
 
@@ -1262,13 +1321,13 @@ __device__ void temperature_residual(const StepParams& P, const DevFactors& F, S
 // The FP32 temperature solve D td = tr of the kernel with one CTA per system:
 // one block walked by warps 2-3, or (tsplit) its two halves by warps 2-3 and 4-5
 // joined through the spikes.  Whole CTA; ends with a barrier.
-__device__ void theta32_chains(const DevFactors& F, SolveSmem& s, int m, int nt, int nbt) {
+__device__ __forceinline__ void theta32_chains(const DevFactors& F, SolveSmem& s, int m, int nt, int nbt) {
     const float* tb = (F.tsplit ? F.tBlk32S : F.tBlk32) + (size_t)m * nbt * 192;
     float *b = reinterpret_cast<float*>(s.tr + 2), *x = reinterpret_cast<float*>(s.td + 2);
     const int ntA = F.tsplit ? 8 * (nbt / 2) : nt;
-    run_chains<RD, 4>(ChainJob<float, 2>{b, x, x, ntA, tb, 2, s.ring_t},
+    run_chains<4>(ChainJob<float, 2>{b, x, x, ntA, tb, 2, s.ring_t},
                       ChainJob<float, 2>{b + 2 * ntA, x + 2 * ntA, x + 2 * ntA, nt - ntA, tb + (size_t)(nbt / 2) * 192, 4,
-                                         s.ring_t + 2 * ring_bytes<float>(RD)},
+                                         s.ring_t + 2 * ring_bytes<float>()},
                       no_job<double, 1>(), no_job<double, 1>(), s.prevs);
     if (F.tsplit) split_join32(s.td + 2, nt, ntA, F.tSpk32 + (size_t)m * nt * 8, F.tRj32 + (size_t)m * 256);
 }
@@ -1295,7 +1354,7 @@ __device__ void temperature_residual_block(const StepParams& P, const DevFactors
 
 // The FP32-refined temperature solve of the kernel with one CTA per system:
 // ir_t corrections x += S32^{-1}(f - L x), every reduction by the whole CTA.
-__device__ void temperature_corrections_roles(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0) {
+__device__ __forceinline__ void temperature_corrections_roles(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0) {
     const int nc = P.nc, nt = nc - 2, nbt = (nt + 7) / 8;
     const int tid = threadIdx.x, nth = blockDim.x;
     for (int it = 0; it < F.ir_t; ++it) {
@@ -1319,15 +1378,17 @@ __device__ __forceinline__ ChainJob<float, 2> theta32_job(const DevFactors& F, c
 // The FP32-refined temperature solve (F.ir_t > 0, MB == 1): x += S32^{-1}(f - L x)
 // for the passes it0 .. ir_t - 1 (pass 0 may have run beside the streamfunction
 // refinement), then the FP64 refinement of the zonal flow (mode 0).
-__device__ void temperature_corrections(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0, bool has_u,
+template <bool IMP>
+__device__ __forceinline__ void temperature_corrections(const StepParams& P, const DevFactors& F, SolveSmem& s, int m0, bool has_u,
                                         int it0) {
     const int nc = P.nc, nt = nc - 2, nbt = (nt + 7) / 8;
     const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5;
     if (F.ir_t) {
-        for (int it = it0; it < F.ir_t; ++it) {
+        if constexpr (IMP) temperature_corrections_roles(P, F, s, m0);
+        for (int it = IMP ? F.ir_t : it0; it < F.ir_t; ++it) {
             temperature_residual(P, F, s, m0, 0);
             __syncthreads();
-            run_chains<RD, 4>(no_job<float, 2>(), no_job<float, 2>(), theta32_job(F, s, m0, nt, nbt, 2), no_job<double, 1>(), s.prevs);
+            run_chains<4>(no_job<float, 2>(), no_job<float, 2>(), theta32_job(F, s, m0, nt, nbt, 2), no_job<double, 1>(), s.prevs);
             if (warp == 2) warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
             __syncthreads();
             schur_update32_dir(s.td, nc, F.tY32 + (size_t)m0 * nt * 2, 0, nth);
@@ -1340,8 +1401,8 @@ __device__ void temperature_corrections(const StepParams& P, const DevFactors& F
 }
 
 // T32: the temperature by FP32 chains refined from FP64 residuals (F.ir_t); DDP:
-// double-float streamfunction chains (explicit buoyancy)
-template <bool T32, bool DDP>
+// double-float streamfunction chains (explicit buoyancy); IMP: implicit buoyancy
+template <bool T32, bool DDP, bool IMP>
 __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                       VecSet mass_out, VecSet imp_out, int want_mass,
                                                       int want_imp, int keep_f) {
@@ -1355,7 +1416,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
     const int np = nc - 4, nt = nc - 2;
     const int nbp = (np + 7) / 8, nbt = (nt + 7) / 8;
     const int nA = 8 * (nbp / 2);  // first half of a split streamfunction block (F.psplit)
-    SolveSmem s = carve(sm, nc);
+    SolveSmem s = carve(sm, nc, T32 && IMP);
     __shared__ __align__(16) double prevs[NTHREADS_S / 32][32];
     s.prevs = prevs;
     const bool has_u = (m0 == 0);
@@ -1381,7 +1442,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         const int n0 = second ? nA : 0, n = m0 == 0 ? 0 : second ? (F.psplit ? np - nA : 0) : F.psplit ? nA : np;
         return ChainJob<CP, 2>{reinterpret_cast<VP*>(b + 4 + n0), reinterpret_cast<VP*>(x + 4 + n0), reinterpret_cast<VP*>(x + 4 + n0), n,
                                blk_p + (second ? (size_t)(nbp / 2) * 192 : 0), (second ? 6 : 0) ^ flip,
-                               s.ring_p + (second ? 2 * ring_bytes<CP>(RD) : 0)};
+                               s.ring_p + (second ? 2 * ring_bytes<CP>() : 0)};
     };
     // the temperature: FP32, or FP64
     using CT = std::conditional_t<T32, float, double>;
@@ -1429,11 +1490,11 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
     //    streamfunction and temperature systems are independent and run together;
     //    with implicit buoyancy (Section 4) the temperature (and zonal flow) goes
     //    first, then g (Ra/Pr)(i m/s_o) C^I theta_new joins the streamfunction rows.
-    const int npass = P.buoy_imp ? 2 : 1;
+    const int npass = IMP ? 2 : 1;
     for (int pass = 0; pass < npass; ++pass) {
-        const bool do_p = !P.buoy_imp || pass == 1;
-        const bool do_t = !P.buoy_imp || pass == 0;
-        if (P.buoy_imp && pass == 1) {
+        const bool do_p = !IMP || pass == 1;
+        const bool do_t = !IMP || pass == 0;
+        if (IMP && pass == 1) {
             if (m0 > 0) {
                 const double cb = F.gdt * P.Ra / P.Pr * (double)m0 / P.s_o;
                 for (int q = 8 + tid; q < 2 * nc; q += nth) {
@@ -1445,9 +1506,18 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         }
         // 2. banded solves by warp pairs: warps 0-1 the streamfunction (6-7 its second
         //    half), 2-3 the temperature, 4-5 the zonal flow (m = 0 only)
-        run_chains<RD, 2>(do_p ? job_p(DDP ? s.pd : s.pf, s.px, false) : no_job<CP, 2>(),
+        // implicit buoyancy: the FP32 temperature solve has the CTA to itself, so its block
+        // goes in halves and its sums over every warp, as in k_solve_roles (1025 x 384:
+        // 268 -> 257 us, 2049 x 384: 516 -> 470)
+        const bool alone_t = T32 && IMP && do_t;
+        if (alone_t) {
+            theta32_chains(F, s, m0, nt, nbt);
+            if (has_u) zonal_chains(F, s, s.uf + 2, s.ux + 2, nt);
+        } else {
+            run_chains<2>(do_p ? job_p(DDP ? s.pd : s.pf, s.px, false) : no_job<CP, 2>(),
                           do_p ? job_p(DDP ? s.pd : s.pf, s.px, true) : no_job<CP, 2>(),
                           do_t ? job_t() : no_job<CT, 2>(), do_t && has_u ? job_u() : no_job<double, 1>(), s.prevs);
+        }
         if (DDP && do_p && m0 > 0) {  // the solution back from double-floats
             if (F.psplit) split_join_dd(reinterpret_cast<ddc*>(s.px) + 4, np, nA, spk_dd, rj_dd, true);
             const ddf* xd = reinterpret_cast<const ddf*>(s.px);
@@ -1462,11 +1532,12 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         //    2 the temperature, 4 the zonal flow
         if (do_p && m0 > 0) rows_dot_part<4>(s.px + 4, np, P.ops.tau_psi_B, part_p);
         if (do_t && !T32) rows_dot_part<2>(s.tx + 2, nt, P.ops.tau_dir_B, part_t);
+        if (alone_t) block_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
         __syncthreads();
         if (warp == 0) {
             if (do_p && m0 > 0) schur_apply<4>(s.px, nullptr, rows_dot_sum(part_p, 8), F.pSinv + (size_t)m0 * 16);
         } else if (warp == 2) {
-            if (do_t) {
+            if (do_t && !alone_t) {
                 if (T32)
                     warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
                 else
@@ -1505,7 +1576,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
             for (int n = tid; n < nc; n += nth) s.tx[n] = to_d2_bits(s.td[n]);
             __syncthreads();
         }
-        if (P.buoy_imp && pass == 0) temperature_corrections(P, F, s, m0, has_u, 0);
+        if (IMP && pass == 0) temperature_corrections<IMP>(P, F, s, m0, has_u, 0);
     }
 
     // 5. one refinement step of the streamfunction solve: r = f - L x (a second
@@ -1513,7 +1584,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
     //    With the FP32-refined temperature solve and explicit buoyancy the first
     //    temperature correction runs beside it: its chain (FP32, warps 2-3) beside
     //    the streamfunction chains (FP64), on disjoint arrays.
-    const bool fuse_t = T32 && !P.buoy_imp;
+    const bool fuse_t = T32 && !IMP;
     if (m0 > 0) {
         for (int q = 8 + tid; q < 2 * nc; q += nth) {
             const int k = q >> 1;
@@ -1532,9 +1603,9 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         if (lane < 8) flat(s.pf)[lane] = -t;  // read by the Schur step below, past the next barrier
     }
     if (fuse_t)
-        run_chains<RD, 2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), job_t(), no_job<double, 1>(), s.prevs);
+        run_chains<2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), job_t(), no_job<double, 1>(), s.prevs);
     else if (m0 > 0)
-        run_chains<RD, 2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), no_job<CT, 2>(), no_job<double, 1>(),
+        run_chains<2>(job_p(s.pf, s.pd, false), job_p(s.pf, s.pd, true), no_job<CT, 2>(), no_job<double, 1>(),
                           s.prevs);
     if (fuse_t) {
         if (warp == 2) warp_schur32_dir(s.td, s.tr, nc, P.ops.tau_dir_B32, F.tSinv32 + (size_t)m0 * 4);
@@ -1560,7 +1631,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
     if (fuse_t)
         for (int n = tid; n < nc; n += nth) s.tx[n] = cadd(s.tx[n], to_d2_bits(s.td[n]));
     __syncthreads();
-    if (!P.buoy_imp) temperature_corrections(P, F, s, m0, has_u, fuse_t ? 1 : 0);
+    if (!IMP) temperature_corrections<IMP>(P, F, s, m0, has_u, fuse_t ? 1 : 0);
 
     // 6. store, then mass / implicit operators for later stages
     for (int q = tid; q < 2 * nc; q += nth) {
@@ -1757,12 +1828,13 @@ __global__ void __launch_bounds__(NTHREADS_S) k_solve_dense(StepParams P, RhsSpe
 // CTA alone, first after the terms of f at that element have been read.  60 KB at
 // N_c = 1365 where five vectors a system took 109 KB (two CTAs).  Bound by FP64 (43%
 // of its rate) and the latency of the chains; with two CTAs an SM 3231 and 1005 us at
-// n_r x n_phi = 2049 x 6144 and 1025 x 3072, with three 2949 and 875.
+// n_r x n_phi = 2049 x 6144 and 1025 x 3072, with three 2949 and 875, 2834 and 770 in the
+// order above, 2505 and 688 with the slimmer steps of Walk.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t solve_roles_smem_bytes(int nc) {
     const size_t b = (size_t)chain_rows(nc);
-    const size_t psi = 2 * b * 16 + 4 * (size_t)ring_bytes<ddc>(RD);          // work vector, solution
-    const size_t th = 5 * b * 8 + 4 * (size_t)ring_bytes<double>(RD);         // solution, FP32 work vector, uf, ux
+    const size_t psi = 2 * b * 16 + 4 * (size_t)ring_bytes<ddc>();          // work vector, solution
+    const size_t th = 5 * b * 8 + 4 * (size_t)ring_bytes<double>();         // solution, FP32 work vector, uf, ux
     return psi > th ? psi : th;
 }
 
@@ -1818,11 +1890,11 @@ __global__ void __launch_bounds__(NTHREADS_S, 3) k_solve_roles(StepParams P, Rhs
             const int n0 = second ? nA : 0, n = second ? (F.psplit ? np - nA : 0) : F.psplit ? nA : np;
             V* v = reinterpret_cast<V*>(work + 4 + n0);
             return ChainJob<C, 2>{v, v, v, n, blk + (second ? (size_t)(nbp / 2) * 192 : 0), second ? 6 : 0,
-                                  ring + (second ? 2 * ring_bytes<C>(RD) : 0)};
+                                  ring + (second ? 2 * ring_bytes<C>() : 0)};
         };
         for (int it = 0; it < 2; ++it) {  // solve, then one refinement step
             double2* sol = it ? work : x;
-            run_chains<RD, 2>(job(false), job(true), no_job<float, 2>(), no_job<double, 1>(), prevs);
+            run_chains<2>(job(false), job(true), no_job<float, 2>(), no_job<double, 1>(), prevs);
             if constexpr (DDP) {
                 if (F.psplit)
                     split_join_dd(reinterpret_cast<ddc*>(work) + 4, np, nA, spk_dd,
@@ -1901,7 +1973,7 @@ __global__ void __launch_bounds__(NTHREADS_S, 3) k_solve_roles(StepParams P, Rhs
         temperature_corrections_roles(P, F, s, m);
     } else {
         double* v = flat(s.tx + 2);
-        run_chains<RD, 2>(no_job<double, 1>(), no_job<double, 1>(),
+        run_chains<2>(no_job<double, 1>(), no_job<double, 1>(),
                           ChainJob<double, 2>{v, v, v, nt, F.tBlk + (size_t)m * nbt * 192, 2, s.ring_t}, no_job<double, 1>(),
                           prevs);
         rows_dot_part<2>(s.tx + 2, nt, P.ops.tau_dir_B, part_s);
@@ -2228,25 +2300,24 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
     // small systems (N_c <= DENSE_NC): the dense inverses, 35 -> 16 us at N_c = 21.
     // Their operations and bytes grow as N_c^2: at N_c = 85 (n_r = 129) the applies
     // alone are 2300 FP64 instructions a warp and mode, 19 us of an SM's FP64 units for
-    // each mode on it, where the chains take 39 us for two.  The options that pick a
+    // each mode on it, where the chains take 35 us for two.  The options that pick a
     // form of the chains keep them.
     if (F.pInv && P.psi_dd < 0 && P.solve_roles <= 0 && !F.ir_t) {
         return launch_chained(k_solve_dense, slab_modes(P), NTHREADS_S, sizeof(double) * dense_smem_doubles(P.nc), st, P, rhs,
                               F, y_out, mass_out, imp_out, want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
     // double-float streamfunction chains with explicit buoyancy (option psi_chain_dd),
-    // by default from N_c > 64: with FP64 ones n_r = 129, 257, 513 took 47.6, 87.8, 335.5
-    // us where these took 45.4, 74.2, 279.3; below, the conversions cost more than the
-    // chains save
+    // by default from N_c > 64: by mode at 129 x 384 and 257 x 768 45.3 and 84.8 us with
+    // FP64 ones, 35.4 and 63.0 with these
     const bool ddp = !P.buoy_imp && F.pBlkDD && (P.psi_dd > 0 || (P.psi_dd < 0 && P.nc > 64));
     // With explicit buoyancy one CTA per system or one per mode.  N_c > 600 (an
     // FP32-refined temperature): per system.  Below, per system for up to a mode an SM,
     // whose two systems then run on two SMs, and from four modes an SM on, where three
     // CTAs of two vectors an SM beat two of seven; between, the modes fit one or two
     // passes of two CTAs an SM, the systems need part of another.  Solve, us, per mode /
-    // per system: n_r = 129, 257, 513 with 129 modes 38.5 / 35.9, 55.2 / 53.1, 88.0 / 76.3; with
-    // 257 modes 45.2 / 53.1, 69.9 / 79.9, 124.8 / 140.0; with 513 modes 92.3 / 98.2, 153.0 /
-    // 154.1, 257.1 / 248.4; with 1025 modes 186.8 / 151.9, 294.9 / 241.3, 520.7 / 404.6.  (By
+    // per system: n_r = 129, 257, 513 with 129 modes 35.4 / 34.2, 50.4 / 49.4, 78.8 / 71.9; with
+    // 257 modes 43.1 / 51.5, 63.0 / 75.6, 112.4 / 128.9; with 513 modes 86.3 / 92.4, 132.7 /
+    // 139.2, 233.4 / 224.9; with 1025 modes 173.3 / 141.3, 263.4 / 218.5, 461.4 / 369.1.  (By
     // the whole number of modes: a slab solves as the whole step does.)
     const int sms = 152;
     const bool per_system = P.nc > 600 || (P.nc > 64 && (P.M <= sms || P.M > 4 * sms));
@@ -2262,8 +2333,10 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
         return launch_chained(kern, 2 * slab_modes(P), NTHREADS_S, smr, st, P, rhs, F, y_out, mass_out, imp_out,
                               want_mass ? 1 : 0, want_imp ? 1 : 0);
     }
-    auto kern = F.ir_t ? (ddp ? k_solve<true, true> : k_solve<true, false>) : (ddp ? k_solve<false, true> : k_solve<false, false>);
-    const size_t sm = sizeof(double) * solve_smem_doubles(P.nc);
+    auto kern = P.buoy_imp ? (F.ir_t ? k_solve<true, false, true> : k_solve<false, false, true>)
+                : F.ir_t   ? (ddp ? k_solve<true, true, false> : k_solve<true, false, false>)
+                           : (ddp ? k_solve<false, true, false> : k_solve<false, false, false>);
+    const size_t sm = sizeof(double) * solve_smem_doubles(P.nc, F.ir_t && P.buoy_imp);
     // the epilogue reads the assembled right-hand sides from shared memory where
     // they fit (up to N_c ~ 1300), else sums the terms again
     int dev = 0, smax = 0;
