@@ -160,10 +160,12 @@ int pizza_init(pizza_ctx **out, int n_r, int n_phi, double E, double Ra,
  *   "solve_roles" with explicit buoyancy, the implicit solve in one CTA per
  *            system (streamfunction; temperature, then the zonal flow for m = 0)
  *            instead of one per mode: 1 always, 0 never, -1 (default) from
- *            N_c > 600, and from N_c > 64 with at most 152 or more than 608 modes.  The same operations but
- *            for the order of some sums: results agree to the accuracy of the
- *            refined solve.  1 also keeps the block chains where N_c <= 42, whose
- *            default is a dense inverse of each system with one refinement;
+ *            N_c > 600, and from N_c > 64 with at most as many modes as the device
+ *            has multiprocessors (152) or more than four times as many.  The same
+ *            operations but for the order of some sums: results agree to the
+ *            accuracy of the refined solve.  1 also keeps the block chains where
+ *            N_c <= 42, whose default is a dense inverse of each system with one
+ *            refinement;
  *   "psi_chain_dd" the block chains of the streamfunction solve (Appendix
  *            A's banded block) in double-float arithmetic on the FP32 pipe
  *            (about 48 significant bits; the Schur step, residual and refinement

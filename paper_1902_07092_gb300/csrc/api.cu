@@ -1489,6 +1489,10 @@ int pizza_init(pizza_ctx** out, int n_r, int n_phi, double E, double Ra, double 
 
     Geom g = make_geom(radius_ratio);
     StepParams& P = ctx->P;
+    if (cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
+        ctx->err = "cudaDeviceGetAttribute failed";
+        return bail(PIZZA_ECUDA);
+    }
     P.n_r = n_r;
     P.n_phi = n_phi;
     P.n_m = ctx->n_m;

@@ -2319,8 +2319,7 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
     // 257 modes 43.1 / 51.5, 63.0 / 75.6, 112.4 / 128.9; with 513 modes 86.3 / 92.4, 132.7 /
     // 139.2, 233.4 / 224.9; with 1025 modes 173.3 / 141.3, 263.4 / 218.5, 461.4 / 369.1.  (By
     // the whole number of modes: a slab solves as the whole step does.)
-    const int sms = 152;
-    const bool per_system = P.nc > 600 || (P.nc > 64 && (P.M <= sms || P.M > 4 * sms));
+    const bool per_system = P.nc > 600 || (P.nc > 64 && (P.M <= P.sms || P.M > 4 * P.sms));
     if (!P.buoy_imp && (P.solve_roles > 0 || (P.solve_roles < 0 && per_system))) {
         const size_t smr = solve_roles_smem_bytes(P.nc);
         auto kern = ddp ? k_solve_roles<true> : k_solve_roles<false>;

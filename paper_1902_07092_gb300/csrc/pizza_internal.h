@@ -160,8 +160,10 @@ struct StepParams {
     // azimuthal kernel folds max |u_s|/ds_k and max |u_phi|/(s_k dphi) of the
     // synthesised state into cfl_max[0], cfl_max[1] (atomic maxima)
     // the solve with explicit buoyancy in one CTA per system instead of one per
-    // mode (option "solve_roles"): 1 always, 0 never, -1 (default) from N_c > 600
+    // mode (option "solve_roles"): 1 always, 0 never, -1 (default) from N_c > 600, and from
+    // N_c > 64 with at most sms or more than 4 sms modes
     int solve_roles;
+    int sms;  // multiprocessors of the device (152)
     // FP64 radial kernels in the three-array layout (option "radial_lean"):
     // 1 from n_r = 129 (the half-length DCT-I), 0 never, -1 (default) from n_r = 1025
     int radial_lean;
