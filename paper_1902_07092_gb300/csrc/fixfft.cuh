@@ -262,47 +262,20 @@ FX_HD unsigned fx_schedule(int lg, bool three, int l1, int& S) {
     return back;
 }
 
-// v 2^(FX_BITS - e) rounded, for |v| < 2^e with e = emax - 1022 given through the
-// biased exponent emax of the block maximum; zero for emax = 0 (a zero or
-// subnormal block) or a subnormal v.
-FX_HD fx64 fx_from_bits(unsigned long long u, int emax) {
-    const int E = (int)(u >> 52) & 0x7ff;
-    // mantissa (53 bits) shifted left by 8, then right by n = emax - E + 1 with rounding
-    const int n = emax - E;  // >= 0
-    const unsigned long long m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 8;
-    if (E == 0 || n > 62) return 0;
-    const fx64 r = (fx64)(((m >> n) + 1) >> 1);
-    return (u >> 63) ? -r : r;
-}
-// a 2^ex as a double, rounded to nearest (ties away from zero); 0 below the
-// normal range, infinity above it
-FX_HD unsigned long long fx_to_bits(fx64 a, int ex) {
-    const unsigned long long s = (unsigned long long)a & 0x8000000000000000ull;
-    unsigned long long m = s ? 0ull - (unsigned long long)a : (unsigned long long)a;
-    if (m == 0) return s;
-#ifdef __CUDA_ARCH__
-    const int lz = __clzll((long long)m);
-#else
-    const int lz = __builtin_clzll(m);
-#endif
-    m <<= lz;
-    const int E = 1023 + 63 - lz + ex;  // biased exponent of the leading bit
-    if (E <= 0) return s;
-    if (E >= 2047) return s | 0x7ff0000000000000ull;
-    return s | (((unsigned long long)(E - 1) << 52) + ((m >> 11) + ((m >> 10) & 1)));
-}
-
 #ifdef __CUDACC__
-// The same on the device: the exponent moves on the integer pipe, the conversion
-// itself issues once on the FP64 pipe (64 cycles of a sub-partition, against 24 and
-// 40 integer instructions for the forms above, which the tests compare them with).
+// v 2^(FX_BITS - e) rounded, for |v| < 2^e with e = emax - 1022 given through the
+// biased exponent emax of the block maximum; zero for emax = 0 (a zero or subnormal
+// block) or a subnormal v.  The exponent moves on the integer pipe; the conversion
+// issues once on the FP64 pipe (64 cycles of a sub-partition, against about 24 integer
+// instructions, and 40 for fx_to).
 __device__ __forceinline__ fx64 fx_from(double v, int emax) {
     const int h = __double2hiint(v), s = FX_BITS + 1022 - emax;
     const int E = (h >> 20) & 0x7ff;
     const fx64 r = __double2ll_rn(__hiloint2double(h + (s << 20), __double2loint(v)));
     return (E == 0 || E + s <= 0) ? 0 : r;
 }
-// emax = 0x7ff (an infinity or NaN in the block): NaN
+// a 2^ex as a double, rounded to nearest; 0 below the normal range, infinity above it;
+// NaN for a bad block (an infinity or NaN in it)
 __device__ __forceinline__ double fx_to(fx64 a, int ex, bool bad) {
     const double d = __ll2double_rn(a);
     int h = __double2hiint(d);
