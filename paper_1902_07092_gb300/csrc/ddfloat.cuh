@@ -1,21 +1,14 @@
-// Double-float arithmetic on the FP32 pipe: a value is the unevaluated sum
-// hi + lo of two floats with |lo| <= ulp(hi)/2, about 48 significant bits.
-// On GB300 the FP32 pipe issues 64 times the FP64 rate, so FP64-accurate
-// transforms whose cost is FP64 issue run faster in this form.
+// Double-float values for the FP32 pipe: a value is the unevaluated sum hi + lo of two
+// floats with |lo| <= ulp(hi)/2, about 48 significant bits.  GB300 issues FP32 64
+// times as fast as FP64, so the block chains of the streamfunction solve, strings of
+// dependent sums that an FP64 refinement follows, run in this form (their sums are
+// beside them, in k_implicit.cu); here are the type and its conversions.
 //
-// Error-free transformations used (published methods):
-//   two-sum (Knuth, TAOCP vol. 2, 4.2.2):   s = a + b,  e = (a - (s - bb)) + (b - bb),
-//                                           bb = s - a;  a + b = s + e exactly;
-//   fast two-sum (Dekker 1971), |a| >= |b|: s = a + b,  e = b - (s - a);
-//   two-product with a fused multiply-add:  p = a b,  e = fma(a, b, -p).
-// Sums use one two-sum of the leading parts plus the trailing parts ("sloppy"
-// addition): its error is bounded relative to |a| + |b|, which is the bound the
-// error analysis of an FFT needs.  Products add the cross terms hi*lo to the
-// two-product's error before the final renormalisation.
+// Error-free transformation used (fast two-sum, Dekker 1971), |a| >= |b|:
+// s = a + b,  e = b - (s - a),  a + b = s + e exactly.
 // Range: that of float (|x| < 3.4e38; below ~1e-38 the trailing part loses bits).
-// The primitives use the _rn intrinsics, which the compiler never contracts
-// into fused multiply-adds: the transformations rely on each operation being
-// rounded on its own.
+// The _rn intrinsics are never contracted into fused multiply-adds: the
+// transformation relies on each operation being rounded on its own.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -32,48 +25,8 @@ __device__ __forceinline__ ddf dd_renorm(float s, float e) {
     const float h = __fadd_rn(s, e);
     return ddf{h, __fsub_rn(e, __fsub_rn(h, s))};
 }
-__device__ __forceinline__ ddf operator+(ddf a, ddf b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    const float bb = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-    return dd_renorm(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
-}
-__device__ __forceinline__ ddf operator-(ddf a) { return ddf{-a.hi, -a.lo}; }
-__device__ __forceinline__ ddf operator-(ddf a, ddf b) { return a + (-b); }
-__device__ __forceinline__ ddf operator*(ddf a, ddf b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e));
-    return dd_renorm(p, e);
-}
-// multiplication by an exact power of two (or any float whose products are exact)
-__device__ __forceinline__ ddf dd_scale2(ddf a, float s) { return ddf{__fmul_rn(a.hi, s), __fmul_rn(a.lo, s)}; }
-
-__device__ __forceinline__ ddf fmat(ddf a, ddf b, ddf c) { return a * b + c; }
-
-// conversions: the nearest float and the float nearest the remainder
-__device__ __forceinline__ ddf dd_from(double v) {
-    const float h = __double2float_rn(v);
-    return ddf{h, __double2float_rn(v - (double)h)};
-}
-__device__ __forceinline__ double dd_to(ddf a) { return (double)a.hi + (double)a.lo; }
-
-// complex double-float
-__device__ __forceinline__ ddc cadd(ddc a, ddc b) { return ddc{a.x + b.x, a.y + b.y}; }
-__device__ __forceinline__ ddc csub(ddc a, ddc b) { return ddc{a.x - b.x, a.y - b.y}; }
-__device__ __forceinline__ ddc cscale(ddc a, ddf s) { return ddc{a.x * s, a.y * s}; }
-__device__ __forceinline__ ddc cmul(ddc a, ddc b) { return ddc{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
-__device__ __forceinline__ ddc cfma(ddc w, ddc b, ddc a) { return cadd(a, cmul(w, b)); }  // a + w b
-__device__ __forceinline__ ddc creflect(ddc a, ddc s) {                                 // 2a - s
-    return ddc{dd_scale2(a.x, 2.f) - s.x, dd_scale2(a.y, 2.f) - s.y};
-}
-__device__ __forceinline__ ddc dd_from(double2 v) { return ddc{dd_from(v.x), dd_from(v.y)}; }
-__device__ __forceinline__ double2 dd_to(ddc a) { return make_double2(dd_to(a.x), dd_to(a.y)); }
-
-// The same conversions taken apart on the IEEE 754 fields with integer and FP32
-// instructions.  On GB300 a conversion between float and double issues on the
-// FP64 unit (2 per clock per SM), which made the conversions of a transform's
-// inputs and outputs cost as much as a quarter of its time.
+// Conversions taken apart on the IEEE 754 fields with integer and FP32 instructions: on
+// GB300 one between float and double issues on the FP64 unit (2 per clock per SM).
 //
 // v = (-1)^s 1.f 2^e (52 fraction bits f) splits into h = the first 24
 // significant bits (truncated) and the remainder r 2^(e-52), r = the low 29 bits
@@ -96,7 +49,6 @@ __device__ __forceinline__ ddf dd_from_bits(double v) {
     const float l = __fmul_rn(rf, __uint_as_float((unsigned)E << 23));          // times 2^e
     return dd_renorm(h, __uint_as_float(__float_as_uint(l) ^ sign));
 }
-__device__ __forceinline__ ddc dd_from_bits(double2 v) { return ddc{dd_from_bits(v.x), dd_from_bits(v.y)}; }
 
 // a float as the double of the same value (exact); subnormal floats give zero
 __device__ __forceinline__ double f2d_bits(float f) {
@@ -125,7 +77,6 @@ __device__ __forceinline__ float f32_from_bits(double v) {
 
 // hi + lo rounded to double: one FP64 add
 __device__ __forceinline__ double dd_to_bits(ddf a) { return f2d_bits(a.hi) + f2d_bits(a.lo); }
-__device__ __forceinline__ double2 dd_to_bits(ddc a) { return make_double2(dd_to_bits(a.x), dd_to_bits(a.y)); }
 
 // hi + lo as a double with integer instructions only.  hi widened to double
 // leaves 29 zero fraction bits below its 24; a renormalised lo (|lo| <= ulp(hi)/2,
@@ -150,14 +101,5 @@ __device__ __forceinline__ double dd_compose(ddf a) {
         H |= L;
     return __longlong_as_double((long long)(H | ((unsigned long long)(hb & 0x80000000u) << 32)));
 }
-__device__ __forceinline__ double2 dd_compose(ddc a) { return make_double2(dd_compose(a.x), dd_compose(a.y)); }
-
-// a double-float times a float (two-product of the leading parts plus lo b)
-__device__ __forceinline__ ddf dd_mulf(ddf a, float b) {
-    const float p = __fmul_rn(a.hi, b);
-    return dd_renorm(p, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p)));
-}
-// i t a for a complex double-float a and a float t
-__device__ __forceinline__ ddc cmul_if(ddc a, float t) { return ddc{-dd_mulf(a.y, t), dd_mulf(a.x, t)}; }
 
 }  // namespace pz
