@@ -38,9 +38,10 @@ constexpr size_t NA_TAB_GRID = na_round(3 * (size_t)NA_MAX_NR);
 constexpr size_t NA_TAB_TWR = na_round(2 * 2 * (size_t)(NA_MAX_NR - 1));
 constexpr size_t NA_TAB_TWP = na_round(2 * (size_t)NA_MAX_NPHI);
 constexpr size_t NA_TAB_TW = NA_TAB_TWR + NA_TAB_TWP;
-// the fixed-point twiddles of both lengths (int4) after the bands
+// the radial transforms' fixed-point twiddles (int4) after the bands; the azimuthal ones
+// run in FP64 here
 constexpr size_t NA_TAB_BAND = na_round(na_band_total());
-constexpr size_t NA_TABLES = NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND + NA_TAB_TW;
+constexpr size_t NA_TABLES = NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND + NA_TAB_TWR;
 static_assert(NA_TAB_GRID % 2 == 0 && NA_TAB_TWR % 2 == 0, "double2 tables must be 16-byte aligned");
 
 static __device__ __align__(256) double2 g_scratch[2 * NA_GRID];
@@ -110,10 +111,8 @@ int na_setup(int dev, int n_r, int n_phi, double eta, cudaStream_t st, DeviceSlo
             std::memcpy(&host[off], b.data(), b.size() * sizeof(double));
             off += (size_t)NA_MAX_NC * NA_WIDTH[id];
         }
-        const auto fxr = fft_twiddles_fx(2 * (n_r - 1)), fxp = fft_twiddles_fx(n_phi);
-        const size_t ofx = NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND;
-        std::memcpy(&host[ofx], fxr.data(), fxr.size() * sizeof(int4));
-        std::memcpy(&host[ofx + NA_TAB_TWR], fxp.data(), fxp.size() * sizeof(int4));
+        const auto fxr = fft_twiddles_fx(2 * (n_r - 1));
+        std::memcpy(&host[NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND], fxr.data(), fxr.size() * sizeof(int4));
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return na_fail(PIZZA_ECUDA, cudaGetErrorString(e));
         e = cudaMemcpyAsync(sl.tables, host.data(), NA_TABLES * sizeof(double), cudaMemcpyHostToDevice, st);
@@ -188,10 +187,8 @@ extern "C" int pizza_explicit_terms_noalloc(int n_r, int n_phi, double Ra, doubl
         P.ops.band[id] = sl->tables + off;
         off += (size_t)NA_MAX_NC * NA_WIDTH[id];
     }
-    const double* fx = sl->tables + NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND;
-    P.fx_r = reinterpret_cast<const int4*>(fx);
+    P.fx_r = reinterpret_cast<const int4*>(sl->tables + NA_TAB_GRID + NA_TAB_TW + NA_TAB_BAND);
     P.radial_dd = -1;  // as by default
-    P.fx_p = reinterpret_cast<const int4*>(fx + NA_TAB_TWR);
     P.ops.tau_psi_B = nullptr;  // the explicit stage uses no tau rows
     P.ops.tau_dir_B = nullptr;
 
