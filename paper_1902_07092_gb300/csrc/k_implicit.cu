@@ -915,8 +915,7 @@ __device__ void apply_row(const StepParams& P, int m, int k, const double2* xp, 
 // same terms in the same order).
 __device__ void epilogue_row(const StepParams& P, const RhsSpec& R, double gdt, int m, int k, const double2* xp,
                              const double2* xt, const double* xu, VecSet mass_out, VecSet imp_out, bool want_mass,
-                             bool want_imp, const double2* fps = nullptr, const double2* fts = nullptr,
-                             const double* fus = nullptr) {
+                             bool want_imp) {
     const int nc = P.nc;
     const double mu = (double)m * m;
     double2 mp = make_double2(0.0, 0.0), mt = make_double2(0.0, 0.0);
@@ -948,12 +947,7 @@ __device__ void epilogue_row(const StepParams& P, const RhsSpec& R, double gdt, 
     if (want_imp) {  // before any store: an output may be one of the terms of f
         double2 fp = make_double2(0.0, 0.0), ft = make_double2(0.0, 0.0);
         double fu = 0.0;
-        if (fps) {  // kept by the caller (the same sums)
-            fp = fps[k];
-            ft = fts[k];
-            if (m == 0) fu = fus[k];
-        }
-        for (int t = 0; t < (fps ? 0 : R.nterms); ++t) {
+        for (int t = 0; t < R.nterms; ++t) {
             const double c = R.t[t].c;
             const double2 vp = R.t[t].v.psi[idx];
             const double2 vt = R.t[t].v.th[idx];
@@ -1180,8 +1174,7 @@ struct SolveSmem {
     char *ring_p, *ring_t, *ring_u;  // the walks' rings of matrices (the zonal flow's over the streamfunction's)
     double (*prevs)[32];             // the walking warps' previous blocks
     // the streamfunction and zonal-flow right-hand sides as assembled (pf and uf
-    // become residuals), for the epilogue; past the end of solve_smem_doubles,
-    // present when the launch adds keep_f_doubles
+    // become residuals), for the epilogue
     double2* fp;
     double* fu;
 };
@@ -1195,10 +1188,9 @@ __host__ __device__ inline int chain_rows(int nc) { return round8(nc) + 8; }
 // done with before it is formed when the buoyancy is implicit: two CTAs on an SM
 // instead of one at N_c = 682 (solve at 1025 x 1536 1100 -> 788 us)
 __host__ __device__ inline size_t solve_smem_doubles(int nc, bool shared_d) {
-    return (size_t)(shared_d ? 12 : 14) * chain_rows(nc) + (4 * ring_bytes<double2>() + 2 * ring_bytes<double>()) / 8;
+    return (size_t)(shared_d ? 12 : 14) * chain_rows(nc) + (4 * ring_bytes<double2>() + 2 * ring_bytes<double>()) / 8 +
+           3 * (size_t)round8(nc);  // (208 KB at N_c = 1365, the largest)
 }
-
-__host__ __device__ inline size_t keep_f_doubles(int nc) { return 3 * (size_t)round8(nc); }
 
 __device__ __forceinline__ SolveSmem carve(double2* base, int nc, bool shared_d) {
     SolveSmem s;
@@ -1405,7 +1397,7 @@ __device__ __forceinline__ void temperature_corrections(const StepParams& P, con
 template <bool T32, bool DDP, bool IMP>
 __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R, DevFactors F, VecSet y_out,
                                                       VecSet mass_out, VecSet imp_out, int want_mass,
-                                                      int want_imp, int keep_f) {
+                                                      int want_imp) {
     chain_wait();
     extern __shared__ double2 sm[];
     __shared__ double part_p[NTHREADS_S / 32][8], part_t[NTHREADS_S / 32][8];
@@ -1479,10 +1471,8 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         flat(s.tf)[q] = at;
         if (T32) reinterpret_cast<float*>(s.tr)[q] = f32_from_bits(at);
         if (has_u && part == 0) s.uf[n] = (n < 2) ? 0.0 : au;
-        if (keep_f) {  // for the epilogue: pf and uf become residuals
-            flat(s.fp)[q] = ap;
-            if (has_u && part == 0) s.fu[n] = s.uf[n];
-        }
+        flat(s.fp)[q] = ap;  // for the epilogue: pf and uf become residuals
+        if (has_u && part == 0) s.fu[n] = s.uf[n];
     }
     __syncthreads();
 
@@ -1643,10 +1633,10 @@ __global__ void __launch_bounds__(NTHREADS_S, 2) k_solve(StepParams P, RhsSpec R
         for (int q = tid; q < 4 * nc; q += nth) {
             if (q < 2 * nc)
                 epilogue_psi_part(P, R, F.gdt, m0, q >> 1, part, s.px, mass_out, imp_out, want_mass, want_imp,
-                                  keep_f ? s.fp : nullptr);
+                                  s.fp);
             else
                 epilogue_theta_part(P, R, F.gdt, m0, (q - 2 * nc) >> 1, part, s.tx, s.ux, mass_out, imp_out, want_mass,
-                                    want_imp, s.tf, keep_f ? s.fu : nullptr);
+                                    want_imp, s.tf, s.fu);
         }
 }
 
@@ -2336,21 +2326,10 @@ cudaError_t launch_solve(const StepParams& P, const RhsSpec& rhs, const DevFacto
                 : F.ir_t   ? (ddp ? k_solve<true, true, false> : k_solve<true, false, false>)
                            : (ddp ? k_solve<false, true, false> : k_solve<false, false, false>);
     const size_t sm = sizeof(double) * solve_smem_doubles(P.nc, F.ir_t && P.buoy_imp);
-    // the epilogue reads the assembled right-hand sides from shared memory where
-    // they fit (up to N_c ~ 1300), else sums the terms again
-    int dev = 0, smax = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
-    cudaFuncAttributes fa;
-    err = cudaFuncGetAttributes(&fa, kern);
-    if (err != cudaSuccess) return err;
-    const size_t smk = sm + sizeof(double) * keep_f_doubles(P.nc);
-    const int keep = smk + fa.sharedSizeBytes <= (size_t)smax ? 1 : 0;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(keep ? smk : sm));
-    if (err != cudaSuccess) return err;
-    return launch_chained(kern, slab_modes(P), NTHREADS_S, keep ? smk : sm, st, P, rhs, F, y_out, mass_out, imp_out,
-                          want_mass ? 1 : 0, want_imp ? 1 : 0, keep);
+    return launch_chained(kern, slab_modes(P), NTHREADS_S, sm, st, P, rhs, F, y_out, mass_out, imp_out, want_mass ? 1 : 0,
+                          want_imp ? 1 : 0);
 }
 
 // acc[0] += sum_n w_n Re theta_hat_0n = Nu - 1 of the state (one warp, a fixed
