@@ -82,7 +82,7 @@ FX_HD fxc fx_sub(fxc a, fxc b) { return fxc{a.x - b.x, a.y - b.y}; }
 // unbiased roundings cancel: a derivative from 2049 grid values comes out 2.7e-11 wrong
 // rounding down, 7.2e-12 with halves up, 2.3e-12 unbiased (7.0e-12 in FP64).  The radial
 // transforms round so (RND); the azimuthal ones, whose spectra no sum differentiates,
-// shift down (1 % of a step less; no worse than FP64 either).
+// shift down (no worse than FP64 either; rounding there too, a step took 0.3 to 0.6 % more).
 // a 2^-s to nearest, halves to even (s >= 1)
 FX_HD fx64 fx_shr(fx64 a, int s) { return (a + ((((fx64)1 << (s - 1)) - 1) + ((a >> s) & 1))) >> s; }
 // a/2 and (a + b)/2, a half to the odd neighbour: one instruction beside the shift

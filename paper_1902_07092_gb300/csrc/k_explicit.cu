@@ -696,9 +696,9 @@ __device__ __forceinline__ void cheb_derivative_part(const double2* c, double2* 
 }
 
 // K1 of the FP64 stage in the batched layout: the equations of k_spec_to_grid with
-// the DCT-I in fixed point.  Bound by the latency of its phases (45 % of the issue
-// slots, 30 % of the FP64 pipe busy at 257 x 768, where the FP64 transforms kept
-// that pipe 60 % busy): 50 -> 25.6 us there, 23 -> 14.9 us at 129 x 384, 67 -> 36 us
+// the DCT-I in fixed point.  Bound by the latency of its phases (39 % of the issue
+// slots, 42 % of the FP64 pipe's at 257 x 768, where the FP64 transforms kept
+// that pipe 60 % busy): 50 -> 24.8 us there, 23 -> 14.8 us at 129 x 384, 67 -> 35 us
 // at 513 x 384 (against the double-float lean layout it replaces at that size).
 __global__ void __launch_bounds__(NTHREADS_FX, 2) k_spec_to_grid_fx(StepParams P, VecSet y, double2* __restrict__ G1,
                                                                    double2* __restrict__ W) {
@@ -830,8 +830,8 @@ __device__ __forceinline__ double band_part(const double* __restrict__ band, con
 // the DCT-I in fixed point, the buoyancy added to N_omega_hat before the one C^I
 // apply (Eq. psi_int applies C^I to their sum), and the banded applies spread
 // over (row, component, operator) so that every warp issues FP64.  257 x 768:
-// 75 -> 43 us (FP64 pipe 66 -> 38 % busy), 129 x 384: 43 -> 24.5, 513 x 384: 114 -> 49 us
-// (from the double-float lean layout).
+// 75 -> 43 us (50 % of the FP64 pipe's slots, 33 % of the issue slots), 129 x 384: 43 ->
+// 24.0, 513 x 384: 114 -> 49 us (from the double-float lean layout).
 // Vectors 0, 1: F1, F2 (to coefficients); 2, 3: their derivatives (to the grid);
 // 4, 5: N_omega (N_u), N_theta (to coefficients).
 __global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P, const double2* G2,
@@ -987,10 +987,11 @@ __global__ void __launch_bounds__(NTHREADS_FX, 2) k_grid_to_spec_fx(StepParams P
 // coefficient on load; the physical values of each field are shifted up by the
 // free leading bits of their largest before the products, whose 60-bit results
 // are transformed back.  FP64 is used for conversions only.  The means of the
-// products (m = 0), which cancel, are summed over the modes in FP64.  Bound by
-// instruction issue (43-54 % of the slots; 16 warps an SM at n_phi = 6144, where
-// two buffers fill its shared memory).  Against the double-float kernel: 257 x 768 37 -> 24.4 us, 33 x 96 22 -> 12.2, 1025 x 3072
-// 443 -> 313, 2049 x 6144 1706 -> 1265 us.
+// products (m = 0), which cancel, are summed over the modes in FP64 (13 us of 327 at
+// 1025 x 3072, 100 of 1363 at 2049 x 6144).  Bound by instruction issue (43 to 49 % of
+// the slots at 257 x 768 .. 1025 x 1536; 16 warps an SM at n_phi = 6144, where two buffers
+// fill its shared memory).  Against the double-float kernel: 257 x 768 37 -> 26.8 us, 33 x
+// 96 22 -> 12.2, 1025 x 3072 443 -> 334, 2049 x 6144 1706 -> 1364 us.
 // ---------------------------------------------------------------------------
 constexpr int PHI_SUMS = 12;
 struct PhiScale {
@@ -1095,8 +1096,10 @@ __device__ void cfl_rates_fx(const StepParams& P, const fxc* R, int k, int sv, i
 
 // PAIR: both packed pairs in one batched transform each way (buffers of 2 n_phi
 // points each); else one after the other, the first pair's physical values
-// and the second products waiting in registers.
-template <bool PAIR>
+// and the second products waiting in registers.  MANY: several modes a lane in the means'
+// sums, read ahead (1025 x 3072 334 us, 340 without); with a mode or two the longer code
+// alone costs 1 us (65 x 192 12.4 -> 13.6, 257 x 768 26.7 -> 28.1).
+template <bool PAIR, bool MANY>
 __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParams P, const double2* G1,
                                                             double2* __restrict__ G2) {
     chain_wait();
@@ -1124,9 +1127,9 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
         // 1536 as with one sum a warp, 85.7 with sixteen.)
         unsigned ex[4] = {0u, 0u, 0u, 0u};
         const int lane = tid & 31;
-        for (int w = tid >> 5; w < PHI_SUMS; w += nth >> 5) {
+        for (int w = tid >> 5; w < PHI_SUMS && 32 * w <= n_m; w += nth >> 5) {
             double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
+#pragma unroll (MANY ? 4 : 1)
             for (int m = 32 * w + lane; m <= n_m; m += 32 * PHI_SUMS) {
                 double2 f[4];
 #pragma unroll
@@ -1140,21 +1143,19 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
                     acc[q] = m ? fma(a.x, b.x, fma(a.y, b.y, acc[q])) : 0.5 * (a.x * b.x);
                 }
             }
-            if (32 * w <= n_m) {
-                // four sums over the warp: halves exchanged twice, then lanes of equal l >> 3 added up
+            // four sums over the warp: halves exchanged twice, then lanes of equal l >> 3 added up
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const int o = 16 >> s, half = 2 >> s;
-                    const bool up = lane & o;
+            for (int s = 0; s < 2; ++s) {
+                const int o = 16 >> s, half = 2 >> s;
+                const bool up = lane & o;
 #pragma unroll
-                    for (int i = 0; i < half; ++i) {
-                        const double send = up ? acc[i] : acc[i + half];
-                        acc[i] = (up ? acc[i + half] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
-                    }
+                for (int i = 0; i < half; ++i) {
+                    const double send = up ? acc[i] : acc[i + half];
+                    acc[i] = (up ? acc[i + half] : acc[i]) + __shfl_xor_sync(0xffffffffu, send, o);
                 }
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
             }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
             if ((lane & 7) == 0) sc.mean[w][lane >> 3] = acc[0];
         }
 #pragma unroll
@@ -1166,7 +1167,8 @@ __global__ void __launch_bounds__(512, PAIR ? 2 : 1) k_phi_products_fx(StepParam
     __syncthreads();
     if (tid >= nth - 32) {  // one warp: lane 4 w + q adds partial sums w and w + 8 of product q
         const int q = tid & 3, w = (tid & 31) >> 2;
-        double v = sc.mean[w][q] + (w + 8 < PHI_SUMS ? sc.mean[w + 8][q] : 0.0);
+        const int ns = min(PHI_SUMS, n_m / 32 + 1);
+        double v = (w < ns ? sc.mean[w][q] : 0.0) + (w + 8 < ns ? sc.mean[w + 8][q] : 0.0);
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (w == 0) sc.mean0[q] = 2.0 * v;
@@ -1843,9 +1845,10 @@ __global__ void __launch_bounds__(NTHREADS_R, lean_ctas<T>()) k_grid_to_spec_lea
 // n_r = 1025): two buffers of K fixed-point entries and one array of n_r FP64 values
 // (98 KB at n_r = 2049: two CTAs of 512 threads share an SM), the vectors of a mode
 // one after another through a half-length DCT-I.  Against double-float transforms
-// in the same layout: 1025 x 3072 343 -> 310 (a1) and 581 -> 433 us (a3), 2049 x 6144
-// 1124 -> 1090 and 1607 -> 1594 us, with roundings about 2^5 smaller; from n_r = 1025,
-// since at 513 the batched layout is faster (a1 52 -> 36, a3 90 -> 49 us at 513 x 384).
+// in the same layout: 1025 x 3072 343 -> 263 (a1) and 581 -> 440 us (a3), 2049 x 6144
+// 1124 -> 889 and 1607 -> 1633 us (1598 with shifts that round down); the derivative of
+// 2049 grid values 1.4e-7 -> 4e-9 off (1.3e-9 by the FP64 transform of this form); from n_r =
+// 1025, since at 513 the batched layout is faster (a1 52 -> 35, a3 90 -> 49 us at 513 x 384).
 // ---------------------------------------------------------------------------
 constexpr int NTHREADS_LX = 512;
 
@@ -2323,7 +2326,8 @@ cudaError_t launch_phi_products(const StepParams& P, const double2* G1, double2*
         const int pair = phi_pair(P, err);
         if (err != cudaSuccess) return err;
         const size_t sm = (pair ? 2 : 1) * smem_phi_products(P);
-        auto kern = pair ? k_phi_products_fx<true> : k_phi_products_fx<false>;
+        auto kern = !pair ? k_phi_products_fx<false, true>
+                    : P.n_m < 768 ? k_phi_products_fx<true, false> : k_phi_products_fx<true, true>;
         err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (err != cudaSuccess) return err;
         return launch_chained(kern, slab_radii(P), nth, sm, st, P, G1, G2);
