@@ -106,6 +106,12 @@ def algorithmic_flops(n_r, n_phi, scheme, radial="integration"):
 # DRAM bytes (read + write) per launch of the roofline kernel from one ncu capture
 # of this workload (summaries under profiles/); null for kernels not captured.
 NCU_TRAFFIC = {
+    # (the mean of the four stages' solves)
+    ("sparse_n257_p768", "solve"): (47.11e6 + 0.001e6, "profiles/imex_step_kernels_n257_p768.md"),
+    ("large_n2049_p6144", "solve"): (6161.6e6 + 312.8e6, "profiles/imex_step_kernels_n2049_p6144.md"),
+    ("large_n2049_p6144", "spec_to_grid"): (97.8e6 + 351.8e6, "profiles/imex_step_kernels_n2049_p6144.md"),
+    ("large_n2049_p6144", "phi_products"): (269.0e6 + 223.3e6, "profiles/imex_step_kernels_n2049_p6144.md"),
+    ("large_n2049_p6144", "grid_to_spec"): (360.1e6 + 72.4e6, "profiles/imex_step_kernels_n2049_p6144.md"),
     ("coll_n257_p768", "solve"): (735.4e6 + 6.9e6, "profiles/collocation_step_kernels_n257_p768.md"),
     ("galerkin_n257_p768", "solve"): (34.58e6 + 0.003e6, "profiles/galerkin_step_kernels_n257_p768.md"),
 }
@@ -283,7 +289,7 @@ def precision_label(wl):
     parts = ["fp64: state, history, stored grid values, field arithmetic at each radius, linear couplings, banded "
              "applies, Schur steps, residuals and refinements in FP64",
              "azimuthal FFTs and products in fixed point with the m = 0 means of the products in FP64"]
-    if wl.get("radial", "integration") == "integration":
+    if wl.get("radial", "integration") != "collocation":
         parts.append("radial DCT-I in fixed point")
     if wl.get("radial", "integration") == "integration" and nc > 64:
         parts.append("block chains of the streamfunction solve in double-float (N_c > 64)")
